@@ -65,7 +65,7 @@ struct sparsk_ctx {
     float2 *rope;
     StepDesc sd;
     int *staged, *tok_dev, *out_tok_dev, *out_depth_dev;
-    int *pf_slot, *pf_pos, *pf_grp_row0, *pf_grp_nrows, *pf_ngrp, *pf_nrows;
+    int *pf_rows;                // row set of a prefill pass, laid out as it is staged (see sparsk_prefill)
     float *h_lo, *h_up;
     float *qbuf;
     float *h_last, *q_last;      // the current rows alone, for the trimmed last layer of the upper pass
@@ -179,12 +179,22 @@ bool dims_ok(const sparsk_dims *d)
     return true;
 }
 
+// Rows of a prefill pass when the caller leaves the choice to the library.  A pass streams every
+// layer's weights once whatever its rows, so it wants as many as one block of the tcgen05 GEMMs
+// takes: a layer of the 40-layer shape takes 153 us at 64 rows and 280 at 256, less than half
+// the time per token (first token after 1,024: 101.6 ms with passes of 64, 49.5 ms with 256).
+// More rows would be a second block, which streams the weights again.
+constexpr int PREFILL_ROWS = GM_MAX_N;
 int cap_rows_of(const sparsk_dims *d)
 {
-    const int pf = d->prefill_rows > 0 ? d->prefill_rows : 64;
+    const int pf = d->prefill_rows > 0 ? d->prefill_rows : PREFILL_ROWS;
     const long dec = (long)d->max_seqs * (d->max_pending + 1);
     return (int)std::max<long>(dec, pf);
 }
+
+// Ints that describe a prefill pass: slot, position and token index of every row, first row and
+// row count of every group (one per prompt that takes part), the two counts.
+size_t prefill_ints(const sparsk_dims *d) { return 3 * (size_t)cap_rows_of(d) + 2 * (size_t)d->max_seqs + 2; }
 
 // Lays the workspace out; with base == NULL only measures it.
 size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
@@ -208,8 +218,7 @@ size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
     sd.counts = w.take<int>(8);
     sd.argmax = w.take<unsigned long long>(B);
     int *staged = w.take<int>(3 * B), *tok = w.take<int>(B), *ot = w.take<int>(B), *od = w.take<int>(B);
-    int *pfs = w.take<int>(R), *pfp = w.take<int>(R), *pfg0 = w.take<int>(1), *pfgn = w.take<int>(1);
-    int *pfng = w.take<int>(1), *pfnr = w.take<int>(1);
+    int *pfr = w.take<int>(prefill_ints(d));
     float *hlo = w.take<float>(B * d->d_model), *hup = w.take<float>(R * d->d_model);
     float *q = w.take<float>(R * qrow);
     int *crows = nullptr, *clist = nullptr;
@@ -238,8 +247,7 @@ size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
     if (c) {
         c->kcache = kc; c->vcache = vc; c->pend_h = ph; c->kv_len = kl; c->pend_cnt = pc; c->rope = rope;
         c->sd = sd; c->staged = staged; c->tok_dev = tok; c->out_tok_dev = ot; c->out_depth_dev = od;
-        c->pf_slot = pfs; c->pf_pos = pfp; c->pf_grp_row0 = pfg0; c->pf_grp_nrows = pfgn;
-        c->pf_ngrp = pfng; c->pf_nrows = pfnr;
+        c->pf_rows = pfr;
         c->conf_rows_dev = crows; c->conf_list_dev = clist; c->conf_ent_dev = cent; c->conf_logits = clog;
         c->h_last = hlast; c->q_last = qlast; c->last_slot = lslot; c->last_pos = lpos;
         c->h_lo = hlo; c->h_up = hup; c->qbuf = q; c->attn_o = ao; c->act = act; c->xnorm = xn; c->qkv_part = qp;
@@ -1074,7 +1082,7 @@ extern "C" int sparsk_create(const sparsk_dims *dims, const sparsk_weights *w, v
     if (!ctx) return SPARSK_EINVAL;
     ctx->magic = CTX_MAGIC;
     ctx->dm = *dims;
-    if (ctx->dm.prefill_rows <= 0) ctx->dm.prefill_rows = 64;
+    if (ctx->dm.prefill_rows <= 0) ctx->dm.prefill_rows = PREFILL_ROWS;
     ctx->stream = (cudaStream_t)cuda_stream;
     ctx->err[0] = 0;
     auto cp = [&](std::vector<const bf16 *> &dst, const void *const *src) {
@@ -1123,7 +1131,7 @@ extern "C" int sparsk_create(const sparsk_dims *dims, const sparsk_weights *w, v
             break;
         }
         for (int i = 0; i < STAGE_RING && rc == SPARSK_OK; i++) {
-            if ((ce = cudaHostAlloc((void **)&ctx->stage_host[i], 3 * sizeof(int) * dims->max_seqs, cudaHostAllocDefault)) != cudaSuccess ||
+            if ((ce = cudaHostAlloc((void **)&ctx->stage_host[i], sizeof(int) * std::max<size_t>(3 * (size_t)dims->max_seqs, prefill_ints(&ctx->dm)), cudaHostAllocDefault)) != cudaSuccess ||
                 (ce = cudaEventCreateWithFlags(&ctx->stage_ev[i], cudaEventDisableTiming)) != cudaSuccess)
                 rc = fail(ctx, SPARSK_ECUDA, "staging setup failed: %s", cudaGetErrorString(ce));
         }
@@ -1442,25 +1450,61 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
         if (ctx->h_pend[s]) return fail(ctx, SPARSK_ESTATE, "prefill: slot %d has pending positions", s);
         if (ctx->h_len[s] + n > d.max_seq_len) return fail(ctx, SPARSK_ECAPACITY, "prefill: slot %d would hold %ld > %d positions", s, ctx->h_len[s] + n, d.max_seq_len);
     }
-    const int chunk = std::min(d.prefill_rows, ctx->cap_rows);
-    for (int i = 0; i < n_seqs; i++) {
-        const int s = slots[i];
-        const int total = offsets[i + 1] - offsets[i];
-        for (int done = 0; done < total; done += chunk) {
-            const int n = std::min(chunk, total - done);
-            const int pos0 = ctx->h_len[s];
-            CU(launch(ctx, prefill_rows_kernel, dim3((n + 255) / 256), dim3(256), 0, ctx->pf_slot, ctx->pf_pos,
-                      ctx->pf_grp_row0, ctx->pf_grp_nrows, s, pos0, n));
-            CU(launch(ctx, set_int_kernel, dim3(1), dim3(1), 0, ctx->pf_ngrp, 1));
-            CU(launch(ctx, set_int_kernel, dim3(1), dim3(1), 0, ctx->pf_nrows, n));
-            CU(launch(ctx, embed_kernel, dim3(n), dim3(128), 0, tokens + offsets[i] + done, ctx->embed, ctx->h_up, n, d.d_model,
-                      d.vocab_text + d.vocab_speech, ctx->sd.counts + CNT_STATUS));
-            RowSet rs{ctx->pf_slot, ctx->pf_pos, ctx->pf_grp_row0, ctx->pf_grp_nrows, ctx->pf_ngrp, ctx->pf_nrows,
-                      n, 1, n, pos0 + n};
-            CU(run_layers(ctx, 1, d.n_layers, ctx->h_up, rs));
-            CU(launch(ctx, set_int_kernel, dim3(1), dim3(1), 0, ctx->kv_len + s, pos0 + n));
-            ctx->h_len[s] = pos0 + n;
+    // Passes of up to `chunk` rows, filled from the prompts in order: the end of one prompt, whole
+    // short ones and the beginning of the next share a pass (each a group of its own), so that only
+    // the last pass of the call runs with fewer rows.
+    const int chunk = std::min(d.prefill_rows, ctx->cap_rows), G_heads = d.n_q_heads / d.n_kv_heads;
+    std::vector<int> slot, pos, tok, g0, gn, base(n_seqs);
+    for (int i = 0; i < n_seqs; i++) base[i] = ctx->h_len[slots[i]];
+    for (int i = 0, done = 0; i < n_seqs;) {
+        slot.clear(); pos.clear(); tok.clear(); g0.clear(); gn.clear();
+        int n = 0, max_grp = 1, max_len = 0, n_big = 0;
+        long sum_len = 0;
+        while (i < n_seqs && n < chunk) {
+            const int s = slots[i], left = offsets[i + 1] - offsets[i] - done, take = std::min(chunk - n, left);
+            if (take > 0) {
+                const int pos0 = base[i] + done;
+                for (int j = 0; j < take; j++) {
+                    slot.push_back(s);
+                    pos.push_back(pos0 + j);
+                    tok.push_back(offsets[i] + done + j);
+                }
+                g0.push_back(n);
+                gn.push_back(take);
+                max_grp = std::max(max_grp, take);
+                max_len = std::max(max_len, pos0 + take);
+                sum_len += pos0 + take;
+                n_big += take * G_heads >= ctx->attn_tc_min_q;
+                n += take;
+                done += take;
+            }
+            if (take == left) {
+                i++;
+                done = 0;
+            }
         }
+        if (n == 0) break;
+        const int ng = (int)g0.size(), ring = ctx->stage_next;
+        ctx->stage_next = (ring + 1) % STAGE_RING;
+        CU(cudaEventSynchronize(ctx->stage_ev[ring]));
+        int *st = ctx->stage_host[ring];
+        std::copy(slot.begin(), slot.end(), st);
+        std::copy(pos.begin(), pos.end(), st + n);
+        std::copy(tok.begin(), tok.end(), st + 2 * n);
+        std::copy(g0.begin(), g0.end(), st + 3 * n);
+        std::copy(gn.begin(), gn.end(), st + 3 * n + ng);
+        st[3 * n + 2 * ng] = ng;
+        st[3 * n + 2 * ng + 1] = n;
+        CU(cudaMemcpyAsync(ctx->pf_rows, st, sizeof(int) * (3 * (size_t)n + 2 * ng + 2), cudaMemcpyHostToDevice, ctx->stream));
+        CU(cudaEventRecord(ctx->stage_ev[ring], ctx->stream));
+        const int *dv = ctx->pf_rows, *d_g0 = dv + 3 * n, *d_gn = d_g0 + ng, *d_cnt = d_gn + ng;
+        CU(launch(ctx, embed_kernel, dim3(n), dim3(128), 0, tokens, dv + 2 * n, ctx->embed, ctx->h_up, n, d.d_model,
+                  d.vocab_text + d.vocab_speech, ctx->sd.counts + CNT_STATUS));
+        RowSet rs{dv, dv + n, d_g0, d_gn, d_cnt, d_cnt + 1, n, ng, max_grp, max_len, n_big};
+        rs.sum_len = sum_len;
+        CU(run_layers(ctx, 1, d.n_layers, ctx->h_up, rs));
+        CU(launch(ctx, prefill_len_kernel, dim3((ng + 127) / 128), dim3(128), 0, ctx->kv_len, dv, dv + n, d_g0, d_gn, ng));
+        for (int g = 0; g < ng; g++) ctx->h_len[slot[g0[g]]] = pos[g0[g]] + gn[g];
     }
     return SPARSK_OK;
 }
@@ -1520,7 +1564,7 @@ static int decode_step_conf(sparsk_ctx *ctx, int32_t n, const int32_t *slots, co
     // the lower-row arrays (positions, one-row groups); "e = L" keeps every head on the lower rows
     CU(launch(ctx, compact_kernel, dim3(1), dim3(1024), 0, ctx->sd, (int)n, (const int *)ctx->kv_len,
               (const int *)ctx->pend_cnt, L, L, B));
-    CU(launch(ctx, embed_kernel, dim3(n), dim3(128), 0, (const int *)ctx->sd.token, ctx->embed, ctx->h_lo, (int)n, d.d_model,
+    CU(launch(ctx, embed_kernel, dim3(n), dim3(128), 0, (const int *)ctx->sd.token, (const int *)nullptr, ctx->embed, ctx->h_lo, (int)n, d.d_model,
               V, ctx->sd.counts + CNT_STATUS));
     if (ctx->dbg_logits) {
         const size_t cnt = (size_t)n * V;
@@ -1752,7 +1796,7 @@ extern "C" int sparsk_decode_step(sparsk_ctx *ctx, int32_t n, const int32_t *slo
               (const int *)token_ids, V, sp));
     CU(launch(ctx, compact_kernel, dim3(1), dim3(1024), 0, ctx->sd, (int)n, (const int *)ctx->kv_len,
               (const int *)ctx->pend_cnt, L, e, B));
-    CU(launch(ctx, embed_kernel, dim3(n), dim3(128), 0, (const int *)ctx->sd.token, ctx->embed, ctx->h_lo, (int)n, d.d_model,
+    CU(launch(ctx, embed_kernel, dim3(n), dim3(128), 0, (const int *)ctx->sd.token, (const int *)nullptr, ctx->embed, ctx->h_lo, (int)n, d.d_model,
               V, ctx->sd.counts + CNT_STATUS));
     if (ctx->dbg_logits) {
         const size_t cnt = (size_t)n * V;

@@ -136,14 +136,15 @@ static __global__ void __launch_bounds__(1024) compact_kernel(StepDesc sd, int n
     }
 }
 
-// h^(0) = E[token]  (Sec. III), fp32 residual stream.
-static __global__ void embed_kernel(const int *__restrict__ tokens, const bf16 *__restrict__ embed,
+// h^(0) = E[token]  (Sec. III), fp32 residual stream.  Row i's token is tokens[i], or
+// tokens[idx[i]] where the rows of a pass are gathered from a longer token array.
+static __global__ void embed_kernel(const int *__restrict__ tokens, const int *__restrict__ idx, const bf16 *__restrict__ embed,
                              float *__restrict__ h, int n, int d, int vocab, int *__restrict__ status)
 {
     griddep_wait();
     const int row = blockIdx.x;
     if (row >= n) return;
-    int tok = tokens[row];
+    int tok = tokens[idx ? idx[row] : row];
     if (tok < 0 || tok >= vocab) {  // never read outside the table; the host reports the flag
         if (threadIdx.x == 0) atomicOr(status, ST_BAD_TOKEN);
         tok = min(max(tok, 0), vocab - 1);
@@ -335,21 +336,14 @@ static __global__ void fill_kernel(float *__restrict__ p, size_t n, float v)
         p[i] = v;
 }
 
-// Prefill bookkeeping: rows of one chunk of one prompt.
-static __global__ void prefill_rows_kernel(int *__restrict__ row_slot, int *__restrict__ row_pos,
-                                    int *__restrict__ grp_row0, int *__restrict__ grp_nrows, int slot,
-                                    int pos0, int n)
+// End of a prefill pass: every group's slot now holds the positions up to the group's last row.
+static __global__ void prefill_len_kernel(int *__restrict__ kv_len, const int *__restrict__ row_slot,
+                                   const int *__restrict__ row_pos, const int *__restrict__ grp_row0,
+                                   const int *__restrict__ grp_nrows, int n_groups)
 {
     griddep_wait();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) {
-        grp_row0[0] = 0;
-        grp_nrows[0] = n;
-    }
-    if (i < n) {
-        row_slot[i] = slot;
-        row_pos[i] = pos0 + i;
-    }
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < n_groups) kv_len[row_slot[grp_row0[g]]] = row_pos[grp_row0[g] + grp_nrows[g] - 1] + 1;
 }
 static __global__ void set_int_kernel(int *p, int v)
 {

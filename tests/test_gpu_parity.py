@@ -257,6 +257,30 @@ def test_attention_items_drawn_from_the_counter(util, options):
     P.close()
 
 
+@pytest.mark.parametrize("rows", [3, 10, 17, 0])
+def test_prompts_share_prefill_passes(util, rows):
+    """Prompts of one call are packed into passes of `rows` rows: pieces that end exactly with a pass,
+    a prompt spread over several passes, several whole prompts in one, one of a single token and
+    one of none; a second call appends to what the slots hold.  The cache of every layer and a
+    cycle decoded on top match the oracle."""
+    dims = synth.model_dims("tiny", 2, 3, 0)
+    w = synth.make_weights(dims, seed=0)
+    lens = [13, 2, 8, 31, 1, 6]                     # one less is ingested: the last token starts decoding
+    prompts = [synth.make_prompts(dims, 1, n, n, seed=40 + i)[0] for i, n in enumerate(lens)]
+    P = util.Pair(dims, w, len(lens), 64, 2, prefill_rows=rows)
+    P.prefill([np.concatenate([p[:len(p) // 2], p[:1]]) for p in prompts])
+    second = [p[len(p) // 2:] for p in prompts]
+    P.prefill(second)
+    for s_, n in enumerate(lens):
+        assert P.g.slot_state(s_) == (n - 1, 0)
+        if n > 1:
+            P.check_cache(s_, range(1, 5), n - 1)
+    for g in range(6):
+        mc = [synth.interleave(g + i, 2, 4) for i in range(len(lens))]
+        P.step([m for m, _ in mc], [c for _, c in mc])
+    P.close()
+
+
 def test_timeout_is_reported_once_and_the_context_recovers(util):
     """A bounded in-kernel wait that runs out: the persistent kernel is told a grid-barrier count
     that no CTA can reach (a host-side test hook; nothing faults or hangs), its wait ends at the
