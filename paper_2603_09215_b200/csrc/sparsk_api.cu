@@ -30,6 +30,7 @@ constexpr size_t TIME_POOL = 16384;           // event pairs available to the ke
 enum { KC_MISC = 0, KC_QKV = 1, KC_ATTN = 2, KC_OPROJ = 3, KC_GATEUP = 4, KC_DOWN = 5, KC_HEAD = 6, KC_MEGA = 7, KC_ALL = 8 };
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+int div_up(int a, int b) { return (a + b - 1) / b; }
 
 struct Carve {
     char *base;
@@ -95,10 +96,11 @@ struct sparsk_ctx {
     float *samp_scratch;         // device [max_seqs][Vt + Vs]
     int64_t launches;
     // tensor-core path: TMA descriptors of every weight matrix and of the activation buffers
-    // (one per box height 16, 32, 64, 128, 256)
+    // (one per box height 16, 32, ..., 256)
     bool tc_ok;
     std::vector<TmaPair> tm_wq, tm_wk, tm_wv, tm_wo, tm_wg, tm_wu, tm_wd, tm_head;
-    TmaPair tm_x[5], tm_ao[5], tm_act[5], tm_x_lo[5], tm_ao_lo[5], tm_act_lo[5];
+    TmaPair tm_x[GM_BOXES], tm_ao[GM_BOXES], tm_act[GM_BOXES], tm_x_lo[GM_BOXES], tm_ao_lo[GM_BOXES], tm_act_lo[GM_BOXES];
+    int gu_rows;                 // weight rows per accumulator of a gate/up unit
     std::vector<CUtensorMap> tm_kc16, tm_vc16;  // per layer: the cache as rows of head_dim numbers, boxes of 16 rows (attn_warp_tma_kernel)
     int attn_tma, attn_tma_ok;               // option (default 1); the maps above exist
     std::vector<CUtensorMap> tm_kc, tm_vc;  // per layer: the cache viewed as [64][slots * Hkv * S rows][hd / 64], boxes of [64][64][2]
@@ -455,7 +457,6 @@ cudaError_t run_head(sparsk_ctx *c, int layer, const float *h, int list, int n_r
 #undef HD_CASE
 }
 
-int div_up(int a, int b);
 
 cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
 {
@@ -620,7 +621,11 @@ bool build_maps(sparsk_ctx *c)
     };
     fill(c->tm_wq, c->wq, qd, d.d_model, 2 * GM_BM); fill(c->tm_wk, c->wk, kd, d.d_model, 2 * GM_BM);
     fill(c->tm_wv, c->wv, kd, d.d_model, 2 * GM_BM); fill(c->tm_wo, c->wo, d.d_model, qd, 2 * GM_BM);
-    fill(c->tm_wg, c->w_gate, d.d_ffn, d.d_model, GM_BM); fill(c->tm_wu, c->w_up, d.d_ffn, d.d_model, GM_BM);
+    // gate/up unit height: the one whose units leave the busiest SM the fewest rows
+    c->gu_rows = GM_BM;
+    for (int r = GM_BM - 8; r >= 32; r -= 8)
+        if (div_up(div_up(d.d_ffn, r), c->n_sm) * r < div_up(div_up(d.d_ffn, c->gu_rows), c->n_sm) * c->gu_rows) c->gu_rows = r;
+    fill(c->tm_wg, c->w_gate, d.d_ffn, d.d_model, c->gu_rows); fill(c->tm_wu, c->w_up, d.d_ffn, d.d_model, c->gu_rows);
     fill(c->tm_wd, c->w_down, d.d_model, d.d_ffn, 2 * GM_BM); fill(c->tm_head, c->head_proj, V, d.d_model, 2 * GM_BM);
     if (d.head_dim == 64 || d.head_dim == 128) {
         const size_t lstride = (size_t)d.max_seqs * d.n_kv_heads * d.max_seq_len * d.head_dim;
@@ -651,8 +656,8 @@ bool build_maps(sparsk_ctx *c)
             c->tm_vc[l] = t.m3;
         }
     }
-    for (int b = 0; b < 5; b++) {
-        const int box = 16 << b;
+    for (int b = 0; b < GM_BOXES; b++) {
+        const int box = 16 * (b + 1);
         ok = ok && encode_maps(fn, &c->tm_x[b], c->xnorm, c->cap_rows, d.d_model, box);
         ok = ok && encode_maps(fn, &c->tm_ao[b], c->attn_o, c->cap_rows, qd, box);
         ok = ok && encode_maps(fn, &c->tm_act[b], c->act, c->cap_rows, d.d_ffn, box);
@@ -663,12 +668,9 @@ bool build_maps(sparsk_ctx *c)
     return ok;
 }
 
-int box_index(int m_rows)
-{
-    int b = 0;
-    while (b < 4 && (16 << b) < std::min(m_rows, GM_MAX_N)) b++;
-    return b;
-}
+// Activation rows per copy: as many as there are, in steps of 16 (a copy of rows that do not exist
+// costs L2 traffic and ring space: 70 rows in a 128-row box left room for one k-block per copy).
+int box_index(int m_rows) { return (std::min(m_rows, GM_MAX_N) + 15) / 16 - 1; }
 
 template <class Epi>
 cudaError_t launch_gemm(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1, const TmaPair &a2, const TmaPair *b_maps,
@@ -684,11 +686,12 @@ cudaError_t launch_gemm(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1, con
         attr_set = true;
     }
     const int bi = box_index(g.m_rows);
-    g.box_n = 16 << bi;
+    g.box_n = 16 * (bi + 1);
+    const int blk_bytes = g.pair ? g.unit_rows * GM_BK * 2 : GM_BLK_BYTES;
     // the ring may be told to stay small enough for two CTAs (of this kernel or of the next one in
     // the stream) to share an SM, so that one's ending overlaps the other's first copies; rows
     // that do not fit such a ring take the whole SM
-    auto stage_bytes = [&](int kb) { return 2 * kb * GM_BLK_BYTES + 2 * kb * g.box_n * GM_BK * 2; };
+    auto stage_bytes = [&](int kb) { return 2 * kb * blk_bytes + 2 * kb * g.box_n * GM_BK * 2; };
     auto plan = [&](int budget) {
         const int room = budget - 1024 - GM_XCHG_BYTES;
         // two k-blocks per copy whenever the inner dimension allows the 3-D view and two stages fit
@@ -712,8 +715,6 @@ cudaError_t launch_gemm(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1, con
     return launch(c, kern, dim3(grid_x, grid_y), dim3(GM_THREADS), smem, a0.m2, a1.m2, a2.m2, b_maps[bi].m2,
                   b_lo_maps[bi].m2, g, epi);
 }
-
-int div_up(int a, int b) { return (a + b - 1) / b; }
 
 cudaError_t run_norm(sparsk_ctx *c, const float *h, const bf16 *gain, const int *row_idx, int n_rows)
 {
@@ -783,7 +784,7 @@ cudaError_t run_layer_tc_back(sparsk_ctx *c, int layer, float *h, const RowSet &
     {
         c->cur_class = KC_GATEUP;
         GemmArgs g{};
-        g.K = d.d_model; g.units[0] = div_up(d.d_ffn, GM_BM); g.pair = 1; g.m_rows = M; g.splits = 1;
+        g.K = d.d_model; g.units[0] = div_up(d.d_ffn, c->gu_rows); g.pair = 1; g.unit_rows = c->gu_rows; g.m_rows = M; g.splits = 1;
         GateUpEnd ep;
         ep.u = c->act; ep.u_lo = c->act_lo; ep.F = d.d_ffn;
         if ((e = launch_gemm(c, c->tm_wg[li], c->tm_wu[li], c->tm_wu[li], c->tm_x, c->tm_x_lo, g, ep)) != cudaSuccess) return e;

@@ -35,6 +35,7 @@ namespace sparsk {
 constexpr int GM_THREADS = 192;
 constexpr int GM_BM = 128;                     // weight rows per accumulator (UMMA M)
 constexpr int GM_BK = 64;                      // inner elements per k-block: one 128-byte swizzle span
+constexpr int GM_BOXES = 16;                   // heights of an activation copy: 16, 32, ..., 256 rows
 constexpr int GM_MAX_N = 256;                  // activation rows per launch block (UMMA N limit)
 constexpr int GM_BLK_BYTES = GM_BM * GM_BK * 2;  // one accumulator's weights for one k-block: 16 KB
 constexpr int GM_MAX_STAGES = 6;
@@ -43,8 +44,11 @@ constexpr int GM_XCHG_BYTES = GM_CHUNK * GM_BM * 4;
 constexpr unsigned long long GM_TIMEOUT_NS = WAIT_TIMEOUT_NS;
 
 // A unit of work is two accumulators of 128 weight rows each: either 256 consecutive rows of one
-// matrix (one TMA box), or 128 rows of matrix 0 and the same 128 rows of matrix 1 ("pair": gate
-// and up, whose results meet in the ending).  The TMA engine spends a fixed few hundred
+// matrix (one TMA box), or `unit_rows` (at most 128) rows of matrix 0 and the same rows of matrix
+// 1 ("pair": gate and up, whose results meet in the ending).  A pair's height is what deals the
+// rows evenly to the SMs: 13,696 rows are 107 units of 128, which leave 41 of 148 SMs without
+// weights to stream, but 143 units of 96; the MMA still covers 128 rows, and what it computes from
+// the bytes behind the 96 is never read.  The TMA engine spends a fixed few hundred
 // nanoseconds per copy whatever its size, so a stage is made of few, large boxes: with a
 // three-dimensional view [64 elements][rows][K/64] of a row-major matrix one box carries two
 // k-blocks of every row.
@@ -54,8 +58,9 @@ struct GemmArgs {
     int row0[3];   // first row of each matrix that belongs to this product (a head's id range)
     int splits;    // cuts of the inner dimension per unit (> 1 only with an additive ending)
     int pair;      // 1: accumulator 1 comes from matrix 1
+    int unit_rows; // pair: weight rows per accumulator (a multiple of 8)
     int m_rows;    // activation rows of the whole launch; block y owns rows [256 y, 256 y + 256)
-    int box_n;     // activation rows per TMA box (16, 32, 64, 128 or 256)
+    int box_n;     // activation rows per TMA box (a multiple of 16, at most 256)
     int stages;    // ring depth
     int kb;        // k-blocks per stage (1 or 2)
     int three_d;   // 1: the descriptors are the [64][rows][K/64] views (needs K % 64 == 0)
@@ -116,6 +121,7 @@ struct TileCtx {
     uint32_t taddr;  // TMEM address of accumulator 0, this thread's lane, column 0
     int acc_stride;  // columns between accumulator 0 and accumulator 1
     float *xchg;     // [GM_CHUNK][128] floats shared by the 128 epilogue threads
+    int unit_rows;   // pair: rows of an accumulator that are the unit's
 };
 
 // ------------------------------------------------------------------ kernel
@@ -134,13 +140,14 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t ring = (smem_u32(gm_smem) + 1023u) & ~1023u;  // swizzled tiles need 1024-byte alignment
-    const int a_bytes = 2 * g.kb * GM_BLK_BYTES;                 // both accumulators' weights of a stage
+    const int blk_bytes = g.pair ? g.unit_rows * GM_BK * 2 : GM_BLK_BYTES;
+    const int a_bytes = 2 * g.kb * blk_bytes;                    // both accumulators' weights of a stage
     const int b_blk = g.box_n * GM_BK * 2;
     const int b_half = g.kb * b_blk;                              // the hi tiles; the lo tiles follow
     const int stage_bytes = a_bytes + 2 * b_half;
     // where accumulator a's rows of k-block j sit inside a stage
-    const int a_blk_stride = g.pair ? GM_BLK_BYTES : 2 * GM_BLK_BYTES;
-    const int a_acc_off = g.pair ? g.kb * GM_BLK_BYTES : GM_BLK_BYTES;
+    const int a_blk_stride = g.pair ? blk_bytes : 2 * blk_bytes;
+    const int a_acc_off = g.pair ? g.kb * blk_bytes : blk_bytes;
     float *xchg = reinterpret_cast<float *>(gm_smem + (ring - smem_u32(gm_smem)) + (size_t)g.stages * stage_bytes);
 
     const int m0 = blockIdx.y * GM_MAX_N;
@@ -193,7 +200,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
             if (t >= g.units[0]) { t -= g.units[0]; mat = 1; }
             if (mat == 1 && t >= g.units[1]) { t -= g.units[1]; mat = 2; }
         }
-        unit_row = t * (g.pair ? GM_BM : 2 * GM_BM);
+        unit_row = t * (g.pair ? g.unit_rows : 2 * GM_BM);
     };
 
     if (warp == 0) {
@@ -300,6 +307,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
         tc.m_end = m_end;
         tc.acc_stride = mma_n;
         tc.xchg = xchg;
+        tc.unit_rows = g.unit_rows;
         uint32_t unit_it = 0;
         bool ok = true;
         for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x, unit_it++) {
@@ -467,7 +475,7 @@ struct GateUpEnd {
             float gt[GM_CHUNK], up[GM_CHUNK];
             tmem_ld16(t.taddr + c0, gt);
             tmem_ld16(t.taddr + t.acc_stride + c0, up);
-            if (f >= F) continue;
+            if (f >= F || t.row >= t.unit_rows) continue;
 #pragma unroll
             for (int c = 0; c < GM_CHUNK; c++) {
                 const int m = t.m0 + c0 + c;

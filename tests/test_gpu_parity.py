@@ -281,6 +281,25 @@ def test_prompts_share_prefill_passes(util, rows):
     P.close()
 
 
+@pytest.mark.parametrize("B", [5, 16, 17, 64, 81, 128, 130])
+def test_tcgen05_passes_of_every_width(util, B):
+    """Batches on the tcgen05 path at the edges of its activation tiles (copies of 16, 32, 48 ... rows),
+    on a shape whose MLP rows are dealt in units lower than the 128 rows an MMA covers."""
+    dims = synth.model_dims("tiny", 2, 3, 0)
+    w = synth.make_weights(dims, seed=3)
+    prompts = synth.make_prompts(dims, B, 3, 12, seed=11)
+    P = util.Pair(dims, w, B, 32, 2, oracle_slots=[0, B // 2, B - 1])
+    P.prefill(prompts)
+    for g in range(6):
+        mc = [synth.interleave(g + i, 2, 4) for i in range(B)]
+        P.step([m for m, _ in mc], [c for _, c in mc])
+    for s_ in (0, B - 1):
+        ln, pend = P.g.slot_state(s_)
+        P.check_cache(s_, range(1, 5), ln - pend)
+    assert P.g.route_counts()["tc"] > 0
+    P.close()
+
+
 def test_timeout_is_reported_once_and_the_context_recovers(util):
     """A bounded in-kernel wait that runs out: the persistent kernel is told a grid-barrier count
     that no CTA can reach (a host-side test hook; nothing faults or hangs), its wait ends at the
