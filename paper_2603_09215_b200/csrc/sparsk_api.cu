@@ -25,6 +25,10 @@ namespace {
 
 constexpr int MAX_SPLITS = AT_MAX_SPLITS;
 constexpr int STAGE_RING = 16;
+// Passes of more rows take gate/up units of 128 rows (see build_maps): a CTA's MMA time does not
+// depend on the unit's height, so lower units only add CTAs.  First token after 1,024 of the 40-layer
+// shape at 256 rows a pass: 51.6 ms with units of 96 rows, 49.8 with 128.
+constexpr int GU_EVEN_ROWS = 128;
 constexpr uint32_t CTX_MAGIC = 0x5350524bu;  // "SPRK"
 constexpr size_t TIME_POOL = 16384;           // event pairs available to the kernel timer
 enum { KC_MISC = 0, KC_QKV = 1, KC_ATTN = 2, KC_OPROJ = 3, KC_GATEUP = 4, KC_DOWN = 5, KC_HEAD = 6, KC_MEGA = 7, KC_ALL = 8 };
@@ -98,9 +102,9 @@ struct sparsk_ctx {
     // tensor-core path: TMA descriptors of every weight matrix and of the activation buffers
     // (one per box height 16, 32, ..., 256)
     bool tc_ok;
-    std::vector<TmaPair> tm_wq, tm_wk, tm_wv, tm_wo, tm_wg, tm_wu, tm_wd, tm_head;
-    TmaPair tm_x[GM_BOXES], tm_ao[GM_BOXES], tm_act[GM_BOXES], tm_x_lo[GM_BOXES], tm_ao_lo[GM_BOXES], tm_act_lo[GM_BOXES];
-    int gu_rows;                 // weight rows per accumulator of a gate/up unit
+    std::vector<TmaPair> tm_wq, tm_wk, tm_wv, tm_wo, tm_wg[2], tm_wu[2], tm_wd, tm_head;
+    TmaPair tm_x[GM_BOXES], tm_ao[GM_BOXES], tm_act[GM_BOXES];
+    int gu_rows[2];              // weight rows per accumulator of a gate/up unit: up to GU_EVEN_ROWS activation rows, beyond
     std::vector<CUtensorMap> tm_kc16, tm_vc16;  // per layer: the cache as rows of head_dim numbers, boxes of 16 rows (attn_warp_tma_kernel)
     int attn_tma, attn_tma_ok;               // option (default 1); the maps above exist
     std::vector<CUtensorMap> tm_kc, tm_vc;  // per layer: the cache viewed as [64][slots * Hkv * S rows][hd / 64], boxes of [64][64][2]
@@ -573,11 +577,11 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Descriptors of a row-major bf16 matrix [rows][cols], 128-byte swizzle, zero fill outside:
+// Descriptors of a row-major 16-bit matrix [rows][cols], 128-byte swizzle, zero fill outside:
 // m2 reads boxes of [box_rows][64]; m3 (only when cols is a multiple of 64) views the matrix as
 // [64][rows][cols/64] and reads [box_rows] rows of two consecutive 64-element blocks at once.
 bool encode_maps(EncodeTiledFn fn, TmaPair *m, const void *base, size_t rows, size_t cols, int box_rows,
-                 CUtensorMapDataType dtype = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16)
+                 CUtensorMapDataType dtype)
 {
     memset(m, 0, sizeof *m);
     if (!base) return true;
@@ -603,6 +607,37 @@ bool encode_maps(EncodeTiledFn fn, TmaPair *m, const void *base, size_t rows, si
     return true;
 }
 
+// Descriptors of an operand of the tcgen05 GEMMs: a row-major bf16 matrix, or (lo) the two planes
+// of an activation matrix.  A box of up to 128 rows carries the same rows of every plane, the lo
+// tile behind the hi tile, a higher one a single plane's.  m2 takes one 64-element block per copy
+// (view [cols][rows][plane]), m3 two (view [64][rows][plane][cols/64]; not for single planes of two).
+bool encode_gemm_maps(EncodeTiledFn fn, TmaPair *m, const bf16 *hi, const bf16 *lo, size_t rows, size_t cols, int box_rows)
+{
+    memset(m, 0, sizeof *m);
+    if (!hi) return true;
+    const cuuint64_t planes = lo ? 2 : 1, row = (cuuint64_t)cols * 2, plane = lo ? (cuuint64_t)((const char *)lo - (const char *)hi) : row * rows;
+    const bool whole = !lo || box_rows <= GM_MAX_N / 2;
+    const cuuint32_t es[4] = {1, 1, 1, 1}, box_planes = whole ? (cuuint32_t)planes : 1u;
+    {
+        const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, planes}, strides[2] = {row, plane};
+        const cuuint32_t box[3] = {(cuuint32_t)GM_BK, (cuuint32_t)box_rows, box_planes};
+        if (fn(&m->m2, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16 *>(hi), dims, strides, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+    }
+    if (cols % GM_BK == 0 && whole) {
+        const cuuint64_t dims[4] = {(cuuint64_t)GM_BK, (cuuint64_t)rows, planes, (cuuint64_t)(cols / GM_BK)};
+        const cuuint64_t strides[3] = {row, plane, (cuuint64_t)GM_BK * 2};
+        const cuuint32_t box[4] = {(cuuint32_t)GM_BK, (cuuint32_t)box_rows, box_planes, 2};
+        if (fn(&m->m3, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16 *>(hi), dims, strides, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+    }
+    return true;
+}
+
 bool build_maps(sparsk_ctx *c)
 {
     const sparsk_dims &d = c->dm;
@@ -617,15 +652,19 @@ bool build_maps(sparsk_ctx *c)
     bool ok = true;
     auto fill = [&](std::vector<TmaPair> &v, const std::vector<const bf16 *> &w, size_t rows, size_t cols, int box) {
         v.resize(L);
-        for (int l = 0; l < L; l++) ok = ok && encode_maps(fn, &v[l], w[l], rows, cols, box);
+        for (int l = 0; l < L; l++) ok = ok && encode_gemm_maps(fn, &v[l], w[l], nullptr, rows, cols, box);
     };
     fill(c->tm_wq, c->wq, qd, d.d_model, 2 * GM_BM); fill(c->tm_wk, c->wk, kd, d.d_model, 2 * GM_BM);
     fill(c->tm_wv, c->wv, kd, d.d_model, 2 * GM_BM); fill(c->tm_wo, c->wo, d.d_model, qd, 2 * GM_BM);
-    // gate/up unit height: the one whose units leave the busiest SM the fewest rows
-    c->gu_rows = GM_BM;
+    // gate/up unit height: the one whose units leave the busiest SM the fewest rows; where the MMAs
+    // and not the weight stream take the time it is what an MMA covers, the full 128
+    c->gu_rows[0] = c->gu_rows[1] = GM_BM;
     for (int r = GM_BM - 8; r >= 32; r -= 8)
-        if (div_up(div_up(d.d_ffn, r), c->n_sm) * r < div_up(div_up(d.d_ffn, c->gu_rows), c->n_sm) * c->gu_rows) c->gu_rows = r;
-    fill(c->tm_wg, c->w_gate, d.d_ffn, d.d_model, c->gu_rows); fill(c->tm_wu, c->w_up, d.d_ffn, d.d_model, c->gu_rows);
+        if (div_up(div_up(d.d_ffn, r), c->n_sm) * r < div_up(div_up(d.d_ffn, c->gu_rows[0]), c->n_sm) * c->gu_rows[0]) c->gu_rows[0] = r;
+    for (int t = 0; t < 2; t++) {
+        fill(c->tm_wg[t], c->w_gate, d.d_ffn, d.d_model, c->gu_rows[t]);
+        fill(c->tm_wu[t], c->w_up, d.d_ffn, d.d_model, c->gu_rows[t]);
+    }
     fill(c->tm_wd, c->w_down, d.d_model, d.d_ffn, 2 * GM_BM); fill(c->tm_head, c->head_proj, V, d.d_model, 2 * GM_BM);
     if (d.head_dim == 64 || d.head_dim == 128) {
         const size_t lstride = (size_t)d.max_seqs * d.n_kv_heads * d.max_seq_len * d.head_dim;
@@ -658,12 +697,9 @@ bool build_maps(sparsk_ctx *c)
     }
     for (int b = 0; b < GM_BOXES; b++) {
         const int box = 16 * (b + 1);
-        ok = ok && encode_maps(fn, &c->tm_x[b], c->xnorm, c->cap_rows, d.d_model, box);
-        ok = ok && encode_maps(fn, &c->tm_ao[b], c->attn_o, c->cap_rows, qd, box);
-        ok = ok && encode_maps(fn, &c->tm_act[b], c->act, c->cap_rows, d.d_ffn, box);
-        ok = ok && encode_maps(fn, &c->tm_x_lo[b], c->xnorm_lo, c->cap_rows, d.d_model, box);
-        ok = ok && encode_maps(fn, &c->tm_ao_lo[b], c->attn_o_lo, c->cap_rows, qd, box);
-        ok = ok && encode_maps(fn, &c->tm_act_lo[b], c->act_lo, c->cap_rows, d.d_ffn, box);
+        ok = ok && encode_gemm_maps(fn, &c->tm_x[b], c->xnorm, c->xnorm_lo, c->cap_rows, d.d_model, box);
+        ok = ok && encode_gemm_maps(fn, &c->tm_ao[b], c->attn_o, c->attn_o_lo, c->cap_rows, qd, box);
+        ok = ok && encode_gemm_maps(fn, &c->tm_act[b], c->act, c->act_lo, c->cap_rows, d.d_ffn, box);
     }
     return ok;
 }
@@ -672,14 +708,14 @@ bool build_maps(sparsk_ctx *c)
 // costs L2 traffic and ring space: 70 rows in a 128-row box left room for one k-block per copy).
 int box_index(int m_rows) { return (std::min(m_rows, GM_MAX_N) + 15) / 16 - 1; }
 
-template <class Epi>
-cudaError_t launch_gemm(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1, const TmaPair &a2, const TmaPair *b_maps,
-                        const TmaPair *b_lo_maps, GemmArgs g, const Epi &epi)
+template <class Epi, bool STACKED>
+cudaError_t launch_gemm_inst(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1, const TmaPair &a2, const TmaPair *b_maps,
+                        GemmArgs g, const Epi &epi)
 {
     static PerDevice<bool> attr_done;
     bool &attr_set = attr_done.here();
     constexpr int SMEM_BUDGET = 220 * 1024;
-    auto kern = wsgemm_kernel<Epi>;
+    auto kern = wsgemm_kernel<Epi, STACKED>;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET);
         if (e != cudaSuccess) return e;
@@ -695,7 +731,7 @@ cudaError_t launch_gemm(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1, con
     auto plan = [&](int budget) {
         const int room = budget - 1024 - GM_XCHG_BYTES;
         // two k-blocks per copy whenever the inner dimension allows the 3-D view and two stages fit
-        g.three_d = (g.K % GM_BK == 0) && 2 * stage_bytes(2) <= room && c->tc_kb != 1;
+        g.three_d = (g.K % GM_BK == 0) && STACKED && 2 * stage_bytes(2) <= room && c->tc_kb != 1;
         g.kb = g.three_d ? 2 : 1;
         g.stages = std::min(GM_MAX_STAGES, room / stage_bytes(g.kb));
         return g.stages >= 2;
@@ -710,10 +746,17 @@ cudaError_t launch_gemm(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1, con
     const int grid_x = std::max(1, std::min(c->n_sm * per_sm, n_units * g.splits));
     const int grid_y = (g.m_rows + GM_MAX_N - 1) / GM_MAX_N;
     if (g.three_d)
-        return launch(c, kern, dim3(grid_x, grid_y), dim3(GM_THREADS), smem, a0.m3, a1.m3, a2.m3, b_maps[bi].m3,
-                      b_lo_maps[bi].m3, g, epi);
-    return launch(c, kern, dim3(grid_x, grid_y), dim3(GM_THREADS), smem, a0.m2, a1.m2, a2.m2, b_maps[bi].m2,
-                  b_lo_maps[bi].m2, g, epi);
+        return launch(c, kern, dim3(grid_x, grid_y), dim3(GM_THREADS), smem, a0.m3, a1.m3, a2.m3, b_maps[bi].m3, g,
+                      epi);
+    return launch(c, kern, dim3(grid_x, grid_y), dim3(GM_THREADS), smem, a0.m2, a1.m2, a2.m2, b_maps[bi].m2, g, epi);
+}
+
+template <class Epi>
+cudaError_t launch_gemm(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1, const TmaPair &a2, const TmaPair *b_maps,
+                        const GemmArgs &g, const Epi &epi)
+{
+    return g.m_rows <= GM_MAX_N / 2 ? launch_gemm_inst<Epi, true>(c, a0, a1, a2, b_maps, g, epi)
+                                    : launch_gemm_inst<Epi, false>(c, a0, a1, a2, b_maps, g, epi);
 }
 
 cudaError_t run_norm(sparsk_ctx *c, const float *h, const bf16 *gain, const int *row_idx, int n_rows)
@@ -752,7 +795,7 @@ cudaError_t run_layer_tc_front(sparsk_ctx *c, int layer, float *h, const RowSet 
         ep.q_out = c->qbuf; ep.kc = kc; ep.vc = vc; ep.rope = c->rope;
         ep.row_slot = rs.slot; ep.row_pos = rs.pos; ep.Hq = d.n_q_heads; ep.Hkv = d.n_kv_heads; ep.hd = d.head_dim;
         ep.S = d.max_seq_len; ep.partial = g.splits > 1 ? c->qkv_part : nullptr;
-        if ((e = launch_gemm(c, c->tm_wq[li], c->tm_wk[li], c->tm_wv[li], c->tm_x, c->tm_x_lo, g, ep)) != cudaSuccess) return e;
+        if ((e = launch_gemm(c, c->tm_wq[li], c->tm_wk[li], c->tm_wv[li], c->tm_x, g, ep)) != cudaSuccess) return e;
         if (g.splits > 1 &&
             (e = launch(c, qkv_finish_kernel, dim3(M), dim3(256), 0, c->qkv_part, c->qbuf, kc, vc, (const float2 *)c->rope,
                         rs.slot, rs.pos, M, d.n_q_heads, d.n_kv_heads, d.head_dim, d.max_seq_len)) != cudaSuccess)
@@ -777,17 +820,18 @@ cudaError_t run_layer_tc_back(sparsk_ctx *c, int layer, float *h, const RowSet &
         g.splits = splits_for(c, g.units[0]);
         ResidEnd ep;
         ep.h = h; ep.n_out = d.d_model; ep.atomic = 1;
-        if ((e = launch_gemm(c, c->tm_wo[li], c->tm_wo[li], c->tm_wo[li], c->tm_ao, c->tm_ao_lo, g, ep)) != cudaSuccess) return e;
+        if ((e = launch_gemm(c, c->tm_wo[li], c->tm_wo[li], c->tm_wo[li], c->tm_ao, g, ep)) != cudaSuccess) return e;
     }
     c->cur_class = KC_MISC;
     if ((e = run_norm(c, h, c->mlp_norm[li], nullptr, M)) != cudaSuccess) return e;
     {
         c->cur_class = KC_GATEUP;
         GemmArgs g{};
-        g.K = d.d_model; g.units[0] = div_up(d.d_ffn, c->gu_rows); g.pair = 1; g.unit_rows = c->gu_rows; g.m_rows = M; g.splits = 1;
+        const int t = M > GU_EVEN_ROWS, rows = c->gu_rows[t];
+        g.K = d.d_model; g.units[0] = div_up(d.d_ffn, rows); g.pair = 1; g.unit_rows = rows; g.m_rows = M; g.splits = 1;
         GateUpEnd ep;
         ep.u = c->act; ep.u_lo = c->act_lo; ep.F = d.d_ffn;
-        if ((e = launch_gemm(c, c->tm_wg[li], c->tm_wu[li], c->tm_wu[li], c->tm_x, c->tm_x_lo, g, ep)) != cudaSuccess) return e;
+        if ((e = launch_gemm(c, c->tm_wg[t][li], c->tm_wu[t][li], c->tm_wu[t][li], c->tm_x, g, ep)) != cudaSuccess) return e;
     }
     {
         c->cur_class = KC_DOWN;
@@ -796,7 +840,7 @@ cudaError_t run_layer_tc_back(sparsk_ctx *c, int layer, float *h, const RowSet &
         g.splits = splits_for(c, g.units[0]);
         ResidEnd ep;
         ep.h = h; ep.n_out = d.d_model; ep.atomic = 1;
-        e = launch_gemm(c, c->tm_wd[li], c->tm_wd[li], c->tm_wd[li], c->tm_act, c->tm_act_lo, g, ep);
+        e = launch_gemm(c, c->tm_wd[li], c->tm_wd[li], c->tm_wd[li], c->tm_act, g, ep);
     }
     c->cur_class = KC_MISC;
     return e;
@@ -821,7 +865,7 @@ cudaError_t run_head_tc(sparsk_ctx *c, int layer, const float *h, int list, int 
     GemmArgs g{};
     g.K = d.d_model; g.units[0] = div_up(ep.hi - ep.lo, 2 * GM_BM); g.row0[0] = ep.lo; g.m_rows = n_rows;
     g.splits = 1;
-    e = launch_gemm(c, c->tm_head[li], c->tm_head[li], c->tm_head[li], c->tm_x, c->tm_x_lo, g, ep);
+    e = launch_gemm(c, c->tm_head[li], c->tm_head[li], c->tm_head[li], c->tm_x, g, ep);
     c->cur_class = KC_MISC;
     return e;
 }

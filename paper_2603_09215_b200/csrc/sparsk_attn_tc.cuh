@@ -67,16 +67,6 @@ __device__ __forceinline__ uint32_t umma_idesc_f16_ex(int n, bool b_mn)
 {
     return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TA_QB >> 4) << 24) | (b_mn ? (1u << 16) : 0u);
 }
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-}
-
 // D (+)= A B with the A operand in TMEM (lane = row, 16-bit elements packed two per column) and B in shared memory.
 __device__ __forceinline__ void umma_f16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t desc_b, uint32_t idesc, int accumulate)
 {

@@ -21,6 +21,12 @@
 // only, and at random initialisation a single bf16 rounding of the activations early in the
 // stack is amplified by every later layer to 2-3 % at the exit of a 28-layer stack.  The second
 // product costs tensor time and L2 traffic, not HBM bytes.
+// Up to 128 rows both terms sit behind one another in a stage and are ONE operand of 2 n rows: an
+// MMA costs some 45 ns however few columns it has (its 128 weight rows have to be fetched from
+// shared memory either way), and with an MMA per term the 32 MMAs of a 64 KB stage held a CTA at
+// 43 GB/s, as much as its share of HBM.  The two products land in columns of their own, which
+// the ending adds.  Event-timed launches, before and after: gate/up of the 40-layer shape 60 -> 50 us
+// at 16 rows and 65 -> 59 at 64, down of the 28-layer shape 35.2 -> 33.2 at 12 rows.
 // Accumulators are double buffered in TMEM so a tile's epilogue overlaps the next tile's MMAs.
 // Every wait is bounded: on a timeout the CTA raises ST_TIMEOUT, stops issuing work, drains its
 // own copies, frees its TMEM and returns.
@@ -63,7 +69,7 @@ struct GemmArgs {
     int box_n;     // activation rows per TMA box (a multiple of 16, at most 256)
     int stages;    // ring depth
     int kb;        // k-blocks per stage (1 or 2)
-    int three_d;   // 1: the descriptors are the [64][rows][K/64] views (needs K % 64 == 0)
+    int three_d;   // 1: the descriptors are the [64][rows][plane][K/64] views (needs K % 64 == 0)
     int *status;   // device status word
 };
 
@@ -96,19 +102,16 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar)
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16])
 {
-    uint32_t r[16];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
           "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr)
         : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
 // What an ending sees of one finished unit.
@@ -122,14 +125,34 @@ struct TileCtx {
     int acc_stride;  // columns between accumulator 0 and accumulator 1
     float *xchg;     // [GM_CHUNK][128] floats shared by the 128 epilogue threads
     int unit_rows;   // pair: rows of an accumulator that are the unit's
+    int lo_off;      // stacked terms: columns from the hi term's product to the lo term's
+
+    // 16 activation rows (from c0 on) of accumulator a
+    template <bool STACKED>
+    __device__ __forceinline__ void load(int a, int c0, float (&v)[GM_CHUNK]) const
+    {
+        const uint32_t at = taddr + (uint32_t)(a * acc_stride + c0);
+        uint32_t r[GM_CHUNK], s[GM_CHUNK];
+        tmem_ld16_nowait(at, r);
+        if (STACKED) {
+            tmem_ld16_nowait(at + (uint32_t)lo_off, s);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < GM_CHUNK; i++) v[i] = __uint_as_float(r[i]) + __uint_as_float(s[i]);
+        } else {
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < GM_CHUNK; i++) v[i] = __uint_as_float(r[i]);
+        }
+    }
 };
 
 // ------------------------------------------------------------------ kernel
-template <class Epi>
+// STACKED: the two terms of the activations are one operand (box_n <= 128; kb is 1 without).
+template <class Epi, bool STACKED>
 __global__ void __launch_bounds__(GM_THREADS, 1)
     wsgemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
                   const __grid_constant__ CUtensorMap map_a2, const __grid_constant__ CUtensorMap map_b,
-                  const __grid_constant__ CUtensorMap map_b_lo,
                   const GemmArgs g, const Epi epi)
 {
     extern __shared__ __align__(1024) unsigned char gm_smem[];
@@ -143,8 +166,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
     const int blk_bytes = g.pair ? g.unit_rows * GM_BK * 2 : GM_BLK_BYTES;
     const int a_bytes = 2 * g.kb * blk_bytes;                    // both accumulators' weights of a stage
     const int b_blk = g.box_n * GM_BK * 2;
-    const int b_half = g.kb * b_blk;                              // the hi tiles; the lo tiles follow
-    const int stage_bytes = a_bytes + 2 * b_half;
+    const int stage_bytes = a_bytes + 2 * g.kb * b_blk;           // per k-block: the hi tile, then the lo tile
     // where accumulator a's rows of k-block j sit inside a stage
     const int a_blk_stride = g.pair ? blk_bytes : 2 * blk_bytes;
     const int a_acc_off = g.pair ? g.kb * blk_bytes : blk_bytes;
@@ -152,7 +174,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
 
     const int m0 = blockIdx.y * GM_MAX_N;
     const int m_end = min(g.m_rows, m0 + GM_MAX_N);
-    const int mma_n = ((m_end - m0) + 15) & ~15;
+    const int mma_n = STACKED ? 2 * g.box_n : ((m_end - m0) + 15) & ~15;
     const int kb_total = (g.K + GM_BK - 1) / GM_BK;
     const int k_stages = (kb_total + g.kb - 1) / g.kb;
     const int n_units = (g.units[0] + (g.pair ? 0 : g.units[1] + g.units[2])) * g.splits;
@@ -235,14 +257,15 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
                 const uint32_t st = ring + (uint32_t)s * stage_bytes;
                 const int blk = ks * g.kb;
                 // lane 0: accumulator 0's weights (or the whole 256-row box); lane 1: accumulator 1's
-                // weights when they come from matrix 1; lanes 2 and 3: the two terms of the activations
-                const CUtensorMap *mp = lane == 0 ? ma : (lane == 1 ? &map_a1 : (lane == 2 ? &map_b : &map_b_lo));
-                const uint32_t dst = lane == 0 ? st : (lane == 1 ? st + a_acc_off : st + a_bytes + (lane == 3 ? b_half : 0));
+                // weights when they come from matrix 1; lane 2: the activations, both terms (lanes 2 and
+                // 3 one each beyond 128 rows)
+                const CUtensorMap *mp = lane == 0 ? ma : (lane == 1 ? &map_a1 : &map_b);
+                const uint32_t dst = lane == 0 ? st : (lane == 1 ? st + a_acc_off : st + a_bytes + (lane == 3 ? b_blk : 0));
                 const int y = lane == 0 ? row : (lane == 1 ? g.row0[1] + unit_row : m0);
-                const bool weights = lane == 0 || (lane == 1 && g.pair), acts = lane == 2 || lane == 3;
+                const bool weights = lane == 0 || (lane == 1 && g.pair), acts = lane == 2 || (lane == 3 && !STACKED);
                 if ((weights && !(pass == 1 && early)) || (acts && pass == 1)) {
-                    if (g.three_d) tma_load_3d(dst, mp, &full_bar[s], 0, y, blk);
-                    else tma_load_2d(dst, mp, &full_bar[s], blk * GM_BK, y);
+                    if (g.three_d) tma_load_4d(dst, mp, &full_bar[s], 0, y, 0, blk);
+                    else tma_load_3d(dst, mp, &full_bar[s], blk * GM_BK, y, lane == 3 ? 1 : 0);
                 }
             }
             if (pass == 0 && it >= (uint32_t)g.stages) break;
@@ -279,17 +302,25 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
                     const uint32_t b_addr = a_addr + a_bytes;
                     for (int j = 0; j < g.kb; j++) {
                         if (ks * g.kb + j >= kb_total) break;  // a box's last k-block may lie outside K
+                        const uint64_t db = umma_desc_sw128(b_addr + j * 2 * b_blk), dl = db + (uint64_t)(b_blk >> 4);
+                        const uint64_t da0 = umma_desc_sw128(a_addr + j * a_blk_stride), da1 = da0 + (uint64_t)(a_acc_off >> 4);
+                        // 16 elements on = 32 bytes on (the descriptors count in 16-byte units)
+                        if (STACKED) {
 #pragma unroll
-                        for (int kk = 0; kk < GM_BK / 16; kk++) {
-                            const uint64_t db = umma_desc_sw128(b_addr + j * b_blk + kk * 32);
-                            const uint64_t dl = umma_desc_sw128(b_addr + b_half + j * b_blk + kk * 32);
-                            const uint64_t da0 = umma_desc_sw128(a_addr + j * a_blk_stride + kk * 32);
-                            const uint64_t da1 = umma_desc_sw128(a_addr + j * a_blk_stride + kk * 32 + a_acc_off);
-                            umma_bf16(d0, da0, db, idesc, accum);
-                            umma_bf16(d0, da0, dl, idesc, 1);
-                            umma_bf16(d0 + mma_n, da1, db, idesc, accum);
-                            umma_bf16(d0 + mma_n, da1, dl, idesc, 1);
-                            accum = 1;
+                            for (int kk = 0; kk < GM_BK / 16; kk++) {
+                                umma_bf16(d0, da0 + kk * 2, db + kk * 2, idesc, accum);
+                                umma_bf16(d0 + mma_n, da1 + kk * 2, db + kk * 2, idesc, accum);
+                                accum = 1;
+                            }
+                        } else {
+#pragma unroll
+                            for (int kk = 0; kk < GM_BK / 16; kk++) {
+                                umma_bf16(d0, da0 + kk * 2, db + kk * 2, idesc, accum);
+                                umma_bf16(d0, da0 + kk * 2, dl + kk * 2, idesc, 1);
+                                umma_bf16(d0 + mma_n, da1 + kk * 2, db + kk * 2, idesc, accum);
+                                umma_bf16(d0 + mma_n, da1 + kk * 2, dl + kk * 2, idesc, 1);
+                                accum = 1;
+                            }
                         }
                     }
                     umma_commit(&empty_bar[s]);  // the stage is free once these MMAs have read it
@@ -308,6 +339,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
         tc.acc_stride = mma_n;
         tc.xchg = xchg;
         tc.unit_rows = g.unit_rows;
+        tc.lo_off = g.box_n;
         uint32_t unit_it = 0;
         bool ok = true;
         for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x, unit_it++) {
@@ -317,7 +349,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
             if (!(ok = mbar_wait(&acc_full[buf], bph, giving_up, g.status))) break;
             tc_fence_after();
             tc.taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * acc_cols);
-            epi.tile(tc);
+            epi.template tile<STACKED>(tc);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[buf]);
@@ -347,6 +379,7 @@ struct QkvEnd {
     float *partial;      // scratch for split sums, or NULL
     int Hq, Hkv, hd, S;
 
+    template <bool STACKED>
     __device__ void tile(const TileCtx &t) const
     {
         const int half = hd >> 1;
@@ -359,7 +392,7 @@ struct QkvEnd {
             const bool hi = i >= half;
             for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
                 float v[GM_CHUNK];
-                tmem_ld16(t.taddr + a * t.acc_stride + c0, v);
+                t.load<STACKED>(a, c0, v);
                 if (partial) {
                     if (n < n_rows_mat) {
 #pragma unroll
@@ -442,13 +475,14 @@ struct ResidEnd {
     float *h;  // [rows][n_out]
     int n_out, atomic;
 
+    template <bool STACKED>
     __device__ void tile(const TileCtx &t) const
     {
         for (int a = 0; a < 2; a++) {
             const int n = t.unit_row + a * GM_BM + t.row;
             for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
                 float v[GM_CHUNK];
-                tmem_ld16(t.taddr + a * t.acc_stride + c0, v);
+                t.load<STACKED>(a, c0, v);
                 if (n >= n_out) continue;
 #pragma unroll
                 for (int c = 0; c < GM_CHUNK; c++) {
@@ -468,13 +502,14 @@ struct GateUpEnd {
     bf16 *u, *u_lo;  // [rows][F]: u + u_lo carries the activation to 16 significant bits
     int F;
 
+    template <bool STACKED>
     __device__ void tile(const TileCtx &t) const
     {
         const int f = t.unit_row + t.row;
         for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
             float gt[GM_CHUNK], up[GM_CHUNK];
-            tmem_ld16(t.taddr + c0, gt);
-            tmem_ld16(t.taddr + t.acc_stride + c0, up);
+            t.load<STACKED>(0, c0, gt);
+            t.load<STACKED>(1, c0, up);
             if (f >= F || t.row >= t.unit_rows) continue;
 #pragma unroll
             for (int c = 0; c < GM_CHUNK; c++) {
@@ -497,6 +532,7 @@ struct HeadEnd {
     float *logits;  // optional [n_seq][V]
     int lo, hi, V;
 
+    template <bool STACKED>
     __device__ void tile(const TileCtx &t) const
     {
         const int lane = threadIdx.x & 31;
@@ -504,7 +540,7 @@ struct HeadEnd {
             const int id = lo + t.unit_row + a * GM_BM + t.row;
             for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
                 float v[GM_CHUNK];
-                tmem_ld16(t.taddr + a * t.acc_stride + c0, v);
+                t.load<STACKED>(a, c0, v);
 #pragma unroll
                 for (int c = 0; c < GM_CHUNK; c++) {
                     const int m = t.m0 + c0 + c;
