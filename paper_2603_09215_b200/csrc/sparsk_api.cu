@@ -761,7 +761,7 @@ cudaError_t launch_gemm(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1, con
 
 cudaError_t run_norm(sparsk_ctx *c, const float *h, const bf16 *gain, const int *row_idx, int n_rows)
 {
-    return launch(c, rmsnorm_rows_kernel, dim3(n_rows), dim3(256), 0, h, gain, row_idx, c->xnorm, c->xnorm_lo, n_rows,
+    return launch(c, rmsnorm_rows_kernel, dim3(n_rows), dim3(RN_THREADS), 0, h, gain, row_idx, c->xnorm, c->xnorm_lo, n_rows,
                   c->dm.d_model, c->dm.rms_eps);
 }
 
@@ -797,8 +797,9 @@ cudaError_t run_layer_tc_front(sparsk_ctx *c, int layer, float *h, const RowSet 
         ep.S = d.max_seq_len; ep.partial = g.splits > 1 ? c->qkv_part : nullptr;
         if ((e = launch_gemm(c, c->tm_wq[li], c->tm_wk[li], c->tm_wv[li], c->tm_x, g, ep)) != cudaSuccess) return e;
         if (g.splits > 1 &&
-            (e = launch(c, qkv_finish_kernel, dim3(M), dim3(256), 0, c->qkv_part, c->qbuf, kc, vc, (const float2 *)c->rope,
-                        rs.slot, rs.pos, M, d.n_q_heads, d.n_kv_heads, d.head_dim, d.max_seq_len)) != cudaSuccess)
+            (e = launch(c, qkv_finish_kernel, dim3(M, div_up((d.n_q_heads + 2 * d.n_kv_heads) * (d.head_dim / 2), QF_THREADS)),
+                        dim3(QF_THREADS), 0, c->qkv_part, c->qbuf, kc, vc, (const float2 *)c->rope,
+                        rs.slot, rs.pos, d.n_q_heads, d.n_kv_heads, d.head_dim, d.max_seq_len)) != cudaSuccess)
             return e;
     }
     c->cur_class = KC_MISC;

@@ -57,7 +57,9 @@ struct PerDevice {
 // writes are visible).  Every kernel here waits before it completes, so completion is transitive:
 // when a kernel's wait returns, everything before it in the stream is done.  The early start is
 // what lets a weight-streaming kernel issue its first weight copies (which depend on nothing)
-// while a small kernel between two of them is still running.
+// while a small kernel between two of them is still running.  The bookkeeping kernels of a step and
+// the copies that stage a row set never let go early, so what they wrote is visible to every kernel
+// of the pass that follows two or more launches later, before its wait as well.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
 

@@ -433,41 +433,42 @@ struct QkvEnd {
 
 // Finishes a q/k/v product whose inner dimension was cut across CTAs: reads the summed row from
 // the scratch, applies the rotary embedding, writes q and appends k, v to the cache, and clears
-// the scratch for the next product.  One block per activation row.
-static __global__ void __launch_bounds__(256) qkv_finish_kernel(float *__restrict__ partial, float *__restrict__ q_out,
+// the scratch for the next product.  Latency is all there is to it, so every thread owns one pair
+// (i, i + hd/2) of one head and nothing waits for anything twice: grid (rows, pairs / 256), with the
+// row's slot, position and rotary factors fetched while the product still runs (the row set of a
+// pass is complete before the pass's first kernel starts; see griddep_wait).  One block per row
+// that walked its pairs one batch of 256 after another held a layer up for 6.8 us at 12 rows, this
+// 2.4 (first dependent load to last store).
+constexpr int QF_THREADS = 256;
+static __global__ void __launch_bounds__(QF_THREADS) qkv_finish_kernel(float *__restrict__ partial, float *__restrict__ q_out,
                                                          kv_t *__restrict__ kc, kv_t *__restrict__ vc,
                                                          const float2 *__restrict__ rope,
                                                          const int *__restrict__ row_slot,
-                                                         const int *__restrict__ row_pos, int n_rows, int Hq, int Hkv,
-                                                         int hd, int S)
+                                                         const int *__restrict__ row_pos, int Hq, int Hkv, int hd, int S)
 {
     griddep_launch();
-    griddep_wait();
-    const int m = blockIdx.x;
-    if (m >= n_rows) return;
-    const int half = hd >> 1, width = (Hq + 2 * Hkv) * hd;
-    float *src = partial + (size_t)m * width;
+    const int m = blockIdx.x, half = hd >> 1, p = blockIdx.y * QF_THREADS + threadIdx.x;
+    const int head = p / half, j = p % half, n_heads = Hq + 2 * Hkv;
+    const bool on = head < n_heads;
     const int slot = row_slot[m], pos = row_pos[m];
-    // q and k heads: one thread per rotary pair
-    for (int p = threadIdx.x; p < (Hq + Hkv) * half; p += blockDim.x) {
-        const int head = p / half, j = p % half;
-        const float a = src[head * hd + j], b = src[head * hd + j + half];
-        const float2 cs = rope[(size_t)pos * half + j];
-        const float ra = a * cs.x - b * cs.y, rb = b * cs.x + a * cs.y;
-        if (head < Hq) {
-            float *dst = q_out + (size_t)m * Hq * hd + head * hd + j;
-            dst[0] = ra;
-            dst[half] = rb;
-        } else {
-            kv_t *dst = kc + (((size_t)slot * Hkv + (head - Hq)) * S + pos) * hd + j;
-            dst[0] = to_kv(ra);
-            dst[half] = to_kv(rb);
-        }
+    const float2 cs = head < Hq + Hkv ? rope[(size_t)pos * half + j] : make_float2(1.f, 0.f);  // values do not turn
+    griddep_wait();
+    if (!on) return;
+    float *src = partial + (size_t)m * n_heads * hd + head * hd + j;
+    const float a = __ldcg(src), b = __ldcg(src + half);
+    const float ra = a * cs.x - b * cs.y, rb = b * cs.x + a * cs.y;
+    if (head < Hq) {
+        float *dst = q_out + (size_t)m * Hq * hd + head * hd + j;
+        dst[0] = ra;
+        dst[half] = rb;
+    } else {
+        const bool key = head < Hq + Hkv;
+        kv_t *dst = (key ? kc : vc) + (((size_t)slot * Hkv + (head - Hq - (key ? 0 : Hkv))) * S + pos) * hd + j;
+        dst[0] = to_kv(ra);
+        dst[half] = to_kv(rb);
     }
-    for (int i = threadIdx.x; i < Hkv * hd; i += blockDim.x)
-        vc[(((size_t)slot * Hkv + i / hd) * S + pos) * hd + i % hd] = to_kv(src[(Hq + Hkv) * hd + i]);
-    __syncthreads();
-    for (int i = threadIdx.x; i < width; i += blockDim.x) src[i] = 0.f;
+    src[0] = 0.f;
+    src[half] = 0.f;
 }
 
 // h[m][n] += (W x_m)[n]; with the inner dimension cut across CTAs the partial sums meet in h.
@@ -560,41 +561,64 @@ struct HeadEnd {
 };
 
 // RMSNorm of selected fp32 rows into the activation matrices the GEMM reads, as two bf16 terms:
-// x + x_lo = h[row_idx ? row_idx[i] : i] / sqrt(mean(h^2) + eps) * gain.
-static __global__ void __launch_bounds__(256) rmsnorm_rows_kernel(const float *__restrict__ h, const bf16 *__restrict__ gain,
+// x + x_lo = h[row_idx ? row_idx[i] : i] / sqrt(mean(h^2) + eps) * gain.  One block per row.  Latency
+// is all there is to it: the gains (cold weights) are fetched while the previous kernel still
+// runs, and a row of up to 8,192 numbers makes one trip from the L2 into registers.  Between the
+// last store of the product before and the first of the product after it: 4.7 us at 12 rows of
+// 3,584 numbers, 6.9 with two trips and cold gains.
+constexpr int RN_THREADS = 512, RN_KEEP = 2;  // 8 numbers per thread and pass; passes kept in registers
+static __global__ void __launch_bounds__(RN_THREADS) rmsnorm_rows_kernel(const float *__restrict__ h, const bf16 *__restrict__ gain,
                                                            const int *__restrict__ row_idx, bf16 *__restrict__ x,
                                                            bf16 *__restrict__ x_lo, int n_rows, int K, float eps)
 {
-    __shared__ float red[8];
+    __shared__ float red[RN_THREADS / 32];
     griddep_launch();
+    const int i = blockIdx.x, k0 = threadIdx.x * 8;
+    uint4 gn[RN_KEEP];
+#pragma unroll
+    for (int p = 0; p < RN_KEEP; p++)
+        gn[p] = k0 + p * RN_THREADS * 8 < K ? *reinterpret_cast<const uint4 *>(gain + k0 + p * RN_THREADS * 8) : make_uint4(0u, 0u, 0u, 0u);
     griddep_wait();
-    const int i = blockIdx.x;
     if (i >= n_rows) return;
     const float *src = h + (size_t)(row_idx ? row_idx[i] : i) * K;
+    float4 v[RN_KEEP][2];
     float ss = 0.f;
-    for (int k = threadIdx.x * 4; k < K; k += 256 * 4) {
-        const float4 v = *reinterpret_cast<const float4 *>(src + k);
-        ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+    auto square = [&](const float4 &a, const float4 &b) {
+        ss += a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w + b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w;
+    };
+#pragma unroll
+    for (int p = 0; p < RN_KEEP; p++) {
+        const int k = k0 + p * RN_THREADS * 8;
+        v[p][0] = k < K ? *reinterpret_cast<const float4 *>(src + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[p][1] = k < K ? *reinterpret_cast<const float4 *>(src + k + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+#pragma unroll
+    for (int p = 0; p < RN_KEEP; p++) square(v[p][0], v[p][1]);
+    for (int k = k0 + RN_KEEP * RN_THREADS * 8; k < K; k += RN_THREADS * 8)
+        square(*reinterpret_cast<const float4 *>(src + k), *reinterpret_cast<const float4 *>(src + k + 4));
     ss = warp_sum(ss);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
     __syncthreads();
     float tot = 0.f;
 #pragma unroll
-    for (int w = 0; w < 8; w++) tot += red[w];
+    for (int w = 0; w < RN_THREADS / 32; w++) tot += red[w];
     const float inv = rsqrtf(tot / (float)K + eps);
-    for (int k = threadIdx.x * 8; k < K; k += 256 * 8) {
-        const float4 a = *reinterpret_cast<const float4 *>(src + k);
-        const float4 b = *reinterpret_cast<const float4 *>(src + k + 4);
-        float gn[8];
-        unpack8(*reinterpret_cast<const uint4 *>(gain + k), gn);
-        const float v[8] = {a.x * inv * gn[0], a.y * inv * gn[1], a.z * inv * gn[2], a.w * inv * gn[3],
-                            b.x * inv * gn[4], b.y * inv * gn[5], b.z * inv * gn[6], b.w * inv * gn[7]};
+    auto put = [&](int k, const float4 &a, const float4 &b, const uint4 &g) {
+        float gf[8];
+        unpack8(g, gf);
+        const float o[8] = {a.x * inv * gf[0], a.y * inv * gf[1], a.z * inv * gf[2], a.w * inv * gf[3],
+                            b.x * inv * gf[4], b.y * inv * gf[5], b.z * inv * gf[6], b.w * inv * gf[7]};
         uint4 hi, lo;
-        split8(v, hi, lo);
+        split8(o, hi, lo);
         *reinterpret_cast<uint4 *>(x + (size_t)i * K + k) = hi;
         *reinterpret_cast<uint4 *>(x_lo + (size_t)i * K + k) = lo;
-    }
+    };
+#pragma unroll
+    for (int p = 0; p < RN_KEEP; p++)
+        if (k0 + p * RN_THREADS * 8 < K) put(k0 + p * RN_THREADS * 8, v[p][0], v[p][1], gn[p]);
+    for (int k = k0 + RN_KEEP * RN_THREADS * 8; k < K; k += RN_THREADS * 8)
+        put(k, *reinterpret_cast<const float4 *>(src + k), *reinterpret_cast<const float4 *>(src + k + 4),
+            *reinterpret_cast<const uint4 *>(gain + k));
 }
 
 }  // namespace sparsk

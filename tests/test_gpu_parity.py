@@ -300,6 +300,22 @@ def test_tcgen05_passes_of_every_width(util, B):
     P.close()
 
 
+@pytest.mark.parametrize("d_model", [4104, 8456])
+def test_wide_rows_on_the_tcgen05_path(util, d_model):
+    """Residual rows wider than what the RMSNorm kernel's threads cover in one pass (4,096 numbers) and
+    than what they keep in registers (8,192), not multiples of 64."""
+    dims = synth.model_dims(dict(MICRO64, d_model=d_model, n_layers=2, d_ffn=96), 1, 2, 0)
+    w = synth.make_weights(dims, seed=2)
+    prompts = synth.make_prompts(dims, 5, 4, 9, seed=3)
+    P = util.Pair(dims, w, 5, 24, 1)
+    P.prefill(prompts)
+    for g in range(5):
+        mc = [synth.interleave(g + i, 1, 4) for i in range(5)]
+        P.step([m for m, _ in mc], [c for _, c in mc])
+    P.check_cache(4, range(1, 3), P.g.slot_state(4)[0] - P.g.slot_state(4)[1])
+    P.close()
+
+
 def test_timeout_is_reported_once_and_the_context_recovers(util):
     """A bounded in-kernel wait that runs out: the persistent kernel is told a grid-barrier count
     that no CTA can reach (a host-side test hook; nothing faults or hangs), its wait ends at the
