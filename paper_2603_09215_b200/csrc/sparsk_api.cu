@@ -264,8 +264,9 @@ size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
     return align_up(w.off, 256);
 }
 
+// cluster: CTAs per cluster along x
 template <class... KArgs, class... Args>
-cudaError_t launch(sparsk_ctx *c, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args)
+cudaError_t launch_clusters(sparsk_ctx *c, int cluster, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args)
 {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
@@ -273,12 +274,17 @@ cudaError_t launch(sparsk_ctx *c, void (*kern)(KArgs...), dim3 grid, dim3 block,
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = c->stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
     if (c->pdl) {
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = cluster;
+        attr[cfg.numAttrs].val.clusterDim.y = 1;
+        attr[cfg.numAttrs++].val.clusterDim.z = 1;
     }
     c->launches++;
     const bool timed = ((c->time_class == c->cur_class && c->time_class != KC_MISC) || c->time_class == KC_ALL) &&
@@ -290,6 +296,12 @@ cudaError_t launch(sparsk_ctx *c, void (*kern)(KArgs...), dim3 grid, dim3 block,
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
     if (timed) cudaEventRecord(c->tev[c->tev_used++], c->stream);
     return e;
+}
+
+template <class... KArgs, class... Args>
+cudaError_t launch(sparsk_ctx *c, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args)
+{
+    return launch_clusters(c, 1, kern, grid, block, smem, args...);
 }
 
 // ---------------------------------------------------------------- GEMV dispatch
@@ -608,16 +620,15 @@ bool encode_maps(EncodeTiledFn fn, TmaPair *m, const void *base, size_t rows, si
 }
 
 // Descriptors of an operand of the tcgen05 GEMMs: a row-major bf16 matrix, or (lo) the two planes
-// of an activation matrix.  A box of up to 128 rows carries the same rows of every plane, the lo
-// tile behind the hi tile, a higher one a single plane's.  m2 takes one 64-element block per copy
-// (view [cols][rows][plane]), m3 two (view [64][rows][plane][cols/64]; not for single planes of two).
+// of an activation matrix: a box carries the same rows of every plane, the lo tile behind the hi
+// tile.  m2 takes one 64-element block per copy (view [cols][rows][plane]), m3 two (view
+// [64][rows][plane][cols/64]).
 bool encode_gemm_maps(EncodeTiledFn fn, TmaPair *m, const bf16 *hi, const bf16 *lo, size_t rows, size_t cols, int box_rows)
 {
     memset(m, 0, sizeof *m);
     if (!hi) return true;
     const cuuint64_t planes = lo ? 2 : 1, row = (cuuint64_t)cols * 2, plane = lo ? (cuuint64_t)((const char *)lo - (const char *)hi) : row * rows;
-    const bool whole = !lo || box_rows <= GM_MAX_N / 2;
-    const cuuint32_t es[4] = {1, 1, 1, 1}, box_planes = whole ? (cuuint32_t)planes : 1u;
+    const cuuint32_t es[4] = {1, 1, 1, 1}, box_planes = (cuuint32_t)planes;
     {
         const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, planes}, strides[2] = {row, plane};
         const cuuint32_t box[3] = {(cuuint32_t)GM_BK, (cuuint32_t)box_rows, box_planes};
@@ -626,7 +637,7 @@ bool encode_gemm_maps(EncodeTiledFn fn, TmaPair *m, const bf16 *hi, const bf16 *
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return false;
     }
-    if (cols % GM_BK == 0 && whole) {
+    if (cols % GM_BK == 0) {
         const cuuint64_t dims[4] = {(cuuint64_t)GM_BK, (cuuint64_t)rows, planes, (cuuint64_t)(cols / GM_BK)};
         const cuuint64_t strides[3] = {row, plane, (cuuint64_t)GM_BK * 2};
         const cuuint32_t box[4] = {(cuuint32_t)GM_BK, (cuuint32_t)box_rows, box_planes, 2};
@@ -704,24 +715,24 @@ bool build_maps(sparsk_ctx *c)
     return ok;
 }
 
-// Activation rows per copy: as many as there are, in steps of 16 (a copy of rows that do not exist
+// Activation rows per copy: as many as a CTA takes, in steps of 16 (a copy of rows that do not exist
 // costs L2 traffic and ring space: 70 rows in a 128-row box left room for one k-block per copy).
-int box_index(int m_rows) { return (std::min(m_rows, GM_MAX_N) + 15) / 16 - 1; }
+int box_index(int rows_per_cta) { return (rows_per_cta + 15) / 16 - 1; }
 
-template <class Epi, bool STACKED>
+template <class Epi, bool DUO>
 cudaError_t launch_gemm_inst(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1, const TmaPair &a2, const TmaPair *b_maps,
                         GemmArgs g, const Epi &epi)
 {
     static PerDevice<bool> attr_done;
     bool &attr_set = attr_done.here();
     constexpr int SMEM_BUDGET = 220 * 1024;
-    auto kern = wsgemm_kernel<Epi, STACKED>;
+    auto kern = wsgemm_kernel<Epi, DUO>;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    const int bi = box_index(g.m_rows);
+    const int bi = box_index(DUO ? (std::min(g.m_rows, GM_MAX_N) + 1) / 2 : g.m_rows);
     g.box_n = 16 * (bi + 1);
     const int blk_bytes = g.pair ? g.unit_rows * GM_BK * 2 : GM_BLK_BYTES;
     // the ring may be told to stay small enough for two CTAs (of this kernel or of the next one in
@@ -731,7 +742,7 @@ cudaError_t launch_gemm_inst(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1
     auto plan = [&](int budget) {
         const int room = budget - 1024 - GM_XCHG_BYTES;
         // two k-blocks per copy whenever the inner dimension allows the 3-D view and two stages fit
-        g.three_d = (g.K % GM_BK == 0) && STACKED && 2 * stage_bytes(2) <= room && c->tc_kb != 1;
+        g.three_d = (g.K % GM_BK == 0) && !DUO && 2 * stage_bytes(2) <= room && c->tc_kb != 1;
         g.kb = g.three_d ? 2 : 1;
         g.stages = std::min(GM_MAX_STAGES, room / stage_bytes(g.kb));
         return g.stages >= 2;
@@ -743,20 +754,22 @@ cudaError_t launch_gemm_inst(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1
     g.splits = std::max(1, std::min(g.splits, k_stages));
     const size_t smem = 1024 + (size_t)g.stages * stage_bytes(g.kb) + GM_XCHG_BYTES;
     const int per_sm = (smem + 1024) * 2 <= 227 * 1024 ? std::max(1, c->gemm_cps) : 1;  // CTAs of this launch that fit an SM
-    const int grid_x = std::max(1, std::min(c->n_sm * per_sm, n_units * g.splits));
+    const int grid_x = DUO ? 2 * std::max(1, std::min(c->n_sm / 2, (n_units + 1) / 2 * g.splits))
+                           : std::max(1, std::min(c->n_sm * per_sm, n_units * g.splits));
     const int grid_y = (g.m_rows + GM_MAX_N - 1) / GM_MAX_N;
     if (g.three_d)
         return launch(c, kern, dim3(grid_x, grid_y), dim3(GM_THREADS), smem, a0.m3, a1.m3, a2.m3, b_maps[bi].m3, g,
                       epi);
-    return launch(c, kern, dim3(grid_x, grid_y), dim3(GM_THREADS), smem, a0.m2, a1.m2, a2.m2, b_maps[bi].m2, g, epi);
+    return launch_clusters(c, DUO ? 2 : 1, kern, dim3(grid_x, grid_y), dim3(GM_THREADS), smem, a0.m2, a1.m2, a2.m2, b_maps[bi].m2,
+                           g, epi);
 }
 
 template <class Epi>
 cudaError_t launch_gemm(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1, const TmaPair &a2, const TmaPair *b_maps,
                         const GemmArgs &g, const Epi &epi)
 {
-    return g.m_rows <= GM_MAX_N / 2 ? launch_gemm_inst<Epi, true>(c, a0, a1, a2, b_maps, g, epi)
-                                    : launch_gemm_inst<Epi, false>(c, a0, a1, a2, b_maps, g, epi);
+    return g.m_rows <= GM_MAX_N / 2 ? launch_gemm_inst<Epi, false>(c, a0, a1, a2, b_maps, g, epi)
+                                    : launch_gemm_inst<Epi, true>(c, a0, a1, a2, b_maps, g, epi);
 }
 
 cudaError_t run_norm(sparsk_ctx *c, const float *h, const bf16 *gain, const int *row_idx, int n_rows)

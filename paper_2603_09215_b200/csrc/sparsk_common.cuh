@@ -158,6 +158,17 @@ __device__ __forceinline__ unsigned long long argmax_key(float logit, int id)
 constexpr unsigned long long WAIT_TIMEOUT_NS = 2000000000ull;
 
 // ------------------------------------------------------------------ mbarrier, TMA and timer wrappers
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// Every thread of every CTA of the cluster.
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ unsigned long long global_ns()
 {
@@ -177,9 +188,31 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
+// The same barrier of CTA `rank` of the cluster: what this CTA wrote before is visible to whoever
+// acquires that phase at cluster scope.
+__device__ __forceinline__ void mbar_arrive_remote(uint64_t *bar, uint32_t rank)
+{
+    asm volatile(
+        "{\n\t.reg .b32 a;\n\t"
+        "mapa.shared::cluster.u32 a, %0, %1;\n\t"
+        "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [a];\n\t}"
+        ::"r"(smem_u32(bar)), "r"(rank)
+        : "memory");
+}
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity)
 {
     uint32_t ok;
+    if (CLUSTER) {
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity)
+            : "memory");
+        return ok != 0;
+    }
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -190,13 +223,15 @@ __device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity)
     return ok != 0;
 }
 // Bounded wait for a phase of an mbarrier.  Returns false if the CTA is giving up (another
-// thread did, or this wait outlasted `limit_ns`); the caller then leaves its loop.
+// thread did, or this wait outlasted `limit_ns`); the caller then leaves its loop.  CLUSTER: threads of
+// another CTA arrive on the barrier.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *giving_up, int *status,
                                           unsigned long long limit_ns = WAIT_TIMEOUT_NS)
 {
     unsigned long long t0 = 0;
     for (uint32_t spin = 0;; ++spin) {
-        if (mbar_test(bar, parity)) return true;
+        if (mbar_test<CLUSTER>(bar, parity)) return true;
         if (spin > 64) __nanosleep(32);
         if ((spin & 255u) == 255u) {
             if (*giving_up) return false;

@@ -27,6 +27,12 @@
 // 43 GB/s, as much as its share of HBM.  The two products land in columns of their own, which
 // the ending adds.  Event-timed launches, before and after: gate/up of the 40-layer shape 60 -> 50 us
 // at 16 rows and 65 -> 59 at 64, down of the 28-layer shape 35.2 -> 33.2 at 12 rows.
+// Beyond 128 rows (prefill, wide batches) the products are bound by the L2: with 256 rows a CTA takes
+// in 64 KB of activations for every 32 KB of weights.  Two CTAs of a cluster then work as one
+// (cta_group::2): each streams its own unit's weights but only half of the activation rows, and an
+// MMA of 256 weight rows reads both halves.  The CTA of rank 0 issues the MMAs for both; the other's
+// warp 1 passes its filled stages on.  Gate/up of the 28-layer shape at 256 rows 115 -> 105 us, a CTA
+// taking in 64 KB a k-block instead of 96; six ragged prompts 214.7 -> 207.1 ms.
 // Consecutive MMAs go to different accumulators: one that adds to the accumulator of the MMA before
 // it waits for it (six ragged prompts at 256 rows a pass: 218.7 -> 214.7 ms).
 // Accumulators are double buffered in TMEM so a tile's epilogue overlaps the next tile's MMAs.
@@ -43,7 +49,7 @@ namespace sparsk {
 constexpr int GM_THREADS = 192;
 constexpr int GM_BM = 128;                     // weight rows per accumulator (UMMA M)
 constexpr int GM_BK = 64;                      // inner elements per k-block: one 128-byte swizzle span
-constexpr int GM_BOXES = 16;                   // heights of an activation copy: 16, 32, ..., 256 rows
+constexpr int GM_BOXES = 8;                    // heights of an activation copy: 16, 32, ..., 128 rows
 constexpr int GM_MAX_N = 256;                  // activation rows per launch block (UMMA N limit)
 constexpr int GM_BLK_BYTES = GM_BM * GM_BK * 2;  // one accumulator's weights for one k-block: 16 KB
 constexpr int GM_MAX_STAGES = 6;
@@ -68,7 +74,7 @@ struct GemmArgs {
     int pair;      // 1: accumulator 1 comes from matrix 1
     int unit_rows; // pair: weight rows per accumulator (a multiple of 8)
     int m_rows;    // activation rows of the whole launch; block y owns rows [256 y, 256 y + 256)
-    int box_n;     // activation rows per TMA box (a multiple of 16, at most 256)
+    int box_n;     // activation rows per TMA box (a multiple of 16, at most 128; a CTA pair: half of the block's)
     int stages;    // ring depth
     int kb;        // k-blocks per stage (1 or 2)
     int three_d;   // 1: the descriptors are the [64][rows][plane][K/64] views (needs K % 64 == 0)
@@ -86,23 +92,40 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr)
            (2ull << 61);
 }
 // Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = 128, N = n.
-__device__ __forceinline__ uint32_t umma_idesc_bf16(int n)
+// (M = 256 for a CTA pair).
+__device__ __forceinline__ uint32_t umma_idesc_bf16(int n, int m)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(GM_BM >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
+template <bool DUO>
 __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc, int accumulate)
 {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
-        : "memory");
+    if (DUO)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(tmem_d), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
+            : "memory");
 }
+// Arrive on a barrier (DUO: on the same barrier of both CTAs) when the MMAs issued so far are done.
+template <bool DUO = false>
 __device__ __forceinline__ void umma_commit(uint64_t *bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
+    if (DUO)
+        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                     ::"r"(smem_u32(bar)), "h"((unsigned short)3)
+                     : "memory");
+    else
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+                     : "memory");
 }
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[16])
 {
@@ -127,16 +150,16 @@ struct TileCtx {
     int acc_stride;  // columns between accumulator 0 and accumulator 1
     float *xchg;     // [GM_CHUNK][128] floats shared by the 128 epilogue threads
     int unit_rows;   // pair: rows of an accumulator that are the unit's
-    int lo_off;      // stacked terms: columns from the hi term's product to the lo term's
+    int lo_off;      // columns from the hi term's product to the lo term's (0: one accumulator holds both)
 
     // 16 activation rows (from c0 on) of accumulator a
-    template <bool STACKED>
+    template <bool DUO>
     __device__ __forceinline__ void load(int a, int c0, float (&v)[GM_CHUNK]) const
     {
         const uint32_t at = taddr + (uint32_t)(a * acc_stride + c0);
         uint32_t r[GM_CHUNK], s[GM_CHUNK];
         tmem_ld16_nowait(at, r);
-        if (STACKED) {
+        if (!DUO) {
             tmem_ld16_nowait(at + (uint32_t)lo_off, s);
             tmem_ld_wait();
 #pragma unroll
@@ -150,8 +173,9 @@ struct TileCtx {
 };
 
 // ------------------------------------------------------------------ kernel
-// STACKED: the two terms of the activations are one operand (box_n <= 128; kb is 1 without).
-template <class Epi, bool STACKED>
+// DUO: a cluster of two CTAs on two units of the same cut (kb is 1); otherwise the two terms of the
+// activations are one operand.
+template <class Epi, bool DUO>
 __global__ void __launch_bounds__(GM_THREADS, 1)
     wsgemm_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_a1,
                   const __grid_constant__ CUtensorMap map_a2, const __grid_constant__ CUtensorMap map_b,
@@ -176,10 +200,13 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
 
     const int m0 = blockIdx.y * GM_MAX_N;
     const int m_end = min(g.m_rows, m0 + GM_MAX_N);
-    const int mma_n = STACKED ? 2 * g.box_n : ((m_end - m0) + 15) & ~15;
+    const int mma_n = 2 * g.box_n;  // columns of an accumulator: both terms' rows, or both CTAs'
     const int kb_total = (g.K + GM_BK - 1) / GM_BK;
     const int k_stages = (kb_total + g.kb - 1) / g.kb;
-    const int n_units = (g.units[0] + (g.pair ? 0 : g.units[1] + g.units[2])) * g.splits;
+    const int rank = DUO ? (int)cluster_rank() : 0;
+    const int n_units0 = g.units[0] + (g.pair ? 0 : g.units[1] + g.units[2]);
+    const int n_units = (DUO ? (n_units0 + 1) / 2 : n_units0) * g.splits;  // work items: (unit or pair of units, cut)
+    const int u0 = DUO ? blockIdx.x >> 1 : blockIdx.x, u_step = DUO ? gridDim.x >> 1 : gridDim.x;
     // accumulator buffers: 2 when they fit, else 1
     const int acc_cols = 2 * mma_n;
     const int n_buf = (2 * acc_cols <= 512) ? 2 : 1;
@@ -188,25 +215,33 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < g.stages; s++) {
-            mbar_init(&full_bar[s], 1);
+            mbar_init(&full_bar[s], DUO && rank == 0 ? 2 : 1);  // own copies; the other CTA's
             mbar_init(&empty_bar[s], 1);
         }
         for (int b = 0; b < 2; b++) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 4);
+            mbar_init(&acc_empty[b], DUO ? 8 : 4);
         }
         giving_up_s = 0;
         never_s = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)),
-                     "r"(alloc_cols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if (DUO) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)),
+                         "r"(alloc_cols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)),
+                         "r"(alloc_cols)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     tc_fence_before();
     __syncthreads();
+    if (DUO) cluster_barrier();  // both CTAs' barriers are set up, both have their TMEM
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_s;
 
@@ -215,12 +250,13 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
     // touches anything, the MMA warp touches no global memory.
     griddep_launch();
 
-    // unit u -> (matrix, first row, split)
+    // work item u -> (matrix, first row, split) of this CTA's unit; the odd unit's partner lies behind
+    // the last row of its matrix: it copies zeros and its ending writes nothing
     auto locate = [&](int u, int &mat, int &unit_row, int &sp) {
-        int t = u / g.splits;
+        int t = DUO ? 2 * (u / g.splits) + rank : u / g.splits;
         sp = u % g.splits;
         mat = 0;
-        if (!g.pair) {
+        if (!g.pair && g.units[1]) {
             if (t >= g.units[0]) { t -= g.units[0]; mat = 1; }
             if (mat == 1 && t >= g.units[1]) { t -= g.units[1]; mat = 2; }
         }
@@ -238,7 +274,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
         // dependency; pass 1 is the whole loop, adding only the activations to those stages
         for (int pass = 0; pass < 2 && ok; pass++) {
         it = 0;
-        for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
+        for (int u = u0; u < n_units && ok; u += u_step) {
             int mat, unit_row, sp;
             locate(u, mat, unit_row, sp);
             const CUtensorMap *ma = mat == 0 ? &map_a0 : (mat == 1 ? &map_a1 : &map_a2);
@@ -259,15 +295,14 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
                 const uint32_t st = ring + (uint32_t)s * stage_bytes;
                 const int blk = ks * g.kb;
                 // lane 0: accumulator 0's weights (or the whole 256-row box); lane 1: accumulator 1's
-                // weights when they come from matrix 1; lane 2: the activations, both terms (lanes 2 and
-                // 3 one each beyond 128 rows)
+                // weights when they come from matrix 1; lane 2: the activations, both terms
                 const CUtensorMap *mp = lane == 0 ? ma : (lane == 1 ? &map_a1 : &map_b);
-                const uint32_t dst = lane == 0 ? st : (lane == 1 ? st + a_acc_off : st + a_bytes + (lane == 3 ? b_blk : 0));
-                const int y = lane == 0 ? row : (lane == 1 ? g.row0[1] + unit_row : m0);
-                const bool weights = lane == 0 || (lane == 1 && g.pair), acts = lane == 2 || (lane == 3 && !STACKED);
+                const uint32_t dst = lane == 0 ? st : (lane == 1 ? st + a_acc_off : st + a_bytes);
+                const int y = lane == 0 ? row : (lane == 1 ? g.row0[1] + unit_row : m0 + rank * g.box_n);
+                const bool weights = lane == 0 || (lane == 1 && g.pair), acts = lane == 2;
                 if ((weights && !(pass == 1 && early)) || (acts && pass == 1)) {
                     if (g.three_d) tma_load_4d(dst, mp, &full_bar[s], 0, y, 0, blk);
-                    else tma_load_3d(dst, mp, &full_bar[s], blk * GM_BK, y, lane == 3 ? 1 : 0);
+                    else tma_load_3d(dst, mp, &full_bar[s], blk * GM_BK, y, 0);
                 }
             }
             if (pass == 0 && it >= (uint32_t)g.stages) break;
@@ -282,23 +317,38 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = umma_idesc_bf16(mma_n);
+        if (DUO && rank != 0) {
+            // the other CTA issues: tell it of every stage that has filled here
+            if (lane == 0) {
+                uint32_t it = 0;
+                bool ok = true;
+                for (int u = u0; u < n_units && ok; u += u_step) {
+                    const int sp = u % g.splits;
+                    const int ks_beg = (int)((long)k_stages * sp / g.splits), ks_end = (int)((long)k_stages * (sp + 1) / g.splits);
+                    for (int ks = ks_beg; ks < ks_end; ks++, it++) {
+                        const int s = it % g.stages;
+                        if (!(ok = mbar_wait(&full_bar[s], (it / g.stages) & 1, giving_up, g.status))) break;
+                        mbar_arrive_remote(&full_bar[s], 0);
+                    }
+                }
+            }
+        } else if (lane == 0) {
+            const uint32_t idesc = umma_idesc_bf16(mma_n, DUO ? 2 * GM_BM : GM_BM);
             uint32_t it = 0, unit_it = 0;
             bool ok = true;
-            for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x, unit_it++) {
+            for (int u = u0; u < n_units && ok; u += u_step, unit_it++) {
                 const int sp = u % g.splits;
                 const int ks_beg = (int)((long)k_stages * sp / g.splits), ks_end = (int)((long)k_stages * (sp + 1) / g.splits);
                 const int buf = unit_it % n_buf;
                 const uint32_t bph = (unit_it / n_buf) & 1;
-                if (!(ok = mbar_wait(&acc_empty[buf], bph ^ 1, giving_up, g.status))) break;
+                if (!(ok = mbar_wait<DUO>(&acc_empty[buf], bph ^ 1, giving_up, g.status))) break;
                 tc_fence_after();
                 const uint32_t d0 = tmem_base + (uint32_t)(buf * acc_cols);
                 int accum = 0;
                 for (int ks = ks_beg; ks < ks_end; ks++, it++) {
                     const int s = it % g.stages;
                     const uint32_t ph = (it / g.stages) & 1;
-                    if (!(ok = mbar_wait(&full_bar[s], ph, giving_up, g.status))) break;
+                    if (!(ok = mbar_wait<DUO>(&full_bar[s], ph, giving_up, g.status))) break;
                     tc_fence_after();
                     const uint32_t a_addr = ring + (uint32_t)s * stage_bytes;
                     const uint32_t b_addr = a_addr + a_bytes;
@@ -307,27 +357,27 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
                         const uint64_t db = umma_desc_sw128(b_addr + j * 2 * b_blk), dl = db + (uint64_t)(b_blk >> 4);
                         const uint64_t da0 = umma_desc_sw128(a_addr + j * a_blk_stride), da1 = da0 + (uint64_t)(a_acc_off >> 4);
                         // 16 elements on = 32 bytes on (the descriptors count in 16-byte units)
-                        if (STACKED) {
+                        if (!DUO) {
 #pragma unroll
                             for (int kk = 0; kk < GM_BK / 16; kk++) {
-                                umma_bf16(d0, da0 + kk * 2, db + kk * 2, idesc, accum);
-                                umma_bf16(d0 + mma_n, da1 + kk * 2, db + kk * 2, idesc, accum);
+                                umma_bf16<DUO>(d0, da0 + kk * 2, db + kk * 2, idesc, accum);
+                                umma_bf16<DUO>(d0 + mma_n, da1 + kk * 2, db + kk * 2, idesc, accum);
                                 accum = 1;
                             }
                         } else {
 #pragma unroll
                             for (int kk = 0; kk < GM_BK / 16; kk++) {
-                                umma_bf16(d0, da0 + kk * 2, db + kk * 2, idesc, accum);
-                                umma_bf16(d0 + mma_n, da1 + kk * 2, db + kk * 2, idesc, accum);
-                                umma_bf16(d0, da0 + kk * 2, dl + kk * 2, idesc, 1);
-                                umma_bf16(d0 + mma_n, da1 + kk * 2, dl + kk * 2, idesc, 1);
+                                umma_bf16<DUO>(d0, da0 + kk * 2, db + kk * 2, idesc, accum);
+                                umma_bf16<DUO>(d0 + mma_n, da1 + kk * 2, db + kk * 2, idesc, accum);
+                                umma_bf16<DUO>(d0, da0 + kk * 2, dl + kk * 2, idesc, 1);
+                                umma_bf16<DUO>(d0 + mma_n, da1 + kk * 2, dl + kk * 2, idesc, 1);
                                 accum = 1;
                             }
                         }
                     }
-                    umma_commit(&empty_bar[s]);  // the stage is free once these MMAs have read it
+                    umma_commit<DUO>(&empty_bar[s]);  // the stage is free once these MMAs have read it
                 }
-                if (ok) umma_commit(&acc_full[buf]);
+                if (ok) umma_commit<DUO>(&acc_full[buf]);
             }
         }
     } else {
@@ -341,28 +391,33 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
         tc.acc_stride = mma_n;
         tc.xchg = xchg;
         tc.unit_rows = g.unit_rows;
-        tc.lo_off = g.box_n;
+        tc.lo_off = DUO ? 0 : g.box_n;
         uint32_t unit_it = 0;
         bool ok = true;
-        for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x, unit_it++) {
+        for (int u = u0; u < n_units && ok; u += u_step, unit_it++) {
             locate(u, tc.matrix, tc.unit_row, tc.split);
             const int buf = unit_it % n_buf;
             const uint32_t bph = (unit_it / n_buf) & 1;
             if (!(ok = mbar_wait(&acc_full[buf], bph, giving_up, g.status))) break;
             tc_fence_after();
             tc.taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * acc_cols);
-            epi.template tile<STACKED>(tc);
+            epi.template tile<DUO>(tc);
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[buf]);
+            if (lane == 0) {
+                if (DUO) mbar_arrive_remote(&acc_empty[buf], 0);
+                else mbar_arrive(&acc_empty[buf]);
+            }
         }
     }
     // ---------------------------------------------------------------- teardown
     tc_fence_before();
     __syncthreads();
+    if (DUO) cluster_barrier();  // neither CTA leaves while the other may still read its shared memory or arrive on its barriers
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(alloc_cols) : "memory");
+        if (DUO) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(alloc_cols) : "memory");
+        else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(alloc_cols) : "memory");
     }
 }
 
@@ -381,7 +436,7 @@ struct QkvEnd {
     float *partial;      // scratch for split sums, or NULL
     int Hq, Hkv, hd, S;
 
-    template <bool STACKED>
+    template <bool DUO>
     __device__ void tile(const TileCtx &t) const
     {
         const int half = hd >> 1;
@@ -394,7 +449,7 @@ struct QkvEnd {
             const bool hi = i >= half;
             for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
                 float v[GM_CHUNK];
-                t.load<STACKED>(a, c0, v);
+                t.load<DUO>(a, c0, v);
                 if (partial) {
                     if (n < n_rows_mat) {
 #pragma unroll
@@ -478,14 +533,14 @@ struct ResidEnd {
     float *h;  // [rows][n_out]
     int n_out, atomic;
 
-    template <bool STACKED>
+    template <bool DUO>
     __device__ void tile(const TileCtx &t) const
     {
         for (int a = 0; a < 2; a++) {
             const int n = t.unit_row + a * GM_BM + t.row;
             for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
                 float v[GM_CHUNK];
-                t.load<STACKED>(a, c0, v);
+                t.load<DUO>(a, c0, v);
                 if (n >= n_out) continue;
 #pragma unroll
                 for (int c = 0; c < GM_CHUNK; c++) {
@@ -505,14 +560,14 @@ struct GateUpEnd {
     bf16 *u, *u_lo;  // [rows][F]: u + u_lo carries the activation to 16 significant bits
     int F;
 
-    template <bool STACKED>
+    template <bool DUO>
     __device__ void tile(const TileCtx &t) const
     {
         const int f = t.unit_row + t.row;
         for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
             float gt[GM_CHUNK], up[GM_CHUNK];
-            t.load<STACKED>(0, c0, gt);
-            t.load<STACKED>(1, c0, up);
+            t.load<DUO>(0, c0, gt);
+            t.load<DUO>(1, c0, up);
             if (f >= F || t.row >= t.unit_rows) continue;
 #pragma unroll
             for (int c = 0; c < GM_CHUNK; c++) {
@@ -535,7 +590,7 @@ struct HeadEnd {
     float *logits;  // optional [n_seq][V]
     int lo, hi, V;
 
-    template <bool STACKED>
+    template <bool DUO>
     __device__ void tile(const TileCtx &t) const
     {
         const int lane = threadIdx.x & 31;
@@ -543,7 +598,7 @@ struct HeadEnd {
             const int id = lo + t.unit_row + a * GM_BM + t.row;
             for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
                 float v[GM_CHUNK];
-                t.load<STACKED>(a, c0, v);
+                t.load<DUO>(a, c0, v);
 #pragma unroll
                 for (int c = 0; c < GM_CHUNK; c++) {
                     const int m = t.m0 + c0 + c;

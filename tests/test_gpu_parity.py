@@ -300,6 +300,23 @@ def test_tcgen05_passes_of_every_width(util, B):
     P.close()
 
 
+@pytest.mark.parametrize("shape", ["tiny", "micro64"])
+@pytest.mark.parametrize("rows", [129, 161, 256, 300])
+def test_prefill_passes_beyond_128_rows(util, rows, shape):
+    """Products of more than 128 rows run on pairs of CTAs, each with half of the activation rows and a
+    unit of weight rows of its own: odd numbers of units, rows that do not split evenly, a second
+    block of rows."""
+    dims = synth.model_dims("tiny" if shape == "tiny" else MICRO64, 2, 3, 0)
+    w = synth.make_weights(dims, seed=4)
+    prompts = synth.make_prompts(dims, 2, 150, 260, seed=8)
+    P = util.Pair(dims, w, 2, 300, 2, prefill_rows=rows)
+    P.prefill(prompts)
+    for s_, p in enumerate(prompts):
+        P.check_cache(s_, range(1, dims["n_layers"] + 1), len(p) - 1)
+    P.step([0, 1], [0, 1])
+    P.close()
+
+
 @pytest.mark.parametrize("d_model", [4104, 8456])
 def test_wide_rows_on_the_tcgen05_path(util, d_model):
     """Residual rows wider than what the RMSNorm kernel's threads cover in one pass (4,096 numbers) and
