@@ -78,7 +78,7 @@ def load():
     for name in ("sparsk_decode_step", "sparsk_decode_step_host"):
         f = getattr(L, name)
         f.restype = C.c_int
-        f.argtypes = [vp, C.c_int32, i32p, vp, u8p, i32p, vp, vp]
+        f.argtypes = [vp, C.c_int32, vp, vp, vp, vp, vp, vp]   # (plain addresses: a typed pointer costs 2 us to make)
     L.sparsk_reset_slot.restype = C.c_int
     L.sparsk_reset_slot.argtypes = [vp, C.c_int32]
     for name in ("sparsk_import_kv", "sparsk_export_kv"):
@@ -280,8 +280,7 @@ class Sparsk:
         sl, ct = _i32(slots), _i32(counters)
         md = np.ascontiguousarray(modality, dtype=np.uint8)
         self._check(self.lib.sparsk_decode_step(
-            self.h, len(sl), sl.ctypes.data_as(C.POINTER(C.c_int32)), token_ids.data_ptr(),
-            md.ctypes.data_as(C.POINTER(C.c_uint8)), ct.ctypes.data_as(C.POINTER(C.c_int32)),
+            self.h, len(sl), sl.ctypes.data, token_ids.data_ptr(), md.ctypes.data, ct.ctypes.data,
             next_tokens.data_ptr(), exit_depths.data_ptr()))
 
     def decode_step_host(self, slots, token_ids, modality, counters, next_tokens: np.ndarray,
@@ -289,8 +288,7 @@ class Sparsk:
         sl, ct, tk = _i32(slots), _i32(counters), _i32(token_ids)
         md = np.ascontiguousarray(modality, dtype=np.uint8)
         self._check(self.lib.sparsk_decode_step_host(
-            self.h, len(sl), sl.ctypes.data_as(C.POINTER(C.c_int32)), tk.ctypes.data,
-            md.ctypes.data_as(C.POINTER(C.c_uint8)), ct.ctypes.data_as(C.POINTER(C.c_int32)),
+            self.h, len(sl), sl.ctypes.data, tk.ctypes.data, md.ctypes.data, ct.ctypes.data,
             next_tokens.ctypes.data, exit_depths.ctypes.data))
 
     def reset_slot(self, slot: int):

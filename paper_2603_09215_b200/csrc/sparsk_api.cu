@@ -69,7 +69,7 @@ struct sparsk_ctx {
     int *kv_len, *pend_cnt;
     float2 *rope;
     StepDesc sd;
-    int *staged, *tok_dev, *out_tok_dev, *out_depth_dev;
+    int *staged, *tok_dev;
     int *pf_rows;                // row set of a prefill pass, laid out as it is staged (see sparsk_prefill)
     float *h_lo, *h_up;
     float *qbuf;
@@ -215,15 +215,14 @@ size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
     int *kl = w.take<int>(B), *pc = w.take<int>(B);
     float2 *rope = w.take<float2>(S * (d->head_dim / 2));
     StepDesc sd;
-    sd.slot = w.take<int>(B); sd.modality = w.take<int>(B); sd.counter = w.take<int>(B);
-    sd.token = w.take<int>(B); sd.depth = w.take<int>(B); sd.lo_pos = w.take<int>(B);
+    sd.slot = w.take<int>(B); sd.modality = w.take<int>(B); sd.depth = w.take<int>(B); sd.lo_pos = w.take<int>(B);
     sd.lo_grp_row0 = w.take<int>(B); sd.lo_grp_nrows = w.take<int>(B);
     sd.up_slot = w.take<int>(R); sd.up_pos = w.take<int>(R); sd.up_src = w.take<int>(R);
     sd.up_grp_row0 = w.take<int>(B); sd.up_grp_nrows = w.take<int>(B); sd.cur_row = w.take<int>(B);
     sd.list_seq = w.take<int>(4 * B); sd.list_row = w.take<int>(4 * B);
     sd.counts = w.take<int>(8);
     sd.argmax = w.take<unsigned long long>(B);
-    int *staged = w.take<int>(3 * B), *tok = w.take<int>(B), *ot = w.take<int>(B), *od = w.take<int>(B);
+    int *staged = w.take<int>(3 * B), *tok = w.take<int>(B);
     int *pfr = w.take<int>(prefill_ints(d));
     float *hlo = w.take<float>(B * d->d_model), *hup = w.take<float>(R * d->d_model);
     float *q = w.take<float>(R * qrow);
@@ -252,7 +251,7 @@ size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
     float2 *pml = w.take<float2>(cells);
     if (c) {
         c->kcache = kc; c->vcache = vc; c->pend_h = ph; c->kv_len = kl; c->pend_cnt = pc; c->rope = rope;
-        c->sd = sd; c->staged = staged; c->tok_dev = tok; c->out_tok_dev = ot; c->out_depth_dev = od;
+        c->sd = sd; c->staged = staged; c->tok_dev = tok;
         c->pf_rows = pfr;
         c->conf_rows_dev = crows; c->conf_list_dev = clist; c->conf_ent_dev = cent; c->conf_logits = clog;
         c->h_last = hlast; c->q_last = qlast; c->last_slot = lslot; c->last_pos = lpos;
@@ -1568,6 +1567,64 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
     return SPARSK_OK;
 }
 
+// --------------------------------------------------------------------------- beginning and end of a step
+// Input tokens of a step: on the device, or host values that ride along as kernel arguments.
+struct StepTokens {
+    const int32_t *dev, *host;
+};
+
+// Hands the step's arrays to the device and runs its first kernel: schedule, compaction (exit layer
+// e), embedding, the parity hook's logits.
+static int step_begin(sparsk_ctx *ctx, int n, const int32_t *slots, StepTokens tokens, const uint8_t *modality,
+                      const int32_t *counters, const SchedParams &sp, int e)
+{
+    const sparsk_dims &d = ctx->dm;
+    const int V = d.vocab_text + d.vocab_speech;
+    StepIn in;
+    const int *staged = nullptr;
+    if (n <= SI_MAX) {
+        for (int i = 0; i < n; i++) {
+            in.slot[i] = slots[i];
+            in.modality[i] = modality[i];
+            in.counter[i] = counters[i];
+            in.token[i] = tokens.host ? tokens.host[i] : 0;
+        }
+    } else {
+        const int ring = ctx->stage_next;
+        ctx->stage_next = (ring + 1) % STAGE_RING;
+        CU(cudaEventSynchronize(ctx->stage_ev[ring]));
+        int *st = ctx->stage_host[ring];
+        for (int i = 0; i < n; i++) {
+            st[i] = slots[i];
+            st[n + i] = modality[i];
+            st[2 * n + i] = counters[i];
+        }
+        CU(cudaMemcpyAsync(ctx->staged, st, sizeof(int) * 3 * n, cudaMemcpyHostToDevice, ctx->stream));
+        CU(cudaEventRecord(ctx->stage_ev[ring], ctx->stream));
+        staged = ctx->staged;
+        if (tokens.host) {
+            memcpy(ctx->io_host, tokens.host, sizeof(int) * n);
+            CU(cudaMemcpyAsync(ctx->tok_dev, ctx->io_host, sizeof(int) * n, cudaMemcpyHostToDevice, ctx->stream));
+            tokens.dev = ctx->tok_dev;
+        }
+    }
+    const size_t n_logits = ctx->dbg_logits ? (size_t)n * V : 0;
+    const int threads = std::max(256, div_up(n, 32) * 32);
+    const int fill = (int)std::min<size_t>((n_logits + threads * 8 - 1) / (threads * 8), 2048);
+    CU(launch(ctx, step_begin_kernel, dim3(1 + n + fill), dim3(threads), 0, ctx->sd, in, n, staged, tokens.dev, V, sp,
+              (const int *)ctx->kv_len, (const int *)ctx->pend_cnt, e, d.max_seqs, ctx->embed, ctx->h_lo, d.d_model,
+              ctx->dbg_logits, n_logits));
+    return SPARSK_OK;
+}
+static int step_finish(sparsk_ctx *ctx, int n, int32_t *next_tokens, int32_t *exit_depths, int *status_out)
+{
+    const int threads = 128;
+    CU(launch(ctx, finish_kernel, dim3(ctx->dbg_hidden ? n : div_up(n, threads)), dim3(threads), 0, ctx->sd, n, ctx->kv_len,
+              ctx->pend_cnt, (int *)next_tokens, (int *)exit_depths, ctx->dm.n_layers, status_out, (const float *)ctx->h_lo,
+              (const float *)ctx->h_up, ctx->dbg_hidden, ctx->dm.d_model));
+    return SPARSK_OK;
+}
+
 // --------------------------------------------------------------------------- decode step, confidence-based exit
 // The step of a context whose dims name a confidence modality (Sec. V-B, compared method 3).
 // Depths are not known beforehand, so the host walks the layers in segments: a segment is a run
@@ -1579,8 +1636,8 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
 // segment are the pending positions not yet carried through its first layer (always the newest
 // ones: an older position has been carried at least as far as a newer one) followed by the
 // current position, i.e. consecutive positions, one attention group.
-static int decode_step_conf(sparsk_ctx *ctx, int32_t n, const int32_t *slots, const int32_t *token_ids,
-                            const uint8_t *modality, const int32_t *counters, int32_t *next_tokens, int32_t *exit_depths)
+static int decode_step_conf(sparsk_ctx *ctx, int32_t n, const int32_t *slots, StepTokens tokens, const uint8_t *modality,
+                            const int32_t *counters, int32_t *next_tokens, int32_t *exit_depths, int *status_out)
 {
     const sparsk_dims &d = ctx->dm;
     const int L = d.n_layers, e = d.exit_layer, B = d.max_seqs, cs = d.conf_start;
@@ -1606,29 +1663,8 @@ static int decode_step_conf(sparsk_ctx *ctx, int32_t n, const int32_t *slots, co
             return fail(ctx, SPARSK_ENOHEAD, "decode_step: layer %d has no exit head", target[i]);
         max_len = std::max(max_len, ctx->h_len[s] + 1);
     }
-    // ---- stage the host arrays; latch tokens; embed
-    const int ring = ctx->stage_next;
-    ctx->stage_next = (ring + 1) % STAGE_RING;
-    CU(cudaEventSynchronize(ctx->stage_ev[ring]));
-    int *st = ctx->stage_host[ring];
-    for (int i = 0; i < n; i++) {
-        st[i] = slots[i];
-        st[n + i] = modality[i];
-        st[2 * n + i] = counters[i];
-    }
-    CU(cudaMemcpyAsync(ctx->staged, st, sizeof(int) * 3 * n, cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaEventRecord(ctx->stage_ev[ring], ctx->stream));
-    CU(launch(ctx, schedule_kernel, dim3((n + 127) / 128), dim3(128), 0, ctx->sd, (int)n, (const int *)ctx->staged,
-              (const int *)token_ids, V, sp));
-    // the lower-row arrays (positions, one-row groups); "e = L" keeps every head on the lower rows
-    CU(launch(ctx, compact_kernel, dim3(1), dim3(1024), 0, ctx->sd, (int)n, (const int *)ctx->kv_len,
-              (const int *)ctx->pend_cnt, L, L, B));
-    CU(launch(ctx, embed_kernel, dim3(n), dim3(128), 0, (const int *)ctx->sd.token, (const int *)nullptr, ctx->embed, ctx->h_lo, (int)n, d.d_model,
-              V, ctx->sd.counts + CNT_STATUS));
-    if (ctx->dbg_logits) {
-        const size_t cnt = (size_t)n * V;
-        CU(launch(ctx, fill_kernel, dim3((unsigned)std::min<size_t>((cnt + 255) / 256, 2048)), dim3(256), 0, ctx->dbg_logits, cnt, -INFINITY));
-    }
+    // "e = L" keeps every head on the lower rows
+    if (const int rc = step_begin(ctx, n, slots, tokens, modality, counters, sp, L)) return rc;
     const int R = ctx->cap_rows;
     size_t arena = 0;  // ints of the pinned arena used so far in this step
     auto region = [&](size_t ints) -> int * {
@@ -1777,11 +1813,7 @@ static int decode_step_conf(sparsk_ctx *ctx, int32_t n, const int32_t *slots, co
     if (!hb) return fail(ctx, SPARSK_ECAPACITY, "decode_step: staging arena exhausted");
     std::copy(depth.begin(), depth.end(), hb);
     CU(cudaMemcpyAsync(ctx->sd.depth, hb, sizeof(int) * n, cudaMemcpyHostToDevice, ctx->stream));
-    if (ctx->dbg_hidden)
-        CU(launch(ctx, debug_hidden_kernel, dim3(n), dim3(128), 0, ctx->sd, (const float *)ctx->h_lo,
-                  (const float *)ctx->h_up, ctx->dbg_hidden, (int)n, d.d_model));
-    CU(launch(ctx, finish_kernel, dim3((n + 127) / 128), dim3(128), 0, ctx->sd, (int)n, ctx->kv_len, ctx->pend_cnt,
-              next_tokens, exit_depths, L));
+    if (const int rc = step_finish(ctx, n, next_tokens, exit_depths, status_out)) return rc;
     for (int i = 0; i < n; i++) {
         ctx->h_len[slots[i]] += 1;
         ctx->h_pend[slots[i]] = (int)ctx->h_fill[slots[i]].size();
@@ -1791,18 +1823,16 @@ static int decode_step_conf(sparsk_ctx *ctx, int32_t n, const int32_t *slots, co
 }
 
 // --------------------------------------------------------------------------- decode step
-extern "C" int sparsk_decode_step(sparsk_ctx *ctx, int32_t n, const int32_t *slots, const int32_t *token_ids,
-                                  const uint8_t *modality, const int32_t *counters, int32_t *next_tokens,
-                                  int32_t *exit_depths)
+static int decode_step(sparsk_ctx *ctx, int32_t n, const int32_t *slots, StepTokens tokens, const uint8_t *modality,
+                       const int32_t *counters, int32_t *next_tokens, int32_t *exit_depths, int *status_out)
 {
-    if (!good(ctx)) return SPARSK_ESTATE;
     const sparsk_dims &d = ctx->dm;
     const int L = d.n_layers, e = d.exit_layer, B = d.max_seqs;
     const SchedParams sp{L, e, d.refresh_period, d.refresh_phase, d.text_period > 0 ? d.text_period : d.refresh_period,
                          d.text_period > 0 ? d.text_phase : d.refresh_phase, d.text_exit};
-    if (n < 1 || n > B || !slots || !token_ids || !modality || !counters || !next_tokens || !exit_depths)
+    if (n < 1 || n > B || !slots || !(tokens.dev || tokens.host) || !modality || !counters || !next_tokens || !exit_depths)
         return fail(ctx, SPARSK_EINVAL, "decode_step: bad arguments (n=%d)", n);
-    if (d.conf_modalities) return decode_step_conf(ctx, n, slots, token_ids, modality, counters, next_tokens, exit_depths);
+    if (d.conf_modalities) return decode_step_conf(ctx, n, slots, tokens, modality, counters, next_tokens, exit_depths, status_out);
     // ---- host mirror of the schedule: validates, and sizes the launches
     std::vector<char> seen(B, 0);
     int n_list[4] = {0, 0, 0, 0};
@@ -1836,48 +1866,25 @@ extern "C" int sparsk_decode_step(sparsk_ctx *ctx, int32_t n, const int32_t *slo
         return fail(ctx, SPARSK_ENOHEAD, "decode_step: layer %d has no exit head", e);
     if (m_up > ctx->cap_rows) return fail(ctx, SPARSK_ECAPACITY, "decode_step: %d upper rows exceed capacity %d", m_up, ctx->cap_rows);
 
-    // ---- stage the host arrays
-    const int ring = ctx->stage_next;
-    ctx->stage_next = (ring + 1) % STAGE_RING;
-    CU(cudaEventSynchronize(ctx->stage_ev[ring]));
-    int *st = ctx->stage_host[ring];
-    for (int i = 0; i < n; i++) {
-        st[i] = slots[i];
-        st[n + i] = modality[i];
-        st[2 * n + i] = counters[i];
-    }
-    CU(cudaMemcpyAsync(ctx->staged, st, sizeof(int) * 3 * n, cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaEventRecord(ctx->stage_ev[ring], ctx->stream));
-
     // ---- schedule, compaction, embedding
     const int V = d.vocab_text + d.vocab_speech;
-    CU(launch(ctx, schedule_kernel, dim3((n + 127) / 128), dim3(128), 0, ctx->sd, (int)n, (const int *)ctx->staged,
-              (const int *)token_ids, V, sp));
-    CU(launch(ctx, compact_kernel, dim3(1), dim3(1024), 0, ctx->sd, (int)n, (const int *)ctx->kv_len,
-              (const int *)ctx->pend_cnt, L, e, B));
-    CU(launch(ctx, embed_kernel, dim3(n), dim3(128), 0, (const int *)ctx->sd.token, (const int *)nullptr, ctx->embed, ctx->h_lo, (int)n, d.d_model,
-              V, ctx->sd.counts + CNT_STATUS));
-    if (ctx->dbg_logits) {
-        const size_t cnt = (size_t)n * V;
-        CU(launch(ctx, fill_kernel, dim3((unsigned)std::min<size_t>((cnt + 255) / 256, 2048)), dim3(256), 0, ctx->dbg_logits, cnt, -INFINITY));
-    }
+    if (const int rc = step_begin(ctx, n, slots, tokens, modality, counters, sp, e)) return rc;
     // ---- lower pass: layers 1..e over all sequences
     RowSet lo{ctx->sd.slot, ctx->sd.lo_pos, ctx->sd.lo_grp_row0, ctx->sd.lo_grp_nrows, ctx->sd.counts + CNT_NSEQ,
               ctx->sd.counts + CNT_NSEQ, n, n, 1, max_len_lo};
     lo.sum_len = sum_len_lo;
     CU(run_layers(ctx, 1, e, ctx->h_lo, lo));
-    // ---- early exits: keep h^(e), read the token from g_e
-    if (n_list[0] + n_list[1]) {
-        CU(launch(ctx, stash_kernel, dim3(n), dim3(128), 0, ctx->sd, (const float *)ctx->h_lo, ctx->pend_h,
-                  (const int *)ctx->pend_cnt, (int)n, d.d_model, L, d.max_pending));
-        for (int l = 0; l < 2; l++)
-            if (n_list[l]) CU(run_head(ctx, e, ctx->h_lo, l, n_list[l]));
-    }
+    // ---- early exits keep h^(e); the upper pass gathers its rows
+    const int n_early = n_list[0] + n_list[1];
+    if (n_early || m_up)
+        CU(launch(ctx, exit_rows_kernel, dim3((n_early ? n : 0) + m_up), dim3(128), 0, ctx->sd, (const float *)ctx->h_lo,
+                  ctx->pend_h, (const int *)ctx->pend_cnt, ctx->h_up, n_early ? n : 0, d.d_model, L, d.max_pending));
+    // ---- early exits read the token from g_e
+    for (int l = 0; l < 2; l++)
+        if (n_list[l]) CU(run_head(ctx, e, ctx->h_lo, l, n_list[l]));
     // ---- upper pass: pending and current positions of full-depth sequences through e+1..L
     const float *h_full = ctx->h_lo;
     if (m_up) {
-        CU(launch(ctx, gather_upper_kernel, dim3(m_up), dim3(128), 0, ctx->sd, (const float *)ctx->h_lo,
-                  (const float *)ctx->pend_h, ctx->h_up, d.d_model, d.max_pending));
         RowSet up{ctx->sd.up_slot, ctx->sd.up_pos, ctx->sd.up_grp_row0, ctx->sd.up_grp_nrows, ctx->sd.counts + CNT_NGRP,
                   ctx->sd.counts + CNT_MUP, m_up, n_grp, max_grp, max_len_up, n_big};
         up.sum_len = sum_len_up;
@@ -1924,11 +1931,7 @@ extern "C" int sparsk_decode_step(sparsk_ctx *ctx, int32_t n, const int32_t *slo
                                  &ctx->launches));
         if (timed) cudaEventRecord(ctx->tev[ctx->tev_used++], ctx->stream);
     }
-    if (ctx->dbg_hidden)
-        CU(launch(ctx, debug_hidden_kernel, dim3(n), dim3(128), 0, ctx->sd, (const float *)ctx->h_lo,
-                  (const float *)ctx->h_up, ctx->dbg_hidden, (int)n, d.d_model));
-    CU(launch(ctx, finish_kernel, dim3((n + 127) / 128), dim3(128), 0, ctx->sd, (int)n, ctx->kv_len, ctx->pend_cnt,
-              next_tokens, exit_depths, L));
+    if (const int rc = step_finish(ctx, n, next_tokens, exit_depths, status_out)) return rc;
     // ---- host mirror follows
     for (int i = 0; i < n; i++) {
         const int s = slots[i];
@@ -1937,6 +1940,14 @@ extern "C" int sparsk_decode_step(sparsk_ctx *ctx, int32_t n, const int32_t *slo
         ctx->h_pend[s] = (depth == L) ? 0 : ctx->h_pend[s] + 1;
     }
     return SPARSK_OK;
+}
+
+extern "C" int sparsk_decode_step(sparsk_ctx *ctx, int32_t n, const int32_t *slots, const int32_t *token_ids,
+                                  const uint8_t *modality, const int32_t *counters, int32_t *next_tokens,
+                                  int32_t *exit_depths)
+{
+    if (!good(ctx)) return SPARSK_ESTATE;
+    return decode_step(ctx, n, slots, {token_ids, nullptr}, modality, counters, next_tokens, exit_depths, nullptr);
 }
 
 extern "C" int sparsk_decode_step_host(sparsk_ctx *ctx, int32_t n, const int32_t *slots, const int32_t *token_ids,
@@ -1952,18 +1963,13 @@ extern "C" int sparsk_decode_step_host(sparsk_ctx *ctx, int32_t n, const int32_t
     for (int i = 0; i < n; i++)
         if (token_ids[i] < 0 || token_ids[i] >= V)
             return fail(ctx, SPARSK_EINVAL, "decode_step_host: token_ids[%d]=%d is outside the vocabulary [0, %d)", i, token_ids[i], V);
-    // Everything crosses the bus through one pinned buffer, so that the copies are truly
-    // asynchronous and the host waits once per step (a copy to or from pageable memory makes the
-    // host wait for it; three of them in a row after the step cost 30 us of idle GPU per step).
+    // The tokens ride along as kernel arguments (or through the pinned buffer, beyond SI_MAX
+    // sequences), and the step's last kernel writes the results and the status word straight into
+    // pinned memory: no copies before or behind the step, one wait.
     const int B = ctx->dm.max_seqs;
     int *io = ctx->io_host;
-    memcpy(io, token_ids, sizeof(int) * n);
-    CU(cudaMemcpyAsync(ctx->tok_dev, io, sizeof(int) * n, cudaMemcpyHostToDevice, ctx->stream));
-    const int rc = sparsk_decode_step(ctx, n, slots, ctx->tok_dev, modality, counters, ctx->out_tok_dev, ctx->out_depth_dev);
+    const int rc = decode_step(ctx, n, slots, {nullptr, token_ids}, modality, counters, io + B, io + 2 * B, io + 3 * B);
     if (rc != SPARSK_OK) return rc;
-    CU(cudaMemcpyAsync(io + B, ctx->out_tok_dev, sizeof(int) * n, cudaMemcpyDeviceToHost, ctx->stream));
-    CU(cudaMemcpyAsync(io + 2 * B, ctx->out_depth_dev, sizeof(int) * n, cudaMemcpyDeviceToHost, ctx->stream));
-    CU(cudaMemcpyAsync(io + 3 * B, ctx->sd.counts + CNT_STATUS, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     CU(cudaStreamSynchronize(ctx->stream));
     memcpy(next_tokens, io + B, sizeof(int) * n);
     memcpy(exit_depths, io + 2 * B, sizeof(int) * n);

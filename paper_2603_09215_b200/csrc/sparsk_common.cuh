@@ -24,7 +24,7 @@ typedef __half kv_t;
 // "upper" rows are, for every sequence that runs full depth, its pending positions
 // followed by its current position (layers e+1..L; Algorithm 1, full-depth branch).
 struct StepDesc {
-    int *slot, *modality, *counter, *token, *depth;  // [B]
+    int *slot, *modality, *depth;                    // [B]
     int *lo_pos;                                     // [B] position of the row = slot length
     int *lo_grp_row0, *lo_grp_nrows;                 // [B] identity groups (1 row each)
     int *up_slot, *up_pos, *up_src;                  // [R] src >= 0: pending index; < 0: lower row -1-src
@@ -57,9 +57,9 @@ struct PerDevice {
 // writes are visible).  Every kernel here waits before it completes, so completion is transitive:
 // when a kernel's wait returns, everything before it in the stream is done.  The early start is
 // what lets a weight-streaming kernel issue its first weight copies (which depend on nothing)
-// while a small kernel between two of them is still running.  The bookkeeping kernels of a step and
-// the copies that stage a row set never let go early, so what they wrote is visible to every kernel
-// of the pass that follows two or more launches later, before its wait as well.
+// while a small kernel between two of them is still running.  The kernel that begins a step and the
+// copies that stage a row set never let go early, and that kernel fences what it wrote: a kernel of
+// the pass that follows finds the row set in the L2 before its wait as well.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
 

@@ -507,7 +507,7 @@ static __global__ void __launch_bounds__(QF_THREADS) qkv_finish_kernel(float *__
     const int m = blockIdx.x, half = hd >> 1, p = blockIdx.y * QF_THREADS + threadIdx.x;
     const int head = p / half, j = p % half, n_heads = Hq + 2 * Hkv;
     const bool on = head < n_heads;
-    const int slot = row_slot[m], pos = row_pos[m];
+    const int slot = __ldcg(row_slot + m), pos = __ldcg(row_pos + m);
     const float2 cs = head < Hq + Hkv ? rope[(size_t)pos * half + j] : make_float2(1.f, 0.f);  // values do not turn
     griddep_wait();
     if (!on) return;

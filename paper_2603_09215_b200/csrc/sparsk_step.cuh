@@ -22,98 +22,141 @@ __host__ __device__ inline int scheduled_depth(int modality, int c, const SchedP
     return (c % p.K == p.r) ? p.L : p.e;
 }
 
-// ---------------------------------------------------------------------------------------
-// Exit schedule (Sec. IV-B.1).  One thread per sequence.  Also latches the input token (clamped
-// into the vocabulary, with a status bit if it was outside) and clears the sequence's argmax cell.
-// ---------------------------------------------------------------------------------------
-static __global__ void schedule_kernel(StepDesc sd, int n, const int *__restrict__ staged /*[3][n]*/,
-                                const int *__restrict__ tokens_in, int vocab, SchedParams sp)
-{
-    griddep_wait();
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b == 0) sd.counts[CNT_NSEQ] = n;
-    if (b >= n) return;
-    int slot = staged[b], mod = staged[n + b], c = staged[2 * n + b];
-    int depth = scheduled_depth(mod, c, sp);
-    int tok = tokens_in[b];
-    if (tok < 0 || tok >= vocab) {
-        atomicOr(&sd.counts[CNT_STATUS], ST_BAD_TOKEN);
-        tok = min(max(tok, 0), vocab - 1);
-    }
-    sd.slot[b] = slot;
-    sd.modality[b] = mod;
-    sd.counter[b] = c;
-    sd.token[b] = tok;
-    sd.depth[b] = depth;
-    sd.argmax[b] = 0ull;
-}
+// What a step is given, as a kernel argument: up to SI_MAX sequences need no copy to the device
+// ahead of the step's first kernel.  Larger steps stage the arrays ([slot][modality][counter], n
+// each) and pass them by pointer.
+constexpr int SI_MAX = 128;
+struct StepIn {
+    int slot[SI_MAX], counter[SI_MAX], token[SI_MAX];
+    unsigned char modality[SI_MAX];
+};
 
-// Exclusive prefix sum over one value per thread of a 1024-thread block; returns the prefix
-// and leaves the block total in *total (shared).
-__device__ __forceinline__ int block_exscan(int v, int *warp_tot /*[32] shared*/, int *total)
+// Exclusive prefix sum over one value per thread of a block; returns the prefix and leaves the
+// block total in *total (shared).
+template <class T>
+__device__ __forceinline__ T block_exscan(T v, T *warp_tot /*[32] shared*/, T *total)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int inc = v;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    T inc = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(0xffffffffu, inc, o);
+        const T t = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += t;
     }
     if (lane == 31) warp_tot[warp] = inc;
     __syncthreads();
     if (warp == 0) {
-        int w = warp_tot[lane];
-        int winc = w;
+        const T w = lane < n_warps ? warp_tot[lane] : T(0);
+        T winc = w;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            int t = __shfl_up_sync(0xffffffffu, winc, o);
+            const T t = __shfl_up_sync(0xffffffffu, winc, o);
             if (lane >= o) winc += t;
         }
         warp_tot[lane] = winc - w;
         if (lane == 31) *total = winc;
     }
     __syncthreads();
-    int res = warp_tot[warp] + inc - v;
+    const T res = warp_tot[warp] + inc - v;
     __syncthreads();
     return res;
 }
 
-// ---------------------------------------------------------------------------------------
-// Active-row compaction.  Sequences that leave at layer e drop out of layers e+1..L; every
-// full-depth sequence contributes its pending positions plus its current one (Algorithm 1,
-// full-depth branch).  Prefix sums give each sequence its offset in the upper row list; four
-// more give the per-(exit, modality) lists the head kernels read.  One block, n <= 1024.
-// ---------------------------------------------------------------------------------------
-static __global__ void __launch_bounds__(1024) compact_kernel(StepDesc sd, int n, const int *__restrict__ kv_len,
-                                                       const int *__restrict__ pend_cnt, int L, int e,
-                                                       int list_stride)
+__device__ __forceinline__ void embed_row(const bf16 *__restrict__ embed, int tok, float *__restrict__ dst, int d)
 {
-    __shared__ int warp_tot[32];
-    __shared__ int total;
+    const bf16 *src = embed + (size_t)tok * d;
+    for (int i = threadIdx.x * 8; i < d; i += blockDim.x * 8) {
+        float f[8];
+        unpack8(*reinterpret_cast<const uint4 *>(src + i), f);
+        float4 *o = reinterpret_cast<float4 *>(dst + i);
+        o[0] = make_float4(f[0], f[1], f[2], f[3]);
+        o[1] = make_float4(f[4], f[5], f[6], f[7]);
+    }
+}
+// A token id clamped into the vocabulary (never read outside the table; the host reports the flag).
+__device__ __forceinline__ int clamp_token(int tok, int vocab, int *status)
+{
+    if (tok < 0 || tok >= vocab) {
+        if (threadIdx.x == 0) atomicOr(status, ST_BAD_TOKEN);
+        tok = min(max(tok, 0), vocab - 1);
+    }
+    return tok;
+}
+
+// ---------------------------------------------------------------------------------------
+// The beginning of a step, one launch.
+//   Block 0: exit schedule (Sec. IV-B.1; a thread per sequence) and active-row compaction.
+//     Sequences that leave at layer e drop out of layers e+1..L; every full-depth sequence
+//     contributes its pending positions plus its current one (Algorithm 1, full-depth branch).
+//     Prefix sums give each sequence its offset in the upper row list, its attention group and its
+//     place in the per-(exit, modality) lists the head kernels read.  n <= 1024.
+//   Blocks 1..n: h^(0) = E[token] of sequence b - 1, fp32.
+//   The rest: -inf into the parity hook's logits (logits may be NULL).
+// All of it is latency.  With the arrays as arguments, one launch here instead of four behind two
+// copies, one launch between the passes and the results written straight to the host, a
+// batch-1 step of the four-layer shape takes 98 us instead of 126.
+// ---------------------------------------------------------------------------------------
+static __global__ void __launch_bounds__(1024) step_begin_kernel(const StepDesc sd, const __grid_constant__ StepIn in, int n,
+                                                          const int *__restrict__ staged, const int *__restrict__ tokens,
+                                                          int vocab, const SchedParams sp, const int *__restrict__ kv_len,
+                                                          const int *__restrict__ pend_cnt, int e, int list_stride,
+                                                          const bf16 *__restrict__ embed, float *__restrict__ h, int d,
+                                                          float *__restrict__ logits, size_t n_logits)
+{
     griddep_wait();
-    const int b = threadIdx.x;
+    if (blockIdx.x > 0) {
+        const int b = blockIdx.x - 1;
+        if (b < n) {
+            embed_row(embed, clamp_token(tokens ? tokens[b] : in.token[b], vocab, &sd.counts[CNT_STATUS]), h + (size_t)b * d, d);
+        } else {
+            const size_t step = (size_t)(gridDim.x - 1 - n) * blockDim.x;
+            for (size_t i = (size_t)(b - n) * blockDim.x + threadIdx.x; i < n_logits; i += step) logits[i] = -INFINITY;
+        }
+        return;
+    }
+    __shared__ int warp_tot[32], total;
+    __shared__ unsigned long long warp_tot_p[32], total_p;
+    const int b = threadIdx.x, L = sp.L;
     const bool on = b < n;
     int slot = 0, depth = 0, mod = 0, len = 0, pend = 0;
     if (on) {
-        slot = sd.slot[b];
-        depth = sd.depth[b];
-        mod = sd.modality[b];
+        slot = staged ? staged[b] : in.slot[b];
+        mod = staged ? staged[n + b] : in.modality[b];
+        depth = scheduled_depth(mod, staged ? staged[2 * n + b] : in.counter[b], sp);
         len = kv_len[slot];
         pend = pend_cnt[slot];
+        sd.slot[b] = slot;
+        sd.modality[b] = mod;
+        sd.depth[b] = depth;
+        sd.argmax[b] = 0ull;
         sd.lo_pos[b] = len;
         sd.lo_grp_row0[b] = b;
         sd.lo_grp_nrows[b] = 1;
     }
     // a sequence needs the upper pass iff it runs L layers and L > e
-    const bool full = on && depth == L;
-    const bool upper = full && e < L;
+    const bool full = on && depth == L, upper = full && e < L;
     const int cnt = upper ? pend + 1 : 0;
     const int off = block_exscan(cnt, warp_tot, &total);
-    if (b == 0) sd.counts[CNT_MUP] = total;
-    const int grp = block_exscan(upper ? 1 : 0, warp_tot, &total);
-    if (b == 0) sd.counts[CNT_NGRP] = total;
-    if (on) sd.cur_row[b] = upper ? off + cnt - 1 : -1;
+    // five 0/1 counts in fields of 12 bits: the four lists (early/text, early/speech, full/text,
+    // full/speech), then the groups
+    const int list = (full ? 2 : 0) + (mod ? 1 : 0);
+    const unsigned long long bits = (on ? 1ull << (12 * list) : 0ull) | (upper ? 1ull << 48 : 0ull);
+    const unsigned long long idx = block_exscan(bits, warp_tot_p, &total_p);
+    if (b == 0) {
+        sd.counts[CNT_NSEQ] = n;
+        sd.counts[CNT_MUP] = total;
+        sd.counts[CNT_NGRP] = (int)(total_p >> 48);
+        for (int l = 0; l < 4; l++) sd.counts[CNT_LIST0 + l] = (int)(total_p >> (12 * l)) & 0xfff;
+    }
+    if (on) {
+        sd.cur_row[b] = upper ? off + cnt - 1 : -1;
+        const int k = (int)(idx >> (12 * list)) & 0xfff;
+        sd.list_seq[list * list_stride + k] = b;
+        // hidden row the head reads: lower row b, or the sequence's current upper row
+        sd.list_row[list * list_stride + k] = upper ? off + cnt - 1 : b;
+    }
     if (upper) {
+        const int grp = (int)(idx >> 48);
         sd.up_grp_row0[grp] = off;
         sd.up_grp_nrows[grp] = cnt;
         for (int j = 0; j < cnt; j++) {
@@ -122,18 +165,8 @@ static __global__ void __launch_bounds__(1024) compact_kernel(StepDesc sd, int n
             sd.up_src[off + j] = (j < pend) ? j : -1 - b;
         }
     }
-    // lists: 0 = early/text, 1 = early/speech, 2 = full/text, 3 = full/speech
-#pragma unroll
-    for (int l = 0; l < 4; l++) {
-        const bool in = on && ((l >> 1) == (full ? 1 : 0)) && ((l & 1) == (mod ? 1 : 0));
-        const int idx = block_exscan(in ? 1 : 0, warp_tot, &total);
-        if (b == 0) sd.counts[CNT_LIST0 + l] = total;
-        if (in) {
-            sd.list_seq[l * list_stride + idx] = b;
-            // hidden row the head reads: lower row b, or the sequence's current upper row
-            sd.list_row[l * list_stride + idx] = (full && e < L) ? off + cnt - 1 : b;
-        }
-    }
+    // kernels of the pass read the row set before their own grid dependency has resolved
+    __threadfence();
 }
 
 // h^(0) = E[token]  (Sec. III), fp32 residual stream.  Row i's token is tokens[i], or
@@ -144,50 +177,36 @@ static __global__ void embed_kernel(const int *__restrict__ tokens, const int *_
     griddep_wait();
     const int row = blockIdx.x;
     if (row >= n) return;
-    int tok = tokens[idx ? idx[row] : row];
-    if (tok < 0 || tok >= vocab) {  // never read outside the table; the host reports the flag
-        if (threadIdx.x == 0) atomicOr(status, ST_BAD_TOKEN);
-        tok = min(max(tok, 0), vocab - 1);
-    }
-    const bf16 *src = embed + (size_t)tok * d;
-    for (int i = threadIdx.x * 8; i < d; i += blockDim.x * 8) {
-        float f[8];
-        unpack8(*reinterpret_cast<const uint4 *>(src + i), f);
-        float4 *dst = reinterpret_cast<float4 *>(h + (size_t)row * d + i);
-        dst[0] = make_float4(f[0], f[1], f[2], f[3]);
-        dst[1] = make_float4(f[4], f[5], f[6], f[7]);
-    }
+    embed_row(embed, clamp_token(tokens[idx ? idx[row] : row], vocab, status), h + (size_t)row * d, d);
 }
 
-// Early-exit rows: h^(e) goes to the pending store (Algorithm 1, early-exit branch).
-static __global__ void stash_kernel(StepDesc sd, const float *__restrict__ h_lo, float *__restrict__ pend_h,
-                             const int *__restrict__ pend_cnt, int n, int d, int L, int max_pending)
+// Between the lower and the upper pass, one launch.
+//   Blocks 0..n_lo-1: early-exit rows: h^(e) goes to the pending store (Algorithm 1, early-exit branch).
+//   Then n_up blocks: upper rows: h^(e) of pending positions comes from the pending store, of the
+//   current position from the lower pass.  (No slot is in both: a sequence exits early or does not.)
+static __global__ void exit_rows_kernel(const StepDesc sd, const float *__restrict__ h_lo, float *__restrict__ pend_h,
+                                 const int *__restrict__ pend_cnt, float *__restrict__ h_up, int n_lo, int d, int L,
+                                 int max_pending)
 {
     griddep_wait();
     const int b = blockIdx.x;
-    if (b >= n || sd.depth[b] == L) return;
-    const int slot = sd.slot[b];
-    const int j = pend_cnt[slot];
-    if (j >= max_pending) return;  // the host refuses such a step before launching
-    const float4 *src = reinterpret_cast<const float4 *>(h_lo + (size_t)b * d);
-    float4 *dst = reinterpret_cast<float4 *>(pend_h + ((size_t)slot * max_pending + j) * d);
-    for (int i = threadIdx.x; i < d / 4; i += blockDim.x) dst[i] = src[i];
-}
-
-// Upper rows: h^(e) of pending positions comes from the pending store, of the current
-// position from the lower pass.
-static __global__ void gather_upper_kernel(StepDesc sd, const float *__restrict__ h_lo,
-                                    const float *__restrict__ pend_h, float *__restrict__ h_up, int d,
-                                    int max_pending)
-{
-    griddep_wait();
-    const int row = blockIdx.x;
-    if (row >= sd.counts[CNT_MUP]) return;
-    const int src = sd.up_src[row];
-    const float *from = (src >= 0) ? pend_h + ((size_t)sd.up_slot[row] * max_pending + src) * d
-                                   : h_lo + (size_t)(-1 - src) * d;
+    const float *from;
+    float *to;
+    if (b < n_lo) {
+        if (sd.depth[b] == L) return;
+        const int slot = sd.slot[b], j = pend_cnt[slot];
+        if (j >= max_pending) return;  // the host refuses such a step before launching
+        from = h_lo + (size_t)b * d;
+        to = pend_h + ((size_t)slot * max_pending + j) * d;
+    } else {
+        const int row = b - n_lo;
+        if (row >= sd.counts[CNT_MUP]) return;
+        const int src = sd.up_src[row];
+        from = src >= 0 ? pend_h + ((size_t)sd.up_slot[row] * max_pending + src) * d : h_lo + (size_t)(-1 - src) * d;
+        to = h_up + (size_t)row * d;
+    }
     const float4 *s4 = reinterpret_cast<const float4 *>(from);
-    float4 *d4 = reinterpret_cast<float4 *>(h_up + (size_t)row * d);
+    float4 *d4 = reinterpret_cast<float4 *>(to);
     for (int i = threadIdx.x; i < d / 4; i += blockDim.x) d4[i] = s4[i];
 }
 
@@ -304,36 +323,34 @@ static __global__ void clear_keys_kernel(unsigned long long *__restrict__ keys, 
     if (i < n) keys[rows[i]] = 0ull;
 }
 
-// End of step: emit tokens and depths, advance lengths, grow or clear the pending sets.
-static __global__ void finish_kernel(StepDesc sd, int n, int *__restrict__ kv_len, int *__restrict__ pend_cnt,
-                              int *__restrict__ next_tokens, int *__restrict__ exit_depths, int L)
+// End of step: emit tokens and depths, advance lengths, grow or clear the pending sets.  The
+// outputs may be pinned host memory (decode_step_host: the results cross the bus as they are
+// written, no copies behind the step); `status_out`, if given, receives the status word.  With
+// `hidden` (parity hook) block b also copies the hidden state sequence b's head read.
+static __global__ void finish_kernel(const StepDesc sd, int n, int *__restrict__ kv_len, int *__restrict__ pend_cnt,
+                              int *__restrict__ next_tokens, int *__restrict__ exit_depths, int L, int *__restrict__ status_out,
+                              const float *__restrict__ h_lo, const float *__restrict__ h_up, float *__restrict__ hidden, int d)
 {
     griddep_wait();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= n) return;
-    const int slot = sd.slot[b], depth = sd.depth[b];
-    next_tokens[b] = (int)(0xffffffffu - (uint32_t)(sd.argmax[b] & 0xffffffffull));
-    exit_depths[b] = depth;
-    kv_len[slot] += 1;
-    pend_cnt[slot] = (depth == L) ? 0 : pend_cnt[slot] + 1;
-}
-
-// Parity hooks: copy the hidden state each head read; pre-fill the logits with -inf.
-static __global__ void debug_hidden_kernel(StepDesc sd, const float *__restrict__ h_lo,
-                                    const float *__restrict__ h_up, float *__restrict__ out, int n, int d)
-{
-    griddep_wait();
-    const int b = blockIdx.x;
-    if (b >= n) return;
-    const int cr = sd.cur_row[b];
-    const float *from = (cr >= 0) ? h_up + (size_t)cr * d : h_lo + (size_t)b * d;
-    for (int i = threadIdx.x; i < d; i += blockDim.x) out[(size_t)b * d + i] = from[i];
-}
-static __global__ void fill_kernel(float *__restrict__ p, size_t n, float v)
-{
-    griddep_wait();
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        p[i] = v;
+    if (b < n) {
+        const int slot = sd.slot[b], depth = sd.depth[b];
+        next_tokens[b] = (int)(0xffffffffu - (uint32_t)(sd.argmax[b] & 0xffffffffull));
+        exit_depths[b] = depth;
+        kv_len[slot] += 1;
+        pend_cnt[slot] = (depth == L) ? 0 : pend_cnt[slot] + 1;
+        if (b == 0 && status_out) *status_out = sd.counts[CNT_STATUS];
+    }
+    if (hidden && blockIdx.x < n) {
+        const int s = blockIdx.x, cr = sd.cur_row[s];
+        const float4 *from = reinterpret_cast<const float4 *>(cr >= 0 ? h_up + (size_t)cr * d : h_lo + (size_t)s * d);
+        float *to = hidden + (size_t)s * d;
+        if (((uintptr_t)hidden & 15) == 0) {
+            for (int i = threadIdx.x; i < d / 4; i += blockDim.x) reinterpret_cast<float4 *>(to)[i] = from[i];
+        } else {
+            for (int i = threadIdx.x; i < d; i += blockDim.x) to[i] = reinterpret_cast<const float *>(from)[i];
+        }
+    }
 }
 
 // End of a prefill pass: every group's slot now holds the positions up to the group's last row.

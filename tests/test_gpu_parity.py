@@ -300,6 +300,43 @@ def test_tcgen05_passes_of_every_width(util, B):
     P.close()
 
 
+@pytest.mark.parametrize("n", [1, 33, 128, 129])
+def test_host_and_device_buffers_give_the_same_step(util, n):
+    """Up to 128 sequences a step's arrays and host tokens travel as kernel arguments, beyond that through
+    staged copies; with tokens on the device the same kernels read them from there.  Slots in an
+    order of their own."""
+    from paper_2603_09215_b200 import binding
+    dims = synth.model_dims("tiny", 2, 3, 0)
+    gw = binding.upload_weights(synth.make_weights(dims, seed=6))
+    prompts = synth.make_prompts(dims, n, 2, 6, seed=12)
+    order = np.random.Generator(np.random.PCG64(1)).permutation(n).astype(np.int32)
+    got = []
+    for host in (True, False):
+        g = binding.Sparsk(dims, gw, n, 16, 2)
+        g.prefill(list(range(n)), [p[:-1] for p in prompts])
+        tok = np.array([int(prompts[s][-1]) for s in order], np.int32)
+        nt, dp = np.zeros(n, np.int32), np.zeros(n, np.int32)
+        d_nt, d_dp = (torch.zeros(n, dtype=torch.int32, device="cuda") for _ in "nd")
+        out = []
+        for step in range(4):
+            mc = [synth.interleave(step + int(s), 2, 4) for s in order]
+            mods, ctrs = [m for m, _ in mc], [c for _, c in mc]
+            if host:
+                g.decode_step_host(order, tok, mods, ctrs, nt, dp)
+            else:
+                g.decode_step(order, torch.from_numpy(tok).cuda(), mods, ctrs, d_nt, d_dp)
+                g.check()
+                nt, dp = d_nt.cpu().numpy(), d_dp.cpu().numpy()
+            out.append((nt.copy(), dp.copy()))
+            tok = (tok * 7 + step) % (dims["vocab_text"] + dims["vocab_speech"])   # the same inputs on both sides
+            tok = tok.astype(np.int32)
+        got.append(out)
+        g.close()
+    for (a, da), (b, db) in zip(*got):
+        assert (da == db).all()
+        assert (a != b).mean() <= 0.02    # near-ties may fall either way: the split sums' order is not fixed
+
+
 @pytest.mark.parametrize("shape", ["tiny", "micro64"])
 @pytest.mark.parametrize("rows", [129, 161, 256, 300])
 def test_prefill_passes_beyond_128_rows(util, rows, shape):
