@@ -372,6 +372,7 @@ struct RowSet {
     int n_big;      // groups with at least attn_tc_min_q query vectors per kv head (0: not counted, assume all)
     const float *q; // the rows' queries if they are not the context's query buffer (NULL: they are)
     long sum_len;   // total of the groups' prefix lengths (host; 0: unknown)
+    bool rows_late; // the arrays are written by a kernel that may still run when the pass's kernels start
 };
 
 cudaError_t run_qkv(sparsk_ctx *c, int layer, const float *h, const RowSet &rs)
@@ -555,6 +556,7 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
     a.split_len = pl.split_len;
     a.n_splits = pl.n_splits;
     a.max_groups = rs.n_groups_h;
+    a.rows_early = !rs.rows_late;
     if (!blocks_tc || (c->attn_tc_min_q > 1 && n_small > 0)) {
         // every group is in the item space (the kernel skips those the other kernel takes)
         const long n_items = (long)rs.n_groups_h * a.n_qblk * d.n_kv_heads * a.n_splits;
@@ -579,8 +581,8 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
         // ticket beyond its last item
         if (a.ticket && n_items > (long)grid * warps) c->attn_ticket_base += (unsigned)n_items;
     }
-    if (d.head_dim == 128) return launch(c, attn_merge_kernel<128>, dim3(rs.n_rows, d.n_q_heads), dim3(128), 0, a, rs.n_rows_dev);
-    return launch(c, attn_merge_kernel<64>, dim3(rs.n_rows, d.n_q_heads), dim3(64), 0, a, rs.n_rows_dev);
+    if (d.head_dim == 128) return launch(c, attn_merge_kernel<128>, dim3(rs.n_rows, d.n_q_heads), dim3(MG_THREADS), 0, a, rs.n_rows_dev);
+    return launch(c, attn_merge_kernel<64>, dim3(rs.n_rows, d.n_q_heads), dim3(MG_THREADS), 0, a, rs.n_rows_dev);
 }
 
 // ---------------------------------------------------------------- tensor-core dispatch
@@ -1907,6 +1909,7 @@ static int decode_step(sparsk_ctx *ctx, int32_t n, const int32_t *slots, StepTok
             RowSet last{ctx->last_slot, ctx->last_pos, ctx->sd.lo_grp_row0, ctx->sd.lo_grp_nrows, ctx->sd.counts + CNT_NGRP,
                         ctx->sd.counts + CNT_NGRP, n_grp, n_grp, 1, max_len_up, 0, ctx->q_last};
             last.sum_len = sum_len_up;
+            last.rows_late = true;
             CU(run_layer_back(ctx, L, ctx->h_last, last));
             CU(launch(ctx, put_current_kernel, dim3(n_grp), dim3(256), 0, ctx->sd, (const float *)ctx->h_last, ctx->h_up,
                       d.d_model));

@@ -67,7 +67,7 @@ extern "C" int sparsk_attention_static(const sparsk_attn_args *args, void *cuda_
         }
         scratch = g_scratch_addr[dev];
     }
-    // Nothing in the area has to start at zero: the two counters are rewritten by every call and,
+    // Nothing in the area has to start at zero: the item counter is cleared by every call that draws and,
     // as long as the groups partition the rows and none exceeds max_grp_rows (the documented
     // precondition of sparsk_attention), every partial cell a call reads is one it wrote first.
     // A row outside every group would be merged from whatever an earlier call left here.

@@ -36,40 +36,71 @@ extern "C" size_t sparsk_attention_scratch_bytes(int32_t n_rows, int32_t n_q_hea
     return 256 + up256(cells * head_dim * sizeof(float)) + up256(cells * sizeof(float2));
 }
 
+// The two launches follow each other as in a decode step: the merge may be resident before the
+// partials are complete and waits for them itself.
+template <class... KArgs, class... Args>
+static cudaError_t launch_dependent(cudaStream_t st, void (*kern)(KArgs...), dim3 grid, int block, size_t smem, Args... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+}
+
+static int n_sm_here()
+{
+    static PerDevice<int> sms;
+    int &n = sms.here();
+    if (n == 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 0;
+    }
+    return n;
+}
+
 // Shared by the entry points of this library that run the two attention kernels outside a
-// context: `scratch` holds two counters, then the split partials.
+// context: `scratch` holds an item counter, then the split partials.
 int sparsk_attention_launch(const sparsk_attn_args *p, char *scratch, cudaStream_t st)
 {
-    int dev = 0, n_sm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return SPARSK_ECUDA;
+    const int n_sm = n_sm_here();
+    if (n_sm == 0) return SPARSK_ECUDA;
     const size_t cells = (size_t)p->n_rows * p->n_q_heads * AT_MAX_SPLITS;
-    int *counts = reinterpret_cast<int *>(scratch);
     AttnArgs a{};
     a.q = (const bf16 *)p->q; a.kc = (const kv_t *)p->k_cache; a.vc = (const kv_t *)p->v_cache;
     a.grp_row0 = p->grp_row0; a.grp_nrows = p->grp_nrows; a.row_slot = p->row_slot; a.row_pos = p->row_pos;
-    a.n_groups = counts;
     a.part_o = reinterpret_cast<float *>(scratch + 256);
     a.part_ml = reinterpret_cast<float2 *>(scratch + 256 + up256(cells * p->head_dim * sizeof(float)));
     a.out = (bf16 *)p->out;
     a.Hq = p->n_q_heads; a.Hkv = p->n_kv_heads; a.S = p->cache_len; a.n_slots = p->n_slots; a.n_rows = p->n_rows;
     a.nq_min = 0; a.nq_max = 1 << 30;
     const int warp_ctas = n_sm * attn_warp_ctas_per_sm(p->head_dim, AW_NST);
+    // Only a bound on the prefixes is known here: with several groups they are taken to be half as long
+    // on average (48 ragged groups of 200 to 3,000 positions: 61.6 us per call planned for the
+    // bound, 57.4 for half of it, 63 for a fifth; uniform ones do not care).
     const AttnPlan pl = attn_plan(warp_ctas * AW_WARPS, p->n_groups, p->max_grp_rows, p->n_q_heads / p->n_kv_heads,
-                                  p->n_kv_heads, p->max_len, 0);
+                                  p->n_kv_heads, p->max_len, 0, p->n_groups > 1 ? (long)p->n_groups * p->max_len / 2 : 0);
     a.n_qblk = pl.n_qblk; a.split_len = pl.split_len; a.n_splits = pl.n_splits;
     a.max_groups = p->n_groups;
-    set_int_kernel<<<1, 1, 0, st>>>(counts, p->n_groups);
-    set_int_kernel<<<1, 1, 0, st>>>(counts + 1, p->n_rows);
     const long n_items = (long)p->n_groups * pl.n_qblk * p->n_kv_heads * pl.n_splits;
     const int grid = (int)std::max<long>(1, std::min<long>(warp_ctas, (n_items + AW_WARPS - 1) / AW_WARPS));
     AttnWarpFn fn;
     if (attn_warp_fn(p->head_dim, AW_NST, &fn) != cudaSuccess) return SPARSK_ECUDA;
-    fn<<<grid, AW_WARPS * 32, AW_WARPS * attn_warp_bytes(p->head_dim, AW_NST), st>>>(a);
-    if (p->head_dim == 128) attn_merge_kernel<128><<<dim3(p->n_rows, p->n_q_heads), 128, 0, st>>>(a, counts + 1);
-    else attn_merge_kernel<64><<<dim3(p->n_rows, p->n_q_heads), 64, 0, st>>>(a, counts + 1);
-    return cudaGetLastError() == cudaSuccess ? SPARSK_OK : SPARSK_ECUDA;
+    if (n_items > (long)grid * AW_WARPS && n_items < (1L << 31)) {  // items beyond the warps' first ones are drawn
+        if (cudaMemsetAsync(scratch, 0, sizeof(unsigned), st) != cudaSuccess) return SPARSK_ECUDA;
+        a.ticket = reinterpret_cast<unsigned *>(scratch);
+    }
+    cudaError_t e = launch_dependent(st, fn, dim3(grid), AW_WARPS * 32, AW_WARPS * attn_warp_bytes(p->head_dim, AW_NST), a);
+    if (e == cudaSuccess)
+        e = launch_dependent(st, p->head_dim == 128 ? attn_merge_kernel<128> : attn_merge_kernel<64>, dim3(p->n_rows, p->n_q_heads),
+                             MG_THREADS, 0, a, (const int *)nullptr);
+    return e == cudaSuccess ? SPARSK_OK : SPARSK_ECUDA;
 }
 
 extern "C" int sparsk_attention(const sparsk_attn_args *args, void *scratch, size_t scratch_bytes, void *cuda_stream)

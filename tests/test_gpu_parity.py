@@ -9,6 +9,8 @@ pytestmark = pytest.mark.gpu
 
 MICRO64 = dict(n_layers=3, d_model=136, n_q_heads=6, n_kv_heads=2, head_dim=64, d_ffn=200,
                vocab_text=301, vocab_speech=99, rms_eps=1e-6, rope_base=10000.0)
+MICRO256 = dict(n_layers=3, d_model=256, n_q_heads=4, n_kv_heads=2, head_dim=64, d_ffn=512,
+                vocab_text=301, vocab_speech=99, rms_eps=1e-6, rope_base=10000.0)
 
 
 @pytest.fixture(scope="module")
@@ -300,6 +302,26 @@ def test_tcgen05_passes_of_every_width(util, B):
     P.close()
 
 
+@pytest.mark.parametrize("options", [{}, {"attn_split": 128, "attn_ctas": 3}, {"attn_tma": 0}, {"attn_tc": 0}])
+@pytest.mark.parametrize("Hq,Hkv", [(7, 1), (32, 2), (4, 2)])
+def test_attention_with_positions_as_the_m_dimension(util, Hq, Hkv, options):
+    """Head dimension 128 on the tcgen05 path: 2 to 32 query vectors per kv head (more go to the kernel for
+    large blocks, or, with that one off, in several blocks of 32), prefixes that end before, on and
+    after a 128-position tile and its half, several splits, many more items than CTAs."""
+    dims = synth.model_dims(dict(MICRO256, n_layers=2, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=128), 1, 4, 0)
+    w = synth.make_weights(dims, seed=13)
+    lens = [2, 63, 65, 128, 129, 130, 200, 257, 390]
+    prompts = [synth.make_prompts(dims, 1, n, n, seed=60 + i)[0] for i, n in enumerate(lens)]
+    P = util.Pair(dims, w, len(lens), 420, 3, options=options, oracle_slots=[0, 2, 3, 4, 7, 8])
+    P.prefill(prompts)
+    for g in range(9):
+        mc = [synth.interleave(g + i, 1, 4) for i in range(len(lens))]
+        P.step([m for m, _ in mc], [c for _, c in mc])
+    assert P.stats["max_flush"] == 3
+    P.check_cache(8, range(1, 3), P.g.slot_state(8)[0] - P.g.slot_state(8)[1])
+    P.close()
+
+
 @pytest.mark.parametrize("n", [1, 33, 128, 129])
 def test_host_and_device_buffers_give_the_same_step(util, n):
     """Up to 128 sequences a step's arrays and host tokens travel as kernel arguments, beyond that through
@@ -404,10 +426,6 @@ def test_timeout_is_reported_once_and_the_context_recovers(util):
     ln, pend = P.g.slot_state(0)
     P.check_cache(0, range(1, 5), ln - pend)
     P.close()
-
-
-MICRO256 = dict(n_layers=3, d_model=256, n_q_heads=4, n_kv_heads=2, head_dim=64, d_ffn=512,
-                vocab_text=301, vocab_speech=99, rms_eps=1e-6, rope_base=10000.0)
 
 
 @pytest.mark.parametrize("K,maxp", [(4, 3), (3, 2)])
