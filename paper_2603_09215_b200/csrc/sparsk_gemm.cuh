@@ -429,6 +429,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
 // buffer, k and v appended to the cache.  With the inner dimension cut across CTAs the partial
 // sums are added into an fp32 scratch [rows][Hq*hd + 2*Hkv*hd] and qkv_finish_kernel does the rest.
 struct QkvEnd {
+    static constexpr bool XCHG = true;  // needs the exchange buffer (when the product is not cut)
     float *q_out;        // [rows][Hq*hd] fp32 (the attention kernels split it into two bf16 terms)
     kv_t *kc, *vc;       // this layer's cache [slot][Hkv][S][hd]
     const float2 *rope;  // [S][hd/2]
@@ -530,6 +531,7 @@ static __global__ void __launch_bounds__(QF_THREADS) qkv_finish_kernel(float *__
 
 // h[m][n] += (W x_m)[n]; with the inner dimension cut across CTAs the partial sums meet in h.
 struct ResidEnd {
+    static constexpr bool XCHG = false;
     float *h;  // [rows][n_out]
     int n_out, atomic;
 
@@ -557,6 +559,7 @@ struct ResidEnd {
 
 // u[m][f] = silu(gate) * up; accumulator 0 holds the gate rows, accumulator 1 the up rows.
 struct GateUpEnd {
+    static constexpr bool XCHG = false;
     bf16 *u, *u_lo;  // [rows][F]: u + u_lo carries the activation to 16 significant bits
     int F;
 
@@ -585,6 +588,7 @@ struct GateUpEnd {
 // Exit head over ids [lo, hi): per activation row the arg max (lowest id on ties) through the
 // same packed 64-bit key the small-batch path uses; optional dump of the logits.
 struct HeadEnd {
+    static constexpr bool XCHG = false;
     const int *seq_of_row;
     unsigned long long *argmax;
     float *logits;  // optional [n_seq][V]
