@@ -743,8 +743,11 @@ cudaError_t launch_gemm_inst(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1
     // (the exchange buffer is taken only by the ending that uses it: without it a third stage fits at up
     // to 16 rows, 123.9 -> 122.1 us a layer of the 28-layer shape at 12)
     const int xchg = Epi::XCHG && g.splits == 1 ? GM_XCHG_BYTES : 0;
+    // an MMA reads 128 rows of a weight tile; where the tiles are lower, what it reads behind the last
+    // one of the last stage has to be the CTA's own memory: the stage's activations, and padding
+    auto pad = [&](int kb) { return std::max(0, GM_BLK_BYTES - blk_bytes - 2 * kb * g.box_n * GM_BK * 2); };
     auto plan = [&](int budget) {
-        const int room = budget - 1024 - xchg;
+        const int room = budget - 1024 - xchg - pad(1);
         // two k-blocks per copy whenever the inner dimension allows the 3-D view and two stages fit
         g.three_d = (g.K % GM_BK == 0) && !DUO && 2 * stage_bytes(2) <= room && c->tc_kb != 1;
         g.kb = g.three_d ? 2 : 1;
@@ -756,7 +759,7 @@ cudaError_t launch_gemm_inst(sparsk_ctx *c, const TmaPair &a0, const TmaPair &a1
     const int n_units = g.units[0] + (g.pair ? 0 : g.units[1] + g.units[2]);
     const int k_stages = ((g.K + GM_BK - 1) / GM_BK + g.kb - 1) / g.kb;
     g.splits = std::max(1, std::min(g.splits, k_stages));
-    const size_t smem = 1024 + (size_t)g.stages * stage_bytes(g.kb) + xchg;
+    const size_t smem = 1024 + (size_t)g.stages * stage_bytes(g.kb) + xchg + pad(g.kb);
     const int per_sm = (smem + 1024) * 2 <= 227 * 1024 ? std::max(1, c->gemm_cps) : 1;  // CTAs of this launch that fit an SM
     const int grid_x = DUO ? 2 * std::max(1, std::min(c->n_sm / 2, (n_units + 1) / 2 * g.splits))
                            : std::max(1, std::min(c->n_sm * per_sm, n_units * g.splits));
