@@ -962,7 +962,7 @@ size_t mega_smem(const sparsk_dims &) { return (size_t)MK_SLOTS * MK_SLOT_BYTES 
 // Can a pass of n_rows rows go through the persistent kernel?
 bool use_mega(const sparsk_ctx *c, int n_rows)
 {
-    return c->mega && c->mk_ok && c->mk_coop && n_rows >= 1 && n_rows <= c->mk_max_rows && (n_rows <= 2 || c->mk_tc_ok) &&
+    return c->mega && c->mk_ok && c->mk_coop && n_rows >= 1 && n_rows <= c->mk_max_rows && (n_rows < MK_TC_ROWS || c->mk_tc_ok) &&
            mk_attn_bytes(c->dm.head_dim) <= MK_AREA_BYTES && c->dm.head_dim % (2 * MK_BOX_ROWS) == 0;
 }
 
@@ -1037,18 +1037,17 @@ cudaError_t run_mega(sparsk_ctx *c, int l_begin, int l_end, float *h, const RowS
     c->mk_trace_n = 1 + 6 * (l_end - l_begin);
     c->mk_bar_base += 6ull * (unsigned long long)(l_end - l_begin) * (unsigned long long)c->n_sm;
     const size_t smem = mega_smem(d);
+    // (three rows run as four with one masked)
     if (d.head_dim == 128) {
         switch (rs.n_rows) {
         case 1: return launch_mega_inst<1, 128>(c, a, smem);
         case 2: return launch_mega_inst<2, 128>(c, a, smem);
-        case 3: return launch_mega_inst<3, 128>(c, a, smem);
         default: return launch_mega_inst<4, 128>(c, a, smem);
         }
     }
     switch (rs.n_rows) {
     case 1: return launch_mega_inst<1, 64>(c, a, smem);
     case 2: return launch_mega_inst<2, 64>(c, a, smem);
-    case 3: return launch_mega_inst<3, 64>(c, a, smem);
     default: return launch_mega_inst<4, 64>(c, a, smem);
     }
 }

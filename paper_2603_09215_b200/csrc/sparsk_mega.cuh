@@ -43,6 +43,7 @@ constexpr int MK_BOX_BYTES = MK_BOX_ROWS * MK_BOX_COLS * 2;  // 8 KB
 constexpr int MK_SLOT_BYTES = 2 * MK_BOX_BYTES;              // two boxes per slot
 constexpr int MK_SLOTS = 8;
 constexpr int MK_MAX_ROWS = 4;
+constexpr int MK_TC_ROWS = 3;                   // rows from which the tensor-core form runs
 constexpr int MK_AREA_BYTES = 88 * 1024;        // shared memory behind the ring
 constexpr int MK_ATT_WARPS = 3;                 // consumer warps that run attention items
 constexpr int MK_ATT_NST = 2;

@@ -34,7 +34,7 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, const MkLayer *L, 
 
 // Merge of the splits: one warp per (row, query head, 32 output dims).  Lane s holds split s's
 // weight (att_splits <= 32); every lane owns one output dim and has all its loads in flight at once.
-template <int HD>
+template <int HD, bool PLANES>
 __device__ __forceinline__ void mk_merge(const MkArgs &a)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -54,7 +54,9 @@ __device__ __forceinline__ void mk_merge(const MkArgs &a)
         float num = 0.f;
 #pragma unroll
         for (int s = 0; s < MK_MAX_SPLITS; s++) num += v[s] * __shfl_sync(0xffffffffu, w_mine, s);
-        a.attn_o[(size_t)cell * HD + d] = den > 0.f ? num / den : 0.f;
+        const float o = den > 0.f ? num / den : 0.f;
+        if (PLANES) mk_put_planes(a.attn_o, a.Hq * HD, a.n_rows, cell / a.Hq, (cell % a.Hq) * HD + d, o);
+        else a.attn_o[(size_t)cell * HD + d] = o;
     }
 }
 

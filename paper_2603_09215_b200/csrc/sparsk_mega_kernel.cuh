@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
                     int row[2];
                     mk_band(ld.type, a, a.layers + ld.l, ld.band(), map, row);
                     const uint32_t dst = smem_u32(ring) + s * MK_SLOT_BYTES + lane * MK_BOX_BYTES;
-                    if (M >= 3)  // the same box as four swizzled 64-column blocks (entries MKW_N on)
+                    if (M >= MK_TC_ROWS)  // the same box as four swizzled 64-column blocks (entries MKW_N on)
                         tma_load_3d(dst, map[lane] + MKW_N, &sh.full[s], 0, row[lane], ld.ks * (MK_BOX_COLS / 64));
                     else
                         tma_load_2d(dst, map[lane], &sh.full[s], ld.ks * MK_BOX_COLS, row[lane]);
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
             // attention and the merge of its splits
             mk_attention<HD>(a, L, area, &sh);
             if (!(ok = mk_grid_barrier(a, &sh, epoch))) break;
-            mk_merge<HD>(a);
+            mk_merge<HD, M >= MK_TC_ROWS>(a);
             if (!(ok = mk_grid_barrier(a, &sh, epoch))) break;
             // O-projection
             if (!(ok = mk_proj<M>(MK_OPROJ, a, L, area, qd, nullptr, a.attn_o, nullptr, ring, &sh, it))) break;

@@ -449,3 +449,22 @@ def test_persistent_kernel_tensor_core_form_for_three_and_four_rows(util, K, max
     P.check_cache(0, range(1, 4), ln - pend)
     print("mega tc", P.stats)
     P.close()
+
+
+@pytest.mark.parametrize("rows", [3, 4])
+@pytest.mark.parametrize("d_ffn", [4352, 4416, 9280])
+def test_persistent_kernel_mlp_windows(util, rows, d_ffn):
+    """Three and four rows in the persistent kernel with an MLP whose activations just fit the shared-memory
+    area (17 steps of 256 columns), just do not, and take several half windows with a ragged end."""
+    dims = synth.model_dims(dict(MICRO256, d_ffn=d_ffn, n_layers=2), 1, 4, 0)
+    w = synth.make_weights(dims, seed=19)
+    prompts = synth.make_prompts(dims, rows, 5, 30, seed=4)
+    P = util.Pair(dims, w, rows, 64, 3)
+    P.prefill(prompts)
+    before = P.g.route_counts()["mega"]
+    for g in range(5):
+        mc = [synth.interleave(g, 1, 4)] * rows
+        P.step([m for m, _ in mc], [c for _, c in mc])
+    assert P.g.route_counts()["mega"] > before
+    P.check_cache(rows - 1, range(1, 3), P.g.slot_state(rows - 1)[0] - P.g.slot_state(rows - 1)[1])
+    P.close()
