@@ -13,9 +13,11 @@
 //               (128-byte swizzle) into a ring of shared-memory stages
 //   warp 1      issues tcgen05.mma for every stage, commits stages back to the producer and
 //               finished accumulators to the epilogue; owns the TMEM allocation
-//   warps 2..5  epilogue: tcgen05.ld of the accumulator (thread = weight row), then the
+//   warps 2..9  epilogue: tcgen05.ld of the accumulator (thread = weight row), then the
 //               operation's own ending: rotary embedding + cache append, residual add,
-//               SiLU(gate) * up, or logits + restricted arg max
+//               SiLU(gate) * up, or logits + restricted arg max.  Two warps per 32 weight rows, an
+//               accumulator each (gate/up: every other chunk of both): nothing overlaps the ending of
+//               a CTA's last unit.  With one warp per 32 rows a layer took 160 us at 64 rows, so 152.
 // The activation operand is carried as two bf16 terms, x = hi + lo with lo = bf16(x - hi), and
 // every weight tile is multiplied by both into the same accumulator: tcgen05 takes bf16 operands
 // only, and at random initialisation a single bf16 rounding of the activations early in the
@@ -46,7 +48,7 @@
 
 namespace sparsk {
 
-constexpr int GM_THREADS = 192;
+constexpr int GM_THREADS = 320;
 constexpr int GM_BM = 128;                     // weight rows per accumulator (UMMA M)
 constexpr int GM_BK = 64;                      // inner elements per k-block: one 128-byte swizzle span
 constexpr int GM_BOXES = 8;                    // heights of an activation copy: 16, 32, ..., 128 rows
@@ -54,7 +56,7 @@ constexpr int GM_MAX_N = 256;                  // activation rows per launch blo
 constexpr int GM_BLK_BYTES = GM_BM * GM_BK * 2;  // one accumulator's weights for one k-block: 16 KB
 constexpr int GM_MAX_STAGES = 6;
 constexpr int GM_CHUNK = 16;                   // accumulator columns per epilogue chunk
-constexpr int GM_XCHG_BYTES = GM_CHUNK * GM_BM * 4;
+constexpr int GM_XCHG_BYTES = 2 * GM_CHUNK * GM_BM * 4;
 constexpr unsigned long long GM_TIMEOUT_NS = WAIT_TIMEOUT_NS;
 
 // A unit of work is two accumulators of 128 weight rows each: either 256 consecutive rows of one
@@ -137,7 +139,7 @@ __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&r)[1
         : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+__device__ __forceinline__ void epi_barrier(int half) { asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory"); }
 
 // What an ending sees of one finished unit.
 struct TileCtx {
@@ -148,8 +150,9 @@ struct TileCtx {
     int m0, m_end;   // activation rows of this launch block: [m0, m_end)
     uint32_t taddr;  // TMEM address of accumulator 0, this thread's lane, column 0
     int acc_stride;  // columns between accumulator 0 and accumulator 1
-    float *xchg;     // [GM_CHUNK][128] floats shared by the 128 epilogue threads
+    float *xchg;     // [GM_CHUNK][128] floats shared by the 128 epilogue threads of a half
     int unit_rows;   // pair: rows of an accumulator that are the unit's
+    int half;        // which of the two warps of these weight rows: the accumulator, or every other chunk
     int lo_off;      // columns from the hi term's product to the lo term's (0: one accumulator holds both)
 
     // 16 activation rows (from c0 on) of accumulator a
@@ -220,7 +223,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
         }
         for (int b = 0; b < 2; b++) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], DUO ? 8 : 4);
+            mbar_init(&acc_empty[b], DUO ? 16 : 8);
         }
         giving_up_s = 0;
         never_s = 0;
@@ -381,7 +384,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
             }
         }
     } else {
-        // ------------------------------------------------------------ epilogue (warps 2..5)
+        // ------------------------------------------------------------ epilogue (warps 2..9)
         griddep_wait();
         const int quad = warp & 3;  // TMEM lanes this warp may read: 32 quad .. 32 quad + 31
         TileCtx tc;
@@ -389,7 +392,8 @@ __global__ void __launch_bounds__(GM_THREADS, 1)
         tc.m0 = m0;
         tc.m_end = m_end;
         tc.acc_stride = mma_n;
-        tc.xchg = xchg;
+        tc.half = (warp - 2) >> 2;
+        tc.xchg = xchg + tc.half * (GM_CHUNK * GM_BM);
         tc.unit_rows = g.unit_rows;
         tc.lo_off = DUO ? 0 : g.box_n;
         uint32_t unit_it = 0;
@@ -444,8 +448,8 @@ struct QkvEnd {
         const int n_rows_mat = (t.matrix == 0 ? Hq : Hkv) * hd;
         const int width = (Hq + 2 * Hkv) * hd;
         const int col0 = t.matrix == 0 ? 0 : (t.matrix == 1 ? Hq * hd : (Hq + Hkv) * hd);
-        for (int a = 0; a < 2; a++) {
-            const int n = t.unit_row + a * GM_BM + t.row;  // row inside its matrix
+        {
+            const int a = t.half, n = t.unit_row + a * GM_BM + t.row;  // row inside its matrix
             const int head = n / hd, i = n % hd, j = i & (half - 1);
             const bool hi = i >= half;
             for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
@@ -464,7 +468,7 @@ struct QkvEnd {
                 if (t.matrix < 2) {
 #pragma unroll
                     for (int c = 0; c < GM_CHUNK; c++) t.xchg[c * GM_BM + t.row] = v[c];
-                    epi_barrier();
+                    epi_barrier(t.half);
                 }
                 if (n < n_rows_mat) {
 #pragma unroll
@@ -483,7 +487,7 @@ struct QkvEnd {
                         }
                     }
                 }
-                if (t.matrix < 2) epi_barrier();
+                if (t.matrix < 2) epi_barrier(t.half);
             }
         }
     }
@@ -538,8 +542,8 @@ struct ResidEnd {
     template <bool DUO>
     __device__ void tile(const TileCtx &t) const
     {
-        for (int a = 0; a < 2; a++) {
-            const int n = t.unit_row + a * GM_BM + t.row;
+        {
+            const int a = t.half, n = t.unit_row + a * GM_BM + t.row;
             for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
                 float v[GM_CHUNK];
                 t.load<DUO>(a, c0, v);
@@ -567,7 +571,7 @@ struct GateUpEnd {
     __device__ void tile(const TileCtx &t) const
     {
         const int f = t.unit_row + t.row;
-        for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
+        for (int c0 = t.half * GM_CHUNK; t.m0 + c0 < t.m_end; c0 += 2 * GM_CHUNK) {
             float gt[GM_CHUNK], up[GM_CHUNK];
             t.load<DUO>(0, c0, gt);
             t.load<DUO>(1, c0, up);
@@ -598,8 +602,8 @@ struct HeadEnd {
     __device__ void tile(const TileCtx &t) const
     {
         const int lane = threadIdx.x & 31;
-        for (int a = 0; a < 2; a++) {
-            const int id = lo + t.unit_row + a * GM_BM + t.row;
+        {
+            const int a = t.half, id = lo + t.unit_row + a * GM_BM + t.row;
             for (int c0 = 0; t.m0 + c0 < t.m_end; c0 += GM_CHUNK) {
                 float v[GM_CHUNK];
                 t.load<DUO>(a, c0, v);
