@@ -499,8 +499,10 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
     const int n_small = rs.n_groups_h - n_big;
     const int warp_ctas = c->attn_ctas > 0 ? c->attn_ctas : c->n_sm * attn_warp_ctas_per_sm(d.head_dim, c->attn_stages);
     const int small_rows = blocks_tc ? std::max(1, std::min(rs.max_grp_rows, (c->attn_tc_min_q - 1) / G)) : rs.max_grp_rows;
+    const bool tma = c->attn_tma && c->attn_tma_ok;
+    a.table = tma && rs.n_groups_h <= AT_TABLE;
     AttnPlan pl = attn_plan(warp_ctas * AW_WARPS, blocks_tc ? std::max(1, n_small) : rs.n_groups_h, small_rows, G,
-                            d.n_kv_heads, rs.max_len, c->attn_split, blocks_tc ? 0 : rs.sum_len);
+                            d.n_kv_heads, rs.max_len, c->attn_split, blocks_tc ? 0 : rs.sum_len, a.table);
     if (blocks_tc) {
         // Groups with many query vectors per kv head go to the tcgen05 kernel (one CTA per SM, tiles
         // of 64 positions), the others to the mma.sync kernel; both launches cover all groups, a CTA
@@ -560,7 +562,6 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
     if (!blocks_tc || (c->attn_tc_min_q > 1 && n_small > 0)) {
         // every group is in the item space (the kernel skips those the other kernel takes)
         const long n_items = (long)rs.n_groups_h * a.n_qblk * d.n_kv_heads * a.n_splits;
-        const bool tma = c->attn_tma && c->attn_tma_ok;
         int warps = AW_WARPS;
         AttnWarpFn fn = nullptr;
         AttnWarpTmaFn fn_tma = nullptr;

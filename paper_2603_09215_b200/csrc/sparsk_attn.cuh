@@ -38,30 +38,49 @@ namespace sparsk {
 constexpr int AT_TP = 16;        // positions per tile
 constexpr int AT_MAX_SPLITS = 32;
 constexpr int AT_MIN_SPLIT = 64;
+constexpr int AT_TABLE = 256;    // groups a CTA's table of items holds
 constexpr int AW_WARPS = 4;      // warps per CTA of the stand-alone kernel
 constexpr int AW_NST = 2;        // ring stages per warp there (default; 3 is the other instantiation)
 
 // How a launch cuts the work: blocks of 16 query vectors per group, and the KV range into
-// splits so that every warp of the persistent grid gets a few items, none shorter than
-// AT_MIN_SPLIT positions (unless forced), at most AT_MAX_SPLITS.
+// splits of equal length, none shorter than AT_MIN_SPLIT positions (unless forced), at most
+// AT_MAX_SPLITS.
 struct AttnPlan {
     int n_qblk, split_len, n_splits;
 };
 // `sum_len` is the total of the groups' prefix lengths when the caller knows it (0: assume every
-// group is as long as the longest): with ragged lengths the splits past a short group's end are
-// empty items, and sizing by the real total keeps the number of items with work near 1.75 per
-// warp whatever the spread of the lengths (shorter items add set-up, longer ones a ragged end).
+// group is as long as the longest).  Two rules:
+// - `table` (the launch deals only items with work, AtTable): one round of items, for at most
+//   three in four of the warps, or for all of them where a group has few splits and one fewer would
+//   make items much longer.  There are at most sum_len / split + n_groups items with work per kv
+//   head and query block, and never more than n_groups * n_splits.  An item more than there are
+//   warps costs a second round on a machine that is then nearly empty; shorter items a
+//   set-up, a partial and a share of the merge each.  Layers (attention and GEMMs) in us, planned for 1.75
+//   items per warp (the other rule) / all warps / three in four / half of them: 64 ragged sequences of 256 to
+//   2,048 positions 163.3 / 157.6 / 156.8 / 158.9, 64 of 8,192 (two kv heads) 230.6 / 225.5 / 224.2 /
+//   228.9, 96 of 1,000 to 2,048 (two) 192.5 / 181.2 / 178.5 / 182.6, 64 of 1,024 (two) 157.2 / 150.2 / 149.2
+//   / 150.3; 12 of 256 to 2,048 125.3 / 123.8 / 123.7 / 123.9; 128 of 256 to 2,048 222.3 / 214.4 / 216.9 /
+//   237.0, 200 of 200 to 1,024 298.5 / 292.7 / 301.7.
+// - otherwise 1.75 items with work per warp, drawn as warps finish (stand-alone calls, which know
+//   a bound on the lengths only: 48 ragged groups of four rows 57 us, 64 to 75 with the rule above).
 inline AttnPlan attn_plan(int n_workers, int n_groups, int max_grp_rows, int G, int Hkv, int max_len, int forced_split,
-                          long sum_len = 0)
+                          long sum_len = 0, bool table = false)
 {
     AttnPlan p;
     const int nq = max_grp_rows * G;
     p.n_qblk = (nq + 15) / 16;
     int split = forced_split;
     if (split <= 0) {
-        const long groups = n_groups < 1 ? 1 : n_groups;
-        const long total = (sum_len > 0 ? sum_len : groups * (long)max_len) * p.n_qblk * Hkv;  // positions x heads to visit
-        split = (int)(total * 4 / (7L * n_workers));  // 1.75 items per warp (measured best at 64 ragged sequences)
+        const long groups = n_groups < 1 ? 1 : n_groups, heads = (long)p.n_qblk * Hkv;
+        const long total = (sum_len > 0 ? sum_len : groups * (long)max_len) * heads;  // positions x heads to visit
+        if (table) {
+            const long base = groups * heads, items = base * 4 > n_workers ? n_workers : n_workers * 3L / 4;
+            const long n = std::max(1L, items / base);
+            split = (int)((max_len + n - 1) / n);
+            if (base < items) split = (int)std::min<long>(split, (total + items - base - 1) / (items - base));
+        } else {
+            split = (int)(total * 4 / (7L * n_workers));
+        }
         if (split < AT_MIN_SPLIT) split = AT_MIN_SPLIT;
         if (split > max_len) split = max_len < 1 ? 1 : max_len;
     }
@@ -95,6 +114,7 @@ struct AttnArgs {
     int n_rows;               // rows in q/out; groups reaching beyond them are skipped
     int nq_min, nq_max;       // only groups with this many query vectors per kv head (another launch takes the rest)
     int max_groups;           // host bound on the number of groups (sizes the item space)
+    int table;                // 1: only items with work are dealt (at most AT_TABLE groups), and the merge reads only their partials
     int rows_early;           // 1: the row and group arrays are complete before the kernel's grid dependency resolves
     // Dynamic dealing of items (optional): a counter that only ever grows.  With W warps and
     // n > W items, warp w starts on item w and ticket ticket_base + t stands for item W + t
@@ -164,16 +184,34 @@ struct AtItem {
     bool valid;                      // false: not an item of this launch (no partial either)
 };
 __device__ __forceinline__ int at_n_groups(const AttnArgs &a) { return a.n_groups ? min(__ldcg(a.n_groups), a.max_groups) : a.max_groups; }
-// Item number idx of a launch -> descriptor (L2: the arrays are in global memory and may have been
-// written while this kernel was already resident).  Straight-line code: every load is clamped instead of
-// skipped, so the loads of one level go out together.
+// The item's span of positions, once its group (ok: one of this launch) is known.
+__device__ __forceinline__ void at_span(const AttnArgs &a, AtItem &it, bool ok)
+{
+    const int G = a.Hq / a.Hkv;
+    it.nq = it.nrows * G;
+    ok = ok && it.qb * 16 < it.nq && it.nq >= a.nq_min && it.nq <= a.nq_max;
+    // positions the item may look at: its split, cut at the last query row's own position (and
+    // at the cache itself: a row that points outside it reads nothing)
+    const bool sane = it.slot >= 0 && it.slot < a.n_slots && it.pos0 >= 0;
+    const int nq_here = min(16, it.nq - it.qb * 16);
+    const int last_row = (it.qb * 16 + nq_here - 1) / G;
+    const int kv_end_all = ok && sane ? min(it.pos0 + last_row + 1, a.S) : 0;
+    it.w_beg = it.sp * a.split_len;
+    it.w_end = min(it.w_beg + a.split_len, kv_end_all);
+    it.n_tiles = it.w_end > it.w_beg ? (it.w_end - it.w_beg + AT_TP - 1) / AT_TP : 0;
+    it.y0 = ((sane ? it.slot : 0) * a.Hkv + it.hk) * a.S;
+    it.valid = ok;
+}
+// Item number idx of a launch -> descriptor, from the row arrays alone: every group has as many items
+// as the longest (L2: the arrays are in global memory and may have been written while this kernel was
+// already resident).  Straight-line code: every load is clamped instead of skipped, so the loads of
+// one level go out together.
 template <bool L2 = false>
 __device__ __forceinline__ AtItem at_resolve(const AttnArgs &a, unsigned idx, unsigned n_items, int n_groups,
                                              const int *grp_row0, const int *grp_nrows, const int *row_slot,
                                              const int *row_pos)
 {
     AtItem it;
-    const int G = a.Hq / a.Hkv;
     unsigned t = idx < n_items ? idx : 0u;
     it.qb = (int)(t % a.n_qblk); t /= a.n_qblk;
     it.hk = (int)(t % a.Hkv); t /= a.Hkv;
@@ -188,19 +226,86 @@ __device__ __forceinline__ AtItem at_resolve(const AttnArgs &a, unsigned idx, un
     const int rc = ok ? it.row0 : 0;
     it.slot = ld(row_slot + rc);
     it.pos0 = ld(row_pos + rc);
-    it.nq = it.nrows * G;
-    ok = ok && it.qb * 16 < it.nq && it.nq >= a.nq_min && it.nq <= a.nq_max;
-    // positions the item may look at: its split, cut at the last query row's own position (and
-    // at the cache itself: a row that points outside it reads nothing)
-    const bool sane = it.slot >= 0 && it.slot < a.n_slots && it.pos0 >= 0;
-    const int nq_here = min(16, it.nq - it.qb * 16);
-    const int last_row = (it.qb * 16 + nq_here - 1) / G;
-    const int kv_end_all = ok && sane ? min(it.pos0 + last_row + 1, a.S) : 0;
-    it.w_beg = it.sp * a.split_len;
-    it.w_end = min(it.w_beg + a.split_len, kv_end_all);
-    it.n_tiles = it.w_end > it.w_beg ? (it.w_end - it.w_beg + AT_TP - 1) / AT_TP : 0;
-    it.y0 = ((sane ? it.slot : 0) * a.Hkv + it.hk) * a.S;
-    it.valid = ok;
+    at_span(a, it, ok);
+    return it;
+}
+// The items that have work, numbered without gaps: a launch of up to AT_TABLE groups deals only
+// those.  With ragged lengths a third to a half of the items that equal counts per group would
+// give are empty, and a split that had to let those through as well would be that much longer.
+// Every CTA makes the table for itself, before its grid dependency resolves where the arrays allow it.
+struct AtTable {
+    int4 grp[AT_TABLE];       // first row, rows, slot, first position
+    int first[AT_TABLE];      // items of the groups before this one (entries past the last group: all items)
+    int total;
+};
+// one thread per group and trip to the L2 (the arrays may have been written while this kernel was
+// already resident), then one warp for the running sum
+__device__ __forceinline__ void at_table_build(const AttnArgs &a, AtTable &tab, int n_groups)
+{
+    const int G = a.Hq / a.Hkv;
+    for (int g = threadIdx.x; g < AT_TABLE; g += blockDim.x) {
+        int items = 0;
+        int4 e = make_int4(0, 0, 0, 0);
+        if (g < n_groups) {
+            e.x = __ldcg(a.grp_row0 + g);
+            e.y = __ldcg(a.grp_nrows + g);
+            if (e.x >= 0 && e.y >= 1 && e.y <= a.n_rows && e.x <= a.n_rows - e.y && e.y * G >= a.nq_min && e.y * G <= a.nq_max) {
+                e.z = __ldcg(a.row_slot + e.x);
+                e.w = __ldcg(a.row_pos + e.x);
+                if (e.z >= 0 && e.z < a.n_slots && e.w >= 0) {
+                    const int len = e.w < a.S - e.y ? e.w + e.y : a.S;
+                    items = min((len + a.split_len - 1) / a.split_len, a.n_splits) * min((e.y * G + 15) / 16, a.n_qblk) * a.Hkv;
+                }
+            }
+        }
+        tab.grp[g] = e;
+        tab.first[g] = items;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        constexpr int PER = AT_TABLE / 32;
+        const int lane = threadIdx.x;
+        int x[PER], sum = 0;
+#pragma unroll
+        for (int i = 0; i < PER; i++) {
+            x[i] = tab.first[lane * PER + i];
+            sum += x[i];
+        }
+        int before = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o *= 2) {
+            const int y = __shfl_up_sync(0xffffffffu, before, o);
+            if (lane >= o) before += y;
+        }
+        if (lane == 31) tab.total = before;
+        before -= sum;
+#pragma unroll
+        for (int i = 0; i < PER; i++) {
+            tab.first[lane * PER + i] = before;
+            before += x[i];
+        }
+    }
+    __syncthreads();
+}
+// Item number idx (the same in all lanes) -> descriptor: the last group whose first item is not
+// past it, found in two ballots; inside a group the split runs slowest, so the query blocks of
+// one (kv head, split) run side by side and all but the first find their K/V tiles in the L2.
+__device__ __forceinline__ AtItem at_table_resolve(const AttnArgs &a, const AtTable &tab, unsigned idx, int lane)
+{
+    constexpr int PER = AT_TABLE / 32;
+    AtItem it;
+    const bool ok = idx < (unsigned)tab.total;
+    const int i = ok ? (int)idx : 0;
+    const int blk = 31 - __clz(__ballot_sync(0xffffffffu, tab.first[lane * PER] <= i));
+    const int g = blk * PER + 31 - __clz(__ballot_sync(0xffffffffu, lane < PER && tab.first[blk * PER + lane % PER] <= i));
+    const int4 e = tab.grp[g];
+    it.row0 = e.x; it.nrows = e.y; it.slot = e.z; it.pos0 = e.w;
+    int t = i - tab.first[g];
+    const int nqb = max(1, min((e.y * (a.Hq / a.Hkv) + 15) / 16, a.n_qblk));
+    it.qb = t % nqb; t /= nqb;
+    it.hk = t % a.Hkv;
+    it.sp = t / a.Hkv;
+    at_span(a, it, ok);
     return it;
 }
 // A warp's K/V ring, in either form: `issue` starts the copies of tile t of the split
@@ -716,6 +821,7 @@ __global__ void __launch_bounds__(WARPS * 32) attn_warp_tma_kernel(const __grid_
                                                                       int *status)
 {
     extern __shared__ __align__(1024) unsigned char awt_smem[];
+    __shared__ AtTable tab;
     __shared__ __align__(8) uint64_t bars[WARPS][NST];
     __shared__ int giving_up_s;
     griddep_launch();
@@ -743,12 +849,17 @@ __global__ void __launch_bounds__(WARPS * 32) attn_warp_tma_kernel(const __grid_
         return n_workers + __shfl_sync(0xffffffffu, t, 0);
     };
     unsigned item = (unsigned)warp * gridDim.x + blockIdx.x;
+    if (a.table) at_table_build(a, tab, n_groups);
+    auto resolve = [&]() {
+        return a.table ? at_table_resolve(a, tab, item, lane)
+                       : at_resolve<true>(a, item, n_items, n_groups, a.grp_row0, a.grp_nrows, a.row_slot, a.row_pos);
+    };
     // the first item is resolved while the kernel before this one still runs, if the row set allows it
-    AtItem it = at_resolve<true>(a, item, n_items, n_groups, a.grp_row0, a.grp_nrows, a.row_slot, a.row_pos);
+    AtItem it = resolve();
     if (a.rows_early) griddep_wait();
     for (bool first = true; item < n_items; first = false) {
         const unsigned next = dynamic ? draw() : item + n_workers;
-        if (!first) it = at_resolve<true>(a, item, n_items, n_groups, a.grp_row0, a.grp_nrows, a.row_slot, a.row_pos);
+        if (!first) it = resolve();
         item = next;
         // after a wait that ran out the warp keeps drawing (the ticket count must come out) but works no more
         if (!it.valid || giving_up_s) continue;
@@ -822,19 +933,25 @@ __global__ void __launch_bounds__(MG_THREADS) attn_merge_kernel(AttnArgs a, cons
     constexpr int V = HD / 4, R = MG_THREADS / V, PER = AT_MAX_SPLITS / R;  // float4s per partial, splits side by side, splits per thread
     __shared__ float4 acc_s[R][V];
     griddep_launch();
-    griddep_wait();
+    if (!a.rows_early) griddep_wait();
     const int row = blockIdx.x, head = blockIdx.y;
-    if (n_rows && row >= *n_rows) return;
+    if (n_rows && row >= __ldcg(n_rows)) return;
+    int n_splits = a.n_splits;
+    if (a.table) {  // the splits this row has: the rest of its cells is not of this call
+        const int slot = __ldcg(a.row_slot + row), pos = __ldcg(a.row_pos + row);
+        n_splits = slot >= 0 && slot < a.n_slots && pos >= 0 ? min(min(pos, a.S - 1) / a.split_len + 1, n_splits) : 0;
+    }
+    if (a.rows_early) griddep_wait();
     const int tid = threadIdx.x, lane = tid & 31, v = tid % V, r = tid / V;
     const size_t cell0 = ((size_t)row * a.Hq + head) * a.n_splits;
     float4 x[PER];
 #pragma unroll
     for (int k = 0; k < PER; k++) {
         const int s = r + k * R;
-        x[k] = s < a.n_splits ? __ldcg(reinterpret_cast<const float4 *>(a.part_o + (cell0 + s) * HD) + v) : make_float4(0.f, 0.f, 0.f, 0.f);
+        x[k] = s < n_splits ? __ldcg(reinterpret_cast<const float4 *>(a.part_o + (cell0 + s) * HD) + v) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    // a.n_splits <= AT_MAX_SPLITS = 32: every warp works all weights out, one split per lane
-    const float2 ml = lane < a.n_splits ? __ldcg(a.part_ml + cell0 + lane) : make_float2(-INFINITY, 0.f);
+    // n_splits <= AT_MAX_SPLITS = 32: every warp works all weights out, one split per lane
+    const float2 ml = lane < n_splits ? __ldcg(a.part_ml + cell0 + lane) : make_float2(-INFINITY, 0.f);
     const float M = warp_max(ml.x);
     const float w = ml.x == -INFINITY ? 0.f : __expf(ml.x - M);
     const float den = warp_sum(ml.y * w);

@@ -302,6 +302,28 @@ def test_tcgen05_passes_of_every_width(util, B):
     P.close()
 
 
+@pytest.mark.parametrize("B", [9, 40, 256, 257])
+@pytest.mark.parametrize("options", [{}, {"attn_split": 16, "attn_ctas": 2}])
+def test_attention_of_many_ragged_sequences(util, B, options):
+    """Up to 256 groups a launch numbers only the attention items with work (the longest prompt has five
+    16-position splits, most have one or two), beyond that every group has as many as the longest;
+    with two CTAs the items outnumber the warps many times over."""
+    dims = synth.model_dims("tiny", 2, 3, 0)
+    w = synth.make_weights(dims, seed=5)
+    lens = [(2, 16, 17, 9, 33, 3, 48)[i % 7] for i in range(B)]
+    lens[B // 2], lens[B - 1] = 70, 31
+    prompts = [synth.make_prompts(dims, 1, n, n, seed=90 + i)[0] for i, n in enumerate(lens)]
+    P = util.Pair(dims, w, B, 96, 2, options=dict(options, mega=0), oracle_slots=[0, 1, B // 2, B - 1])
+    P.prefill(prompts)
+    for g in range(4):
+        mc = [synth.interleave(g + i, 2, 4) for i in range(B)]
+        P.step([m for m, _ in mc], [c for _, c in mc])
+    for s_ in (1, B // 2, B - 1):
+        ln, pend = P.g.slot_state(s_)
+        P.check_cache(s_, range(1, 5), ln - pend)
+    P.close()
+
+
 @pytest.mark.parametrize("options", [{}, {"attn_split": 128, "attn_ctas": 3}, {"attn_tma": 0}, {"attn_tc": 0}])
 @pytest.mark.parametrize("Hq,Hkv", [(7, 1), (32, 2), (4, 2)])
 def test_attention_with_positions_as_the_m_dimension(util, Hq, Hkv, options):
