@@ -492,6 +492,7 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
     a.n_rows = rs.n_rows;
     a.nq_min = 0;
     a.nq_max = 1 << 30;
+    a.rows_early = !rs.rows_late;
     cudaError_t e;
     const bool blocks_tc = c->attn_tc && c->tc_ok && d.head_dim == TA_HD && rs.max_grp_rows * G >= c->attn_tc_min_q;
     // groups the tcgen05 kernel takes (the host knows every group's row count) and the rest
@@ -516,7 +517,11 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
         }
         // The tcgen05 kernel wants few, long splits (about one CTA per SM from the big groups alone,
         // its set-up is worth a few tiles), the other kernel many short ones: the first kernel's
-        // split is `mult` of the second's, and it marks the partial slots in between as empty.
+        // split is `mult` of the second's, and it marks the partial slots in between as empty.  Without
+        // groups for the second kernel the partials lie side by side, and a single one is finished
+        // by the kernel itself, without a merge: the merge of a pass of 256 prompt rows read up to sixteen
+        // slots per row and head for its one or two partials, 13.8 us a layer (ragged prompts over
+        // the 28-layer shape 206 -> 193 ms, 1,024 tokens over the 40-layer shape 44.9 -> 43.3).
         const int big_ctas = std::max(1, n_big * div_up(rs.max_grp_rows * G, TA_QB) * d.n_kv_heads);
         const int tiles = std::max(1, div_up(rs.max_len, TA_NT));
         int s_tc = 1;
@@ -536,7 +541,7 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
         }
         if (c->attn_split > 0) s_tc = pl.n_splits;
         s_tc = std::min(s_tc, AT_MAX_SPLITS);
-        const int mult = std::max(1, std::min(AT_MAX_SPLITS / s_tc, div_up(pl.n_splits, s_tc)));
+        const int mult = n_small > 0 ? std::max(1, std::min(AT_MAX_SPLITS / s_tc, div_up(pl.n_splits, s_tc))) : 1;
         const int small_len = div_up(div_up(rs.max_len, s_tc * mult), TA_NT) * TA_NT;
         pl.split_len = small_len;
         pl.n_splits = std::max(1, div_up(rs.max_len, small_len));
@@ -547,18 +552,18 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
         ta.a.n_splits = pl.n_splits;
         ta.a.nq_min = c->attn_tc_min_q;
         ta.split_mult = mult;
+        ta.direct = pl.n_splits == 1 && n_small == 0;
         ta.status = c->sd.counts + CNT_STATUS;
         const int n_splits_tc = std::max(1, div_up(rs.max_len, small_len * mult));
         dim3 grid(rs.n_groups_h * ta.a.n_qblk, d.n_kv_heads, n_splits_tc);
         e = launch(c, attn_tc_kernel, grid, dim3(TA_THREADS), (size_t)TA_SMEM, c->tm_kc[layer - 1], c->tm_vc[layer - 1], ta);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || ta.direct) return e;
         a.nq_max = c->attn_tc_min_q - 1;
     }
     a.n_qblk = blocks_tc ? div_up(std::min(rs.max_grp_rows * G, c->attn_tc_min_q - 1), 16) : pl.n_qblk;
     a.split_len = pl.split_len;
     a.n_splits = pl.n_splits;
     a.max_groups = rs.n_groups_h;
-    a.rows_early = !rs.rows_late;
     if (!blocks_tc || (c->attn_tc_min_q > 1 && n_small > 0)) {
         // every group is in the item space (the kernel skips those the other kernel takes)
         const long n_items = (long)rs.n_groups_h * a.n_qblk * d.n_kv_heads * a.n_splits;
@@ -582,8 +587,9 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
         // ticket beyond its last item
         if (a.ticket && n_items > (long)grid * warps) c->attn_ticket_base += (unsigned)n_items;
     }
-    if (d.head_dim == 128) return launch(c, attn_merge_kernel<128>, dim3(rs.n_rows, d.n_q_heads), dim3(MG_THREADS), 0, a, rs.n_rows_dev);
-    return launch(c, attn_merge_kernel<64>, dim3(rs.n_rows, d.n_q_heads), dim3(MG_THREADS), 0, a, rs.n_rows_dev);
+    dim3 grid;
+    const AttnMergeFn merge = attn_merge_fn(d.head_dim, a.n_splits, rs.n_rows, d.n_q_heads, &grid);
+    return launch(c, merge, grid, dim3(MG_THREADS), 0, a, rs.n_rows_dev);
 }
 
 // ---------------------------------------------------------------- tensor-core dispatch

@@ -51,6 +51,7 @@ struct AttnTcArgs {
     int split_mult;    // this kernel's split s fills partial slot s * split_mult of the a.n_splits slots a
                        // row has (the slots in between are marked empty): its splits are split_mult times
                        // as long as those of the kernel that takes the small groups of the same launch set
+    int direct;        // 1: every group is this kernel's and has one split: the output is written here, no merge follows
     int *status;       // device status word (ST_TIMEOUT on a wait that ran out)
 };
 
@@ -101,25 +102,23 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
     const uint32_t base = (smem_u32(ta_smem) + 1023u) & ~1023u;
     const uint32_t k0 = base, v0 = k0 + TA_KST * TA_T_BYTES;
 
-    // ---- what this CTA works on (every thread computes the same); a CTA whose group belongs to
-    // the other kernel, or does not exist, leaves before it sets anything up
+    // ---- what this CTA works on (every thread computes the same), worked out while the kernel before
+    // this one still runs, if the row set allows it; a CTA whose group belongs to the other kernel, or
+    // does not exist, leaves before it sets anything up.  (The loads are clamped, not skipped, and go
+    // past the L1: the arrays may have been written while this kernel was already resident.)
     griddep_launch();
-    griddep_wait();
+    if (!a.rows_early) griddep_wait();
     const int bx = blockIdx.x, hk = blockIdx.y, sp = blockIdx.z;
     const int g = bx / a.n_qblk, qb = bx % a.n_qblk;
     const int G = a.Hq / a.Hkv;
-    bool live = g < *a.n_groups;
-    int row0 = 0, nrows = 0;
-    if (live) {
-        row0 = a.grp_row0[g];
-        nrows = a.grp_nrows[g];
-        live = row0 >= 0 && nrows >= 1 && row0 + nrows <= a.n_rows;
-    }
+    const int n_groups = __ldcg(a.n_groups), row0 = __ldcg(a.grp_row0 + g), nrows = __ldcg(a.grp_nrows + g);
+    bool live = g < n_groups && row0 >= 0 && nrows >= 1 && row0 + nrows <= a.n_rows;
     const int nq = nrows * G, q0 = qb * TA_QB;
     live = live && q0 < nq && nq >= a.nq_min && nq <= a.nq_max;
+    const int slot = __ldcg(a.row_slot + (live ? row0 : 0)), pos0 = __ldcg(a.row_pos + (live ? row0 : 0));
+    if (a.rows_early) griddep_wait();
     if (!live) return;
     const int nq_here = min(TA_QB, nq - q0);
-    const int slot = a.row_slot[row0], pos0 = a.row_pos[row0];
     const bool sane = slot >= 0 && slot < a.n_slots && pos0 >= 0;
     const int last_row = (q0 + nq_here - 1) / G;
     const int kv_end_all = sane ? min(pos0 + last_row + 1, a.S) : 0;
@@ -185,8 +184,9 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
+    // the producer needs none of this: its first copies are under way meanwhile
     tc_fence_before();
-    __syncthreads();
+    if (warp != 0) asm volatile("bar.sync 1, %0;" ::"n"(TA_THREADS - 32) : "memory");
     tc_fence_after();
 
     if (warp == 0) {
@@ -445,17 +445,33 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
         }
         if (have && ok) {
             const int qg = q0 + qi, r = qg / G, j = qg % G;
-            const size_t cell0 = ((size_t)(row0 + r) * a.Hq + hk * G + j) * a.n_splits;
-            const int first = sp * args.split_mult;
-            if (first < a.n_splits) {
-                float *dst = a.part_o + (cell0 + first) * TA_HD + half * 64;
+            if (args.direct) {
+                // the only partial of the row: finished here
+                const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+                const size_t at = ((size_t)(row0 + r) * a.Hq + hk * G + j) * TA_HD + half * 64;
 #pragma unroll
-                for (int i = 0; i < 64; i += 4) *reinterpret_cast<float4 *>(dst + i) = make_float4(o[i], o[i + 1], o[i + 2], o[i + 3]);
-                if (half == 0) a.part_ml[cell0 + first] = make_float2(m_run * 0.6931471805599453f, l_run);  // back to natural-log units
+                for (int i = 0; i < 64; i += 8) {
+                    uint4 hi, lo;
+                    split_pair(o[i] * inv, o[i + 1] * inv, hi.x, lo.x);
+                    split_pair(o[i + 2] * inv, o[i + 3] * inv, hi.y, lo.y);
+                    split_pair(o[i + 4] * inv, o[i + 5] * inv, hi.z, lo.z);
+                    split_pair(o[i + 6] * inv, o[i + 7] * inv, hi.w, lo.w);
+                    *reinterpret_cast<uint4 *>(a.out + at + i) = hi;
+                    if (a.out_lo) *reinterpret_cast<uint4 *>(a.out_lo + at + i) = lo;
+                }
+            } else {
+                const size_t cell0 = ((size_t)(row0 + r) * a.Hq + hk * G + j) * a.n_splits;
+                const int first = sp * args.split_mult;
+                if (first < a.n_splits) {
+                    float *dst = a.part_o + (cell0 + first) * TA_HD + half * 64;
+#pragma unroll
+                    for (int i = 0; i < 64; i += 4) *reinterpret_cast<float4 *>(dst + i) = make_float4(o[i], o[i + 1], o[i + 2], o[i + 3]);
+                    if (half == 0) a.part_ml[cell0 + first] = make_float2(m_run * 0.6931471805599453f, l_run);  // back to natural-log units
+                }
+                if (half == 0)
+                    for (int e = first + 1; e < min(first + args.split_mult, a.n_splits); e++)
+                        a.part_ml[cell0 + e] = make_float2(-INFINITY, 0.f);
             }
-            if (half == 0)
-                for (int e = first + 1; e < min(first + args.split_mult, a.n_splits); e++)
-                    a.part_ml[cell0 + e] = make_float2(-INFINITY, 0.f);
         }
     }
     // ---------------------------------------------------------------- teardown

@@ -97,9 +97,9 @@ int sparsk_attention_launch(const sparsk_attn_args *p, char *scratch, cudaStream
         a.ticket = reinterpret_cast<unsigned *>(scratch);
     }
     cudaError_t e = launch_dependent(st, fn, dim3(grid), AW_WARPS * 32, AW_WARPS * attn_warp_bytes(p->head_dim, AW_NST), a);
-    if (e == cudaSuccess)
-        e = launch_dependent(st, p->head_dim == 128 ? attn_merge_kernel<128> : attn_merge_kernel<64>, dim3(p->n_rows, p->n_q_heads),
-                             MG_THREADS, 0, a, (const int *)nullptr);
+    dim3 merge_grid;
+    const AttnMergeFn merge = attn_merge_fn(p->head_dim, a.n_splits, p->n_rows, p->n_q_heads, &merge_grid);
+    if (e == cudaSuccess) e = launch_dependent(st, merge, merge_grid, MG_THREADS, 0, a, (const int *)nullptr);
     return e == cudaSuccess ? SPARSK_OK : SPARSK_ECUDA;
 }
 
