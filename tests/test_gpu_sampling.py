@@ -58,6 +58,22 @@ def test_tokens_land_where_the_reference_puts_them(mods, Vt, Vs, scale, seed):
     print("exact", exact, "of", n)
 
 
+@pytest.mark.parametrize("Vt,Vs", [(8192, 8193), (24576, 24577), (511, 513), (8191, 31)])
+def test_ranges_at_the_ends_of_the_kernel_forms(mods, Vt, Vs):
+    """16 weights a thread up to 8,192 ids, 48 up to 24,576, a cluster beyond; ranges that leave threads without ids."""
+    smp, binding = mods
+    n = 12
+    z = synth.make_logits(n, Vt + Vs, 1.0, Vt)
+    z[::4, 1::2] = z[::4, 0:1]  # some rows with half of their ids tied
+    u = synth.make_uniforms(n, Vs)
+    got = _run(binding, z, u, [i % 2 for i in range(n)], Vt, Vs)
+    for i in range(n):
+        lo, hi = (Vt, Vt + Vs) if i % 2 else (0, Vt)
+        ref = smp.nucleus_sample(z[i], lo, hi, T, TOP_P, float(u[i]))
+        assert lo <= got[i] < hi
+        assert smp.landing_error(ref, int(got[i]), float(u[i])) <= LAND_TOL, (i, int(got[i]), ref["token"])
+
+
 def test_worked_example_limits_and_ties(mods):
     smp, binding = mods
     z = np.log(np.array([[0.05, 0.5, 0.15, 0.3]] * 4, dtype=np.float32))
