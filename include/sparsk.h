@@ -189,8 +189,8 @@ int sparsk_set_debug(sparsk_ctx *ctx, float *exit_hidden /*device or NULL*/,
  * large value keeps everything on the GEMV path), "mega" (0/1: run passes of up to
  * four rows as one persistent kernel per layer range; default 1), "mega_max_rows" (1..4: the
  * largest pass that kernel takes; default 4. Passes of three and four rows use its tensor-core
- * inner loop, which needs d_model, d_ffn and n_heads * head_dim to be multiples of 64; other
- * shapes stop at two rows), "gemm_kb" (1: one 64-element block of the inner
+ * inner loop, which needs d_model, d_ffn and n_heads * head_dim to be multiples of 64 and d_model
+ * to be at most 4,352; other shapes stop at two rows), "gemm_kb" (1: one 64-element block of the inner
  * dimension per TMA copy instead of two; 0 = automatic), "attn_split" (positions
  * per KV split), "attn_dynamic" (0/1: the attention kernel's warps draw their work items from a
  * counter as they finish instead of taking every n-th one; default 1), "attn_ctas" (CTAs of that

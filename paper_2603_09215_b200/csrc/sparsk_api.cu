@@ -921,8 +921,14 @@ bool build_mega(sparsk_ctx *c)
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
-    // the swizzled three-dimensional view needs inner dimensions that are whole 64-element blocks
-    c->mk_tc_ok = d.d_model % 64 == 0 && d.d_ffn % 64 == 0 && qd % 64 == 0;
+    // The swizzled three-dimensional view needs inner dimensions that are whole 64-element blocks, and
+    // the RMSNorm of the form leaves whole residual rows in the activation area: 4,352 numbers.
+    // Passes of three and four wider rows take the tcgen05 path, which is the faster one there in
+    // any case.  us a layer at three / four rows: 4,352 numbers (MLP 11,776) 111 / 111 here and 117
+    // there; a form that normalised a window at a time took 117 / 165 at 4,416, 142 / 204 at 5,120
+    // (MLP 13,824) and 165 / 237 at 5,888 (15,360) where the tcgen05 path takes 113, 134 and 155.
+    c->mk_tc_ok = d.d_model % 64 == 0 && d.d_ffn % 64 == 0 && qd % 64 == 0 &&
+                  div_up(d.d_model, MK_BOX_COLS) <= mk_tc_window(MK_MAX_ROWS);
     auto enc_sw = [&](CUtensorMap *m, const void *base, size_t rows, size_t cols) {
         const cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64)};
         const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, 128};

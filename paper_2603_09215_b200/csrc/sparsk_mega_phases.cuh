@@ -334,8 +334,9 @@ __device__ __forceinline__ bool mk_project_tc(int type, const MkArgs &a, const M
     float *red = reinterpret_cast<float *>(area + MK_AREA_BYTES - MK_TC_RED_BYTES);
     MkWalk walk;
     walk.init(type, a);
-    // The activations of a whole phase at once, or pieces of at most `win` k-steps that follow the CTA's
-    // segments through two buffers.
+    // The activations of a whole phase at once, or pieces of at most `win` k-steps of `x` that follow the
+    // CTA's segments through two buffers.  Phases that start from `h` always get the whole row (the
+    // host sends wider residual rows elsewhere: mk_tc_ok).
     const bool whole = walk.k_steps <= mk_tc_window(M);
     const int win = whole ? walk.k_steps : mk_tc_window(M) / 2;
     const int ncols = win * MK_BOX_COLS, rs = ncols + 8;

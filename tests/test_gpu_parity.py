@@ -490,3 +490,28 @@ def test_persistent_kernel_mlp_windows(util, rows, d_ffn):
     assert P.g.route_counts()["mega"] > before
     P.check_cache(rows - 1, range(1, 3), P.g.slot_state(rows - 1)[0] - P.g.slot_state(rows - 1)[1])
     P.close()
+
+
+@pytest.mark.parametrize("d_model,route", [(4352, "mega"), (4416, "tc"), (5120, "tc")])
+@pytest.mark.parametrize("rows", [1, 3, 4])
+def test_three_and_four_wide_rows(util, rows, d_model, route):
+    """Residual rows that just fit the persistent kernel's activation area as three or four rows, and rows
+    that do not, which take the tcgen05 path: batches of three and four, and one sequence whose
+    refresh carries three pending rows."""
+    dims = synth.model_dims(dict(MICRO256, d_model=d_model, n_layers=2, d_ffn=128), 1, 4, 0)
+    w = synth.make_weights(dims, seed=23)
+    prompts = synth.make_prompts(dims, rows, 5, 20, seed=7)
+    P = util.Pair(dims, w, rows, 64, 3)
+    P.prefill(prompts)
+    other = "tc" if route == "mega" else "mega"
+    for g in range(6):
+        before = P.g.route_counts()
+        P.step([0 if g == 0 else 1] * rows, [0 if g == 0 else g - 1] * rows)
+        after = P.g.route_counts()
+        if rows >= 3 or g == 5:              # g = 5 is the refresh: three pending rows and the current one
+            assert after[route] > before[route]
+        if (rows >= 3 and g < 5) or (rows == 1 and route == "mega"):
+            assert after[other] == before[other]
+    assert P.stats["max_flush"] == 3
+    P.check_cache(rows - 1, range(1, 3), P.g.slot_state(rows - 1)[0] - P.g.slot_state(rows - 1)[1])
+    P.close()
