@@ -675,11 +675,10 @@ bool build_maps(sparsk_ctx *c)
     };
     fill(c->tm_wq, c->wq, qd, d.d_model, 2 * GM_BM); fill(c->tm_wk, c->wk, kd, d.d_model, 2 * GM_BM);
     fill(c->tm_wv, c->wv, kd, d.d_model, 2 * GM_BM); fill(c->tm_wo, c->wo, d.d_model, qd, 2 * GM_BM);
-    // gate/up unit height: the one whose units leave the busiest SM the fewest rows; where the MMAs
-    // and not the weight stream take the time it is what an MMA covers, the full 128
-    c->gu_rows[0] = c->gu_rows[1] = GM_BM;
-    for (int r = GM_BM - 8; r >= 32; r -= 8)
-        if (div_up(div_up(d.d_ffn, r), c->n_sm) * r < div_up(div_up(d.d_ffn, c->gu_rows[0]), c->n_sm) * c->gu_rows[0]) c->gu_rows[0] = r;
+    // gate/up unit height: dealt evenly to the SMs, or, where the MMAs and not the weight stream take
+    // the time, what an MMA covers, the full 128
+    c->gu_rows[0] = gateup_unit_rows(d.d_ffn, c->n_sm);
+    c->gu_rows[1] = GM_BM;
     for (int t = 0; t < 2; t++) {
         fill(c->tm_wg[t], c->w_gate, d.d_ffn, d.d_model, c->gu_rows[t]);
         fill(c->tm_wu[t], c->w_up, d.d_ffn, d.d_model, c->gu_rows[t]);

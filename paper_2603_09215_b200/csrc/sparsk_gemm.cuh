@@ -68,6 +68,19 @@ constexpr unsigned long long GM_TIMEOUT_NS = WAIT_TIMEOUT_NS;
 // nanoseconds per copy whatever its size, so a stage is made of few, large boxes: with a
 // three-dimensional view [64 elements][rows][K/64] of a row-major matrix one box carries two
 // k-blocks of every row.
+// Height of such a pair: the lowest (a multiple of 8) with which the busiest SM still takes as few units one
+// after another as with 128 rows.  More, lower units would leave it fewer rows, but a k-block of a
+// unit costs at least its MMAs and copies, 0.53 us, and below 88 rows that is more than its weights
+// take to arrive (0.77 us for 128).  Gate/up of 8,192 x 28,672 at 5 / 128 rows: 206 / 292 us with units of 128
+// rows (two each), 331 / 588 with 40 (five), 158 / 265 with 104 (two).
+inline int gateup_unit_rows(int F, int n_sm)
+{
+    const long units = (((long)F + GM_BM - 1) / GM_BM + n_sm - 1) / n_sm * n_sm;  // as many as cost the same time
+    int r = GM_BM;
+    while (r > 32 && ((long)F + r - 9) / (r - 8) <= units) r -= 8;
+    return r;
+}
+
 struct GemmArgs {
     int K;         // inner dimension
     int units[3];  // units of matrix 0, 1, 2 (pair: units[0] only)

@@ -302,6 +302,20 @@ def test_tcgen05_passes_of_every_width(util, B):
     P.close()
 
 
+@pytest.mark.parametrize("B", [5, 128])
+def test_mlp_whose_gateup_units_take_two_rounds(util, B):
+    """28,672 MLP rows: units of 104 rows, two for most SMs."""
+    dims = synth.model_dims(dict(MICRO256, d_ffn=28672, n_layers=2), 1, 2, 0)
+    w = synth.make_weights(dims, seed=17)
+    prompts = synth.make_prompts(dims, B, 3, 9, seed=5)
+    P = util.Pair(dims, w, B, 16, 1, oracle_slots=[0, B - 1])
+    P.prefill(prompts)
+    for g in range(3):
+        mc = [synth.interleave(g + i, 1, 4) for i in range(B)]
+        P.step([m for m, _ in mc], [c for _, c in mc])
+    P.close()
+
+
 @pytest.mark.parametrize("B", [9, 40, 256, 257])
 @pytest.mark.parametrize("options", [{}, {"attn_split": 16, "attn_ctas": 2}])
 def test_attention_of_many_ragged_sequences(util, B, options):
