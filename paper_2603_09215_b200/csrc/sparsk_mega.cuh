@@ -218,6 +218,7 @@ struct MkShared {
     uint64_t full[MK_SLOTS], empty[MK_SLOTS];
     int giving_up, never;
     int row_slot[MK_MAX_ROWS], row_pos[MK_MAX_ROWS], grp_row0[MK_MAX_ROWS], grp_nrows[MK_MAX_ROWS];  // copies of the row set
+    int row_splits[MK_MAX_ROWS];         // splits of the attention phase that hold positions of the row
     float red[MK_CW];
     float red_rows[MK_MAX_ROWS][MK_CW];  // per-row partial sums of squares (tensor-core form: all rows at once)
 };

@@ -34,20 +34,22 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, const MkLayer *L, 
 
 // Merge of the splits: one warp per (row, query head, 32 output dims).  Lane s holds split s's
 // weight (att_splits <= 32); every lane owns one output dim and has all its loads in flight at once.
+// Only the splits that hold positions of the row are read: nobody writes the partials of the others, and
+// what they hold (NaN for one) would outlast a weight of zero.
 template <int HD, bool PLANES>
-__device__ __forceinline__ void mk_merge(const MkArgs &a)
+__device__ __forceinline__ void mk_merge(const MkArgs &a, const MkShared *sh)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int PARTS = HD / 32;
     const int n_items = a.n_rows * a.Hq * PARTS;
     for (int item = warp * gridDim.x + blockIdx.x; item < n_items; item += gridDim.x * MK_CW) {
-        const int cell = item / PARTS, d = (item % PARTS) * 32 + lane;
+        const int cell = item / PARTS, d = (item % PARTS) * 32 + lane, live = sh->row_splits[cell / a.Hq];
         const size_t cell0 = (size_t)cell * a.att_splits;
         float2 ml = make_float2(-INFINITY, 0.f);
-        if (lane < a.att_splits) ml = a.part_ml[cell0 + lane];
+        if (lane < live) ml = a.part_ml[cell0 + lane];
         float v[MK_MAX_SPLITS];
 #pragma unroll
-        for (int s = 0; s < MK_MAX_SPLITS; s++) v[s] = s < a.att_splits ? a.part_o[(cell0 + s) * HD + d] : 0.f;
+        for (int s = 0; s < MK_MAX_SPLITS; s++) v[s] = s < live ? a.part_o[(cell0 + s) * HD + d] : 0.f;
         const float M = warp_max(ml.x);
         const float w_mine = ml.x == -INFINITY ? 0.f : __expf(ml.x - M);
         const float den = warp_sum(ml.y * w_mine);

@@ -71,13 +71,15 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
         }
         sh.giving_up = 0;
         sh.never = 0;
-        for (int i = 0; i < MK_MAX_ROWS; i++) {
-            sh.row_slot[i] = i < a.n_rows ? a.row_slot[i] : -1;
-            sh.row_pos[i] = i < a.n_rows ? a.row_pos[i] : -1;
-            sh.grp_row0[i] = i < a.n_groups ? a.grp_row0[i] : -1;
-            sh.grp_nrows[i] = i < a.n_groups ? a.grp_nrows[i] : 0;
-        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1 && lane < MK_MAX_ROWS) {
+        const int i = lane;
+        sh.row_slot[i] = i < a.n_rows ? a.row_slot[i] : -1;
+        sh.row_pos[i] = i < a.n_rows ? a.row_pos[i] : -1;
+        sh.row_splits[i] = i < a.n_rows ? min(a.row_pos[i] / a.att_split_len + 1, a.att_splits) : 0;
+        sh.grp_row0[i] = i < a.n_groups ? a.grp_row0[i] : -1;
+        sh.grp_nrows[i] = i < a.n_groups ? a.grp_nrows[i] : 0;
     }
     __syncthreads();
 
@@ -132,7 +134,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
             // attention and the merge of its splits
             mk_attention<HD>(a, L, area, &sh);
             if (!(ok = mk_grid_barrier(a, &sh, epoch))) break;
-            mk_merge<HD, M >= MK_TC_ROWS>(a);
+            mk_merge<HD, M >= MK_TC_ROWS>(a, &sh);
             if (!(ok = mk_grid_barrier(a, &sh, epoch))) break;
             // O-projection
             if (!(ok = mk_proj<M>(MK_OPROJ, a, L, area, qd, nullptr, a.attn_o, nullptr, ring, &sh, it))) break;

@@ -464,6 +464,38 @@ def test_timeout_is_reported_once_and_the_context_recovers(util):
     P.close()
 
 
+@pytest.mark.parametrize("options", [{}, {"mega": 0}])
+@pytest.mark.parametrize("B", [2, 3])
+@pytest.mark.parametrize("hd", [64, 128])
+def test_partials_of_an_earlier_step_do_not_leak(util, hd, B, options):
+    """A short sequence beside a long one leaves most of its attention splits empty; what their partials hold
+    from an earlier step (here NaN: a cache that was imported broken, and mended afterwards) must
+    not reach the output."""
+    dims = synth.model_dims(dict(MICRO256, head_dim=hd), 2, 3, 0)
+    w = synth.make_weights(dims, seed=29)
+    lens = [300, 40, 20][:B]
+    prompts = [synth.make_prompts(dims, 1, n, n, seed=70 + i)[0] for i, n in enumerate(lens)]
+    P = util.Pair(dims, w, B, 330, 2, options=options)
+    P.prefill(prompts)
+    layers, n = range(1, dims["n_layers"] + 1), lens[0] - 1
+    good = {l: tuple(t.clone() for t in P.g.export_kv(0, l, 0, n)) for l in layers}
+    for l in layers:
+        P.g.import_kv(0, l, 0, good[l][0], torch.full_like(good[l][1], float("nan")))
+    tok, dep = np.zeros(B, np.int32), np.zeros(B, np.int32)
+    for row in range(1, B):                      # the long sequence in the place of every short one
+        order = list(range(B))
+        order[0], order[row] = order[row], order[0]
+        P.g.decode_step_host(order, np.ones(B, np.int32), [0] * B, [0] * B, tok, dep)
+        for s_ in range(B):
+            P.g.set_len(s_, lens[s_] - 1)
+    for l in layers:
+        P.g.import_kv(0, l, 0, *good[l])
+    for g in range(3):
+        mc = [synth.interleave(g, 1, 4)] * B
+        P.step([m for m, _ in mc], [c for _, c in mc])
+    P.close()
+
+
 @pytest.mark.parametrize("K,maxp", [(4, 3), (3, 2)])
 def test_persistent_kernel_tensor_core_form_for_three_and_four_rows(util, K, maxp):
     """Flushes of two and three pending rows (passes of three and four rows) inside the persistent
