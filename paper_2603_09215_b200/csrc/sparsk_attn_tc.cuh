@@ -106,7 +106,6 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
     // this one still runs, if the row set allows it; a CTA whose group belongs to the other kernel, or
     // does not exist, leaves before it sets anything up.  (The loads are clamped, not skipped, and go
     // past the L1: the arrays may have been written while this kernel was already resident.)
-    griddep_launch();
     if (!a.rows_early) griddep_wait();
     const int bx = blockIdx.x, hk = blockIdx.y, sp = blockIdx.z;
     const int g = bx / a.n_qblk, qb = bx % a.n_qblk;
@@ -116,8 +115,10 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
     const int nq = nrows * G, q0 = qb * TA_QB;
     live = live && q0 < nq && nq >= a.nq_min && nq <= a.nq_max;
     const int slot = __ldcg(a.row_slot + (live ? row0 : 0)), pos0 = __ldcg(a.row_pos + (live ? row0 : 0));
-    if (a.rows_early) griddep_wait();
-    if (!live) return;
+    if (!live) {
+        if (a.rows_early) griddep_wait();
+        return;
+    }
     const int nq_here = min(TA_QB, nq - q0);
     const bool sane = slot >= 0 && slot < a.n_slots && pos0 >= 0;
     const int last_row = (q0 + nq_here - 1) / G;
@@ -155,6 +156,12 @@ __global__ void __launch_bounds__(TA_THREADS, 1)
     tc_fence_before();
     __syncthreads();  // the TMEM base address is known
     tc_fence_after();
+    // The next kernel may come only now: a CTA of it beside this one would otherwise take the TMEM and
+    // wait for this kernel to finish while this one waits for the TMEM.  (The wait for the kernel
+    // before stands behind the allocation: all its CTAs have theirs, or this kernel would not be
+    // here, and need nothing of this one to finish.)
+    griddep_launch();
+    if (a.rows_early) griddep_wait();
     const uint32_t tmem_base = tmem_base_s;
     const uint32_t t_s0 = tmem_base + TA_C_S, t_o = tmem_base + TA_C_O, t_p = tmem_base + TA_C_P, t_q = tmem_base + TA_C_Q;
 

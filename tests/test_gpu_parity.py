@@ -412,6 +412,22 @@ def test_prefill_passes_beyond_128_rows(util, rows, shape):
     P.close()
 
 
+@pytest.mark.parametrize("kb", [48, 110])
+@pytest.mark.parametrize("rows", [40, 128, 256])
+def test_prompt_attention_beside_small_gemm_rings(util, rows, kb):
+    """Rings small enough for a GEMM CTA to share an SM with the tcgen05 attention of a prompt pass, which has
+    no merge between the two: the attention takes its tensor memory before it lets the GEMM come."""
+    dims = synth.model_dims(dict(MICRO256, n_q_heads=8, head_dim=128), 2, 3, 0)
+    w = synth.make_weights(dims, seed=9)
+    prompts = synth.make_prompts(dims, 3, 60, 300, seed=2)
+    P = util.Pair(dims, w, 3, 320, 2, prefill_rows=rows, options={"gemm_smem_kb": kb}, oracle_slots=[0, 2])
+    P.prefill(prompts)
+    for s_ in (0, 2):
+        P.check_cache(s_, range(1, 4), len(prompts[s_]) - 1)
+    P.step([0, 1, 0], [0, 1, 0])
+    P.close()
+
+
 @pytest.mark.parametrize("d_model", [4104, 8456])
 def test_wide_rows_on_the_tcgen05_path(util, d_model):
     """Residual rows wider than what the RMSNorm kernel's threads cover in one pass (4,096 numbers) and
