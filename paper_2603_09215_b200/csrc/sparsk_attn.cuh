@@ -942,7 +942,15 @@ __device__ __forceinline__ void at_store_merged(const AttnArgs &a, int row, int 
     split_pair(num.x * inv, num.y * inv, hi.x, lo.x);
     split_pair(num.z * inv, num.w * inv, hi.y, lo.y);
     const size_t o = ((size_t)row * a.Hq + head) * HD + v * 4;
-    *reinterpret_cast<uint2 *>(a.out + o) = hi;
+    if (((uintptr_t)a.out & 7) == 0) {
+        *reinterpret_cast<uint2 *>(a.out + o) = hi;
+    } else {  // a caller's buffer may start at any element
+        unsigned short *to = reinterpret_cast<unsigned short *>(a.out + o);
+        to[0] = (unsigned short)hi.x;
+        to[1] = (unsigned short)(hi.x >> 16);
+        to[2] = (unsigned short)hi.y;
+        to[3] = (unsigned short)(hi.y >> 16);
+    }
     if (a.out_lo) *reinterpret_cast<uint2 *>(a.out_lo + o) = lo;
 }
 template <int HD>

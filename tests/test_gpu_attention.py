@@ -65,6 +65,34 @@ def test_attention_matches_oracle(Hq, Hkv, hd, S, groups):
     assert err <= REL_TOL, err
 
 
+@pytest.mark.parametrize("hd", [64, 128])
+@pytest.mark.parametrize("last", [40, 2500])
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_output_may_start_at_any_element(hd, last, offset):
+    """Few splits (a warp merges a row's head) and many (a block does): an output buffer that starts 2, 4 or 6
+    bytes past an 8-byte boundary receives the same bits, and nothing around it is written."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2603_09215_b200 import binding
+    Hq, Hkv = 6, 2
+    q, k, v, row_slot, row_pos, g0, gn = make_case(5, 2, Hq, Hkv, hd, 2600, [(0, last, 3), (1, 11, 1)])
+    dev = "cuda"
+    t = lambda a: torch.tensor(a, dtype=torch.int32, device=dev)
+    keep = [q.to(dev), k.to(dev), v.to(dev), t(row_slot), t(row_pos), t(g0), t(gn)]
+    n = q.shape[0] * Hq * hd
+    scratch = torch.empty(binding.attention_scratch_bytes(q.shape[0], Hq, hd), dtype=torch.uint8, device=dev)
+    got = []
+    for off in (0, offset):
+        buf = torch.full((n + 16,), 7.0, dtype=torch.bfloat16, device=dev)
+        out = buf[off:off + n].view(q.shape[0], Hq * hd)
+        args = binding.attn_args(*keep[:3], out, *keep[3:], max(gn), max(row_pos) + 1, Hq)
+        assert binding.attention(args, scratch) == binding.OK
+        torch.cuda.synchronize()
+        assert bool((buf[:off] == 7.0).all()) and bool((buf[off + n:] == 7.0).all())
+        got.append(out.clone())
+    assert bool(torch.isfinite(got[0].float()).all()) and torch.equal(got[0], got[1])
+
+
 def test_attention_rejects_bad_arguments():
     if not torch.cuda.is_available():
         pytest.skip("needs a CUDA device")
