@@ -70,7 +70,7 @@ struct sparsk_ctx {
     float2 *rope;
     StepDesc sd;
     int *staged, *tok_dev;
-    int *pf_rows;                // row set of a prefill pass, laid out as it is staged (see sparsk_prefill)
+    int *pf_rows;                // row set of a prefill pass: slot and position of every row, the groups, the two counts
     float *h_lo, *h_up;
     float *qbuf;
     float *h_last, *q_last;      // the current rows alone, for the trimmed last layer of the upper pass
@@ -198,9 +198,9 @@ int cap_rows_of(const sparsk_dims *d)
     return (int)std::max<long>(dec, pf);
 }
 
-// Ints that describe a prefill pass: slot, position and token index of every row, first row and
-// row count of every group (one per prompt that takes part), the two counts.
-size_t prefill_ints(const sparsk_dims *d) { return 3 * (size_t)cap_rows_of(d) + 2 * (size_t)d->max_seqs + 2; }
+// Ints that describe a prefill pass: slot and position of every row, first row and row count of every
+// group (one per prompt that takes part), the two counts.
+size_t prefill_ints(const sparsk_dims *d) { return 2 * (size_t)cap_rows_of(d) + 2 * (size_t)d->max_seqs + 2; }
 
 // Lays the workspace out; with base == NULL only measures it.
 size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
@@ -1208,7 +1208,7 @@ extern "C" int sparsk_create(const sparsk_dims *dims, const sparsk_weights *w, v
             break;
         }
         for (int i = 0; i < STAGE_RING && rc == SPARSK_OK; i++) {
-            if ((ce = cudaHostAlloc((void **)&ctx->stage_host[i], sizeof(int) * std::max<size_t>(3 * (size_t)dims->max_seqs, prefill_ints(&ctx->dm)), cudaHostAllocDefault)) != cudaSuccess ||
+            if ((ce = cudaHostAlloc((void **)&ctx->stage_host[i], 3 * sizeof(int) * dims->max_seqs, cudaHostAllocDefault)) != cudaSuccess ||
                 (ce = cudaEventCreateWithFlags(&ctx->stage_ev[i], cudaEventDisableTiming)) != cudaSuccess)
                 rc = fail(ctx, SPARSK_ECUDA, "staging setup failed: %s", cudaGetErrorString(ce));
         }
@@ -1531,29 +1531,36 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
     // short ones and the beginning of the next share a pass (each a group of its own), so that only
     // the last pass of the call runs with fewer rows.
     const int chunk = std::min(d.prefill_rows, ctx->cap_rows), G_heads = d.n_q_heads / d.n_kv_heads;
-    std::vector<int> slot, pos, tok, g0, gn, base(n_seqs);
-    for (int i = 0; i < n_seqs; i++) base[i] = ctx->h_len[slots[i]];
+    int *const r_slot = ctx->pf_rows, *const r_pos = r_slot + ctx->cap_rows, *const r_g0 = r_pos + ctx->cap_rows,
+              *const r_gn = r_g0 + d.max_seqs, *const r_cnt = r_gn + d.max_seqs;
+    PromptPieces in;
     for (int i = 0, done = 0; i < n_seqs;) {
-        slot.clear(); pos.clear(); tok.clear(); g0.clear(); gn.clear();
-        int n = 0, max_grp = 1, max_len = 0, n_big = 0;
+        int n = 0, ng = 0, k = 0, max_grp = 1, max_len = 0, n_big = 0;  // rows, groups (k of them in `in`) of the pass
         long sum_len = 0;
+        auto begin = [&](bool last) {  // the k pieces in hand
+            const int rows = in.row0[k] - in.row0[0], first = ng - k, pieces = k;
+            k = 0;
+            return launch(ctx, prompt_begin_kernel, dim3(rows), dim3(128), 0, in, pieces, first, last, tokens, r_slot, r_pos, r_g0,
+                          r_gn, r_cnt, ctx->embed, ctx->h_up, d.d_model, d.vocab_text + d.vocab_speech, ctx->sd.counts + CNT_STATUS);
+        };
         while (i < n_seqs && n < chunk) {
             const int s = slots[i], left = offsets[i + 1] - offsets[i] - done, take = std::min(chunk - n, left);
             if (take > 0) {
-                const int pos0 = base[i] + done;
-                for (int j = 0; j < take; j++) {
-                    slot.push_back(s);
-                    pos.push_back(pos0 + j);
-                    tok.push_back(offsets[i] + done + j);
-                }
-                g0.push_back(n);
-                gn.push_back(take);
+                if (k == PP_MAX) CU(begin(false));
+                const int pos0 = ctx->h_len[s];
+                in.row0[k] = n;
+                in.slot[k] = s;
+                in.pos[k] = pos0;
+                in.token[k] = offsets[i] + done;
+                in.row0[++k] = n + take;
+                ng++;
                 max_grp = std::max(max_grp, take);
                 max_len = std::max(max_len, pos0 + take);
                 sum_len += pos0 + take;
                 n_big += take * G_heads >= ctx->attn_tc_min_q;
                 n += take;
                 done += take;
+                ctx->h_len[s] = pos0 + take;
             }
             if (take == left) {
                 i++;
@@ -1561,27 +1568,12 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
             }
         }
         if (n == 0) break;
-        const int ng = (int)g0.size(), ring = ctx->stage_next;
-        ctx->stage_next = (ring + 1) % STAGE_RING;
-        CU(cudaEventSynchronize(ctx->stage_ev[ring]));
-        int *st = ctx->stage_host[ring];
-        std::copy(slot.begin(), slot.end(), st);
-        std::copy(pos.begin(), pos.end(), st + n);
-        std::copy(tok.begin(), tok.end(), st + 2 * n);
-        std::copy(g0.begin(), g0.end(), st + 3 * n);
-        std::copy(gn.begin(), gn.end(), st + 3 * n + ng);
-        st[3 * n + 2 * ng] = ng;
-        st[3 * n + 2 * ng + 1] = n;
-        CU(cudaMemcpyAsync(ctx->pf_rows, st, sizeof(int) * (3 * (size_t)n + 2 * ng + 2), cudaMemcpyHostToDevice, ctx->stream));
-        CU(cudaEventRecord(ctx->stage_ev[ring], ctx->stream));
-        const int *dv = ctx->pf_rows, *d_g0 = dv + 3 * n, *d_gn = d_g0 + ng, *d_cnt = d_gn + ng;
-        CU(launch(ctx, embed_kernel, dim3(n), dim3(128), 0, tokens, dv + 2 * n, ctx->embed, ctx->h_up, n, d.d_model,
-                  d.vocab_text + d.vocab_speech, ctx->sd.counts + CNT_STATUS));
-        RowSet rs{dv, dv + n, d_g0, d_gn, d_cnt, d_cnt + 1, n, ng, max_grp, max_len, n_big};
+        CU(begin(true));
+        RowSet rs{r_slot, r_pos, r_g0, r_gn, r_cnt, r_cnt + 1, n, ng, max_grp, max_len, n_big};
         rs.sum_len = sum_len;
         CU(run_layers(ctx, 1, d.n_layers, ctx->h_up, rs));
-        CU(launch(ctx, prefill_len_kernel, dim3((ng + 127) / 128), dim3(128), 0, ctx->kv_len, dv, dv + n, d_g0, d_gn, ng));
-        for (int g = 0; g < ng; g++) ctx->h_len[slot[g0[g]]] = pos[g0[g]] + gn[g];
+        CU(launch(ctx, prefill_len_kernel, dim3((ng + 127) / 128), dim3(128), 0, ctx->kv_len, (const int *)r_slot, (const int *)r_pos,
+                  (const int *)r_g0, (const int *)r_gn, ng));
     }
     return SPARSK_OK;
 }

@@ -57,8 +57,8 @@ struct PerDevice {
 // writes are visible).  Every kernel here waits before it completes, so completion is transitive:
 // when a kernel's wait returns, everything before it in the stream is done.  The early start is
 // what lets a weight-streaming kernel issue its first weight copies (which depend on nothing)
-// while a small kernel between two of them is still running.  The kernel that begins a step and the
-// copies that stage a row set never let go early, and that kernel fences what it wrote: a kernel of
+// while a small kernel between two of them is still running.  The kernels that begin a step or a prompt
+// pass, and the copies that stage a row set, never let go early, and those kernels fence what they wrote: a kernel of
 // the pass that follows finds the row set in the L2 before its wait as well.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;"); }

@@ -169,15 +169,45 @@ static __global__ void __launch_bounds__(1024) step_begin_kernel(const StepDesc 
     __threadfence();
 }
 
-// h^(0) = E[token]  (Sec. III), fp32 residual stream.  Row i's token is tokens[i], or
-// tokens[idx[i]] where the rows of a pass are gathered from a longer token array.
-static __global__ void embed_kernel(const int *__restrict__ tokens, const int *__restrict__ idx, const bf16 *__restrict__ embed,
-                             float *__restrict__ h, int n, int d, int vocab, int *__restrict__ status)
+// The beginning of a prompt pass: its pieces (consecutive tokens of one prompt each) as a kernel
+// argument, up to PP_MAX a launch, so that nothing of a pass lives in host memory once it is
+// enqueued.  Block r works row r of the launch out: its slot and position, its group's entry if it
+// is the group's first, h^(0) = E[token] (Sec. III).  The pass's last launch also leaves the counts.
+constexpr int PP_MAX = 128;
+struct PromptPieces {
+    int row0[PP_MAX + 1];                          // first row of the pass (entry n: the end)
+    int slot[PP_MAX], pos[PP_MAX], token[PP_MAX];  // slot, first position, first index into the tokens
+};
+static __global__ void prompt_begin_kernel(const __grid_constant__ PromptPieces in, int n, int grp0, bool last,
+                                    const int *__restrict__ tokens, int *__restrict__ row_slot, int *__restrict__ row_pos,
+                                    int *__restrict__ grp_row0, int *__restrict__ grp_nrows, int *__restrict__ counts,
+                                    const bf16 *__restrict__ embed, float *__restrict__ h, int d, int vocab,
+                                    int *__restrict__ status)
 {
     griddep_wait();
-    const int row = blockIdx.x;
-    if (row >= n) return;
-    embed_row(embed, clamp_token(tokens[idx ? idx[row] : row], vocab, status), h + (size_t)row * d, d);
+    const int row = in.row0[0] + blockIdx.x;
+    int g = 0, end = n;  // the piece that holds the row
+    while (end - g > 1) {
+        const int mid = (g + end) >> 1;
+        if (in.row0[mid] <= row) g = mid;
+        else end = mid;
+    }
+    const int at = row - in.row0[g];
+    if (threadIdx.x == 0) {
+        row_slot[row] = in.slot[g];
+        row_pos[row] = in.pos[g] + at;
+        if (at == 0) {
+            grp_row0[grp0 + g] = row;
+            grp_nrows[grp0 + g] = in.row0[g + 1] - row;
+        }
+        if (last && blockIdx.x == 0) {
+            counts[0] = grp0 + n;
+            counts[1] = in.row0[n];
+        }
+    }
+    embed_row(embed, clamp_token(tokens[in.token[g] + at], vocab, status), h + (size_t)row * d, d);
+    // kernels of the pass read the row set before their own grid dependency has resolved
+    __threadfence();
 }
 
 // Between the lower and the upper pass, one launch.

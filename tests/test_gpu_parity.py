@@ -283,6 +283,66 @@ def test_prompts_share_prefill_passes(util, rows):
     P.close()
 
 
+@pytest.mark.parametrize("n", [128, 129, 300])
+def test_many_prompts_in_one_prefill_pass(util, n):
+    """A pass's pieces travel as kernel arguments, 128 a launch: as many, one more, and three launches over two
+    passes of 256 rows; the piece behind a full launch holds several tokens."""
+    dims = synth.model_dims("tiny", 2, 3, 0)
+    w = synth.make_weights(dims, seed=2)
+    lens = [4 if i % 64 == 0 and i else 2 for i in range(n)]
+    prompts = [synth.make_prompts(dims, 1, k, k, seed=200 + i)[0] for i, k in enumerate(lens)]
+    seen = sorted({0, 1, 64, 127, 128, n // 2, n - 1} & set(range(n)))
+    P = util.Pair(dims, w, n, 16, 2, oracle_slots=seen)
+    P.prefill(prompts)
+    for s_ in seen:
+        assert P.g.slot_state(s_) == (lens[s_] - 1, 0)
+        P.check_cache(s_, range(1, 5), lens[s_] - 1)
+    P.step([0] * n, [0] * n)
+    P.close()
+
+
+def test_captured_prefill_replays_and_leaves_the_context_usable(util):
+    """Nothing of a prompt pass lives in host memory once it is enqueued: a captured one gives the same cache
+    when it is replayed after other prompts, on tokens written to the captured buffer meanwhile, and the
+    context goes on working."""
+    import ctypes as C
+    from paper_2603_09215_b200 import binding
+    dims = synth.model_dims("tiny", 2, 3, 0)
+    gw = binding.upload_weights(synth.make_weights(dims, seed=1))
+    st = torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())
+    n = 40
+    prompts = [p[:n] for p in synth.make_prompts(dims, 3, n, n, seed=6)]
+    with torch.cuda.stream(st):
+        g = binding.Sparsk(dims, gw, 2, 64, 2, stream=st)
+        tokens = torch.from_numpy(np.ascontiguousarray(prompts[0], dtype=np.int32)).cuda()
+        slot, offs = (C.c_int32 * 1)(0), (C.c_int32 * 2)(0, n)
+        prefill = lambda: g._check(g.lib.sparsk_prefill(g.h, 1, slot, tokens.data_ptr(), offs))
+        prefill()
+        st.synchronize()
+        ref = []
+        for p in prompts:                       # what each prompt's cache is, without a capture
+            g.reset_slot(0)
+            g.prefill([0], [p])
+            ref.append([t.clone() for l in range(1, 5) for t in g.export_kv(0, l, 0, n)])
+        g.reset_slot(0)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            prefill()
+        for i in range(20):                     # more passes than any ring of staging buffers holds
+            g.reset_slot(1)
+            g.prefill([1], [prompts[2]])
+        for i in (0, 1):
+            tokens.copy_(torch.from_numpy(np.ascontiguousarray(prompts[i], dtype=np.int32)))
+            graph.replay()
+            got = [t for l in range(1, 5) for t in g.export_kv(0, l, 0, n)]
+            st.synchronize()
+            for a, b in zip(got, ref[i]):       # (the split sums' order is not fixed)
+                assert float((a.float() - b.float()).abs().max()) <= 5e-3 * float(b.float().abs().max())
+        g.check()
+        g.close()
+
+
 @pytest.mark.parametrize("B", [5, 16, 17, 64, 81, 128, 130])
 def test_tcgen05_passes_of_every_width(util, B):
     """Batches on the tcgen05 path at the edges of its activation tiles (copies of 16, 32, 48 ... rows),
