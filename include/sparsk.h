@@ -71,7 +71,9 @@ typedef struct {
     int32_t max_seqs;       /* number of sequence slots */
     int32_t max_seq_len;    /* positions per slot */
     int32_t max_pending;    /* pending positions per slot; >= K-1 for the periodic schedule */
-    int32_t prefill_rows;   /* rows per prefill pass (0 = default) */
+    int32_t prefill_rows;   /* rows per prefill pass; 0 = 256.  The workspace holds activations and
+                               attention partials for as many rows (28 query heads of 128 numbers:
+                               0.45 MiB of partials a row), so a smaller number makes it smaller */
     int32_t text_period;    /* K of text steps when they follow the rule (text_exit 1 or 2); 0 = the
                                same K and r as speech steps.  Sec. V-E: the two modalities may need
                                different policies */
@@ -323,7 +325,7 @@ int64_t sparsk_launch_count(const sparsk_ctx *ctx);
 int sparsk_conf_entropies(const sparsk_ctx *ctx, int32_t n_seqs, float *out /*host*/);
 
 /* Which implementation the layer passes so far went through (a pass = one layer over one row
- * set): layer_passes[0] persistent layer-range kernel (1-2 rows), [1] tcgen05 kernels launched
+ * set): layer_passes[0] persistent layer-range kernel (1-4 rows), [1] tcgen05 kernels launched
  * per projection, [2] small-batch GEMV kernels.  Lets a benchmark
  * attribute bytes to the kernel it times without re-deriving the choice.  No counterpart in the
  * paper: measurement only. */

@@ -100,7 +100,7 @@ struct sparsk_ctx {
     float *samp_scratch;         // device [max_seqs][Vt + Vs]
     int64_t launches;
     // tensor-core path: TMA descriptors of every weight matrix and of the activation buffers
-    // (one per box height 16, 32, ..., 256)
+    // (one per box height 16, 32, ..., 128)
     bool tc_ok;
     std::vector<TmaPair> tm_wq, tm_wk, tm_wv, tm_wo, tm_wg[2], tm_wu[2], tm_wd, tm_head;
     TmaPair tm_x[GM_BOXES], tm_ao[GM_BOXES], tm_act[GM_BOXES];
@@ -110,11 +110,11 @@ struct sparsk_ctx {
     std::vector<CUtensorMap> tm_kc, tm_vc;  // per layer: the cache viewed as [64][slots * Hkv * S rows][hd / 64], boxes of [64][64][2]
     int attn_stages;                        // K/V ring depth of the warp-per-item attention kernel (2 or 3)
     int attn_tc, attn_tc_min_q;             // tcgen05 attention for blocks of at least this many query vectors
-    // persistent layer-range kernel (one or two rows)
+    // persistent layer-range kernel (one to four rows)
     MkLayer *mk_layers;            // device [L]
     unsigned long long *mk_bar;    // device: grid barrier counter; mk_bar_base mirrors its value
     int *mk_abort;                 // device
-    float *mk_attn_o, *mk_act;     // device fp32 [MK_MAX_ROWS][Hq*hd], [MK_MAX_ROWS][F]
+    float *mk_attn_o, *mk_act;     // device fp32 [MK_MAX_ROWS][Hq*hd], [MK_MAX_ROWS][F] (see MkArgs)
     unsigned long long *mk_trace;  // device [1 + 6 L]
     int mk_trace_n;                // entries the last launch wrote
     unsigned long long mk_bar_base;
@@ -1015,7 +1015,7 @@ cudaError_t launch_mega_inst(sparsk_ctx *c, const MkArgs &a, size_t smem)
     return e;
 }
 
-// Layers [l_begin, l_end) (0-based) over a row set of one or two rows, in one launch.
+// Layers [l_begin, l_end) (0-based) over a row set of one to four rows, in one launch.
 cudaError_t run_mega(sparsk_ctx *c, int l_begin, int l_end, float *h, const RowSet &rs)
 {
     const sparsk_dims &d = c->dm;

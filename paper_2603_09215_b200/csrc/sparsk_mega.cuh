@@ -1,6 +1,6 @@
-// Persistent layer-range kernel for passes of one or two rows.
+// Persistent layer-range kernel for passes of one to four rows.
 //
-// At one or two rows a decode step is nothing but a stream of weights from HBM (Sec. IV-B.3),
+// At so few rows a decode step is nothing but a stream of weights from HBM (Sec. IV-B.3),
 // and one kernel per projection leaves HBM idle at every kernel boundary.  This kernel runs a
 // whole range of layers in ONE cooperative launch, one CTA per SM:
 //
@@ -17,11 +17,12 @@
 //   * warps 0..15 are consumers.  Per layer they run six phases separated by grid-wide barriers:
 //     RMSNorm + q/k/v + rotary embedding + cache append; attention partials; merge of the
 //     splits; O-projection + residual; RMSNorm + gate/up + SiLU; down-projection + residual.
-//     In a projection phase a CTA owns "bands" of 32 weight rows; warp w owns row w of each of
+//     In a projection phase a CTA owns "bands" of 32 weight rows; with one or two rows warp w owns row w of each of
 //     the band's two 16-row boxes (a rotary pair, a gate/up pair, or two plain rows), reads one
 //     16-byte unit per lane per box, keeps fp32 sums across the whole inner dimension and
 //     shuffles once per band.  Activations sit in shared memory as fp32, and the attention
-//     output and the MLP activation travel between phases as fp32: at random initialisation a
+//     output and the MLP activation travel between phases as fp32 (three and four rows: two bf16
+//     terms of 16 significant bits, see sparsk_mega_phases.cuh): at random initialisation a
 //     rounding early in the stack is amplified by every later layer, and bf16 activations alone
 //     put the exit states of a 28-layer stack 2-3 % from the fp64 reference.
 //
@@ -49,7 +50,7 @@ constexpr int MK_ATT_WARPS = 3;                 // consumer warps that run atten
 constexpr int MK_ATT_NST = 2;
 constexpr int MK_MAX_SPLITS = 32;             // the merge keeps one split per lane
 
-// The area behind the ring holds the activations of a projection phase (M rows of bf16; when
+// The area behind the ring holds the activations of a projection phase (M rows; when
 // M rows of the whole inner dimension do not fit, a window of k-steps that is reloaded as the
 // phase moves along), or the attention warps' query blocks and K/V rings.
 inline size_t mk_attn_bytes(int head_dim)
@@ -79,7 +80,7 @@ struct MkArgs {
     const int *row_slot, *row_pos, *grp_row0, *grp_nrows;
     int n_rows, n_groups;
     float *q_buf;                // [rows][Hq*hd]
-    float *attn_o, *act;         // [rows][Hq*hd], [rows][F]
+    float *attn_o, *act;         // [rows][Hq*hd], [rows][F]; three and four rows: bf16 planes [hi rows][lo rows][..] instead
     float *part_o;
     float2 *part_ml;
     const float2 *rope;

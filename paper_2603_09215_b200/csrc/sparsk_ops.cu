@@ -82,8 +82,12 @@ int sparsk_attention_launch(const sparsk_attn_args *p, char *scratch, cudaStream
     a.nq_min = 0; a.nq_max = 1 << 30;
     const int warp_ctas = n_sm * attn_warp_ctas_per_sm(p->head_dim, AW_NST);
     // Only a bound on the prefixes is known here: with several groups they are taken to be half as long
-    // on average (48 ragged groups of 200 to 3,000 positions: 61.6 us per call planned for the
-    // bound, 57.4 for half of it, 63 for a fifth; uniform ones do not care).
+    // on average.  That suits ragged lengths and costs uniform ones.  us a call back to back, planned
+    // for the bound / for half of it (28 query heads of 128, 4 kv heads, unless given): 48 groups of 200 to
+    // 3,000 positions, every third of four rows 63.1 / 59.8, all of one row 46.4 / 45.2, one of 3,000
+    // among 47 of 100 25.6 / 23.1, 64 of 500 to 4,000 and four rows (32 heads, 2 kv heads) 126.0 / 116.6;
+    // against that 48 of 3,000 each 63.5 / 67.0, with four rows 100.7 / 119.0, 32 of 2,048 and eight rows (32
+    // heads, 8 kv heads) 96.0 / 115.9.  (A fifth: 63 for the first.)
     const AttnPlan pl = attn_plan(warp_ctas * AW_WARPS, p->n_groups, p->max_grp_rows, p->n_q_heads / p->n_kv_heads,
                                   p->n_kv_heads, p->max_len, 0, p->n_groups > 1 ? (long)p->n_groups * p->max_len / 2 : 0);
     a.n_qblk = pl.n_qblk; a.split_len = pl.split_len; a.n_splits = pl.n_splits;
