@@ -399,22 +399,24 @@ def test_attention_of_many_ragged_sequences(util, B, options):
 
 
 @pytest.mark.parametrize("options", [{}, {"attn_split": 128, "attn_ctas": 3}, {"attn_tma": 0}, {"attn_tc": 0}])
-@pytest.mark.parametrize("Hq,Hkv", [(7, 1), (32, 2), (4, 2)])
-def test_attention_with_positions_as_the_m_dimension(util, Hq, Hkv, options):
-    """Head dimension 128 on the tcgen05 path: 2 to 32 query vectors per kv head (more go to the kernel for
-    large blocks, or, with that one off, in several blocks of 32), prefixes that end before, on and
-    after a 128-position tile and its half, several splits, many more items than CTAs."""
+@pytest.mark.parametrize("Hq,Hkv", [(7, 1), (8, 1), (9, 1), (32, 2), (4, 2)])
+def test_attention_forms_of_few_and_many_query_vectors(util, Hq, Hkv, options):
+    """Head dimension 128 on the tcgen05 path: single rows of 2 to 16 query vectors per kv head, on both sides
+    of the transposed item form (up to eight), and refresh blocks of four rows in blocks of 16 query vectors or,
+    from 33 on, in the tcgen05 kernel (unless that is off); prefixes that end before, on and after a
+    16-position tile, the 64 positions of a large block's tile and of the shortest split, and a forced
+    split of 128."""
     dims = synth.model_dims(dict(MICRO256, n_layers=2, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=128), 1, 4, 0)
     w = synth.make_weights(dims, seed=13)
-    lens = [2, 63, 65, 128, 129, 130, 200, 257, 390]
+    lens = [2, 15, 16, 17, 63, 64, 65, 128, 129, 130, 257, 390]
     prompts = [synth.make_prompts(dims, 1, n, n, seed=60 + i)[0] for i, n in enumerate(lens)]
-    P = util.Pair(dims, w, len(lens), 420, 3, options=options, oracle_slots=[0, 2, 3, 4, 7, 8])
+    P = util.Pair(dims, w, len(lens), 420, 3, options=options, oracle_slots=[0, 2, 3, 5, 6, 7, 9, 11])
     P.prefill(prompts)
     for g in range(9):
         mc = [synth.interleave(g + i, 1, 4) for i in range(len(lens))]
         P.step([m for m, _ in mc], [c for _, c in mc])
     assert P.stats["max_flush"] == 3
-    P.check_cache(8, range(1, 3), P.g.slot_state(8)[0] - P.g.slot_state(8)[1])
+    P.check_cache(11, range(1, 3), P.g.slot_state(11)[0] - P.g.slot_state(11)[1])
     P.close()
 
 
