@@ -307,8 +307,8 @@ int sparsk_kernel_time_by_class(sparsk_ctx *ctx, double *total_ms /*host [8]*/, 
 int sparsk_check(sparsk_ctx *ctx);
 
 /* Phase clock of the persistent layer-range kernel: its first CTA records the GPU's nanosecond
- * timer when it starts and after each of the six phases of every layer (q/k/v, attention,
- * merge, O-projection, gate/up, down-projection).  Copies the entries of the most recent launch
+ * timer when it starts and after each of the four phases of every layer (q/k/v; attention;
+ * merge of its splits and O-projection; MLP).  Copies the entries of the most recent launch
  * to out_ns (host), synchronising the stream; returns how many were written (at most
  * `capacity`), or a negative code.  No counterpart in the paper: measurement only. */
 int sparsk_phase_trace(sparsk_ctx *ctx, int64_t *out_ns /*host*/, int32_t capacity);

@@ -114,8 +114,9 @@ struct sparsk_ctx {
     MkLayer *mk_layers;            // device [L]
     unsigned long long *mk_bar;    // device: grid barrier counter; mk_bar_base mirrors its value
     int *mk_abort;                 // device
-    float *mk_attn_o, *mk_act;     // device fp32 [MK_MAX_ROWS][Hq*hd], [MK_MAX_ROWS][F] (see MkArgs)
-    unsigned long long *mk_trace;  // device [1 + 6 L]
+    float *mk_h2;                  // device fp32 [MK_MAX_ROWS][d] (see MkArgs)
+    MkCols mk_cols16, mk_cols32;   // how the MLP's columns are dealt to the CTAs, at one and two and at three and four rows
+    unsigned long long *mk_trace;  // device [1 + MK_PHASES L]
     int mk_trace_n;                // entries the last launch wrote
     unsigned long long mk_bar_base;
     int mega, mk_ok, mk_coop, mk_max_rows;
@@ -244,9 +245,11 @@ size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
     unsigned long long *mkb = w.take<unsigned long long>(1);
     int *mka = w.take<int>(1);
     unsigned *atk = w.take<unsigned>(1);
-    float *mkao = w.take<float>((size_t)MK_MAX_ROWS * qrow), *mkact = w.take<float>((size_t)MK_MAX_ROWS * d->d_ffn);
-    unsigned long long *mkt = w.take<unsigned long long>(1 + 6 * L);
-    const size_t cells = std::max<size_t>(R * MAX_SPLITS, (size_t)MK_MAX_ROWS * MK_MAX_SPLITS) * d->n_q_heads;
+    float *mkh2 = w.take<float>((size_t)MK_MAX_ROWS * d->d_model);
+    unsigned long long *mkt = w.take<unsigned long long>(1 + MK_PHASES * L);
+    // attention partials: of the launches, and of the persistent kernel (see MkRuns)
+    const size_t runs = (size_t)MK_MAX_CTAS + (size_t)MK_MAX_ROWS * d->n_kv_heads;
+    const size_t cells = std::max<size_t>(R * MAX_SPLITS * d->n_q_heads, runs * MK_MAX_ROWS * (d->n_q_heads / d->n_kv_heads));
     float *po = w.take<float>(cells * d->head_dim);
     float2 *pml = w.take<float2>(cells);
     if (c) {
@@ -257,7 +260,7 @@ size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
         c->h_last = hlast; c->q_last = qlast; c->last_slot = lslot; c->last_pos = lpos;
         c->h_lo = hlo; c->h_up = hup; c->qbuf = q; c->attn_o = ao; c->act = act; c->xnorm = xn; c->qkv_part = qp;
         c->attn_o_lo = aol; c->act_lo = actl; c->xnorm_lo = xnl;
-        c->mk_layers = mkl; c->mk_bar = mkb; c->mk_abort = mka; c->mk_attn_o = mkao; c->mk_act = mkact; c->mk_trace = mkt;
+        c->mk_layers = mkl; c->mk_bar = mkb; c->mk_abort = mka; c->mk_h2 = mkh2; c->mk_trace = mkt;
         c->part_o = po; c->part_ml = pml; c->attn_ticket = atk;
     }
     return align_up(w.off, 256);
@@ -909,7 +912,6 @@ bool build_mega(sparsk_ctx *c)
         return false;
     EncodeTiledFn fn = (EncodeTiledFn)fp;
     const size_t qd = (size_t)d.n_q_heads * d.head_dim, kd = (size_t)d.n_kv_heads * d.head_dim;
-    const size_t lstride = (size_t)d.max_seqs * d.n_kv_heads * d.max_seq_len * d.head_dim;
     // [16 rows][256 columns] boxes of a row-major matrix, no swizzle, zero fill outside
     auto enc = [&](CUtensorMap *m, const void *base, size_t rows, size_t cols) {
         const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
@@ -920,14 +922,25 @@ bool build_mega(sparsk_ctx *c)
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
-    // The swizzled three-dimensional view needs inner dimensions that are whole 64-element blocks, and
+    // [64 rows][cols columns] boxes of O and down
+    auto enc_col = [&](CUtensorMap *m, const void *base, size_t rows, size_t cols, int box_cols) {
+        const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+        const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
+        const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)MK_CBOX_ROWS};
+        const cuuint32_t es[2] = {1, 1};
+        return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    c->mk_cols16 = mk_cols(d.d_ffn, MK_BOX_ROWS, c->n_sm);
+    c->mk_cols32 = mk_cols(d.d_ffn, 2 * MK_BOX_ROWS, c->n_sm);
+    // The swizzled three-dimensional views need inner dimensions that are whole 64-element blocks, and
     // the RMSNorm of the form leaves whole residual rows in the activation area: 4,352 numbers.
     // Passes of three and four wider rows take the tcgen05 path, which is the faster one there in
     // any case.  us a layer at three / four rows: 4,352 numbers (MLP 11,776) 111 / 111 here and 117
     // there; a form that normalised a window at a time took 117 / 165 at 4,416, 142 / 204 at 5,120
     // (MLP 13,824) and 165 / 237 at 5,888 (15,360) where the tcgen05 path takes 113, 134 and 155.
-    c->mk_tc_ok = d.d_model % 64 == 0 && d.d_ffn % 64 == 0 && qd % 64 == 0 &&
-                  div_up(d.d_model, MK_BOX_COLS) <= mk_tc_window(MK_MAX_ROWS);
+    c->mk_tc_ok = d.d_model % 64 == 0 && d.d_ffn % 64 == 0 && qd % 64 == 0 && mk_tc_fits(MK_MAX_ROWS, d.d_model, c->mk_cols32.most);
     auto enc_sw = [&](CUtensorMap *m, const void *base, size_t rows, size_t cols) {
         const cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64)};
         const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, 128};
@@ -935,6 +948,15 @@ bool build_mega(sparsk_ctx *c)
         const cuuint32_t es[3] = {1, 1, 1};
         return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, es,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    auto enc_col_sw = [&](CUtensorMap *m, const void *base, size_t rows, size_t cols, int box_cols) {
+        const cuuint64_t dims[3] = {32, (cuuint64_t)rows, (cuuint64_t)(cols / 32)};
+        const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, 64};
+        const cuuint32_t box[3] = {32, (cuuint32_t)MK_CBOX_ROWS, (cuuint32_t)(box_cols / 32)};
+        const cuuint32_t es[3] = {1, 1, 1};
+        return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, es,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
     c->mk_host.resize(d.n_layers);
@@ -947,19 +969,27 @@ bool build_mega(sparsk_ctx *c)
         const size_t cols[MKW_N] = {(size_t)d.d_model, (size_t)d.d_model, (size_t)d.d_model, qd, (size_t)d.d_model,
                                     (size_t)d.d_model, (size_t)d.d_ffn};
         for (int k = 0; k < MKW_N; k++) {
-            ok = ok && enc(&m.map[k], mats[k], rows[k], cols[k]);
-            if (c->mk_tc_ok) ok = ok && enc_sw(&m.map[MKW_N + k], mats[k], rows[k], cols[k]);
+            if (k == MKW_O || k == MKW_D) {
+                ok = ok && enc_col(&m.map[k], mats[k], rows[k], cols[k], k == MKW_O ? d.head_dim : c->mk_cols16.box);
+                if (c->mk_tc_ok) ok = ok && enc_col_sw(&m.map[MKW_N + k], mats[k], rows[k], cols[k], k == MKW_O ? d.head_dim : c->mk_cols32.box);
+            } else {
+                ok = ok && enc(&m.map[k], mats[k], rows[k], cols[k]);
+                if (c->mk_tc_ok) ok = ok && enc_sw(&m.map[MKW_N + k], mats[k], rows[k], cols[k]);
+            }
+        }
+        if (c->attn_tma_ok) {
+            m.kmap = c->tm_kc16[l];
+            m.vmap = c->tm_vc16[l];
         }
         m.attn_gain = c->attn_norm[l];
         m.mlp_gain = c->mlp_norm[l];
-        m.kc = c->kcache + l * lstride;
-        m.vc = c->vcache + l * lstride;
     }
     if (!ok) return false;
     if (cudaMemcpyAsync(c->mk_layers, c->mk_host.data(), sizeof(MkLayer) * d.n_layers, cudaMemcpyHostToDevice,
                         c->stream) != cudaSuccess ||
         cudaMemsetAsync(c->mk_bar, 0, sizeof(unsigned long long), c->stream) != cudaSuccess ||
-        cudaMemsetAsync(c->mk_abort, 0, sizeof(int), c->stream) != cudaSuccess)
+        cudaMemsetAsync(c->mk_abort, 0, sizeof(int), c->stream) != cudaSuccess ||
+        cudaMemsetAsync(c->mk_h2, 0, sizeof(float) * MK_MAX_ROWS * (size_t)d.d_model, c->stream) != cudaSuccess)
         return false;
     c->mk_bar_base = 0;
     int dev = 0, coop = 0;
@@ -969,18 +999,21 @@ bool build_mega(sparsk_ctx *c)
     return true;
 }
 
-size_t mega_smem(const sparsk_dims &) { return (size_t)MK_SLOTS * MK_SLOT_BYTES + MK_AREA_BYTES + 1024; }
-
 // Can a pass of n_rows rows go through the persistent kernel?
 bool use_mega(const sparsk_ctx *c, int n_rows)
 {
+    const int m = n_rows >= MK_TC_ROWS ? MK_MAX_ROWS : n_rows;  // (three rows run as four with one masked)
     return c->mega && c->mk_ok && c->mk_coop && n_rows >= 1 && n_rows <= c->mk_max_rows && (n_rows < MK_TC_ROWS || c->mk_tc_ok) &&
-           mk_attn_bytes(c->dm.head_dim) <= MK_AREA_BYTES && c->dm.head_dim % (2 * MK_BOX_ROWS) == 0;
+           c->attn_tma_ok && c->n_sm <= MK_MAX_CTAS &&
+           (size_t)MK_MAX_ROWS * c->dm.n_kv_heads * (c->dm.max_seq_len / AT_TP + 1) * MK_MAX_CTAS < (1ull << 31) &&  // (32-bit shares)
+           mk_attn_fits(m, c->dm.n_q_heads / c->dm.n_kv_heads, c->dm.head_dim) &&
+           (n_rows >= MK_TC_ROWS || mk_act_window(m, m * c->mk_cols16.most * 4 + mk_sums_bytes(m)) >= 1);
 }
 
 template <int M, int HD>
-cudaError_t launch_mega_inst(sparsk_ctx *c, const MkArgs &a, size_t smem)
+cudaError_t launch_mega_inst(sparsk_ctx *c, const MkArgs &a)
 {
+    constexpr size_t smem = mk_smem_bytes(M);
     static PerDevice<int> grid_dev;  // 0: not asked yet, 1: one CTA per SM fits, 2: it does not
     int &grid_ok = grid_dev.here();
     auto kern = mega_kernel<M, HD>;
@@ -1023,21 +1056,14 @@ cudaError_t run_mega(sparsk_ctx *c, int l_begin, int l_end, float *h, const RowS
     a.layers = c->mk_layers; a.layer_begin = l_begin; a.layer_end = l_end; a.h = h;
     a.row_slot = rs.slot; a.row_pos = rs.pos; a.grp_row0 = rs.grp_row0; a.grp_nrows = rs.grp_nrows;
     a.n_rows = rs.n_rows; a.n_groups = rs.n_groups_h;
-    a.q_buf = c->qbuf; a.attn_o = c->mk_attn_o; a.act = c->mk_act; a.part_o = c->part_o; a.part_ml = c->part_ml;
+    a.h2 = c->mk_h2;
+    a.kc = c->kcache; a.vc = c->vcache;
+    a.kv_layer = (size_t)d.max_seqs * d.n_kv_heads * d.max_seq_len * d.head_dim;
+    a.q_buf = c->qbuf; a.part_o = c->part_o; a.part_ml = c->part_ml;
     a.rope = c->rope;
     a.d = d.d_model; a.Hq = d.n_q_heads; a.Hkv = d.n_kv_heads; a.hd = d.head_dim; a.F = d.d_ffn; a.S = d.max_seq_len;
     a.n_slots = d.max_seqs; a.eps = d.rms_eps;
-    // KV cut: an item for every attention warp of the machine if there are that many 16-position tiles
-    const int G = d.n_q_heads / d.n_kv_heads;
-    const int n_qblk = (rs.max_grp_rows * G + 15) / 16;
-    const int base = std::max(1, rs.n_groups_h * n_qblk * d.n_kv_heads);
-    const int tiles = std::max(1, (rs.max_len + AT_TP - 1) / AT_TP);
-    int splits = c->attn_split > 0 ? (rs.max_len + c->attn_split - 1) / c->attn_split
-                                   : (c->n_sm * MK_ATT_WARPS + base - 1) / base;
-    splits = std::max(1, std::min(splits, std::min(MK_MAX_SPLITS, tiles)));
-    a.att_qblk = n_qblk;
-    a.att_split_len = ((rs.max_len + splits - 1) / splits + AT_TP - 1) / AT_TP * AT_TP;
-    a.att_splits = std::max(1, (rs.max_len + a.att_split_len - 1) / a.att_split_len);
+    a.cols = rs.n_rows >= MK_TC_ROWS ? c->mk_cols32 : c->mk_cols16;
     a.bar = c->mk_bar; a.bar_base = c->mk_bar_base; a.abort_word = c->mk_abort; a.status = c->sd.counts + CNT_STATUS;
     if (c->inject_timeout) {
         // the launch is told a barrier count that is never reached: its first grid barrier runs
@@ -1046,21 +1072,20 @@ cudaError_t run_mega(sparsk_ctx *c, int l_begin, int l_end, float *h, const RowS
         c->inject_timeout = 0;
     }
     a.trace = c->mk_trace;
-    c->mk_trace_n = 1 + 6 * (l_end - l_begin);
-    c->mk_bar_base += 6ull * (unsigned long long)(l_end - l_begin) * (unsigned long long)c->n_sm;
-    const size_t smem = mega_smem(d);
+    c->mk_trace_n = 1 + MK_PHASES * (l_end - l_begin);
+    c->mk_bar_base += (unsigned long long)MK_PHASES * (unsigned long long)(l_end - l_begin) * (unsigned long long)c->n_sm;
     // (three rows run as four with one masked)
     if (d.head_dim == 128) {
         switch (rs.n_rows) {
-        case 1: return launch_mega_inst<1, 128>(c, a, smem);
-        case 2: return launch_mega_inst<2, 128>(c, a, smem);
-        default: return launch_mega_inst<4, 128>(c, a, smem);
+        case 1: return launch_mega_inst<1, 128>(c, a);
+        case 2: return launch_mega_inst<2, 128>(c, a);
+        default: return launch_mega_inst<4, 128>(c, a);
         }
     }
     switch (rs.n_rows) {
-    case 1: return launch_mega_inst<1, 64>(c, a, smem);
-    case 2: return launch_mega_inst<2, 64>(c, a, smem);
-    default: return launch_mega_inst<4, 64>(c, a, smem);
+    case 1: return launch_mega_inst<1, 64>(c, a);
+    case 2: return launch_mega_inst<2, 64>(c, a);
+    default: return launch_mega_inst<4, 64>(c, a);
     }
 }
 
@@ -1414,6 +1439,7 @@ static int act_on_status(sparsk_ctx *ctx, int status)
     if (status & ST_TIMEOUT) {
         CU(cudaMemsetAsync(ctx->mk_bar, 0, sizeof(unsigned long long), ctx->stream));
         CU(cudaMemsetAsync(ctx->mk_abort, 0, sizeof(int), ctx->stream));
+        CU(cudaMemsetAsync(ctx->mk_h2, 0, sizeof(float) * MK_MAX_ROWS * (size_t)ctx->dm.d_model, ctx->stream));
         CU(cudaMemsetAsync(ctx->attn_ticket, 0, sizeof(unsigned), ctx->stream));
         ctx->mk_bar_base = 0;
         ctx->attn_ticket_base = 0;

@@ -331,6 +331,7 @@ struct AtRing {
     // element offset of 16-byte chunk c of row `row` inside a tile
     __device__ __forceinline__ static int off(int row, int c) { return TMA ? at_swz<HD>(row, c) : row * KP + c * 8; }
     __device__ __forceinline__ int stage(int t) const { return (int)((seq0 + (uint32_t)t) % NS); }
+    __device__ __forceinline__ int pos(int t) const { return w_beg + t * AT_TP; }  // first position of tile t
     // TMA form: the tile whose first cache row is y, as tile number `seq` of this warp.  Rows past a
     // split's end arrive as whatever the cache holds there (zeros beyond the cache): the scores
     // mask them, the value rows are cleared after landing.
@@ -419,34 +420,44 @@ __device__ __forceinline__ uint32_t movmatrix_t(uint32_t x)
     return y;
 }
 
+// Where an item leaves what it found for query vector qg of its group (unnormalised sum of values;
+// running maximum and sum): the partial cells of the launch-wide merge.
+template <int HD>
+struct AtCells {
+    float *po;
+    float2 *pml;
+    int row0, Hq, h0, G, splits, sp;
+    __device__ __forceinline__ AtCells(const AttnArgs &a, const AtItem &it)
+        : po(a.part_o), pml(a.part_ml), row0(it.row0), Hq(a.Hq), h0(it.hk * (a.Hq / a.Hkv)), G(a.Hq / a.Hkv), splits(a.n_splits),
+          sp(it.sp)
+    {
+    }
+    __device__ __forceinline__ size_t cell(int qg) const { return ((size_t)(row0 + qg / G) * Hq + h0 + qg % G) * splits + sp; }
+    __device__ __forceinline__ float *o(int qg) const { return po + cell(qg) * HD; }
+    __device__ __forceinline__ float2 *ml(int qg) const { return pml + cell(qg); }
+    // an empty split: max = -inf, sum = 0 is all the merge looks at
+    __device__ __forceinline__ void empty(int q0, int n, int lane) const
+    {
+        for (int qi = lane; qi < n; qi += 32) *ml(q0 + qi) = make_float2(-INFINITY, 0.f);
+    }
+};
+
 // One item, by one warp: query vectors [16 qb, 16 qb + 16) of a group (rows row0 .. row0 + nrows - 1
-// of slot `slot`, the first at position pos0), kv head hk, split sp.  `wr` is the warp's ring of
-// NS stages.  Writes the item's partial.
+// of slot `slot`, the first at position pos0) and kv head hk, over the tiles that `ring` (already
+// started) delivers, none of whose positions from w_end on counts.  Leaves the item's partial in `cells`.
 // QREG: the query fragments stay in registers for the whole item (32 registers at head dimension
 // 128); otherwise they are parked in `qs` ([16][HD + 8] of shared memory) and re-read per tile,
 // for callers whose register budget is spoken for.
-template <int HD, int NS, bool QREG, bool TMA = false>
-__device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, kv_t *wr, kv_t *qs, int lane,
-                                          AttnTma *tm = nullptr)
+template <int HD, bool QREG, class Ring, class Cells>
+__device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, Ring &ring, const Cells &cells, kv_t *qs, int lane)
 {
-    typedef AtRing<HD, NS, TMA> Ring;
     constexpr int KP = HD + 8;      // padded row of the parked queries: ldmatrix rows fall into distinct banks
     constexpr float LOG2E = 1.4426950408889634f, LN2 = 0.6931471805599453f;
-    const int G = a.Hq / a.Hkv, splits = a.n_splits;
-    const int qb = it.qb, hk = it.hk, sp = it.sp, row0 = it.row0, pos0 = it.pos0;
+    const int G = a.Hq / a.Hkv;
+    const int qb = it.qb, hk = it.hk, row0 = it.row0, pos0 = it.pos0;
     const int nq = it.nq, q0 = qb * 16;
     const int nq_here = min(16, nq - q0);
-    const int w_beg = it.w_beg, w_end = it.w_end, n_tiles = it.n_tiles;
-    if (n_tiles == 0) {
-        // an empty split: max = -inf, sum = 0 is all the merge looks at
-        for (int qi = lane; qi < nq_here; qi += 32) {
-            const int qg = q0 + qi;
-            a.part_ml[((size_t)(row0 + qg / G) * a.Hq + hk * G + qg % G) * splits + sp] = make_float2(-INFINITY, 0.f);
-        }
-        return;
-    }
-    Ring ring(a, it, wr, lane, tm);
-    ring.start();
+    const int w_end = it.w_end, n_tiles = ring.n_tiles;
 
     // the queries, as A fragments (row = lane / 4 and + 8, columns 2 (lane % 4) + {0, 1, 8, 9} of
     // every 16-column step), while the first tiles are on their way
@@ -515,7 +526,7 @@ __device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, k
     for (int t = 0; t < n_tiles; t++) {
         const kv_t *Kt, *Vt;
         if (!ring.wait(t, Kt, Vt)) return;
-        const int p0 = w_beg + t * AT_TP;
+        const int p0 = ring.pos(t);
 
         // S = Q K^T for 16 positions, in log2 units; two accumulator chains
         float s[2][4], s2[2][4];
@@ -616,13 +627,10 @@ __device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, k
         l += __shfl_xor_sync(0xffffffffu, l, 2);
         const int qi = (lane >> 2) + hf * 8;
         if (qi < nq_here) {
-            const int qg = q0 + qi, r = qg / G, j = qg % G;
-            const size_t cell = ((size_t)(row0 + r) * a.Hq + hk * G + j) * splits + sp;
-            if ((lane & 3) == 0) a.part_ml[cell] = make_float2(m_run[hf] * LN2, l);  // max back in natural-log units
+            if ((lane & 3) == 0) *cells.ml(q0 + qi) = make_float2(m_run[hf] * LN2, l);  // max back in natural-log units
+            float *po = cells.o(q0 + qi) + (lane & 3) * 2;
 #pragma unroll
-            for (int nt = 0; nt < HD / 8; nt++)
-                *reinterpret_cast<float2 *>(a.part_o + cell * HD + nt * 8 + (lane & 3) * 2) =
-                    make_float2(o[nt][hf * 2], o[nt][hf * 2 + 1]);
+            for (int nt = 0; nt < HD / 8; nt++) *reinterpret_cast<float2 *>(po + nt * 8) = make_float2(o[nt][hf * 2], o[nt][hf * 2 + 1]);
         }
     }
 }
@@ -635,21 +643,13 @@ __device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, k
 // O^T = V^T P^T through two 8x8 register transposes, and V^T is read with transposing ldmatrix.
 // Half the MMAs, half the accumulators and a quarter of the exponentials of the other form;
 // the partial it writes is the same.
-template <int HD, int NS, bool TMA>
-__device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it, kv_t *wr, int lane, AttnTma *tm = nullptr)
+template <int HD, class Ring, class Cells>
+__device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it, Ring &ring, const Cells &cells, int lane)
 {
     constexpr float LOG2E = 1.4426950408889634f, LN2 = 0.6931471805599453f;
-    typedef AtRing<HD, NS, TMA> Ring;
-    const int G = a.Hq / a.Hkv, splits = a.n_splits;
-    const int hk = it.hk, sp = it.sp, row0 = it.row0, pos0 = it.pos0;
+    const int G = a.Hq / a.Hkv;
+    const int hk = it.hk, row0 = it.row0, pos0 = it.pos0, w_end = it.w_end;
     const int nq = it.nq;  // <= 8
-    if (it.n_tiles == 0) {
-        for (int qi = lane; qi < nq; qi += 32)
-            a.part_ml[((size_t)(row0 + qi / G) * a.Hq + hk * G + qi % G) * splits + sp] = make_float2(-INFINITY, 0.f);
-        return;
-    }
-    Ring ring(a, it, wr, lane, tm);
-    ring.start();
 
     // the queries as B fragments: column lane / 4, elements 2 (lane % 4) + {0, 1, 8, 9} of every
     // 16-element step, scaled by log2(e) / sqrt(hd)
@@ -693,7 +693,7 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
     for (int t = 0; t < ring.n_tiles; t++) {
         const kv_t *Kt, *Vt;
         if (!ring.wait(t, Kt, Vt)) return;
-        const int p0 = ring.w_beg + t * AT_TP;
+        const int p0 = ring.pos(t);
         // S^T for 16 positions x 8 query vectors, two accumulator chains
         float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -705,14 +705,14 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
             mma_f16(s1, kb, qf[ks + 1][0], qf[ks + 1][1]);
         }
         // online softmax down the columns; accumulator rows are positions lane / 4 and + 8
-        const bool full = p0 + AT_TP <= ring.w_end && p0 + AT_TP - 1 <= pos0;
+        const bool full = p0 + AT_TP <= w_end && p0 + AT_TP - 1 <= pos0;
         float pv[2][2], alpha[2];
 #pragma unroll
         for (int e = 0; e < 2; e++) {
 #pragma unroll
             for (int j = 0; j < 2; j++) {
                 const int p = p0 + (lane >> 2) + j * 8;
-                const bool ok = full || (p < ring.w_end && p <= limit[e]);
+                const bool ok = full || (p < w_end && p <= limit[e]);
                 pv[e][j] = ok ? s0[j * 2 + e] + s1[j * 2 + e] : -INFINITY;
             }
             float tmax = fmaxf(pv[e][0], pv[e][1]);
@@ -762,15 +762,31 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
         l += __shfl_xor_sync(0xffffffffu, l, 16);
         const int qi = (lane & 3) * 2 + e;
         if (qi < nq) {
-            const size_t cell = ((size_t)(row0 + qi / G) * a.Hq + hk * G + qi % G) * splits + sp;
-            if ((lane >> 2) == 0) a.part_ml[cell] = make_float2(m_run[e] * LN2, l);
+            if ((lane >> 2) == 0) *cells.ml(qi) = make_float2(m_run[e] * LN2, l);
+            float *po = cells.o(qi) + (lane >> 2);
 #pragma unroll
             for (int mt = 0; mt < HD / 16; mt++) {
-                a.part_o[cell * HD + mt * 16 + (lane >> 2)] = o[mt][e];
-                a.part_o[cell * HD + mt * 16 + 8 + (lane >> 2)] = o[mt][2 + e];
+                po[mt * 16] = o[mt][e];
+                po[mt * 16 + 8] = o[mt][2 + e];
             }
         }
     }
+}
+
+// An item of the launches below: its ring, its form, its partial.  At most eight query vectors take the
+// transposed form.
+template <int HD, int NS, bool TMA>
+__device__ __forceinline__ void attn_split_item(const AttnArgs &a, const AtItem &it, kv_t *wr, int lane, AttnTma *tm = nullptr)
+{
+    const AtCells<HD> cells(a, it);
+    if (it.n_tiles == 0) {
+        cells.empty(it.qb * 16, min(16, it.nq - it.qb * 16), lane);
+        return;
+    }
+    AtRing<HD, NS, TMA> ring(a, it, wr, lane, tm);
+    ring.start();
+    if (it.nq <= 8) attn_item_t<HD>(a, it, ring, cells, lane);
+    else attn_item<HD, true>(a, it, ring, cells, nullptr, lane);
 }
 
 // Persistent grid of warps; item i = ((sp * groups + g) * Hkv + hk) * n_qblk + qb: the query
@@ -806,8 +822,7 @@ __global__ void __launch_bounds__(AW_WARPS * 32) attn_warp_kernel(AttnArgs a)
         const AtItem it = at_resolve(a, item, n_items, n_groups, a.grp_row0, a.grp_nrows, a.row_slot, a.row_pos);
         item = next;
         if (!it.valid) continue;
-        if (it.nq <= 8) attn_item_t<HD, NST, false>(a, it, wr, lane);
-        else attn_item<HD, NST, true>(a, it, wr, nullptr, lane);
+        attn_split_item<HD, NST, false>(a, it, wr, lane);
     }
 }
 
@@ -863,8 +878,7 @@ __global__ void __launch_bounds__(WARPS * 32) attn_warp_tma_kernel(const __grid_
         item = next;
         // after a wait that ran out the warp keeps drawing (the ticket count must come out) but works no more
         if (!it.valid || giving_up_s) continue;
-        if (it.nq <= 8) attn_item_t<HD, NST, true>(a, it, wr, lane, &tm);
-        else attn_item<HD, NST, true, true>(a, it, wr, nullptr, lane, &tm);
+        attn_split_item<HD, NST, true>(a, it, wr, lane, &tm);
     }
 }
 inline size_t attn_warp_tma_bytes(int head_dim, int stages, int warps)

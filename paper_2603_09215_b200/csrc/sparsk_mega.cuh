@@ -4,32 +4,46 @@
 // and one kernel per projection leaves HBM idle at every kernel boundary.  This kernel runs a
 // whole range of layers in ONE cooperative launch, one CTA per SM:
 //
-//   * warps 16..19 are producers.  They walk the same list of phases as everyone else but only
-//     ever look at weights, which depend on nothing, so they keep TMA copies of [16 rows x 256
-//     columns] weight boxes flowing into an 8-slot shared-memory ring across phase and layer
-//     boundaries.  Producer p owns the ring slots p and p + 4 and cycles them on its own (one
-//     thread needs a few hundred nanoseconds per copy, so four run side by side).  The ring is
-//     what keeps HBM streaming while the consumers sit in a barrier or in the attention phases.
+//   * warps 16..19 are producers.  They walk the same list of work as everyone else but only
+//     ever look at weights and at the cache, which depend on nothing this launch computes (the few
+//     cache rows that do are patched in by their readers), so they keep TMA copies flowing into a
+//     ring of 16 KB shared-memory slots across phase and layer boundaries.  Producer p owns the
+//     slots p, p + 4, ... and cycles them on its own (one thread needs a few hundred nanoseconds
+//     per copy, so four run side by side).  The ring is what keeps HBM streaming while the
+//     consumers sit in a barrier.  Twelve slots cover 4.2 us of HBM; no more than eight are on
+//     their way at once (148 SMs, 16 KB boxes from HBM: 6.1 / 6.9 / 7.03 / 6.6 TB/s with 4 / 6 / 8 / 12
+//     slots on their way, 7.01 with twelve slots of which eight are).
 //     (Asking the L2 for weights further ahead was measured in three forms and lost each time:
 //     tensor or bulk prefetches running ahead of the copies made every phase slower, gate/up by
 //     30-80 %; a burst for the next gate/up bands during the attention phases delayed the
 //     attention's own cache reads by as much as it later saved.)
-//   * warps 0..15 are consumers.  Per layer they run six phases separated by grid-wide barriers:
-//     RMSNorm + q/k/v + rotary embedding + cache append; attention partials; merge of the
-//     splits; O-projection + residual; RMSNorm + gate/up + SiLU; down-projection + residual.
-//     In a projection phase a CTA owns "bands" of 32 weight rows; with one or two rows warp w owns row w of each of
-//     the band's two 16-row boxes (a rotary pair, a gate/up pair, or two plain rows), reads one
-//     16-byte unit per lane per box, keeps fp32 sums across the whole inner dimension and
-//     shuffles once per band.  Activations sit in shared memory as fp32, and the attention
-//     output and the MLP activation travel between phases as fp32 (three and four rows: two bf16
-//     terms of 16 significant bits, see sparsk_mega_phases.cuh): at random initialisation a
-//     rounding early in the stack is amplified by every later layer, and bf16 activations alone
-//     put the exit states of a 28-layer stack 2-3 % from the fp64 reference.
+//   * warps 0..15 are consumers.  Per layer they run four phases separated by grid-wide barriers:
+//     RMSNorm + q/k/v + rotary embedding + cache append; attention partials; O-projection;
+//     RMSNorm + gate/up + SiLU + down-projection.
+//     - Row form (q/k/v, gate/up: a sum is needed whole before anything can be done with it): a
+//       CTA owns "bands" of 32 weight rows in two 16-row boxes (rotary pairs, gate/up pairs, or
+//       plain rows) over the whole inner dimension.
+//     - Column form (O, down: sums that are added to the residual stream): a CTA owns columns of the
+//       matrix, i.e. a stretch of the inner dimension, for many or all weight rows, and adds its
+//       share of every output.  So it needs only the few activations of its columns, which sit in
+//       registers: of the attention output the one or two heads it owns, whose splits it merges for
+//       itself (no merge phase), and of the MLP activation exactly what its own gate/up bands made
+//       (no barrier between gate/up and down).  The additions of the 148 CTAs to one row are 0.6 us
+//       of L2 atomics beside a stream of 20.
+//     Activations are fp32 (three and four rows: two bf16 terms of 16 significant bits, see
+//     sparsk_mega_phases.cuh): at random initialisation a rounding early in the stack is amplified by
+//     every later layer, and bf16 activations alone put the exit states of a 28-layer stack 2-3 %
+//     from the fp64 reference.
+//     While some CTA still reads the residual stream at the start of the MLP, another may be done with
+//     its gate/up bands: the down-projection therefore adds into a buffer of its own (h2), which the
+//     next layer's first RMSNorm reads along with h and the attention phase folds into h.
 //
 // Every wait (ring slot, grid barrier) is bounded by a wall-clock limit; on a timeout the CTA
 // raises ST_TIMEOUT, tells the other CTAs through the abort word, lets its copies land and
 // returns.
 #pragma once
+
+#include <cstddef>
 
 #include "sparsk_attn.cuh"
 #include "sparsk_gemm.cuh"
@@ -39,60 +53,86 @@ namespace sparsk {
 constexpr int MK_CW = 16;                       // consumer warps
 constexpr int MK_PW = 4;                        // producer warps
 constexpr int MK_THREADS = (MK_CW + MK_PW) * 32;
-constexpr int MK_BOX_ROWS = 16, MK_BOX_COLS = 256;
+constexpr int MK_BOX_ROWS = 16, MK_BOX_COLS = 256;           // row form: two such boxes per slot
 constexpr int MK_BOX_BYTES = MK_BOX_ROWS * MK_BOX_COLS * 2;  // 8 KB
-constexpr int MK_SLOT_BYTES = 2 * MK_BOX_BYTES;              // two boxes per slot
-constexpr int MK_SLOTS = 8;
+constexpr int MK_CBOX_ROWS = 64, MK_CBOX_COLS = 128;         // column form: one box of 64 rows and up to 128 columns per slot
+constexpr int MK_SLOT_BYTES = 2 * MK_BOX_BYTES;
+constexpr int MK_IN_FLIGHT = 8;                 // slots on their way at once
 constexpr int MK_MAX_ROWS = 4;
 constexpr int MK_TC_ROWS = 3;                   // rows from which the tensor-core form runs
-constexpr int MK_AREA_BYTES = 88 * 1024;        // shared memory behind the ring
-constexpr int MK_ATT_WARPS = 3;                 // consumer warps that run attention items
-constexpr int MK_ATT_NST = 2;
-constexpr int MK_MAX_SPLITS = 32;             // the merge keeps one split per lane
+constexpr int MK_GROUPS = 4;                    // a slot of weights is the work of one of four groups of four warps
+constexpr int MK_MAX_CTAS = 192;                // bounds the number of attention partials
+constexpr int MK_SHARED_BYTES = 3072;           // MkShared, behind the area, with two to four rows
+constexpr int MK_SHARED_FEW_BYTES = 2048;       // the part of it that one row needs
 
-// The area behind the ring holds the activations of a projection phase (M rows; when
-// M rows of the whole inner dimension do not fit, a window of k-steps that is reloaded as the
-// phase moves along), or the attention warps' query blocks and K/V rings.
-inline size_t mk_attn_bytes(int head_dim)
+// The ring, then the area: the activations of a row-form phase (M rows; with one or two rows, when they
+// do not fit whole, a window of k-steps that is reloaded as the phase moves along) and what the CTA's
+// own bands make of them, or the attention's parked queries and partials, or the merged heads.
+// Several rows' activations need the larger area.  A multiple of four slots: a weight slot always belongs
+// to the same four warps, so that nobody waits for a slot's next fill before its present one has landed.
+__host__ __device__ constexpr int mk_slots(int M) { return M >= 2 ? 8 : 12; }
+__host__ __device__ constexpr int mk_area_bytes(int M) { return M >= 2 ? 88 * 1024 : 33792; }
+__host__ __device__ constexpr size_t mk_smem_bytes(int M)
 {
-    return (size_t)MK_ATT_WARPS * (16 * (head_dim + 8) * 2 + attn_warp_bytes(head_dim, MK_ATT_NST));
+    return (size_t)mk_slots(M) * MK_SLOT_BYTES + mk_area_bytes(M) + (M >= 2 ? MK_SHARED_BYTES : MK_SHARED_FEW_BYTES);
 }
-// k-steps of M fp32 activation rows that fit the area
-__host__ __device__ inline int mk_act_window(int M) { return MK_AREA_BYTES / (M * MK_BOX_COLS * 4); }
+// k-steps of M fp32 activation rows that fit the area beside `own` bytes
+__host__ __device__ inline int mk_act_window(int M, int own) { return (mk_area_bytes(M) - own) / (M * MK_BOX_COLS * 4); }
 
 enum { MKW_Q = 0, MKW_K, MKW_V, MKW_O, MKW_G, MKW_U, MKW_D, MKW_N };
-enum { MK_QKV = 0, MK_ATTN = 1, MK_MERGE = 2, MK_OPROJ = 3, MK_GATEUP = 4, MK_DOWN = 5 };
+enum { MK_QKV = 0, MK_ATTN = 1, MK_OPROJ = 2, MK_MLP = 3, MK_PHASES = 4 };
 
 // One layer's worth of what the phases need (device array, one entry per layer).
 struct MkLayer {
-    // per matrix (MKW_*): [16 rows x 256 columns] boxes without swizzle (passes of one or two rows),
-    // then, MKW_N entries on, the same boxes as four 64-column blocks with the 128-byte swizzle
-    // (view [64][rows][K/64], box {64, 16, 4}; passes of three and four rows read them with ldmatrix)
+    // per matrix (MKW_*), for passes of one or two rows: [16 rows x 256 columns] boxes, of O and down
+    // [64 rows x head_dim or MkCols::box columns] boxes, all without swizzle; then, MKW_N entries on, for
+    // passes of three and four rows, which read them with ldmatrix: the same boxes as 64-column blocks with
+    // the 128-byte swizzle (view [64][rows][K/64], box {64, 16, 4}), of O and down as 32-column blocks
+    // with the 64-byte swizzle (view [32][rows][K/32], box {32, 64, columns / 32})
     CUtensorMap map[14];
+    CUtensorMap kmap, vmap;  // the cache as rows of head_dim numbers, boxes of 16 (AttnTma's)
     const bf16 *attn_gain, *mlp_gain;
-    kv_t *kc, *vc;  // this layer's cache [slot][Hkv][S][hd]
 };
+
+// How the MLP's inner dimension is dealt: contiguous units of `unit` columns (16: a gate/up band; 32 with
+// three and four rows) to every CTA, at most `most` columns, walked in `chunks` boxes of `box` columns.
+// A box may reach into the next CTA's columns; the activations that meet those are zeros.
+struct MkCols {
+    int unit, most, box, chunks;
+};
+inline MkCols mk_cols(int F, int unit, int n_cta)
+{
+    const int n = (F + unit - 1) / unit, per = (n + n_cta - 1) / n_cta, lim = MK_CBOX_COLS / unit;
+    MkCols c;
+    c.unit = unit;
+    c.chunks = (per + lim - 1) / lim;
+    const int in_box = (per + c.chunks - 1) / c.chunks;
+    c.box = in_box * unit;
+    c.most = c.box * c.chunks;
+    return c;
+}
 
 struct MkArgs {
     const MkLayer *layers;       // device
     int layer_begin, layer_end;  // 0-based, [begin, end)
     float *h;                    // residual stream of the pass [rows][d]
+    float *h2;                   // [MK_MAX_ROWS][d], zero between launches: what the down-projection has added since h was last whole
     const int *row_slot, *row_pos, *grp_row0, *grp_nrows;
     int n_rows, n_groups;
+    kv_t *kc, *vc;               // cache of the first layer [slot][Hkv][S][hd], and what lies between two layers'
+    size_t kv_layer;             // (arithmetic: a pointer read from `layers` would be a trip to HBM in every layer)
     float *q_buf;                // [rows][Hq*hd]
-    float *attn_o, *act;         // [rows][Hq*hd], [rows][F]; three and four rows: bf16 planes [hi rows][lo rows][..] instead
-    float *part_o;
+    float *part_o;               // attention partials, see MkRuns
     float2 *part_ml;
     const float2 *rope;
     int d, Hq, Hkv, hd, F, S, n_slots;
     float eps;
-    int att_splits, att_split_len;  // KV cut of the attention phase
-    int att_qblk;                   // blocks of 16 query vectors per group
+    MkCols cols;
     unsigned long long *bar;        // grid barrier counter (monotonic)
     unsigned long long bar_base;    // its value when this launch starts
     int *abort_word;                // nonzero: some CTA gave up
     int *status;
-    unsigned long long *trace;      // [1 + 6 * layers]: CTA 0's clock at the start and after every phase
+    unsigned long long *trace;      // [1 + MK_PHASES * layers]: CTA 0's clock at the start and after every phase
 };
 
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p)
@@ -109,122 +149,137 @@ __device__ __forceinline__ int ld_volatile_i32(const int *p)
 }
 __device__ __forceinline__ void mk_consumer_sync() { asm volatile("bar.sync 2, %0;" ::"n"(MK_CW * 32) : "memory"); }
 
-// Bands and k-steps of a projection phase.
-struct MkShape {
-    int n_bands, k_steps;
-};
-__device__ __forceinline__ MkShape mk_shape(int type, const MkArgs &a)
-{
-    MkShape s;
-    const int half = a.hd >> 1;
-    switch (type) {
-    case MK_QKV:
-        s.n_bands = (a.Hq + a.Hkv) * (half / MK_BOX_ROWS) + (a.Hkv * a.hd + 2 * MK_BOX_ROWS - 1) / (2 * MK_BOX_ROWS);
-        s.k_steps = (a.d + MK_BOX_COLS - 1) / MK_BOX_COLS;
-        break;
-    case MK_OPROJ:
-        s.n_bands = (a.d + 2 * MK_BOX_ROWS - 1) / (2 * MK_BOX_ROWS);
-        s.k_steps = (a.Hq * a.hd + MK_BOX_COLS - 1) / MK_BOX_COLS;
-        break;
-    case MK_GATEUP:
-        s.n_bands = (a.F + MK_BOX_ROWS - 1) / MK_BOX_ROWS;
-        s.k_steps = (a.d + MK_BOX_COLS - 1) / MK_BOX_COLS;
-        break;
-    case MK_DOWN:
-        s.n_bands = (a.d + 2 * MK_BOX_ROWS - 1) / (2 * MK_BOX_ROWS);
-        s.k_steps = (a.F + MK_BOX_COLS - 1) / MK_BOX_COLS;
-        break;
-    default:
-        s.n_bands = 0;
-        s.k_steps = 0;
+// Row form: bands and k-steps.  q/k/v deals whole bands round-robin (144 bands fill 148 SMs well), gate/up
+// contiguous bands, because what they make is what the CTA's columns of the down-projection need.
+struct MkBands {
+    int j, end, step, k_steps;
+    __device__ void init(int type, const MkArgs &a)
+    {
+        const int half = a.hd >> 1;
+        k_steps = (a.d + MK_BOX_COLS - 1) / MK_BOX_COLS;
+        if (type == MK_QKV) {
+            j = blockIdx.x;
+            end = (a.Hq + a.Hkv) * (half / MK_BOX_ROWS) + (a.Hkv * a.hd + 2 * MK_BOX_ROWS - 1) / (2 * MK_BOX_ROWS);
+            step = gridDim.x;
+        } else {
+            const int per = a.cols.unit / MK_BOX_ROWS, n = (a.F + a.cols.unit - 1) / a.cols.unit;
+            j = (int)(blockIdx.x * (unsigned)n / gridDim.x) * per;
+            end = min((int)((blockIdx.x + 1) * (unsigned)n / gridDim.x) * per, (a.F + MK_BOX_ROWS - 1) / MK_BOX_ROWS);
+            step = 1;
+        }
     }
-    return s;
-}
-// Descriptor and first row of the two boxes of band b.
-__device__ __forceinline__ void mk_band(int type, const MkArgs &a, const MkLayer *L, int b, const CUtensorMap *(&map)[2],
-                                        int (&row)[2])
+};
+// Descriptor and first row of box `b` (0 or 1) of a band.
+__device__ __forceinline__ void mk_band(int type, const MkArgs &a, const MkLayer *L, int band, int b, const CUtensorMap *&map, int &row)
 {
     const int half = a.hd >> 1, per_head = half / MK_BOX_ROWS;
-    switch (type) {
-    case MK_QKV: {
+    if (type == MK_QKV) {
         const int nq = a.Hq * per_head, nk = a.Hkv * per_head;
-        if (b < nq + nk) {
-            const bool isq = b < nq;
-            const int bb = isq ? b : b - nq;
-            map[0] = map[1] = &L->map[isq ? MKW_Q : MKW_K];
-            row[0] = (bb / per_head) * a.hd + (bb % per_head) * MK_BOX_ROWS;
-            row[1] = row[0] + half;
+        if (band < nq + nk) {
+            const bool isq = band < nq;
+            const int bb = isq ? band : band - nq;
+            map = &L->map[isq ? MKW_Q : MKW_K];
+            row = (bb / per_head) * a.hd + (bb % per_head) * MK_BOX_ROWS + b * half;
         } else {
-            map[0] = map[1] = &L->map[MKW_V];
-            row[0] = (b - nq - nk) * 2 * MK_BOX_ROWS;
-            row[1] = row[0] + MK_BOX_ROWS;
+            map = &L->map[MKW_V];
+            row = ((band - nq - nk) * 2 + b) * MK_BOX_ROWS;
         }
-        break;
-    }
-    case MK_GATEUP:
-        map[0] = &L->map[MKW_G];
-        map[1] = &L->map[MKW_U];
-        row[0] = row[1] = b * MK_BOX_ROWS;
-        break;
-    default:
-        map[0] = map[1] = &L->map[type == MK_OPROJ ? MKW_O : MKW_D];
-        row[0] = b * 2 * MK_BOX_ROWS;
-        row[1] = row[0] + MK_BOX_ROWS;
+    } else {
+        map = &L->map[b ? MKW_U : MKW_G];
+        row = band * MK_BOX_ROWS;
     }
 }
 
-// This CTA's share of a projection phase, as segments (band, k-steps [ks0, ks1)).  q/k/v and
-// gate/up deal whole bands round-robin (144 and F/16 bands fill 148 SMs well).  The two residual
-// projections have d/32 bands, fewer than there are SMs, and an additive ending, so their
-// (band, k-step) pairs are laid end to end and cut into equal contiguous shares; a share that
-// ends inside a band adds its partial sums into the residual stream with atomics.
-struct MkSeg {
-    int band, ks0, ks1;
-};
-struct MkWalk {
-    int k_steps, n_bands, j;
-    bool stream;
-    long pos, hi;
-    __device__ void init(int type, const MkArgs &a)
+// Column form, O-projection: the (head, box of 64 weight rows) pairs laid end to end, head by head, and cut
+// into equal contiguous shares [lo, hi).
+struct MkHeads {
+    int boxes, lo, hi;
+    __device__ void init(const MkArgs &a)
     {
-        const MkShape shp = mk_shape(type, a);
-        k_steps = shp.k_steps;
-        n_bands = shp.n_bands;
-        stream = type == MK_OPROJ || type == MK_DOWN;
-        j = blockIdx.x;
-        const long T = (long)n_bands * k_steps;
-        pos = (long)blockIdx.x * T / gridDim.x;
-        hi = (long)(blockIdx.x + 1) * T / gridDim.x;
-    }
-    __device__ bool next(MkSeg &s)
-    {
-        if (stream) {
-            if (pos >= hi) return false;
-            s.band = (int)(pos / k_steps);
-            s.ks0 = (int)(pos % k_steps);
-            s.ks1 = (int)min((long)k_steps, s.ks0 + (hi - pos));
-            pos += s.ks1 - s.ks0;
-            return true;
-        }
-        if (j >= n_bands || k_steps < 1) return false;
-        s.band = j;
-        s.ks0 = 0;
-        s.ks1 = k_steps;
-        j += gridDim.x;
-        return true;
+        boxes = (a.d + MK_CBOX_ROWS - 1) / MK_CBOX_ROWS;
+        const unsigned T = (unsigned)a.Hq * boxes;
+        lo = (int)(blockIdx.x * T / gridDim.x);
+        hi = (int)((blockIdx.x + 1) * T / gridDim.x);
     }
 };
 
 struct MkShared {
-    uint64_t full[MK_SLOTS], empty[MK_SLOTS];
-    int giving_up, never;
+    uint64_t full[mk_slots(1)], empty[mk_slots(1)];
+    int giving_up, never, go_on;
     int row_slot[MK_MAX_ROWS], row_pos[MK_MAX_ROWS], grp_row0[MK_MAX_ROWS], grp_nrows[MK_MAX_ROWS];  // copies of the row set
-    int row_splits[MK_MAX_ROWS];         // splits of the attention phase that hold positions of the row
-    float red[MK_CW];
-    float red_rows[MK_MAX_ROWS][MK_CW];  // per-row partial sums of squares (tensor-core form: all rows at once)
+    int row_grp[MK_MAX_ROWS];            // group of a row
+    int grp_tiles[MK_MAX_ROWS];          // 16-position tiles of a group's prefix
+    int att_base[MK_MAX_ROWS + 1];       // tiles x kv heads of the groups before this one
+    int att_ctas;                        // CTAs that the tiles are dealt to: none of them goes without
+    int att_t0, att_t1;                  // this CTA's share of them
+    float red_rows[MK_MAX_ROWS][MK_CW];  // per-row partial sums of squares
+    float2 rope[MK_MAX_ROWS][64];        // rotary factors of the rows' positions; one row has room for as many
+};
+static_assert(sizeof(MkShared) <= MK_SHARED_BYTES, "MkShared outgrew its place");
+static_assert(offsetof(MkShared, rope) + sizeof(float2) * 64 <= MK_SHARED_FEW_BYTES, "MkShared outgrew its place");
+
+// A warp's place in the ring: slot and the parity of its present fill.
+template <int SLOTS>
+struct MkPos {
+    int s;
+    uint32_t ph;
+    __device__ __forceinline__ void skip(int n)   // n < SLOTS
+    {
+        s += n;
+        if (s >= SLOTS) {
+            s -= SLOTS;
+            ph ^= 1u;
+        }
+    }
+    __device__ __forceinline__ void skip_many(int n)
+    {
+        const int t = s + n, r = t / SLOTS;
+        s = t - r * SLOTS;
+        ph ^= (uint32_t)r & 1u;
+    }
 };
 
-// Consumers only: wait until every CTA has arrived at this barrier.
+// Attention: the tiles of 16 positions of all (group, kv head) pairs laid end to end and cut into equal
+// contiguous shares, so that every SM reads as much of the cache as the next (with fewer tiles than SMs, one each
+// for as many SMs); a run is what a share has of one pair.  The run of pair p in CTA c leaves partial number
+// c + p (both only ever grow from one run to the next), for every query vector of the pair.
+struct MkRun {
+    int g, hk, tile0, n;   // group, kv head, first tile, tiles
+};
+struct MkRuns {
+    int t, end;
+    __device__ void init(const MkShared *sh)
+    {
+        t = sh->att_t0;
+        end = sh->att_t1;
+    }
+    __device__ bool next(const MkShared *sh, MkRun &r)
+    {
+        if (t >= end) return false;
+        int g = 0;
+#pragma unroll
+        for (int i = 1; i < MK_MAX_ROWS; i++)
+            if (t >= sh->att_base[i]) g = i;   // (groups without tiles share their successor's base)
+        const int tiles = sh->grp_tiles[g], rem = t - sh->att_base[g];
+        r.g = g;
+        r.hk = rem / tiles;
+        r.tile0 = rem - r.hk * tiles;
+        r.n = min(tiles - r.tile0, end - t);
+        t += r.n;
+        return true;
+    }
+};
+// CTA whose share holds tile t
+__device__ __forceinline__ int mk_run_cta(const MkShared *sh, int t)
+{
+    return (int)((((unsigned)t + 1u) * (unsigned)sh->att_ctas - 1u) / (unsigned)sh->att_base[MK_MAX_ROWS]);
+}
+// query vectors of a partial
+__device__ __forceinline__ int mk_part_rows(const MkArgs &a) { return a.n_rows * (a.Hq / a.Hkv); }
+
+// Consumers only: wait until every CTA has arrived at this barrier.  A warp whose wait for a ring slot ran out
+// stays until here, without working, because the barriers among the CTA's warps have no time limit;
+// here all of them learn of it and leave together.
 __device__ __forceinline__ bool mk_grid_barrier(const MkArgs &a, MkShared *sh, unsigned long long &epoch)
 {
     mk_consumer_sync();
@@ -237,11 +292,12 @@ __device__ __forceinline__ bool mk_grid_barrier(const MkArgs &a, MkShared *sh, u
         for (uint32_t spin = 0;; ++spin) {
             if (ld_acquire_u64(a.bar) >= epoch) break;
             if ((spin & 63u) == 63u) {
-                if (ld_volatile_i32(a.abort_word) || sh->giving_up) {
-                    // another CTA (or an earlier launch that was never cleaned up after) gave up:
+                if (ld_volatile_i32(a.abort_word) || *(volatile int *)&sh->giving_up) {
+                    // this CTA or another (or an earlier launch that was never cleaned up after) gave up:
                     // leave too, and say so, so that skipping the rest is never silent
                     sh->giving_up = 1;
                     atomicOr(a.status, ST_TIMEOUT);
+                    atomicExch(a.abort_word, 1);
                     break;
                 }
                 const unsigned long long now = global_ns();
@@ -254,10 +310,11 @@ __device__ __forceinline__ bool mk_grid_barrier(const MkArgs &a, MkShared *sh, u
                 }
             }
         }
+        sh->go_on = !*(volatile int *)&sh->giving_up;
         if (blockIdx.x == 0 && a.trace) a.trace[(epoch - a.bar_base) / gridDim.x] = global_ns();
     }
     mk_consumer_sync();
-    return *(volatile int *)&sh->giving_up == 0;
+    return sh->go_on != 0;  // one answer for all warps
 }
 
 }  // namespace sparsk

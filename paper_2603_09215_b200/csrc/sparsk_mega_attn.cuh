@@ -1,65 +1,226 @@
-// Attention and split-merge phases of the persistent layer-range kernel (see sparsk_mega.cuh).
+// Attention phase of the persistent layer-range kernel and the merge of its partials (see sparsk_mega.cuh).
 #pragma once
 
 namespace sparsk {
 
-// Items (group, query block, kv head, split) are dealt to MK_ATT_WARPS warps of every CTA; a warp
-// runs its item alone (attn_item of the stand-alone kernel): 16 query vectors (query heads of the
-// kv head, for the group's rows) parked in shared memory (this kernel's register budget is spoken
-// for), its own two-stage K/V ring inside the activation area, one partial per item.
+// A warp's view of a run's ring items: items sub, sub + nsub, ... of the run, two 16-position tiles each (K and
+// V, with the 128-byte swizzle, as the producers' TMA copies leave them), in the form attn_item asks for.
+// The tiles were on their way before this launch's q/k/v projection had written the current rows' keys and
+// values: those rows are copied over from the cache, and value rows past the end are cleared (they meet a
+// weight of exactly zero, which must not meet a NaN).  Every warp that reads a tile does both for itself.
+template <int HD, int SLOTS>
+struct MkTiles {
+    static constexpr int TILE = AT_TP * HD;   // numbers of one matrix's tile
+    unsigned char *ring;
+    MkShared *sh;
+    int *status;
+    const kv_t *kbase, *vbase;    // the cache of (slot, kv head)
+    MkPos<SLOTS> at0;             // ring place of the run's first tiles
+    int tile0, sub, nsub;
+    int new0, end;                // the pass's own positions: [new0, end), end = the prefix's length
+    int arrivals;                 // this warp's share of a slot's release
+    int n_tiles, lane;
+
+    __device__ __forceinline__ static int off(int row, int c) { return at_swz<HD>(row, c); }
+    __device__ __forceinline__ int item(int t) const { return sub + nsub * (t >> 1); }
+    __device__ __forceinline__ MkPos<SLOTS> place(int t) const
+    {
+        MkPos<SLOTS> p = at0;
+        p.skip_many(item(t));
+        return p;
+    }
+    __device__ __forceinline__ int pos(int t) const { return (tile0 + 2 * item(t) + (t & 1)) * AT_TP; }
+    __device__ __forceinline__ bool wait(int t, const kv_t *&Kt, const kv_t *&Vt) const
+    {
+        const MkPos<SLOTS> at = place(t);
+        if (!(t & 1) && !mbar_wait(&sh->full[at.s], at.ph, &sh->giving_up, status)) return false;
+        kv_t *kt = reinterpret_cast<kv_t *>(ring + (size_t)at.s * MK_SLOT_BYTES) + (t & 1) * 2 * TILE, *vt = kt + TILE;
+        const int p0 = pos(t);
+        if (p0 + AT_TP > new0) {
+            constexpr int CH = HD / 8;
+            for (int k = lane; k < AT_TP * CH; k += 32) {
+                const int r = k / CH, c = k % CH, p = p0 + r;
+                if (p < new0) continue;
+                const size_t o = (size_t)p * HD + c * 8;
+                if (p < end) *reinterpret_cast<uint4 *>(&kt[off(r, c)]) = __ldcg(reinterpret_cast<const uint4 *>(kbase + o));
+                *reinterpret_cast<uint4 *>(&vt[off(r, c)]) = p < end ? __ldcg(reinterpret_cast<const uint4 *>(vbase + o)) : make_uint4(0u, 0u, 0u, 0u);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the slot's next copy
+        }
+        __syncwarp();
+        Kt = kt;
+        Vt = vt;
+        return true;
+    }
+    __device__ __forceinline__ void release(int t) const
+    {
+        __syncwarp();
+        if ((t & 1) || t == n_tiles - 1) {
+            if (lane == 0) mbar_arrive_n(&sh->empty[place(t).s], (uint32_t)arrivals);
+        }
+    }
+    __device__ __forceinline__ void finish() const {}
+};
+// Where it leaves its partial: the run's place in global memory, or the area, when several warps share the run.
 template <int HD>
-__device__ __forceinline__ void mk_attention(const MkArgs &a, const MkLayer *L, unsigned char *area, const MkShared *sh)
+struct MkCells {
+    float *po;
+    float2 *pml;
+    __device__ __forceinline__ float *o(int qg) const { return po + (ptrdiff_t)qg * HD; }
+    __device__ __forceinline__ float2 *ml(int qg) const { return pml + qg; }
+};
+// Parked queries of one block of sixteen; one warp's partial of such a block and its sums.
+template <int HD>
+__host__ __device__ constexpr int mk_park_bytes() { return 16 * (HD + 8) * 2; }
+template <int HD>
+__host__ __device__ constexpr int mk_cell_bytes() { return 16 * HD * 4 + 16 * 8; }
+// Shapes the phase can run: a warp and a place for its queries per block of query vectors of a group.
+inline bool mk_attn_fits(int M, int G, int head_dim)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (warp >= MK_ATT_WARPS) return;
-    // per warp: its 16 query vectors, then the K/V ring
-    kv_t *qs = reinterpret_cast<kv_t *>(area) + (size_t)warp * (16 + MK_ATT_NST * 2 * AT_TP) * (HD + 8);
-    kv_t *wr = qs + 16 * (HD + 8);
-    AttnArgs at{};
-    at.q = nullptr; at.q32 = a.q_buf; at.kc = L->kc; at.vc = L->vc;
-    at.part_o = a.part_o; at.part_ml = a.part_ml;
-    at.Hq = a.Hq; at.Hkv = a.Hkv; at.S = a.S; at.n_slots = a.n_slots; at.n_rows = a.n_rows;
-    at.n_qblk = a.att_qblk; at.n_splits = a.att_splits; at.split_len = a.att_split_len; at.max_groups = a.n_groups;
-    at.nq_min = 0; at.nq_max = 1 << 30;
-    const unsigned n_workers = gridDim.x * MK_ATT_WARPS, worker = warp * gridDim.x + blockIdx.x;
-    const unsigned n_items = (unsigned)a.n_groups * a.att_qblk * a.Hkv * a.att_splits;
-    for (unsigned item = worker; item < n_items; item += n_workers) {
-        const AtItem it = at_resolve(at, item, n_items, a.n_groups, sh->grp_row0, sh->grp_nrows, sh->row_slot, sh->row_pos);
-        if (!it.valid) continue;
-        // a single row's query heads (at most eight per kv head) take the transposed form
-        if (it.nq <= 8) attn_item_t<HD, MK_ATT_NST, false>(at, it, wr, lane);
-        else attn_item<HD, MK_ATT_NST, false>(at, it, wr, qs, lane);
+    const int blocks = (M * G + 15) / 16;
+    return blocks <= MK_CW && blocks * (head_dim == 128 ? mk_park_bytes<128>() : mk_park_bytes<64>()) <= mk_area_bytes(M);
+}
+
+// The CTA's runs, one after another.  Up to four warps per block of sixteen query vectors share a run (as many as the area
+// has room for partials), every nsub-th slot each; their partials meet in the area.
+template <int M, int HD>
+__device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned char *area, unsigned char *ring, MkShared *sh,
+                                             MkPos<mk_slots(M)> &at)
+{
+    constexpr int SLOTS = mk_slots(M);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = a.Hq / a.Hkv;
+    AttnArgs aa{};
+    aa.q32 = a.q_buf; aa.Hq = a.Hq; aa.Hkv = a.Hkv;
+    const int stride = mk_part_rows(a);
+    MkRuns runs;
+    runs.init(sh);
+    MkRun r;
+    while (runs.next(sh, r)) {
+        const int nq = sh->grp_nrows[r.g] * G, n_qblk = (nq + 15) / 16, n_items = (r.n + 1) / 2;
+        const int room = (mk_area_bytes(M) - n_qblk * mk_park_bytes<HD>()) / (n_qblk * mk_cell_bytes<HD>());
+        int nsub = min(min(4, MK_CW / n_qblk), min(room, n_items));
+        if (nsub < 1) nsub = 1;
+        if (SLOTS % nsub) nsub = 2;  // a slot's successive fills stay with one warp
+        const int qb = warp % n_qblk, sub = warp / n_qblk;
+        // (the warps of a block all park its queries, the same numbers in the same place)
+        kv_t *park = reinterpret_cast<kv_t *>(area) + (size_t)qb * 16 * (HD + 8);
+        unsigned char *cells = area + n_qblk * mk_park_bytes<HD>();
+        const size_t part = (size_t)(blockIdx.x + r.g * a.Hkv + r.hk) * stride;
+        if (sub < nsub) {
+            const int row0 = sh->grp_row0[r.g], pos0 = sh->row_pos[row0];
+            AtItem item;
+            item.qb = qb; item.hk = r.hk; item.row0 = row0; item.nrows = sh->grp_nrows[r.g]; item.pos0 = pos0; item.nq = nq;
+            item.w_end = min(pos0 + (min(qb * 16 + 16, nq) - 1) / G + 1, a.S);
+            MkTiles<HD, SLOTS> tiles;
+            tiles.ring = ring; tiles.sh = sh; tiles.status = a.status;
+            const size_t rows0 = ((size_t)sh->row_slot[row0] * a.Hkv + r.hk) * a.S;
+            tiles.kbase = a.kc + l * a.kv_layer + rows0 * HD; tiles.vbase = a.vc + l * a.kv_layer + rows0 * HD;
+            tiles.at0 = at; tiles.tile0 = r.tile0; tiles.sub = sub; tiles.nsub = nsub;
+            tiles.new0 = pos0; tiles.end = min(pos0 + item.nrows, a.S);
+            tiles.arrivals = qb == 0 ? MK_CW - (n_qblk - 1) : 1;
+            const int mine = (n_items - sub + nsub - 1) / nsub;
+            tiles.n_tiles = 2 * mine - ((r.n & 1) && (n_items - 1) % nsub == sub ? 1 : 0);
+            tiles.lane = lane;
+            MkCells<HD> out;
+            if (nsub > 1) {
+                // query vector qg of block qb at row qg - 16 qb of the warp's cells
+                unsigned char *c = cells + (size_t)(sub * n_qblk + qb) * mk_cell_bytes<HD>();
+                out.po = reinterpret_cast<float *>(c) - (ptrdiff_t)qb * 16 * HD;
+                out.pml = reinterpret_cast<float2 *>(c + 16 * HD * 4) - qb * 16;
+            } else {
+                out.po = a.part_o + part * HD;
+                out.pml = a.part_ml + part;
+            }
+            if (nq <= 8) attn_item_t<HD>(aa, item, tiles, out, lane);
+            else attn_item<HD, false>(aa, item, tiles, out, park, lane);
+        }
+        at.skip_many(n_items);
+        mk_consumer_sync();
+        if (nsub > 1) {
+            for (int k = threadIdx.x; k < nq * (HD / 4); k += MK_CW * 32) {
+                const int qg = k / (HD / 4), c4 = k % (HD / 4), blk = qg / 16, ql = qg % 16;
+                float mx = -INFINITY, sum = 0.f;
+                float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int s = 0; s < nsub; s++)
+                    mx = fmaxf(mx, reinterpret_cast<const float2 *>(cells + (size_t)(s * n_qblk + blk) * mk_cell_bytes<HD>() + 16 * HD * 4)[ql].x);
+                for (int s = 0; s < nsub; s++) {
+                    const unsigned char *c = cells + (size_t)(s * n_qblk + blk) * mk_cell_bytes<HD>();
+                    const float2 ml = reinterpret_cast<const float2 *>(c + 16 * HD * 4)[ql];
+                    const float w = ml.x == -INFINITY ? 0.f : __expf(ml.x - mx);
+                    const float4 p = reinterpret_cast<const float4 *>(c)[ql * (HD / 4) + c4];
+                    sum += ml.y * w;
+                    o.x += p.x * w; o.y += p.y * w; o.z += p.z * w; o.w += p.w * w;
+                }
+                *reinterpret_cast<float4 *>(a.part_o + (part + qg) * HD + c4 * 4) = o;
+                if (c4 == 0) a.part_ml[part + qg] = make_float2(mx, sum);
+            }
+            mk_consumer_sync();  // the next run may use the area
+        }
     }
 }
 
-// Merge of the splits: one warp per (row, query head, 32 output dims).  Lane s holds split s's
-// weight (att_splits <= 32); every lane owns one output dim and has all its loads in flight at once.
-// Only the splits that hold positions of the row are read: nobody writes the partials of the others, and
-// what they hold (NaN for one) would outlast a weight of zero.
-template <int HD, bool PLANES>
-__device__ __forceinline__ void mk_merge(const MkArgs &a, const MkShared *sh)
+// Merge of the partials of query heads hq and, with NH = 2, hq + 1, for all rows: 16 / (M NH) warps per row and head, a
+// share of the partials each, then the shares meet in scr.  Leaves the output of head i, row m at column c
+// through put(i, m, c, value).
+template <int M, int HD, int NH, class Put>
+__device__ __forceinline__ void mk_merge_heads(const MkArgs &a, const MkShared *sh, int hq, float *scr, const Put &put)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int PARTS = HD / 32;
-    const int n_items = a.n_rows * a.Hq * PARTS;
-    for (int item = warp * gridDim.x + blockIdx.x; item < n_items; item += gridDim.x * MK_CW) {
-        const int cell = item / PARTS, d = (item % PARTS) * 32 + lane, live = sh->row_splits[cell / a.Hq];
-        const size_t cell0 = (size_t)cell * a.att_splits;
-        float2 ml = make_float2(-INFINITY, 0.f);
-        if (lane < live) ml = a.part_ml[cell0 + lane];
-        float v[MK_MAX_SPLITS];
+    constexpr int WPR = MK_CW / (M * NH), LN = HD / 4;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = a.Hq / a.Hkv;
+    const int hm = warp / WPR, h = hq + hm / M, hk = h / G, m = hm % M, wi = warp % WPR, stride = mk_part_rows(a);
+    float2 *scr_ml = reinterpret_cast<float2 *>(scr + MK_CW * HD);
+    float mx = -INFINITY, l = 0.f;
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int g = m < a.n_rows ? sh->row_grp[m] : -1, tiles = g >= 0 ? sh->grp_tiles[g] : 0;
+    if (tiles > 0) {
+        const int t0 = sh->att_base[g] + hk * tiles;
+        const int cf = mk_run_cta(sh, t0), cl = mk_run_cta(sh, t0 + tiles - 1);
+        const size_t cell0 = (size_t)(g * a.Hkv + hk) * stride + (m - sh->grp_row0[g]) * G + h - hk * G;
+        constexpr int U = 5;
+        for (int c0 = cf + wi; c0 <= cl; c0 += WPR * U) {
+            float2 ml[U];
+            float4 v[U];
 #pragma unroll
-        for (int s = 0; s < MK_MAX_SPLITS; s++) v[s] = s < live ? a.part_o[(cell0 + s) * HD + d] : 0.f;
-        const float M = warp_max(ml.x);
-        const float w_mine = ml.x == -INFINITY ? 0.f : __expf(ml.x - M);
-        const float den = warp_sum(ml.y * w_mine);
-        float num = 0.f;
+            for (int u = 0; u < U; u++) {
+                const int c = c0 + u * WPR;
+                const size_t cell = cell0 + (size_t)c * stride;
+                ml[u] = c <= cl ? a.part_ml[cell] : make_float2(-INFINITY, 0.f);
+                v[u] = c <= cl && lane < LN ? reinterpret_cast<const float4 *>(a.part_o + cell * HD)[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            float top = mx;
 #pragma unroll
-        for (int s = 0; s < MK_MAX_SPLITS; s++) num += v[s] * __shfl_sync(0xffffffffu, w_mine, s);
-        const float o = den > 0.f ? num / den : 0.f;
-        if (PLANES) mk_put_planes(a.attn_o, a.Hq * HD, a.n_rows, cell / a.Hq, (cell % a.Hq) * HD + d, o);
-        else a.attn_o[(size_t)cell * HD + d] = o;
+            for (int u = 0; u < U; u++) top = fmaxf(top, ml[u].x);
+            if (top == -INFINITY) continue;  // (the same in all lanes)
+            const float old = __expf(mx - top);
+            l *= old;
+            o.x *= old; o.y *= old; o.z *= old; o.w *= old;
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                const float w = ml[u].x == -INFINITY ? 0.f : __expf(ml[u].x - top);
+                l += ml[u].y * w;
+                o.x += v[u].x * w; o.y += v[u].y * w; o.z += v[u].z * w; o.w += v[u].w * w;
+            }
+            mx = top;
+        }
     }
+    if (lane < LN) reinterpret_cast<float4 *>(scr + warp * HD)[lane] = o;
+    if (lane == 0) scr_ml[warp] = make_float2(mx, l);
+    mk_consumer_sync();
+    for (int k = threadIdx.x; k < NH * M * HD; k += MK_CW * 32) {
+        const int at = k / HD, c = k % HD;
+        float top = -INFINITY, den = 0.f, num = 0.f;
+#pragma unroll
+        for (int w = 0; w < WPR; w++) top = fmaxf(top, scr_ml[at * WPR + w].x);
+#pragma unroll
+        for (int w = 0; w < WPR; w++) {
+            const float2 ml = scr_ml[at * WPR + w];
+            const float f = ml.x == -INFINITY ? 0.f : __expf(ml.x - top);
+            den += ml.y * f;
+            num += scr[(at * WPR + w) * HD + c] * f;
+        }
+        put(at / M, at % M, c, den > 0.f ? num / den : 0.f);
+    }
+    mk_consumer_sync();
 }
 
 }  // namespace sparsk

@@ -3,149 +3,273 @@
 
 namespace sparsk {
 
-// Walks this CTA's ring items in consumption order: for every layer, for the four projection
-// phases, for every segment the CTA owns, for every k-step.
-struct MkCursor {
-    int l, type, ks;
-    MkWalk walk;
-    MkSeg seg;
-    uint32_t idx;
-    bool done;
-
-    __device__ void settle(const MkArgs &a)
-    {
-        // move to the next phase that has work for this CTA
-        for (;;) {
-            if (l >= a.layer_end) {
-                done = true;
-                return;
+// ------------------------------------------------------------------ producers
+// One producer warp: walks the CTA's ring items in consumption order and issues every fourth.
+template <int M, int HD>
+__device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring, MkShared *sh, int p)
+{
+    constexpr int SLOTS = mk_slots(M);
+    constexpr bool TC = M >= MK_TC_ROWS;
+    const int lane = threadIdx.x & 31;
+    uint32_t idx = 0;   // ring item
+    bool ok = true;
+    // waits until item idx's slot is free and no more than MK_IN_FLIGHT items (counting this one) are on
+    // their way, and announces `bytes`; item idx - MK_IN_FLIGHT was this warp's own
+    static_assert(MK_IN_FLIGHT % MK_PW == 0 && SLOTS % MK_PW == 0, "a producer waits for items of its own");
+    auto open = [&](uint32_t bytes) {
+        const int s = idx % SLOTS;
+        int go = 1;
+        if (lane == 0) {
+            if (SLOTS > MK_IN_FLIGHT && idx >= MK_IN_FLIGHT) {
+                const uint32_t o = idx - MK_IN_FLIGHT;
+                go = mbar_wait(&sh->full[o % SLOTS], (o / SLOTS) & 1, &sh->giving_up, a.status) ? 1 : 0;
             }
-            walk.init(type, a);
-            if (walk.next(seg)) {
-                ks = seg.ks0;
-                return;
-            }
-            next_phase();
+            if (go) go = mbar_wait(&sh->empty[s], ((idx / SLOTS) & 1) ^ 1, &sh->giving_up, a.status) ? 1 : 0;
+            if (go) mbar_expect_tx(&sh->full[s], bytes);
         }
-    }
-    __device__ void next_phase()
-    {
-        type = type == MK_QKV ? MK_OPROJ : (type == MK_OPROJ ? MK_GATEUP : (type == MK_GATEUP ? MK_DOWN : MK_QKV));
-        if (type == MK_QKV) l++;
-    }
-    __device__ void init(const MkArgs &a)
-    {
-        l = a.layer_begin;
-        type = MK_QKV;
-        idx = 0;
-        done = false;
-        settle(a);
-    }
-    __device__ void advance(const MkArgs &a)
-    {
+        ok = __shfl_sync(0xffffffffu, go, 0) != 0;
+        return ok;
+    };
+    auto rows = [&](int type, const MkLayer *L) {
+        MkBands w;
+        w.init(type, a);
+        for (; w.j < w.end; w.j += w.step)
+            for (int ks = 0; ks < w.k_steps; ks++, idx++) {
+                if ((int)(idx % MK_PW) != p) continue;
+                if (!open(MK_SLOT_BYTES)) return;
+                if (lane < 2) {
+                    const CUtensorMap *map;
+                    int row;
+                    mk_band(type, a, L, w.j, lane, map, row);
+                    const int s = idx % SLOTS;
+                    const uint32_t dst = smem_u32(ring) + s * MK_SLOT_BYTES + lane * MK_BOX_BYTES;
+                    // (three and four rows: the same box as four swizzled 64-column blocks)
+                    if (TC) tma_load_3d(dst, map + MKW_N, &sh->full[s], 0, row, ks * (MK_BOX_COLS / 64));
+                    else tma_load_2d(dst, map, &sh->full[s], ks * MK_BOX_COLS, row);
+                }
+            }
+    };
+    auto column_box = [&](const CUtensorMap *map, int cols, int col0, int row0) {
+        if ((int)(idx % MK_PW) == p) {
+            if (!open((uint32_t)(MK_CBOX_ROWS * cols * 2))) return;
+            if (lane == 0) {
+                const int s = idx % SLOTS;
+                const uint32_t dst = smem_u32(ring) + s * MK_SLOT_BYTES;
+                if (TC) tma_load_3d(dst, map + MKW_N, &sh->full[s], 0, row0, col0 / 32);
+                else tma_load_2d(dst, map, &sh->full[s], col0, row0);
+            }
+        }
         idx++;
-        if (++ks < seg.ks1) return;
-        if (walk.next(seg)) {
-            ks = seg.ks0;
-            return;
+    };
+    for (int l = a.layer_begin; l < a.layer_end && ok; l++) {
+        const MkLayer *L = a.layers + l;
+        rows(MK_QKV, L);
+        if (!ok) break;
+        MkRuns runs;
+        runs.init(sh);
+        MkRun r;
+        while (ok && runs.next(sh, r)) {
+            const int y0 = (sh->row_slot[sh->grp_row0[r.g]] * a.Hkv + r.hk) * a.S;
+            for (int i = 0; i < r.n; i += 2, idx++) {
+                if ((int)(idx % MK_PW) != p) continue;
+                const int n = min(2, r.n - i);
+                if (!open((uint32_t)(n * 2 * AT_TP * HD * sizeof(kv_t)))) break;
+                if (lane < 2 * n) {
+                    const int s = idx % SLOTS, y = y0 + (r.tile0 + i + (lane >> 1)) * AT_TP;
+                    const uint32_t dst = smem_u32(ring) + s * MK_SLOT_BYTES + lane * (AT_TP * HD * (uint32_t)sizeof(kv_t));
+                    const CUtensorMap *map = lane & 1 ? &L->vmap : &L->kmap;
+                    if (HD > 64) tma_load_3d(dst, map, &sh->full[s], 0, y, 0);
+                    else tma_load_2d(dst, map, &sh->full[s], 0, y);
+                }
+            }
         }
-        next_phase();
-        settle(a);
+        if (!ok) break;
+        MkHeads w;
+        w.init(a);
+        for (int i = w.lo; i < w.hi && ok; i++) column_box(&L->map[MKW_O], HD, (i / w.boxes) * HD, (i % w.boxes) * MK_CBOX_ROWS);
+        if (!ok) break;
+        rows(MK_MLP, L);
+        if (!ok) break;
+        MkBands b;
+        b.init(MK_MLP, a);
+        if (b.j < b.end)
+            for (int c = 0; c < a.cols.chunks && ok; c++)
+                for (int i = 0; i < w.boxes && ok; i++)
+                    column_box(&L->map[MKW_D], a.cols.box, b.j * MK_BOX_ROWS + c * a.cols.box, i * MK_CBOX_ROWS);
     }
-    __device__ int band() const { return seg.band; }
-};
+    // never leave with copies in flight: every slot this producer filled must have landed
+    // (consumers that gave up no longer free slots, so wait on the full barriers, 2 ms each)
+    if (lane == 0) {
+        const uint32_t total = idx;  // items before the point where this producer stopped
+        for (int s = p; s < SLOTS; s += MK_PW)
+            if (total > (uint32_t)s) mbar_wait(&sh->full[s], ((total - 1 - s) / SLOTS) & 1, &sh->never, nullptr, 2000000ull);
+    }
+}
+
+// ------------------------------------------------------------------ consumers: O-projection and MLP
+template <int M, int HD>
+__device__ __forceinline__ void mk_oproj(const MkArgs &a, unsigned char *area, unsigned char *ring, MkShared *sh,
+                                         MkPos<mk_slots(M)> &at)
+{
+    MkHeads w;
+    w.init(a);
+    constexpr bool TC = M >= MK_TC_ROWS;
+    constexpr int RS = HD + 8;
+    // two merged heads, as fp32 rows or as two planes each
+    float *const x = reinterpret_cast<float *>(area);
+    bf16 *const planes = reinterpret_cast<bf16 *>(area);
+    float *scr = reinterpret_cast<float *>(area + 8 * 1024);
+    static_assert((TC ? 2 * 2 * M * RS * 2 : 2 * M * HD * 4) <= 8 * 1024, "two heads' activations");
+    auto put = [&](int i, int m, int c, float v) {
+        if constexpr (TC) mk_put_planes<M>(planes + i * 2 * M * RS, RS, m, c, v);
+        else x[(i * M + m) * HD + c] = v;
+    };
+    // a share reaches into a second head as often as not, into a third one only with more heads than CTAs
+    for (int i = w.lo; i < w.hi;) {
+        const int hq = i / w.boxes;
+        if (i != w.lo) mk_consumer_sync();  // everyone is done with the heads before
+        if ((hq + 1) * w.boxes < w.hi) mk_merge_heads<M, HD, 2>(a, sh, hq, scr, put);
+        else mk_merge_heads<M, HD, 1>(a, sh, hq, scr, put);
+        for (int k = 0; k < 2 && i < w.hi; k++) {
+            const int r0 = i - (hq + k) * w.boxes, n = min(w.boxes - r0, w.hi - i);
+            if constexpr (TC) mk_columns_tc<M>(a, a.h, r0, r0 + n, HD, planes + k * 2 * M * RS, RS, ring, sh, at);
+            else mk_columns<M, HD / 8>(a, a.h, r0, r0 + n, HD, x + k * M * HD, HD, ring, sh, at);
+            i += n;
+            at.skip_many(n);
+        }
+    }
+}
+
+template <int M>
+__device__ __forceinline__ void mk_mlp(const MkArgs &a, int l, unsigned char *area, unsigned char *ring, MkShared *sh,
+                                       const MkGains &gains, MkPos<mk_slots(M)> &at)
+{
+    const int boxes = (a.d + MK_CBOX_ROWS - 1) / MK_CBOX_ROWS;
+    MkBands w;
+    w.init(MK_MLP, a);
+    if (w.j >= w.end) return;
+    const bf16 *gain = a.layers[l].mlp_gain;
+    // columns of the last box that are the next CTA's meet zeros
+    if constexpr (M >= MK_TC_ROWS) {
+        const int rs = a.cols.most + 8;
+        bf16 *planes = reinterpret_cast<bf16 *>(area);
+        float *red = reinterpret_cast<float *>(area + mk_tc_planes_bytes(M, w.k_steps * MK_BOX_COLS));
+        bf16 *u = reinterpret_cast<bf16 *>(reinterpret_cast<unsigned char *>(red) + MK_TC_RED_BYTES);
+        for (int i = threadIdx.x; i < M * rs; i += MK_CW * 32) reinterpret_cast<uint32_t *>(u)[i] = 0u;
+        mk_rows_tc<M>(MK_MLP, a, l, planes, red, nullptr, gain, gains, u, rs, ring, sh, at);
+        mk_consumer_sync();
+        for (int c = 0; c < a.cols.chunks; c++, at.skip_many(boxes))
+            mk_columns_tc<M>(a, a.h2, 0, boxes, a.cols.box, u + c * a.cols.box, rs, ring, sh, at);
+    } else {
+        const int own = M * a.cols.most * 4 + mk_sums_bytes(M);
+        float *u = reinterpret_cast<float *>(area + mk_area_bytes(M) - own), *sums = u + M * a.cols.most;
+        for (int i = threadIdx.x; i < M * a.cols.most; i += MK_CW * 32) u[i] = 0.f;
+        mk_rows<M>(MK_MLP, a, l, reinterpret_cast<float *>(area), sums, own, nullptr, gain, gains, u, a.cols.most, ring, sh, at);
+        mk_consumer_sync();
+        for (int c = 0; c < a.cols.chunks; c++, at.skip_many(boxes)) {
+            const float *x = u + c * a.cols.box;
+            if (a.cols.box <= 64) mk_columns<M, 8>(a, a.h2, 0, boxes, a.cols.box, x, a.cols.most, ring, sh, at);
+            else mk_columns<M, 16>(a, a.h2, 0, boxes, a.cols.box, x, a.cols.most, ring, sh, at);
+        }
+    }
+}
+
+// h += h2, h2 = 0: `n` threads of every CTA, this one the i-th of them.
+__device__ __forceinline__ void mk_fold(const MkArgs &a, int i, int n)
+{
+    const int total = a.n_rows * a.d / 4;
+    for (int k = (int)blockIdx.x + i * (int)gridDim.x; k < total; k += n * (int)gridDim.x) {
+        float4 *p = reinterpret_cast<float4 *>(a.h) + k, *q = reinterpret_cast<float4 *>(a.h2) + k;
+        const float4 x = *p, y = *q;
+        *p = make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w);
+        *q = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
 
 template <int M, int HD>
 __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
 {
-    extern __shared__ __align__(1024) unsigned char mk_smem[];
-    __shared__ MkShared sh;
-    // the swizzled boxes of the tensor-core form need the ring on a 1024-byte boundary
-    unsigned char *ring = mk_smem + ((1024u - (smem_u32(mk_smem) & 1023u)) & 1023u);  // MK_SLOTS x 16 KB
-    unsigned char *area = ring + (size_t)MK_SLOTS * MK_SLOT_BYTES;     // activations / attention rings
+    extern __shared__ __align__(1024) unsigned char mk_smem[];  // (nothing else is in shared memory: the swizzled boxes need 1024)
+    unsigned char *ring = mk_smem;
+    unsigned char *area = ring + (size_t)mk_slots(M) * MK_SLOT_BYTES;
+    MkShared *sh = reinterpret_cast<MkShared *>(area + mk_area_bytes(M));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < MK_SLOTS; s++) {
-            mbar_init(&sh.full[s], 1);
-            mbar_init(&sh.empty[s], MK_CW);
+        for (int s = 0; s < mk_slots(M); s++) {
+            mbar_init(&sh->full[s], 1);
+            mbar_init(&sh->empty[s], MK_CW);
         }
-        sh.giving_up = 0;
-        sh.never = 0;
+        sh->giving_up = 0;
+        sh->never = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1 && lane < MK_MAX_ROWS) {
-        const int i = lane;
-        sh.row_slot[i] = i < a.n_rows ? a.row_slot[i] : -1;
-        sh.row_pos[i] = i < a.n_rows ? a.row_pos[i] : -1;
-        sh.row_splits[i] = i < a.n_rows ? min(a.row_pos[i] / a.att_split_len + 1, a.att_splits) : 0;
-        sh.grp_row0[i] = i < a.n_groups ? a.grp_row0[i] : -1;
-        sh.grp_nrows[i] = i < a.n_groups ? a.grp_nrows[i] : 0;
+    if (warp == 1) {
+        if (lane < MK_MAX_ROWS) {
+            const int i = lane;
+            sh->row_slot[i] = i < a.n_rows ? a.row_slot[i] : -1;
+            sh->row_pos[i] = i < a.n_rows ? a.row_pos[i] : -1;
+            sh->row_grp[i] = -1;
+            sh->grp_row0[i] = i < a.n_groups ? a.grp_row0[i] : -1;
+            sh->grp_nrows[i] = i < a.n_groups ? a.grp_nrows[i] : 0;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            int base = 0;
+            for (int g = 0; g < MK_MAX_ROWS; g++) {
+                const int r0 = sh->grp_row0[g], n = sh->grp_nrows[g];
+                const bool sane = r0 >= 0 && n >= 1 && r0 + n <= a.n_rows && sh->row_slot[r0] >= 0 && sh->row_slot[r0] < a.n_slots &&
+                                  sh->row_pos[r0] >= 0;
+                const int tiles = sane ? (min(sh->row_pos[r0] + n, a.S) + AT_TP - 1) / AT_TP : 0;
+                sh->grp_tiles[g] = tiles;
+                sh->att_base[g] = base;
+                base += tiles * a.Hkv;
+                for (int r = 0; sane && r < n; r++) sh->row_grp[r0 + r] = g;
+            }
+            sh->att_base[MK_MAX_ROWS] = base;
+            const unsigned n = (unsigned)min((int)gridDim.x, base), c = blockIdx.x;
+            sh->att_ctas = (int)n;
+            sh->att_t0 = c < n ? (int)(c * (unsigned)base / n) : 0;
+            sh->att_t1 = c < n ? (int)((c + 1) * (unsigned)base / n) : 0;
+        }
+    }
+    if (warp >= 2 && warp < 2 + M && warp - 2 < a.n_rows) {
+        const int i = warp - 2, pos = a.row_pos[i];
+        for (int j = lane; j < HD / 2; j += 32) sh->rope[i][j] = pos >= 0 ? a.rope[(size_t)pos * (HD / 2) + j] : make_float2(1.f, 0.f);
     }
     __syncthreads();
 
     if (warp >= MK_CW) {
-        // ------------------------------------------------------------ producers
-        const int p = warp - MK_CW;  // owns items p, p + 4, ... and with them ring slots p and p + 4
-        MkCursor ld;
-        ld.init(a);
-        bool ok = true;
-        while (!ld.done && ok) {
-            if ((int)(ld.idx % MK_PW) == p) {
-                const int s = ld.idx % MK_SLOTS;
-                int go = 1;
-                if (lane == 0) {
-                    go = mbar_wait(&sh.empty[s], ((ld.idx / MK_SLOTS) & 1) ^ 1, &sh.giving_up, a.status) ? 1 : 0;
-                    if (go) mbar_expect_tx(&sh.full[s], MK_SLOT_BYTES);
-                }
-                go = __shfl_sync(0xffffffffu, go, 0);
-                if (!(ok = go != 0)) break;
-                if (lane < 2) {
-                    const CUtensorMap *map[2];
-                    int row[2];
-                    mk_band(ld.type, a, a.layers + ld.l, ld.band(), map, row);
-                    const uint32_t dst = smem_u32(ring) + s * MK_SLOT_BYTES + lane * MK_BOX_BYTES;
-                    if (M >= MK_TC_ROWS)  // the same box as four swizzled 64-column blocks (entries MKW_N on)
-                        tma_load_3d(dst, map[lane] + MKW_N, &sh.full[s], 0, row[lane], ld.ks * (MK_BOX_COLS / 64));
-                    else
-                        tma_load_2d(dst, map[lane], &sh.full[s], ld.ks * MK_BOX_COLS, row[lane]);
-                }
-            }
-            ld.advance(a);
-        }
-        // never leave with copies in flight: every slot this producer filled must have landed
-        // (consumers that gave up no longer free slots, so wait on the full barriers, 2 ms each)
-        if (lane == 0) {
-            const uint32_t total = ld.idx;  // items before the point where this producer stopped
-            for (int s = p; s < MK_SLOTS; s += MK_PW)
-                if (total > (uint32_t)s) mbar_wait(&sh.full[s], ((total - 1 - s) / MK_SLOTS) & 1, &sh.never, nullptr, 2000000ull);
-        }
+        mk_produce<M, HD>(a, ring, sh, warp - MK_CW);
     } else {
-        // ------------------------------------------------------------ consumers
-        uint32_t it = 0;
+        constexpr bool TC = M >= MK_TC_ROWS;
+        MkPos<mk_slots(M)> at{0, 0u};
         unsigned long long epoch = a.bar_base;
         if (blockIdx.x == 0 && threadIdx.x == 0 && a.trace) a.trace[0] = global_ns();
         bool ok = true;
-        const int qd = a.Hq * a.hd;
+        MkGains gains;
+        gains.load(a.layers[a.layer_begin].attn_gain, a.d);
         for (int l = a.layer_begin; l < a.layer_end && ok; l++) {
-            const MkLayer *L = a.layers + l;
-            // q/k/v
-            if (!(ok = mk_proj<M>(MK_QKV, a, L, area, a.d, a.h, nullptr, L->attn_gain, ring, &sh, it))) break;
-            if (!(ok = mk_grid_barrier(a, &sh, epoch))) break;
-            // attention and the merge of its splits
-            mk_attention<HD>(a, L, area, &sh);
-            if (!(ok = mk_grid_barrier(a, &sh, epoch))) break;
-            mk_merge<HD, M >= MK_TC_ROWS>(a, &sh);
-            if (!(ok = mk_grid_barrier(a, &sh, epoch))) break;
-            // O-projection
-            if (!(ok = mk_proj<M>(MK_OPROJ, a, L, area, qd, nullptr, a.attn_o, nullptr, ring, &sh, it))) break;
-            if (!(ok = mk_grid_barrier(a, &sh, epoch))) break;
-            // MLP
-            if (!(ok = mk_proj<M>(MK_GATEUP, a, L, area, a.d, a.h, nullptr, L->mlp_gain, ring, &sh, it))) break;
-            if (!(ok = mk_grid_barrier(a, &sh, epoch))) break;
-            if (!(ok = mk_proj<M>(MK_DOWN, a, L, area, a.F, nullptr, a.act, nullptr, ring, &sh, it))) break;
-            if (!(ok = mk_grid_barrier(a, &sh, epoch))) break;
+            const bf16 *gain = a.layers[l].attn_gain;
+            if constexpr (TC) {
+                const int whole = (a.d + MK_BOX_COLS - 1) / MK_BOX_COLS * MK_BOX_COLS;
+                mk_rows_tc<M>(MK_QKV, a, l, reinterpret_cast<bf16 *>(area), reinterpret_cast<float *>(area + mk_tc_planes_bytes(M, whole)),
+                              a.h2, gain, gains, nullptr, 0, ring, sh, at);
+            } else {
+                mk_rows<M>(MK_QKV, a, l, reinterpret_cast<float *>(area), reinterpret_cast<float *>(area + mk_area_bytes(M) - mk_sums_bytes(M)),
+                           mk_sums_bytes(M), a.h2, gain, gains, nullptr, 0, ring, sh, at);
+            }
+            if (!(ok = mk_grid_barrier(a, sh, epoch))) break;
+            if (warp == MK_CW - 1) mk_fold(a, lane, 32);
+            mk_attention<M, HD>(a, l, area, ring, sh, at);
+            if (!(ok = mk_grid_barrier(a, sh, epoch))) break;
+            mk_oproj<M, HD>(a, area, ring, sh, at);
+            gains.load(a.layers[l].mlp_gain, a.d);
+            if (!(ok = mk_grid_barrier(a, sh, epoch))) break;
+            mk_mlp<M>(a, l, area, ring, sh, gains, at);
+            if (l + 1 < a.layer_end) gains.load(a.layers[l + 1].attn_gain, a.d);
+            ok = mk_grid_barrier(a, sh, epoch);
         }
-        if (!ok && threadIdx.x == 0) sh.giving_up = 1;
+        if (ok) mk_fold(a, (int)threadIdx.x, MK_CW * 32);
     }
     __syncthreads();
 }

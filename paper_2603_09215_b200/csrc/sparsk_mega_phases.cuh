@@ -1,4 +1,4 @@
-// Phases of the persistent layer-range kernel (see sparsk_mega.cuh) and the kernel itself.
+// Projection phases of the persistent layer-range kernel (see sparsk_mega.cuh).
 #pragma once
 
 namespace sparsk {
@@ -15,238 +15,43 @@ __device__ __forceinline__ int mk_act_slot(int i)
     return (i - ci) + ((ci >> 2) & 1) * (MK_BOX_COLS / 2) + (ci >> 3) * 4;
 }
 
-// Columns [c0, c0 + ncols) of the M activation rows, as fp32, row m at act + m * ncols (in the
-// layout of mk_act_slot).  With h:
-// x = h / sqrt(mean(h^2) + eps) * gain; otherwise a copy of the fp32 rows x.  Columns at or
-// beyond K are zeros (the last weight box is zero-filled there too).  ncols is a multiple of 256.
-template <int M>
-__device__ __forceinline__ void mk_load_act(float *act, int c0, int ncols, int K, const float *h, const float *x,
-                                            const bf16 *gain, float eps, MkShared *sh)
+// Four numbers of the residual stream from element i on: h, or h + h2 where the down-projection's sums have
+// not been folded into h yet.
+__device__ __forceinline__ float4 mk_resid(const float *h, const float *h2, size_t i)
 {
+    float4 v = *reinterpret_cast<const float4 *>(h + i);
+    if (h2) {
+        const float4 w = *reinterpret_cast<const float4 *>(h2 + i);
+        v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
+    }
+    return v;
+}
+
+// The gains a thread needs for the columns it keeps in registers in mk_norm.  They are cold (every layer's are read once a
+// launch), so they are asked for while the CTA waits for the grid barrier before the norm.
+constexpr int MK_KEEP = 2;
+struct MkGains {
+    uint2 g[MK_KEEP];
+    __device__ __forceinline__ void load(const bf16 *gain, int K)
+    {
+#pragma unroll
+        for (int k = 0; k < MK_KEEP; k++) {
+            const int i = ((int)threadIdx.x + k * MK_CW * 32) * 4;
+            g[k] = i < K ? *reinterpret_cast<const uint2 *>(gain + i) : make_uint2(0u, 0u);
+        }
+    }
+};
+
+// x = (h + h2) / sqrt(mean((h + h2)^2) + eps) * gain for the M rows, left through put(row, column, four numbers); columns at
+// or beyond K, up to ncols, and rows from n_rows on are zeros.  Rows of up to MK_KEEP float4s per thread stay in
+// registers between the sum of squares and the scaling: one trip to the L2.
+template <int M, class Put>
+__device__ __forceinline__ void mk_norm(int ncols, int K, int n_rows, const float *h, const float *h2, const bf16 *gain,
+                                        const MkGains &gains, float eps, MkShared *sh, const Put &put)
+{
+    constexpr int T = MK_CW * 32, KEEP = MK_KEEP;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int T = MK_CW * 32;
-    mk_consumer_sync();  // everyone is done with what the area held
-#pragma unroll
-    for (int m = 0; m < M; m++) {
-        float *dst = act + (size_t)m * ncols;
-        if (h) {
-            const float *src = h + (size_t)m * K;
-            // a row that is loaded whole is parked in the area on its way through the sum of
-            // squares and scaled in place afterwards: one trip to the L2 instead of two
-            const bool whole = c0 == 0 && ncols >= K;
-            float ss = 0.f;
-            for (int i = tid * 4; i < (whole ? ncols : K); i += T * 4) {
-                const float4 v = i < K ? *reinterpret_cast<const float4 *>(src + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-                ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-                if (whole) *reinterpret_cast<float4 *>(dst + mk_act_slot(i)) = v;
-            }
-            ss = warp_sum(ss);
-            if (lane == 0) sh->red[warp] = ss;
-            mk_consumer_sync();
-            float tot = 0.f;
-#pragma unroll
-            for (int w = 0; w < MK_CW; w++) tot += sh->red[w];
-            mk_consumer_sync();
-            const float inv = rsqrtf(tot / (float)K + eps);
-            if (whole) {
-                for (int i = tid * 4; i < K; i += T * 4) {   // the thread's own float4s again
-                    float4 *q = reinterpret_cast<float4 *>(dst + mk_act_slot(i));
-                    const float4 p = *q;
-                    const uint2 g2 = *reinterpret_cast<const uint2 *>(gain + i);
-                    *q = make_float4(p.x * inv * bf_lo(g2.x), p.y * inv * bf_hi(g2.x), p.z * inv * bf_lo(g2.y),
-                                     p.w * inv * bf_hi(g2.y));
-                }
-            } else {
-                for (int i = tid * 4; i < ncols; i += T * 4) {
-                    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-                    const int k = c0 + i;
-                    if (k < K) {
-                        const float4 p = *reinterpret_cast<const float4 *>(src + k);
-                        const uint2 g2 = *reinterpret_cast<const uint2 *>(gain + k);
-                        o = make_float4(p.x * inv * bf_lo(g2.x), p.y * inv * bf_hi(g2.x), p.z * inv * bf_lo(g2.y),
-                                        p.w * inv * bf_hi(g2.y));
-                    }
-                    *reinterpret_cast<float4 *>(dst + mk_act_slot(i)) = o;
-                }
-            }
-        } else {
-            const float *src = x + (size_t)m * K;
-            for (int i = tid * 4; i < ncols; i += T * 4)
-                *reinterpret_cast<float4 *>(dst + mk_act_slot(i)) =
-                    c0 + i < K ? *reinterpret_cast<const float4 *>(src + c0 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    }
-    mk_consumer_sync();
-}
-
-// Column k of activation row m as two bf16 terms, in a buffer that is [n_rows hi][n_rows lo][K].
-__device__ __forceinline__ void mk_put_planes(float *buf, int K, int n_rows, int m, int k, float x)
-{
-    bf16 *p = reinterpret_cast<bf16 *>(buf);
-    const bf16 hi = __float2bfloat16(x);
-    p[(size_t)m * K + k] = hi;
-    p[(size_t)(n_rows + m) * K + k] = __float2bfloat16(x - __bfloat162float(hi));
-}
-
-// ------------------------------------------------------------------ what a finished pair of sums becomes
-// v0 = row `rib` of band b's first box, v1 = the same row of its second box (a rotary pair, a
-// gate/up pair, or two plain rows), for activation row m.  PLANES: what the next phase reads as
-// activations is left as the two bf16 planes of the tensor-core form ([hi rows][lo rows][K]).
-template <bool PLANES>
-__device__ __forceinline__ void mk_finish(int type, const MkArgs &a, const MkLayer *L, const MkShared *sh, int b, int rib,
-                                          int m, float v0, float v1)
-{
-    const int half = a.hd >> 1, per_head = half / MK_BOX_ROWS;
-    switch (type) {
-    case MK_QKV: {
-        const int nq = a.Hq * per_head, nk = a.Hkv * per_head;
-        const int slot_id = sh->row_slot[m], pos = sh->row_pos[m];
-        if (b < nq + nk) {
-            const bool isq = b < nq;
-            const int bb = isq ? b : b - nq;
-            const int head = bb / per_head, i = (bb % per_head) * MK_BOX_ROWS + rib;
-            const float2 cs = a.rope[(size_t)pos * half + i];
-            const float ra = v0 * cs.x - v1 * cs.y, rb = v1 * cs.x + v0 * cs.y;
-            if (isq) {
-                float *dst = a.q_buf + (size_t)m * a.Hq * a.hd + head * a.hd + i;
-                dst[0] = ra;
-                dst[half] = rb;
-            } else {
-                kv_t *dst = L->kc + (((size_t)slot_id * a.Hkv + head) * a.S + pos) * a.hd + i;
-                dst[0] = to_kv(ra);
-                dst[half] = to_kv(rb);
-            }
-        } else {
-            const int n0 = (b - nq - nk) * 2 * MK_BOX_ROWS + rib, n1 = n0 + MK_BOX_ROWS;
-            const int kvd = a.Hkv * a.hd;
-            if (n0 < kvd) L->vc[(((size_t)slot_id * a.Hkv + n0 / a.hd) * a.S + pos) * a.hd + n0 % a.hd] = to_kv(v0);
-            if (n1 < kvd) L->vc[(((size_t)slot_id * a.Hkv + n1 / a.hd) * a.S + pos) * a.hd + n1 % a.hd] = to_kv(v1);
-        }
-        break;
-    }
-    case MK_GATEUP: {
-        const int f = b * MK_BOX_ROWS + rib;
-        if (f < a.F) {
-            const float u = v0 / (1.f + __expf(-v0)) * v1;
-            if (PLANES) mk_put_planes(a.act, a.F, a.n_rows, m, f, u);
-            else a.act[(size_t)m * a.F + f] = u;
-        }
-        break;
-    }
-    default: {
-        const int n0 = b * 2 * MK_BOX_ROWS + rib, n1 = n0 + MK_BOX_ROWS;
-        // shares of a band held by different CTAs meet in the residual stream
-        if (n0 < a.d) atomicAdd(a.h + (size_t)m * a.d + n0, v0);
-        if (n1 < a.d) atomicAdd(a.h + (size_t)m * a.d + n1, v1);
-    }
-    }
-}
-
-// ------------------------------------------------------------------ projection phase (consumers)
-// The activations of the phase come from `h` (normalised with `gain`) or from the fp32 rows `x`,
-// K columns each.  If M rows of the whole inner dimension fit the area they are loaded once;
-// otherwise the area holds a window of k-steps that follows the CTA's segments.
-template <int M>
-__device__ __forceinline__ bool mk_project(int type, const MkArgs &a, const MkLayer *L, float *act, int K,
-                                           const float *h, const float *x, const bf16 *gain, unsigned char *ring,
-                                           MkShared *sh, uint32_t &it)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    MkWalk walk;
-    walk.init(type, a);
-    const int window = mk_act_window(M);
-    const bool whole = walk.k_steps <= window;
-    int win0 = 0, win1 = 0;  // k-steps the area holds: [win0, win1)
-    if (whole) {
-        win1 = walk.k_steps;
-        mk_load_act<M>(act, 0, win1 * MK_BOX_COLS, K, h, x, gain, a.eps, sh);
-    }
-    const int ncols = whole ? walk.k_steps * MK_BOX_COLS : window * MK_BOX_COLS;
-    MkSeg seg;
-    while (walk.next(seg)) {
-        const int b = seg.band;
-        float acc[2][M];
-#pragma unroll
-        for (int r = 0; r < 2; r++)
-#pragma unroll
-            for (int m = 0; m < M; m++) acc[r][m] = 0.f;
-        for (int ks = seg.ks0; ks < seg.ks1; ks++, it++) {
-            if (ks < win0 || ks >= win1) {  // uniform across the CTA: move the window
-                win0 = ks;
-                win1 = min(walk.k_steps, ks + window);
-                mk_load_act<M>(act, win0 * MK_BOX_COLS, ncols, K, h, x, gain, a.eps, sh);
-            }
-            const int s = it % MK_SLOTS;
-            if (!mbar_wait(&sh->full[s], (it / MK_SLOTS) & 1, &sh->giving_up, a.status)) return false;
-            const unsigned char *slot = ring + (size_t)s * MK_SLOT_BYTES + (size_t)warp * MK_BOX_COLS * 2 + lane * 16;
-            float w0[8], w1[8];
-            unpack8(*reinterpret_cast<const uint4 *>(slot), w0);
-            unpack8(*reinterpret_cast<const uint4 *>(slot + MK_BOX_BYTES), w1);
-#pragma unroll
-            for (int m = 0; m < M; m++) {
-                const float *xp = act + (size_t)m * ncols + (ks - win0) * MK_BOX_COLS + lane * 4;
-                const float4 xa = *reinterpret_cast<const float4 *>(xp), xb = *reinterpret_cast<const float4 *>(xp + MK_BOX_COLS / 2);
-                const float xv[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
-#pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    acc[0][m] = fmaf(w0[j], xv[j], acc[0][m]);
-                    acc[1][m] = fmaf(w1[j], xv[j], acc[1][m]);
-                }
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sh->empty[s]);
-        }
-#pragma unroll
-        for (int r = 0; r < 2; r++)
-#pragma unroll
-            for (int m = 0; m < M; m++) acc[r][m] = warp_sum(acc[r][m]);
-        // lane m finishes activation row m
-        float v0 = acc[0][0], v1 = acc[1][0];
-#pragma unroll
-        for (int m = 1; m < M; m++)
-            if (lane == m) {
-                v0 = acc[0][m];
-                v1 = acc[1][m];
-            }
-        if (lane < M) mk_finish<false>(type, a, L, sh, b, warp, lane, v0, v1);
-    }
-    return true;
-}
-
-// ------------------------------------------------------------------ three and four rows: tensor-core form
-// With three or four activation rows the CUDA-core inner loop above is bound by shared-memory
-// reads (every warp reads all rows' activations for its two weight rows).  Here a slot's two
-// boxes arrive as four 64-column blocks each with the 128-byte swizzle, warp w takes box w / 8
-// and the 32-column slice w % 8 of it, and multiplies with mma.sync m16n8k16: A = 16 weight rows
-// x 16 columns (ldmatrix, conflict-free under the swizzle), B = 16 columns x 8 columns of which the
-// first M are the rows' hi terms and the next M their lo terms (two bf16 terms, 16 significant
-// bits, as on the tcgen05 path): one instruction for both, added at the end of a band, where
-// the eight slices of a box meet in shared memory.
-// The planes that the attention and the MLP leave for the next phase are copied as they are; the MLP's
-// do not fit whole, so they come in two half windows, one on its way while the other is read.
-// A layer of the 28-layer shape: 102.7 -> 99.0 us at three rows, 104.9 -> 99.0 at four (an instruction per
-// term, fp32 activations split on every load and blocking windows before).
-constexpr int MK_TC_RED_BYTES = 2 * 2 * 8 * 16 * 8 * 4;  // [parity][box][slice][16 rows][8 n] floats = 16 KB
-__host__ __device__ inline int mk_tc_window(int M)
-{
-    return (MK_AREA_BYTES - MK_TC_RED_BYTES - 2 * 2 * M * 16) / (M * MK_BOX_COLS * 2 * 2);
-}
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// The activation rows, normalised, as two bf16 planes of M rows (those beyond n_rows are zeros): hi at planes + m * rs, lo at planes + (M + m)
-// * rs, rs = ncols + 8 elements (the padding spreads the rows over the banks); columns at or
-// beyond K are zeros.  Rows of up to KEEP float4s per thread stay in registers between the sum of
-// squares and the scaling: one trip to the L2.
-template <int M>
-__device__ __forceinline__ void mk_norm_tc(bf16 *planes, int ncols, int K, int n_rows, const float *h, const bf16 *gain, float eps, MkShared *sh)
-{
-    constexpr int T = MK_CW * 32, KEEP = 2;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rs = ncols + 8;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 v[M][KEEP];
     float ss[M];
 #pragma unroll
@@ -254,7 +59,7 @@ __device__ __forceinline__ void mk_norm_tc(bf16 *planes, int ncols, int K, int n
 #pragma unroll
         for (int m = 0; m < M; m++) {
             const int i = (tid + k * T) * 4;
-            v[m][k] = i < K && m < n_rows ? *reinterpret_cast<const float4 *>(h + (size_t)m * K + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[m][k] = i < K && m < n_rows ? mk_resid(h, h2, (size_t)m * K + i) : zero;
         }
 #pragma unroll
     for (int m = 0; m < M; m++) {
@@ -266,7 +71,7 @@ __device__ __forceinline__ void mk_norm_tc(bf16 *planes, int ncols, int K, int n
 #pragma unroll
         for (int m = 0; m < M; m++) {
             if (m >= n_rows) break;
-            const float4 x = *reinterpret_cast<const float4 *>(h + (size_t)m * K + i);
+            const float4 x = mk_resid(h, h2, (size_t)m * K + i);
             ss[m] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
         }
 #pragma unroll
@@ -283,136 +88,394 @@ __device__ __forceinline__ void mk_norm_tc(bf16 *planes, int ncols, int K, int n
         for (int w = 0; w < MK_CW; w++) tot += sh->red_rows[m][w];
         inv[m] = rsqrtf(tot / (float)K + eps);
     }
-    auto put = [&](int m, int i, const float4 &x, const uint2 &g2) {
-        uint2 hi, lo;
-        split_pair(x.x * inv[m] * bf_lo(g2.x), x.y * inv[m] * bf_hi(g2.x), hi.x, lo.x);
-        split_pair(x.z * inv[m] * bf_lo(g2.y), x.w * inv[m] * bf_hi(g2.y), hi.y, lo.y);
-        *reinterpret_cast<uint2 *>(planes + (size_t)m * rs + i) = hi;
-        *reinterpret_cast<uint2 *>(planes + (size_t)(M + m) * rs + i) = lo;
+    auto scaled = [&](int m, const float4 &x, const uint2 &g) {
+        return make_float4(x.x * inv[m] * bf_lo(g.x), x.y * inv[m] * bf_hi(g.x), x.z * inv[m] * bf_lo(g.y), x.w * inv[m] * bf_hi(g.y));
     };
 #pragma unroll
     for (int k = 0; k < KEEP; k++) {
         const int i = (tid + k * T) * 4;
         if (i >= ncols) continue;
-        const uint2 g2 = i < K ? *reinterpret_cast<const uint2 *>(gain + i) : make_uint2(0u, 0u);
 #pragma unroll
-        for (int m = 0; m < M; m++) put(m, i, v[m][k], g2);
+        for (int m = 0; m < M; m++) put(m, i, scaled(m, v[m][k], gains.g[k]));
     }
     for (int i = (tid + KEEP * T) * 4; i < ncols; i += T * 4) {
-        const uint2 g2 = i < K ? *reinterpret_cast<const uint2 *>(gain + i) : make_uint2(0u, 0u);
+        const uint2 g = i < K ? *reinterpret_cast<const uint2 *>(gain + i) : make_uint2(0u, 0u);
 #pragma unroll
-        for (int m = 0; m < M; m++)
-            put(m, i, i < K && m < n_rows ? *reinterpret_cast<const float4 *>(h + (size_t)m * K + i) : make_float4(0.f, 0.f, 0.f, 0.f), g2);
+        for (int m = 0; m < M; m++) put(m, i, scaled(m, i < K && m < n_rows ? mk_resid(h, h2, (size_t)m * K + i) : zero, g));
     }
     mk_consumer_sync();
 }
-// Starts the copies of columns [c0, c0 + ncols) of the plane rows in global memory ([n_rows hi][n_rows
-// lo][K]; zeros beyond K, a multiple of 8) to planes of M rows with row stride rs.
+
+// Columns [c0, c0 + ncols) of M rows that do not fit the area whole, as fp32, row m at act + m * ncols (in the
+// layout of mk_act_slot); ncols is a multiple of 256.
 template <int M>
-__device__ __forceinline__ void mk_copy_planes(bf16 *planes, int rs, int c0, int ncols, int K, int n_rows, const float *x)
+__device__ __forceinline__ void mk_norm_window(float *act, int c0, int ncols, int K, const float *h, const float *h2,
+                                               const bf16 *gain, float eps, MkShared *sh)
 {
-    const bf16 *src = reinterpret_cast<const bf16 *>(x);
-    const int per_row = ncols / 8;
-    for (int idx = threadIdx.x; idx < 2 * M * per_row; idx += MK_CW * 32) {
-        const int r = idx / per_row, i = (idx - r * per_row) * 8, k = c0 + i;
-        const bool ok = k < K && r % M < n_rows;
-        const size_t from = (size_t)((r / M) * n_rows + r % M) * K + k;
-        cp_async16(planes + (size_t)r * rs + i, src + (ok ? from : 0), ok ? 16 : 0);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int T = MK_CW * 32;
+#pragma unroll
+    for (int m = 0; m < M; m++) {
+        const size_t row = (size_t)m * K;
+        float ss = 0.f;
+        for (int i = tid * 4; i < K; i += T * 4) {
+            const float4 v = mk_resid(h, h2, row + i);
+            ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+        }
+        ss = warp_sum(ss);
+        if (lane == 0) sh->red_rows[m][warp] = ss;
     }
-    cp_async_commit();
+    mk_consumer_sync();  // also: everyone is done with what the area held
+#pragma unroll
+    for (int m = 0; m < M; m++) {
+        const size_t row = (size_t)m * K;
+        float *dst = act + (size_t)m * ncols;
+        float tot = 0.f;
+#pragma unroll
+        for (int w = 0; w < MK_CW; w++) tot += sh->red_rows[m][w];
+        const float inv = rsqrtf(tot / (float)K + eps);
+        for (int i = tid * 4; i < ncols; i += T * 4) {
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int k = c0 + i;
+            if (k < K) {
+                const float4 p = mk_resid(h, h2, row + k);
+                const uint2 g2 = *reinterpret_cast<const uint2 *>(gain + k);
+                o = make_float4(p.x * inv * bf_lo(g2.x), p.y * inv * bf_hi(g2.x), p.z * inv * bf_lo(g2.y),
+                                p.w * inv * bf_hi(g2.y));
+            }
+            *reinterpret_cast<float4 *>(dst + mk_act_slot(i)) = o;
+        }
+    }
+    mk_consumer_sync();
 }
 
+// Two fp32 numbers in a register pair; a * b + c on both at once.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 mk_pair(float lo, float hi)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ f32x2 mk_fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ float mk_sum2(f32x2 a)
+{
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+    return lo + hi;
+}
+// eight bf16 weights as four pairs
+__device__ __forceinline__ void mk_unpack(const uint4 &w, f32x2 (&p)[4])
+{
+    p[0] = mk_pair(bf_lo(w.x), bf_hi(w.x));
+    p[1] = mk_pair(bf_lo(w.y), bf_hi(w.y));
+    p[2] = mk_pair(bf_lo(w.z), bf_hi(w.z));
+    p[3] = mk_pair(bf_lo(w.w), bf_hi(w.w));
+}
+
+// The sums over LANES neighbouring lanes of N <= LANES numbers each (powers of two).  After every step a lane holds
+// half as many sums, each of twice as many lanes; in the end sum k is v[0] of the LANES / N lanes from LANES / N * k on.
+template <int N, int LANES>
+__device__ __forceinline__ void mk_exchange(float (&v)[N], int lane)
+{
+    int off = LANES / 2;
+#pragma unroll
+    for (int n = N / 2; n > 0; n >>= 1, off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int k = 0; k < N / 2; k++) {
+            if (k >= n) break;
+            const float give = up ? v[k] : v[k + n], keep = up ? v[k + n] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+        }
+    }
+#pragma unroll
+    for (; off > 0; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+}
+
+// ------------------------------------------------------------------ what a finished pair of sums becomes
+// v0 = row `rib` of q/k/v band b's first box, v1 = the same row of its second box (a rotary pair or two
+// plain rows), for activation row m of layer l.
+__device__ __forceinline__ void mk_finish_qkv(const MkArgs &a, int l, const MkShared *sh, int b, int rib, int m, float v0, float v1)
+{
+    const int half = a.hd >> 1, per_head = half / MK_BOX_ROWS;
+    const int nq = a.Hq * per_head, nk = a.Hkv * per_head;
+    const int slot_id = sh->row_slot[m], pos = sh->row_pos[m];
+    if (b < nq + nk) {
+        const bool isq = b < nq;
+        const int bb = isq ? b : b - nq;
+        const int head = bb / per_head, i = (bb % per_head) * MK_BOX_ROWS + rib;
+        const float2 cs = sh->rope[m][i];
+        const float ra = v0 * cs.x - v1 * cs.y, rb = v1 * cs.x + v0 * cs.y;
+        if (isq) {
+            float *dst = a.q_buf + (size_t)m * a.Hq * a.hd + head * a.hd + i;
+            dst[0] = ra;
+            dst[half] = rb;
+        } else {
+            kv_t *dst = a.kc + l * a.kv_layer + (((size_t)slot_id * a.Hkv + head) * a.S + pos) * a.hd + i;
+            dst[0] = to_kv(ra);
+            dst[half] = to_kv(rb);
+        }
+    } else {
+        const int n0 = (b - nq - nk) * 2 * MK_BOX_ROWS + rib, n1 = n0 + MK_BOX_ROWS;
+        const int kvd = a.Hkv * a.hd;
+        kv_t *vc = a.vc + l * a.kv_layer;
+        if (n0 < kvd) vc[(((size_t)slot_id * a.Hkv + n0 / a.hd) * a.S + pos) * a.hd + n0 % a.hd] = to_kv(v0);
+        if (n1 < kvd) vc[(((size_t)slot_id * a.Hkv + n1 / a.hd) * a.S + pos) * a.hd + n1 % a.hd] = to_kv(v1);
+    }
+}
+__device__ __forceinline__ float mk_silu_mul(float gate, float up) { return gate / (1.f + __expf(-gate)) * up; }
+
+// ------------------------------------------------------------------ one and two rows
+// Waits for a slot and takes eight 16-byte units per lane out of it: `stride` bytes apart, the second four from `second` on.  The
+// slot is free for its next fill before its products are formed.  False: the wait ran out.
+template <int SLOTS>
+__device__ __forceinline__ bool mk_take(uint4 (&w)[8], const unsigned char *ring, MkShared *sh, const MkPos<SLOTS> &p, int off, int stride,
+                                        int second, int *status)
+{
+    if (!mbar_wait(&sh->full[p.s], p.ph, &sh->giving_up, status)) return false;
+    const unsigned char *src = ring + (size_t)p.s * MK_SLOT_BYTES + off;
+#pragma unroll
+    for (int r = 0; r < 8; r++) w[r] = *reinterpret_cast<const uint4 *>(src + (r >= 4 ? second : 0) + (r & 3) * stride);
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive_n(&sh->empty[p.s], MK_CW / MK_GROUPS);
+    return true;
+}
+
+// Row form.  A slot s is the work of the four warps of group s mod 4, four rows of both boxes each; the groups' sums of a row
+// meet in shared memory once per eight bands.  (All sixteen warps on every slot, a row of both boxes each, took
+// 0.35 us a slot from a full ring, as long as HBM takes to fill it; in groups 0.2: a warp spends some ten cycles an
+// instruction, and waiting, releasing and reading the activations cost as much as the products.)
+// If M rows of the whole inner dimension fit the area they are loaded once; otherwise the area
+// holds a window of k-steps that is reloaded as the phase moves along.  gate/up leaves its results in u: column
+// (band - first band) * 16 + row of the box, of activation row m at u + m * u_stride.
+constexpr int MK_BATCH = 8;  // bands whose sums wait in shared memory
+__host__ __device__ constexpr int mk_sums_bytes(int M) { return MK_BATCH * 2 * MK_BOX_ROWS * M * MK_GROUPS * 4; }
+
 template <int M>
-__device__ __forceinline__ bool mk_project_tc(int type, const MkArgs &a, const MkLayer *L, unsigned char *area, int K,
-                                              const float *h, const float *x, const bf16 *gain, unsigned char *ring,
-                                              MkShared *sh, uint32_t &it)
+__device__ __forceinline__ void mk_rows(int type, const MkArgs &a, int l, float *act, float *sums, int own, const float *h2,
+                                        const bf16 *gain, const MkGains &gains, float *u, int u_stride, unsigned char *ring,
+                                        MkShared *sh, MkPos<mk_slots(M)> &at)
+{
+    constexpr int ROWS = MK_BOX_ROWS / (MK_CW / MK_GROUPS), N = 2 * ROWS * M;  // rows of a box per warp; sums per warp
+    static_assert(ROWS == 4, "mk_take");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / MK_GROUPS, sub = warp % MK_GROUPS;
+    MkBands w;
+    w.init(type, a);
+    if (w.j >= w.end) return;
+    const int first = w.j, n_bands = (w.end - w.j + w.step - 1) / w.step, room = mk_act_window(M, own);
+    const bool whole = w.k_steps <= room;
+    const int window = whole ? w.k_steps : room, ncols = window * MK_BOX_COLS;
+    bool live = true;        // false: a wait ran out, this warp only keeps the barriers whole
+    if (whole)
+        mk_norm<M>(ncols, a.d, a.n_rows, a.h, h2, gain, gains, a.eps, sh,
+                   [&](int m, int i, const float4 &x) { *reinterpret_cast<float4 *>(act + (size_t)m * ncols + mk_act_slot(i)) = x; });
+    for (int b0 = 0; b0 < n_bands; b0 += MK_BATCH) {
+        const int nb = min(MK_BATCH, n_bands - b0);
+        for (int b = 0; b < nb; b++) {
+            f32x2 acc[2 * ROWS][M];
+#pragma unroll
+            for (int r = 0; r < 2 * ROWS; r++)
+#pragma unroll
+                for (int m = 0; m < M; m++) acc[r][m] = 0ull;
+            for (int win0 = 0; win0 < w.k_steps; win0 += window) {
+                const int n = min(window, w.k_steps - win0);
+                if (!whole) mk_norm_window<M>(act, win0 * MK_BOX_COLS, ncols, a.d, a.h, h2, gain, a.eps, sh);
+                const int ahead = (grp - at.s) & (MK_GROUPS - 1);
+                MkPos<mk_slots(M)> p = at;
+                p.skip(ahead);
+                for (int k = ahead; k < n && live; k += MK_GROUPS, p.skip(MK_GROUPS)) {
+                    uint4 wt[2 * ROWS];
+                    if (!(live = mk_take(wt, ring, sh, p, sub * ROWS * MK_BOX_COLS * 2 + lane * 16, MK_BOX_COLS * 2, MK_BOX_BYTES, a.status))) break;
+                    f32x2 xv[M][4];
+#pragma unroll
+                    for (int m = 0; m < M; m++) {
+                        const float *xp = act + (size_t)m * ncols + k * MK_BOX_COLS + lane * 4;
+                        const ulonglong2 xa = *reinterpret_cast<const ulonglong2 *>(xp), xb = *reinterpret_cast<const ulonglong2 *>(xp + MK_BOX_COLS / 2);
+                        xv[m][0] = xa.x; xv[m][1] = xa.y; xv[m][2] = xb.x; xv[m][3] = xb.y;
+                    }
+#pragma unroll
+                    for (int r = 0; r < 2 * ROWS; r++) {
+                        f32x2 wp[4];
+                        mk_unpack(wt[r], wp);
+#pragma unroll
+                        for (int m = 0; m < M; m++)
+#pragma unroll
+                            for (int j = 0; j < 4; j++) acc[r][m] = mk_fma2(wp[j], xv[m][j], acc[r][m]);
+                    }
+                }
+                at.skip_many(n);
+            }
+            float v[N];
+#pragma unroll
+            for (int r = 0; r < 2 * ROWS; r++)
+#pragma unroll
+                for (int m = 0; m < M; m++) v[r * M + m] = mk_sum2(acc[r][m]);
+            mk_exchange<N, 32>(v, lane);
+            // sum k of N sits in the 32 / N lanes from 32 / N k on
+            const int k = lane / (32 / N), r = k / M, m = k % M;
+            if (lane % (32 / N) == 0)
+                sums[((b * 2 * MK_BOX_ROWS + (r / ROWS) * MK_BOX_ROWS + sub * ROWS + r % ROWS) * M + m) * MK_GROUPS + grp] = v[0];
+        }
+        mk_consumer_sync();
+        for (int i = threadIdx.x; i < nb * MK_BOX_ROWS * M; i += MK_CW * 32) {
+            const int m = i % M, rib = i / M % MK_BOX_ROWS, b = i / M / MK_BOX_ROWS;
+            const float4 s0 = reinterpret_cast<const float4 *>(sums)[(b * 2 * MK_BOX_ROWS + rib) * M + m];
+            const float4 s1 = reinterpret_cast<const float4 *>(sums)[(b * 2 * MK_BOX_ROWS + MK_BOX_ROWS + rib) * M + m];
+            const float v0 = (s0.x + s0.y) + (s0.z + s0.w), v1 = (s1.x + s1.y) + (s1.z + s1.w);
+            if (type == MK_QKV) mk_finish_qkv(a, l, sh, first + (b0 + b) * w.step, rib, m, v0, v1);
+            else u[m * u_stride + (b0 + b) * MK_BOX_ROWS + rib] = mk_silu_mul(v0, v1);
+        }
+        if (b0 + MK_BATCH < n_bands) mk_consumer_sync();
+    }
+}
+
+// Column form.
+// Boxes [r0, r1) of 64 weight rows x `cols` columns, the first of them at ring place `at`: dst[m][row] += W[row][its
+// columns] . x_m, x_m (cols numbers) at x + m * x_stride in shared memory.  A slot s is the work of the four
+// warps of group s mod 4, sixteen rows each.  LPR lanes share a row, eight columns each, whose activations they hold
+// in registers: the products of a box need nothing but the weights from shared memory, and the sums of
+// sixteen rows meet in 8 (one row of activations) or 15 (two) shuffles.
+template <int M, int LPR>
+__device__ __forceinline__ void mk_columns(const MkArgs &a, float *dst, int r0, int r1, int cols, const float *x, int x_stride,
+                                           unsigned char *ring, MkShared *sh, MkPos<mk_slots(M)> at)
+{
+    constexpr int RPL = 32 / LPR, NL = 16 / RPL;  // rows per load, loads per box
+    static_assert(NL <= 8, "mk_take");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / MK_GROUPS, sub = warp % MK_GROUPS;
+    const int li = lane & (LPR - 1), row_in = lane / LPR;
+    const bool on = li * 8 < cols;
+    f32x2 xv[M][4];
+#pragma unroll
+    for (int m = 0; m < M; m++) {
+        const ulonglong2 z = make_ulonglong2(0ull, 0ull);
+        const ulonglong2 xa = on ? *reinterpret_cast<const ulonglong2 *>(x + m * x_stride + li * 8) : z;
+        const ulonglong2 xb = on ? *reinterpret_cast<const ulonglong2 *>(x + m * x_stride + li * 8 + 4) : z;
+        xv[m][0] = xa.x; xv[m][1] = xa.y; xv[m][2] = xb.x; xv[m][3] = xb.y;
+    }
+    // (lanes without columns read their row's first ones, and drop them)
+    const int ahead = (grp - at.s) & (MK_GROUPS - 1), stride = RPL * cols * 2, off = (sub * 16 + row_in) * cols * 2 + (on ? li * 16 : 0);
+    at.skip(ahead);
+    for (int r = r0 + ahead; r < r1; r += MK_GROUPS, at.skip(MK_GROUPS)) {
+        uint4 wt[8];
+        if (!mk_take(wt, ring, sh, at, off, stride, NL > 4 ? 4 * stride : 0, a.status)) return;
+        float v[NL * M];
+#pragma unroll
+        for (int i = 0; i < NL; i++) {
+            f32x2 w[4];
+            mk_unpack(on ? wt[i] : make_uint4(0u, 0u, 0u, 0u), w);
+#pragma unroll
+            for (int m = 0; m < M; m++) {
+                f32x2 t = mk_fma2(w[0], xv[m][0], 0ull);
+#pragma unroll
+                for (int j = 1; j < 4; j++) t = mk_fma2(w[j], xv[m][j], t);
+                v[i * M + m] = mk_sum2(t);
+            }
+        }
+        // NL * M = LPR / 2 * M sums over LPR lanes: one each with two activation rows, one per pair of lanes with one
+        mk_exchange<NL * M, LPR>(v, lane);
+        const int m = M == 1 ? 0 : li & 1, row = r * MK_CBOX_ROWS + sub * 16 + (li >> 1) * RPL + row_in;
+        if ((M == 2 || !(li & 1)) && row < a.d) atomicAdd(dst + (size_t)m * a.d + row, v[0]);
+    }
+}
+
+// ------------------------------------------------------------------ three and four rows: tensor-core form
+// The same two forms with mma.sync m16n8k16: A = 16 weight rows x 16 columns (ldmatrix, conflict-free under the
+// copies' swizzle), B = 16 columns x 8 columns of which the first M are the rows' hi terms and the next M their lo
+// terms (two bf16 terms, 16 significant bits, as on the tcgen05 path): one instruction for both, added at
+// the end.  In the row form a warp of a slot's four takes one box and half of its columns, and the eight shares of a
+// box (four groups, two halves) meet in shared memory at the end of a band.
+constexpr int MK_TC_RED_BYTES = 2 * 2 * 8 * 16 * 8 * 4;  // [parity][box][share][16 rows][8 n] floats = 16 KB
+// The area with three and four rows: planes of d columns, the band sums, planes of the CTA's own `most` columns.
+__host__ __device__ inline size_t mk_tc_planes_bytes(int M, int cols) { return (size_t)2 * M * (cols + 8) * 2; }
+inline bool mk_tc_fits(int M, int d, int most)
+{
+    const int whole = (d + MK_BOX_COLS - 1) / MK_BOX_COLS * MK_BOX_COLS;
+    return mk_tc_planes_bytes(M, whole) + MK_TC_RED_BYTES + mk_tc_planes_bytes(M, most) <= (size_t)mk_area_bytes(M);
+}
+__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Column c of activation row m as two bf16 terms, in planes of M rows: hi rows, then lo rows.
+template <int M>
+__device__ __forceinline__ void mk_put_planes(bf16 *planes, int rs, int m, int c, float x)
+{
+    const bf16 hi = __float2bfloat16(x);
+    planes[(size_t)m * rs + c] = hi;
+    planes[(size_t)(M + m) * rs + c] = __float2bfloat16(x - __bfloat162float(hi));
+}
+__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
+// Row form.  gate/up leaves its results as planes of their own, u_planes, row stride u_rs.
+template <int M>
+__device__ __forceinline__ void mk_rows_tc(int type, const MkArgs &a, int l, bf16 *planes, float *red, const float *h2,
+                                           const bf16 *gain, const MkGains &gains, bf16 *u_planes, int u_rs, unsigned char *ring,
+                                           MkShared *sh, MkPos<mk_slots(M)> &at)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
-    const int box = warp >> 3, slice = warp & 7;
-    bf16 *planes = reinterpret_cast<bf16 *>(area);
-    float *red = reinterpret_cast<float *>(area + MK_AREA_BYTES - MK_TC_RED_BYTES);
-    MkWalk walk;
-    walk.init(type, a);
-    // The activations of a whole phase at once, or pieces of at most `win` k-steps of `x` that follow the
-    // CTA's segments through two buffers.  Phases that start from `h` always get the whole row (the
-    // host sends wider residual rows elsewhere: mk_tc_ok).
-    const bool whole = walk.k_steps <= mk_tc_window(M);
-    const int win = whole ? walk.k_steps : mk_tc_window(M) / 2;
-    const int ncols = win * MK_BOX_COLS, rs = ncols + 8;
-    bf16 *const buf[2] = {planes, planes + (whole ? 0 : 2 * M * rs)};
-    MkWalk ahead = walk;  // the piece to copy next
-    MkSeg aseg;
-    bool a_more = !whole && ahead.next(aseg);
-    int a_ks = a_more ? aseg.ks0 : 0;
-    uint32_t issued = 0, piece = 0;
-    auto copy_next = [&]() {
-        if (!a_more) {
-            cp_async_commit();  // (keeps one group per piece)
-            return;
-        }
-        const int n = min(win, aseg.ks1 - a_ks);
-        mk_copy_planes<M>(buf[issued & 1], rs, a_ks * MK_BOX_COLS, n * MK_BOX_COLS, K, a.n_rows, x);
-        issued++;
-        if ((a_ks += n) == aseg.ks1 && (a_more = ahead.next(aseg))) a_ks = aseg.ks0;
-    };
-    if (h) {
-        mk_norm_tc<M>(planes, ncols, K, a.n_rows, h, gain, a.eps, sh);
-    } else if (whole) {
-        mk_consumer_sync();  // everyone is done with what the area held
-        mk_copy_planes<M>(planes, rs, 0, ncols, K, a.n_rows, x);
-        cp_async_wait<0>();
-        mk_consumer_sync();
-    } else {
-        mk_consumer_sync();
-        copy_next();
-        copy_next();
-    }
+    const int grp = warp / MK_GROUPS, box = (warp >> 1) & 1, half = warp & 1;
+    MkBands w;
+    w.init(type, a);
+    if (w.j >= w.end) return;
+    // row stride: the padding spreads the rows over the banks
+    const int first = w.j, ncols = w.k_steps * MK_BOX_COLS, rs = ncols + 8;
+    mk_norm<M>(ncols, a.d, a.n_rows, a.h, h2, gain, gains, a.eps, sh, [&](int m, int i, const float4 &x) {
+        uint2 hi, lo;
+        split_pair(x.x, x.y, hi.x, lo.x);
+        split_pair(x.z, x.w, hi.y, lo.y);
+        *reinterpret_cast<uint2 *>(planes + (size_t)m * rs + i) = hi;
+        *reinterpret_cast<uint2 *>(planes + (size_t)(M + m) * rs + i) = lo;
+    });
     // this lane's row address inside a 64-column block for ldmatrix: matrices (rows 0-7, k 0-7),
     // (rows 8-15, k 0-7), (rows 0-7, k 8-15), (rows 8-15, k 8-15)
     const int lrow = (lane & 7) + ((lane >> 3) & 1) * 8, lchk = lane >> 4;
-    const uint32_t a_off = (uint32_t)box * MK_BOX_BYTES + (uint32_t)(slice >> 1) * (MK_BOX_ROWS * 128) + (uint32_t)lrow * 128;
-    MkSeg seg;
+    const uint32_t a_off = (uint32_t)box * MK_BOX_BYTES + (uint32_t)half * (2 * MK_BOX_ROWS * 128) + (uint32_t)lrow * 128;
+    const bf16 *act = planes + (size_t)g * rs + half * 128 + 2 * t;
+    static_assert(2 * M == 8, "a plane row per column of the B operand");
     uint32_t band_it = 0;
-    while (walk.next(seg)) {
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int p0 = seg.ks0; p0 < seg.ks1; piece++) {
-            const int p1 = whole ? seg.ks1 : min(seg.ks1, p0 + win), base = whole ? 0 : p0;
-            if (!whole) {
-                cp_async_wait<1>();  // this piece has landed; the next may be on its way
-                mk_consumer_sync();
-            }
-            const bf16 *act = buf[whole ? 0 : piece & 1] + (size_t)g * rs + slice * 32 + 2 * t;
-            for (int ks = p0; ks < p1; ks++, it++) {
-                const int s = it % MK_SLOTS;
-                if (!mbar_wait(&sh->full[s], (it / MK_SLOTS) & 1, &sh->giving_up, a.status)) return false;
-                const uint32_t slot = smem_u32(ring) + (uint32_t)s * MK_SLOT_BYTES + a_off;
-                const bf16 *bp = act + (ks - base) * MK_BOX_COLS;
+    bool live = true;        // false: a wait ran out, this warp only keeps the barriers whole
+    for (; w.j < w.end; w.j += w.step) {
+        float acc[4] = {0.f, 0.f, 0.f, 0.f}, acc2[4] = {0.f, 0.f, 0.f, 0.f};
+        const int ahead = (grp - at.s) & (MK_GROUPS - 1);
+        MkPos<mk_slots(M)> p = at;
+        p.skip(ahead);
+        for (int ks = ahead; ks < w.k_steps && live; ks += MK_GROUPS, p.skip(MK_GROUPS)) {
+            if (!(live = mbar_wait(&sh->full[p.s], p.ph, &sh->giving_up, a.status))) break;
+            const uint32_t slot = smem_u32(ring) + (uint32_t)p.s * MK_SLOT_BYTES + a_off;
+            const bf16 *bp = act + ks * MK_BOX_COLS;
+            uint32_t af[8][4];
 #pragma unroll
-                for (int j = 0; j < 2; j++) {
-                    uint32_t af[4];
-                    const uint32_t chunk = (uint32_t)((slice & 1) * 4 + j * 2 + lchk);
-                    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                                 : "=r"(af[0]), "=r"(af[1]), "=r"(af[2]), "=r"(af[3])
-                                 : "r"(slot + ((chunk ^ (uint32_t)(lrow & 7)) << 4)));
-                    uint32_t b0 = 0, b1 = 0;
-                    if (g < 2 * M) {
-                        b0 = *reinterpret_cast<const uint32_t *>(bp + j * 16);
-                        b1 = *reinterpret_cast<const uint32_t *>(bp + j * 16 + 8);
-                    }
-                    mma_bf16_16816(acc, af, b0, b1);
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&sh->empty[s]);
+            for (int j = 0; j < 8; j++)
+                ldsm_x4(af[j], slot + (uint32_t)(j >> 2) * (MK_BOX_ROWS * 128) + (((uint32_t)((j & 3) * 2 + lchk) ^ (uint32_t)(lrow & 7)) << 4));
+            __syncwarp();
+            if (lane == 0) mbar_arrive_n(&sh->empty[p.s], MK_CW / MK_GROUPS);
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+                const uint32_t b0 = *reinterpret_cast<const uint32_t *>(bp + j * 16), b1 = *reinterpret_cast<const uint32_t *>(bp + j * 16 + 8);
+                if (j & 1) mma_bf16_16816(acc2, af[j], b0, b1);
+                else mma_bf16_16816(acc, af[j], b0, b1);
             }
-            if (!whole) {
-                mk_consumer_sync();  // everyone is done with this buffer
-                copy_next();
-            }
-            p0 = p1;
         }
-        // the eight slices of each box meet: [parity][box][slice][16 rows][8 n]
-        float *mine = red + ((((band_it & 1) * 2 + box) * 8 + slice) * 16) * 8;
+        at.skip_many(w.k_steps);
+#pragma unroll
+        for (int e = 0; e < 4; e++) acc[e] += acc2[e];
+        // the eight shares of each box meet: [parity][box][share][16 rows][8 n]
+        float *mine = red + ((((band_it & 1) * 2 + box) * 8 + grp * 2 + half) * 16) * 8;
         *reinterpret_cast<float2 *>(mine + g * 8 + 2 * t) = make_float2(acc[0], acc[1]);
         *reinterpret_cast<float2 *>(mine + (g + 8) * 8 + 2 * t) = make_float2(acc[2], acc[3]);
         mk_consumer_sync();
@@ -426,22 +489,68 @@ __device__ __forceinline__ bool mk_project_tc(int type, const MkArgs &a, const M
                 v0 += r0[sl * 16 * 8] + r0[sl * 16 * 8 + M];
                 v1 += r1[sl * 16 * 8] + r1[sl * 16 * 8 + M];
             }
-            if (m < a.n_rows) mk_finish<true>(type, a, L, sh, seg.band, rib, m, v0, v1);
+            if (type == MK_QKV) {
+                if (m < a.n_rows) mk_finish_qkv(a, l, sh, w.j, rib, m, v0, v1);
+            } else {
+                const int c = (w.j - first) * MK_BOX_ROWS + rib;
+                mk_put_planes<M>(u_planes, u_rs, m, c, mk_silu_mul(v0, v1));  // (rows beyond n_rows: their planes are zeros)
+            }
         }
         band_it++;
     }
-    cp_async_wait<0>();
-    return true;
 }
 
-// Few rows: CUDA-core form with fp32 activations; from MK_TC_ROWS on: tensor-core form.
+// Column form (see mk_columns): a warp's sixteen rows are the A operand, the activations of the columns sit in
+// registers as B operands, and a box's sums need no other warp.  x: planes of M rows, row stride x_rs.
 template <int M>
-__device__ __forceinline__ bool mk_proj(int type, const MkArgs &a, const MkLayer *L, unsigned char *area, int K,
-                                        const float *h, const float *x, const bf16 *gain, unsigned char *ring, MkShared *sh,
-                                        uint32_t &it)
+__device__ __forceinline__ void mk_columns_tc(const MkArgs &a, float *dst, int r0, int r1, int cols, const bf16 *x, int x_rs,
+                                              unsigned char *ring, MkShared *sh, MkPos<mk_slots(M)> at)
 {
-    if (M >= MK_TC_ROWS) return mk_project_tc<M>(type, a, L, area, K, h, x, gain, ring, sh, it);
-    return mk_project<M>(type, a, L, reinterpret_cast<float *>(area), K, h, x, gain, ring, sh, it);
+    constexpr int KS = MK_CBOX_COLS / 16;
+    static_assert(2 * M == 8, "the exchange below adds column n + M to column n");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / MK_GROUPS, sub = warp % MK_GROUPS;
+    const int g = lane >> 2, t = lane & 3, nk = cols / 16;
+    uint32_t b[KS][2];
+#pragma unroll
+    for (int k = 0; k < KS; k++) {
+        b[k][0] = b[k][1] = 0u;
+        if (k < nk) {
+            b[k][0] = *reinterpret_cast<const uint32_t *>(x + (size_t)g * x_rs + k * 16 + 2 * t);
+            b[k][1] = *reinterpret_cast<const uint32_t *>(x + (size_t)g * x_rs + k * 16 + 8 + 2 * t);
+        }
+    }
+    const int lrow = sub * 16 + (lane & 7) + ((lane >> 3) & 1) * 8, lchk = lane >> 4;
+    const int ahead = (grp - at.s) & (MK_GROUPS - 1);
+    at.skip(ahead);
+    for (int r = r0 + ahead; r < r1; r += MK_GROUPS, at.skip(MK_GROUPS)) {
+        if (!mbar_wait(&sh->full[at.s], at.ph, &sh->giving_up, a.status)) return;
+        const uint32_t slot = smem_u32(ring) + (uint32_t)at.s * MK_SLOT_BYTES + (uint32_t)lrow * 64;
+        float acc[4] = {0.f, 0.f, 0.f, 0.f}, acc2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int k = 0; k < KS; k++) {
+            if (k < nk) {
+                uint32_t af[4];
+                const uint32_t chunk = (uint32_t)((k & 1) * 2 + lchk);
+                ldsm_x4(af, slot + (uint32_t)(k >> 1) * (MK_CBOX_ROWS * 64) + ((chunk ^ (uint32_t)((lrow >> 1) & 3)) << 4));
+                if (k & 1) mma_bf16_16816(acc2, af, b[k][0], b[k][1]);
+                else mma_bf16_16816(acc, af, b[k][0], b[k][1]);
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive_n(&sh->empty[at.s], MK_CW / MK_GROUPS);
+        // lanes t < 2 hold hi terms of rows 2 t and 2 t + 1, lanes t + 2 the lo terms of the same; the lower ones finish weight row g,
+        // the upper ones g + 8
+#pragma unroll
+        for (int e = 0; e < 4; e++) acc[e] += acc2[e];
+        const bool up = t >= 2;
+        const float y0 = (up ? acc[2] : acc[0]) + __shfl_xor_sync(0xffffffffu, up ? acc[0] : acc[2], 2);
+        const float y1 = (up ? acc[3] : acc[1]) + __shfl_xor_sync(0xffffffffu, up ? acc[1] : acc[3], 2);
+        const int row = r * MK_CBOX_ROWS + sub * 16 + g + (up ? 8 : 0), m = (t & 1) * 2;
+        if (row < a.d) {
+            if (m < a.n_rows) atomicAdd(dst + (size_t)m * a.d + row, y0);
+            if (m + 1 < a.n_rows) atomicAdd(dst + (size_t)(m + 1) * a.d + row, y1);
+        }
+    }
 }
 
 }  // namespace sparsk

@@ -639,3 +639,37 @@ def test_three_and_four_wide_rows(util, rows, d_model, route):
     assert P.stats["max_flush"] == 3
     P.check_cache(rows - 1, range(1, 3), P.g.slot_state(rows - 1)[0] - P.g.slot_state(rows - 1)[1])
     P.close()
+
+
+@pytest.mark.parametrize("shape,lens", [
+    # a CTA's MLP columns: none for most CTAs, a lone band, boxes that reach into the next CTA's columns
+    (dict(d_model=256, n_q_heads=4, n_kv_heads=2, head_dim=64, d_ffn=64), (1,)),
+    (dict(d_model=200, n_q_heads=6, n_kv_heads=3, head_dim=64, d_ffn=712), (17, 30)),
+    # 148 SMs x 128 columns and a little: two boxes a CTA; nine bands a CTA meet in two batches of sums
+    (dict(d_model=64, n_q_heads=2, n_kv_heads=1, head_dim=128, d_ffn=19200), (33,)),
+    (dict(d_model=128, n_q_heads=2, n_kv_heads=2, head_dim=64, d_ffn=19008), (5, 64, 16)),
+    # sixteen query heads a kv head (blocks of sixteen query vectors) and more cache tiles than SMs, several a CTA
+    (dict(d_model=192, n_q_heads=16, n_kv_heads=1, head_dim=64, d_ffn=320), (900, 3)),
+    (dict(d_model=128, n_q_heads=8, n_kv_heads=4, head_dim=64, d_ffn=256), (1300, 15, 48, 700)),
+    # a residual row wider than the registers of the norm hold, and with two rows than the area
+    (dict(d_model=4352, n_q_heads=2, n_kv_heads=1, head_dim=64, d_ffn=128), (20,)),
+    (dict(d_model=11264, n_q_heads=2, n_kv_heads=1, head_dim=64, d_ffn=64), (18, 9)),
+])
+def test_persistent_kernel_at_the_edges_of_its_shares(util, shape, lens):
+    """One to four rows through the persistent kernel (and the flushes of what they leave pending where those are
+    as few) where the shares of its CTAs are empty, ragged, or more than one box, run or window."""
+    dims = synth.model_dims(dict(n_layers=3, vocab_text=96, vocab_speech=64, rms_eps=1e-6, rope_base=10000.0, **shape), 2, 3, 0)
+    w = synth.make_weights(dims, seed=3)
+    rng = np.random.default_rng(5)
+    prompts = [rng.integers(0, 160, size=n + 1).astype(np.int32) for n in lens]
+    P = util.Pair(dims, w, len(lens), max(lens) + 16, 2, prefill_rows=64)
+    P.prefill(prompts)
+    before = P.g.route_counts()["mega"]
+    for g in range(7):
+        mc = [synth.interleave(g + i, 1, 4) for i in range(len(lens))]
+        P.step([m for m, _ in mc], [c for _, c in mc])
+    assert P.g.route_counts()["mega"] > before
+    for s_ in range(len(lens)):
+        ln, pend = P.g.slot_state(s_)
+        P.check_cache(s_, range(1, 4), ln - pend)
+    P.close()
