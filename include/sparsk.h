@@ -71,9 +71,11 @@ typedef struct {
     int32_t max_seqs;       /* number of sequence slots */
     int32_t max_seq_len;    /* positions per slot */
     int32_t max_pending;    /* pending positions per slot; >= K-1 for the periodic schedule */
-    int32_t prefill_rows;   /* rows per prefill pass; 0 = 256.  The workspace holds activations and
-                               attention partials for as many rows (28 query heads of 128 numbers:
-                               0.45 MiB of partials a row), so a smaller number makes it smaller */
+    int32_t prefill_rows;   /* rows per prefill pass; 0 = 1,024, or as many as the slots hold positions
+                               (256 at least).  The workspace holds activations for as many rows
+                               (28-layer shape: 0.15 MiB a row) and attention partials for up to
+                               256 of them (28 query heads of 128 numbers: 0.45 MiB a row), so a
+                               smaller number makes it smaller */
     int32_t text_period;    /* K of text steps when they follow the rule (text_exit 1 or 2); 0 = the
                                same K and r as speech steps.  Sec. V-E: the two modalities may need
                                different policies */

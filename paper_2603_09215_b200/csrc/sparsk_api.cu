@@ -186,17 +186,26 @@ bool dims_ok(const sparsk_dims *d)
     return true;
 }
 
-// Rows of a prefill pass when the caller leaves the choice to the library.  A pass streams every
-// layer's weights once whatever its rows, so it wants as many as one block of the tcgen05 GEMMs
-// takes: a layer of the 40-layer shape takes 153 us at 64 rows and 280 at 256, less than half
-// the time per token (first token after 1,024: 101.6 ms with passes of 64, 49.5 ms with 256).
-// More rows would be a second block, which streams the weights again.
-constexpr int PREFILL_ROWS = GM_MAX_N;
-int cap_rows_of(const sparsk_dims *d)
+// Rows of a prefill pass when the caller leaves the choice to the library.  The GEMMs are bound by the tensor cores
+// from 256 rows on (one block of rows), so more rows save no weight traffic, but they give every launch several
+// blocks of rows: what a launch costs beyond its products (boundary, ramp, ending) is paid once for all of them,
+// the projections with few units need fewer cuts of the inner dimension and so add fewer partials, and
+// units that are no multiple of the SMs leave less of the last wave empty.  First token after 1,024: 42.0 ms with
+// passes of 256 rows and 33.2 with 1,024 (40-layer shape), 30.9 and 27.0 (28-layer shape); after three times 700
+// 63.4 and 54.6.
+constexpr int PREFILL_ROWS = 4 * GM_MAX_N;
+// Never more rows than the cache has positions.
+int prefill_rows_of(const sparsk_dims *d)
 {
-    const int pf = d->prefill_rows > 0 ? d->prefill_rows : PREFILL_ROWS;
-    const long dec = (long)d->max_seqs * (d->max_pending + 1);
-    return (int)std::max<long>(dec, pf);
+    return d->prefill_rows > 0 ? d->prefill_rows : (int)std::min<long>(PREFILL_ROWS, std::max<long>(GM_MAX_N, (long)d->max_seqs * d->max_seq_len));
+}
+long decode_rows_of(const sparsk_dims *d) { return (long)d->max_seqs * (d->max_pending + 1); }
+int cap_rows_of(const sparsk_dims *d) { return (int)std::max<long>(decode_rows_of(d), prefill_rows_of(d)); }
+// (row, split) pairs the attention partials have room for: every split of a step's rows or of one block of prompt rows.  Passes of more
+// prompt rows have fewer splits (run_attn).
+size_t part_rows_of(const sparsk_dims *d)
+{
+    return (size_t)std::max<long>(decode_rows_of(d), std::min(prefill_rows_of(d), GM_MAX_N)) * MAX_SPLITS;
 }
 
 // Ints that describe a prefill pass: slot and position of every row, first row and row count of every
@@ -247,9 +256,9 @@ size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
     unsigned *atk = w.take<unsigned>(1);
     float *mkh2 = w.take<float>((size_t)MK_MAX_ROWS * d->d_model);
     unsigned long long *mkt = w.take<unsigned long long>(1 + MK_PHASES * L);
-    // attention partials: of the launches, and of the persistent kernel (see MkRuns)
+    // attention partials: of the launches, and of the persistent kernel (see MkRun)
     const size_t runs = (size_t)MK_MAX_CTAS + (size_t)MK_MAX_ROWS * d->n_kv_heads;
-    const size_t cells = std::max<size_t>(R * MAX_SPLITS * d->n_q_heads, runs * MK_MAX_ROWS * (d->n_q_heads / d->n_kv_heads));
+    const size_t cells = std::max<size_t>(std::max(R, part_rows_of(d)) * d->n_q_heads, runs * MK_MAX_ROWS * (d->n_q_heads / d->n_kv_heads));
     float *po = w.take<float>(cells * d->head_dim);
     float2 *pml = w.take<float2>(cells);
     if (c) {
@@ -497,6 +506,7 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
     a.nq_max = 1 << 30;
     a.rows_early = !rs.rows_late;
     cudaError_t e;
+    const int max_splits = (int)std::min<size_t>(AT_MAX_SPLITS, std::max<size_t>(1, part_rows_of(&d) / rs.n_rows));
     const bool blocks_tc = c->attn_tc && c->tc_ok && d.head_dim == TA_HD && rs.max_grp_rows * G >= c->attn_tc_min_q;
     // groups the tcgen05 kernel takes (the host knows every group's row count) and the rest
     const int n_big = blocks_tc ? (rs.n_big > 0 ? rs.n_big : rs.n_groups_h) : 0;
@@ -507,6 +517,10 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
     a.table = tma && rs.n_groups_h <= AT_TABLE;
     AttnPlan pl = attn_plan(warp_ctas * AW_WARPS, blocks_tc ? std::max(1, n_small) : rs.n_groups_h, small_rows, G,
                             d.n_kv_heads, rs.max_len, c->attn_split, blocks_tc ? 0 : rs.sum_len, a.table);
+    if (pl.n_splits > max_splits) {
+        pl.split_len = div_up(div_up(rs.max_len, max_splits), AT_TP) * AT_TP;
+        pl.n_splits = div_up(rs.max_len, pl.split_len);
+    }
     if (blocks_tc) {
         // Groups with many query vectors per kv head go to the tcgen05 kernel (one CTA per SM, tiles
         // of 64 positions), the others to the mma.sync kernel; both launches cover all groups, a CTA
@@ -530,7 +544,7 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
         int s_tc = 1;
         {   // the split count whose CTAs fill whole waves of one CTA per SM best (at least 8 tiles each)
             double best = -1.0;
-            const int s_max = std::max(1, std::min(AT_MAX_SPLITS, tiles / 8));
+            const int s_max = std::max(1, std::min(max_splits, tiles / 8));
             for (int sc = 1; sc <= s_max; sc++) {
                 const long n = (long)big_ctas * sc, waves = (n + c->n_sm - 1) / c->n_sm;
                 const double eff = (double)n / (double)(waves * c->n_sm);
@@ -543,8 +557,8 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
             }
         }
         if (c->attn_split > 0) s_tc = pl.n_splits;
-        s_tc = std::min(s_tc, AT_MAX_SPLITS);
-        const int mult = n_small > 0 ? std::max(1, std::min(AT_MAX_SPLITS / s_tc, div_up(pl.n_splits, s_tc))) : 1;
+        s_tc = std::min(s_tc, max_splits);
+        const int mult = n_small > 0 ? std::max(1, std::min(max_splits / s_tc, div_up(pl.n_splits, s_tc))) : 1;
         const int small_len = div_up(div_up(rs.max_len, s_tc * mult), TA_NT) * TA_NT;
         pl.split_len = small_len;
         pl.n_splits = std::max(1, div_up(rs.max_len, small_len));
@@ -794,9 +808,10 @@ cudaError_t run_norm(sparsk_ctx *c, const float *h, const bf16 *gain, const int 
                   c->dm.d_model, c->dm.rms_eps);
 }
 
-// How many cuts of the inner dimension fill the machine when a product has `units` units.
-int splits_for(const sparsk_ctx *c, int units)
+// How many cuts of the inner dimension fill the machine when a product has `units` units for every block of rows.
+int splits_for(const sparsk_ctx *c, int units, int m_rows)
 {
+    units *= div_up(m_rows, GM_MAX_N);
     const int ctas = c->n_sm * std::max(1, c->gemm_cps);
     return units * 2 <= ctas ? ctas / units : 1;
 }
@@ -819,7 +834,7 @@ cudaError_t run_layer_tc_front(sparsk_ctx *c, int layer, float *h, const RowSet 
         GemmArgs g{};
         g.K = d.d_model; g.units[0] = div_up(qd, 2 * GM_BM); g.units[1] = g.units[2] = div_up(kd, 2 * GM_BM);
         g.m_rows = M;
-        g.splits = splits_for(c, g.units[0] + g.units[1] + g.units[2]);
+        g.splits = splits_for(c, g.units[0] + g.units[1] + g.units[2], M);
         QkvEnd ep;
         ep.q_out = c->qbuf; ep.kc = kc; ep.vc = vc; ep.rope = c->rope;
         ep.row_slot = rs.slot; ep.row_pos = rs.pos; ep.Hq = d.n_q_heads; ep.Hkv = d.n_kv_heads; ep.hd = d.head_dim;
@@ -847,7 +862,7 @@ cudaError_t run_layer_tc_back(sparsk_ctx *c, int layer, float *h, const RowSet &
         c->cur_class = KC_OPROJ;
         GemmArgs g{};
         g.K = qd; g.units[0] = div_up(d.d_model, 2 * GM_BM); g.m_rows = M;
-        g.splits = splits_for(c, g.units[0]);
+        g.splits = splits_for(c, g.units[0], M);
         ResidEnd ep;
         ep.h = h; ep.n_out = d.d_model; ep.atomic = 1;
         if ((e = launch_gemm(c, c->tm_wo[li], c->tm_wo[li], c->tm_wo[li], c->tm_ao, g, ep)) != cudaSuccess) return e;
@@ -867,7 +882,7 @@ cudaError_t run_layer_tc_back(sparsk_ctx *c, int layer, float *h, const RowSet &
         c->cur_class = KC_DOWN;
         GemmArgs g{};
         g.K = d.d_ffn; g.units[0] = div_up(d.d_model, 2 * GM_BM); g.m_rows = M;
-        g.splits = splits_for(c, g.units[0]);
+        g.splits = splits_for(c, g.units[0], M);
         ResidEnd ep;
         ep.h = h; ep.n_out = d.d_model; ep.atomic = 1;
         e = launch_gemm(c, c->tm_wd[li], c->tm_wd[li], c->tm_wd[li], c->tm_act, g, ep);
@@ -1184,7 +1199,7 @@ extern "C" int sparsk_create(const sparsk_dims *dims, const sparsk_weights *w, v
     if (!ctx) return SPARSK_EINVAL;
     ctx->magic = CTX_MAGIC;
     ctx->dm = *dims;
-    if (ctx->dm.prefill_rows <= 0) ctx->dm.prefill_rows = PREFILL_ROWS;
+    ctx->dm.prefill_rows = prefill_rows_of(dims);
     ctx->stream = (cudaStream_t)cuda_stream;
     ctx->err[0] = 0;
     auto cp = [&](std::vector<const bf16 *> &dst, const void *const *src) {

@@ -474,6 +474,23 @@ def test_prefill_passes_beyond_128_rows(util, rows, shape):
     P.close()
 
 
+@pytest.mark.parametrize("options", [{}, {"attn_split": 16}, {"attn_tc": 0}, {"attn_tc": 0, "attn_split": 16, "attn_tma": 0}])
+def test_prefill_passes_of_several_row_blocks(util, options):
+    """The library's own choice of rows a pass: a pass of 1,024 rows (four blocks of rows; attention partials have room
+    for an eighth of the splits, whatever was asked for) with two groups for the tcgen05 attention and one below its
+    size, then a pass with what is left."""
+    dims = synth.model_dims(dict(MICRO256, n_q_heads=8, head_dim=128), 2, 3, 0)
+    w = synth.make_weights(dims, seed=9)
+    rng = np.random.default_rng(6)
+    prompts = [rng.integers(0, 400, size=n).astype(np.int32) for n in (701, 4, 431)]
+    P = util.Pair(dims, w, 3, 720, 2, options=options)
+    P.prefill(prompts)
+    for s_, p in enumerate(prompts):
+        P.check_cache(s_, range(1, 4), len(p) - 1)
+    P.step([0, 1, 0], [0, 1, 0])
+    P.close()
+
+
 @pytest.mark.parametrize("kb", [48, 110])
 @pytest.mark.parametrize("rows", [40, 128, 256])
 def test_prompt_attention_beside_small_gemm_rings(util, rows, kb):
