@@ -62,8 +62,8 @@ constexpr int MK_MAX_ROWS = 4;
 constexpr int MK_TC_ROWS = 3;                   // rows from which the tensor-core form runs
 constexpr int MK_GROUPS = 4;                    // a slot of weights is the work of one of four groups of four warps
 constexpr int MK_MAX_CTAS = 192;                // bounds the number of attention partials
-constexpr int MK_SHARED_BYTES = 3072;           // MkShared, behind the area, with two to four rows
-constexpr int MK_SHARED_FEW_BYTES = 2048;       // the part of it that one row needs
+constexpr int MK_SHARED_BYTES = 2560;           // MkShared, behind the area, with two to four rows
+constexpr int MK_SHARED_FEW_BYTES = 1536;       // the part of it that one row needs
 
 // The ring, then the area: the activations of a row-form phase (M rows; with one or two rows, when they
 // do not fit whole, a window of k-steps that is reloaded as the phase moves along) and what the CTA's
@@ -122,7 +122,7 @@ struct MkArgs {
     kv_t *kc, *vc;               // cache of the first layer [slot][Hkv][S][hd], and what lies between two layers'
     size_t kv_layer;             // (arithmetic: a pointer read from `layers` would be a trip to HBM in every layer)
     float *q_buf;                // [rows][Hq*hd]
-    float *part_o;               // attention partials, see MkRuns
+    float *part_o;               // attention partials, see MkRun
     float2 *part_ml;
     const float2 *rope;
     int d, Hq, Hkv, hd, F, S, n_slots;
@@ -203,6 +203,29 @@ struct MkHeads {
     }
 };
 
+// Attention: the tiles of 16 positions of all (group, kv head) pairs laid end to end and cut into equal
+// contiguous shares, so that every SM reads as much of the cache as the next (with fewer tiles than SMs, one each
+// for as many SMs); a run is what a share has of one pair.  The run of pair p in CTA c leaves partial number
+// c + p (both only ever grow from one run to the next), for every query vector of the pair.
+struct MkRun {
+    int g, hk, tile0, n;            // group, kv head, first tile, tiles
+    int row0, nrows, pos0, cache0;  // the group's rows; first cache row of (slot, kv head)
+    int nq, n_qblk;                 // query vectors, blocks of sixteen of them
+};
+// What a row of weights of the q/k/v projection becomes: a rotary pair of q or k, or two numbers of v.
+struct MkFin {
+    float2 cs;      // rotary factors
+    size_t off;     // of the first number, the second is `second` behind it
+    int second, kind;
+};
+enum { MK_FIN_Q = 0, MK_FIN_K, MK_FIN_V, MK_FIN_NONE };
+// The partials of one (row, query head): those of the CTAs [cf, cl], `cell0` plus the CTA's number times mk_part_rows.
+struct MkMerge {
+    int cf, cl, cell0;
+};
+
+// A launch's constants are worked out once: a warp spends some ten cycles an instruction here, so the
+// divisions that turn a share into rows and heads held every layer up by 2 us.
 struct MkShared {
     uint64_t full[mk_slots(1)], empty[mk_slots(1)];
     int giving_up, never, go_on;
@@ -212,11 +235,16 @@ struct MkShared {
     int att_base[MK_MAX_ROWS + 1];       // tiles x kv heads of the groups before this one
     int att_ctas;                        // CTAs that the tiles are dealt to: none of them goes without
     int att_t0, att_t1;                  // this CTA's share of them
+    MkRun run0;                          // its first run
+    MkBands bands[2];                    // this CTA's bands of q/k/v and of gate/up
+    MkHeads heads;                       // and of the O-projection
+    int head0;                           // first head of those
+    MkMerge merge[2][MK_MAX_ROWS];       // its first two heads
     float red_rows[MK_MAX_ROWS][MK_CW];  // per-row partial sums of squares
-    float2 rope[MK_MAX_ROWS][64];        // rotary factors of the rows' positions; one row has room for as many
+    MkFin fin[MK_BOX_ROWS * MK_MAX_ROWS];  // of the first q/k/v band, [row of the box][activation row]; one row has room for as many
 };
 static_assert(sizeof(MkShared) <= MK_SHARED_BYTES, "MkShared outgrew its place");
-static_assert(offsetof(MkShared, rope) + sizeof(float2) * 64 <= MK_SHARED_FEW_BYTES, "MkShared outgrew its place");
+static_assert(offsetof(MkShared, fin) + sizeof(MkFin) * MK_BOX_ROWS <= MK_SHARED_FEW_BYTES, "MkShared outgrew its place");
 
 // A warp's place in the ring: slot and the parity of its present fill.
 template <int SLOTS>
@@ -239,36 +267,25 @@ struct MkPos {
     }
 };
 
-// Attention: the tiles of 16 positions of all (group, kv head) pairs laid end to end and cut into equal
-// contiguous shares, so that every SM reads as much of the cache as the next (with fewer tiles than SMs, one each
-// for as many SMs); a run is what a share has of one pair.  The run of pair p in CTA c leaves partial number
-// c + p (both only ever grow from one run to the next), for every query vector of the pair.
-struct MkRun {
-    int g, hk, tile0, n;   // group, kv head, first tile, tiles
-};
-struct MkRuns {
-    int t, end;
-    __device__ void init(const MkShared *sh)
-    {
-        t = sh->att_t0;
-        end = sh->att_t1;
-    }
-    __device__ bool next(const MkShared *sh, MkRun &r)
-    {
-        if (t >= end) return false;
-        int g = 0;
+// The run that begins with tile t of a share that ends before `end`.
+__device__ __forceinline__ void mk_run_at(const MkArgs &a, const MkShared *sh, int t, int end, MkRun &r)
+{
+    int g = 0;
 #pragma unroll
-        for (int i = 1; i < MK_MAX_ROWS; i++)
-            if (t >= sh->att_base[i]) g = i;   // (groups without tiles share their successor's base)
-        const int tiles = sh->grp_tiles[g], rem = t - sh->att_base[g];
-        r.g = g;
-        r.hk = rem / tiles;
-        r.tile0 = rem - r.hk * tiles;
-        r.n = min(tiles - r.tile0, end - t);
-        t += r.n;
-        return true;
-    }
-};
+    for (int i = 1; i < MK_MAX_ROWS; i++)
+        if (t >= sh->att_base[i]) g = i;   // (groups without tiles share their successor's base)
+    const int tiles = sh->grp_tiles[g], rem = t - sh->att_base[g];
+    r.g = g;
+    r.hk = rem / tiles;
+    r.tile0 = rem - r.hk * tiles;
+    r.n = min(tiles - r.tile0, end - t);
+    r.row0 = sh->grp_row0[g];
+    r.nrows = sh->grp_nrows[g];
+    r.pos0 = sh->row_pos[r.row0];
+    r.cache0 = (sh->row_slot[r.row0] * a.Hkv + r.hk) * a.S;
+    r.nq = r.nrows * (a.Hq / a.Hkv);
+    r.n_qblk = (r.nq + 15) / 16;
+}
 // CTA whose share holds tile t
 __device__ __forceinline__ int mk_run_cta(const MkShared *sh, int t)
 {

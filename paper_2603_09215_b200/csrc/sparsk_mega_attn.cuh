@@ -91,35 +91,34 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = a.Hq / a.Hkv;
     AttnArgs aa{};
     aa.q32 = a.q_buf; aa.Hq = a.Hq; aa.Hkv = a.Hkv;
-    const int stride = mk_part_rows(a);
-    MkRuns runs;
-    runs.init(sh);
-    MkRun r;
-    while (runs.next(sh, r)) {
-        const int nq = sh->grp_nrows[r.g] * G, n_qblk = (nq + 15) / 16, n_items = (r.n + 1) / 2;
-        const int room = (mk_area_bytes(M) - n_qblk * mk_park_bytes<HD>()) / (n_qblk * mk_cell_bytes<HD>());
-        int nsub = min(min(4, MK_CW / n_qblk), min(room, n_items));
-        if (nsub < 1) nsub = 1;
+    const int stride = mk_part_rows(a), end = sh->att_t1;
+    int t = sh->att_t0;
+    MkRun r = sh->run0;
+    while (t < end) {
+        const int nq = r.nq, n_qblk = r.n_qblk, n_items = (r.n + 1) / 2;
+        int nsub = min(4, n_items);
+        if (nsub > 1) {
+            const int room = (mk_area_bytes(M) - n_qblk * mk_park_bytes<HD>()) / (n_qblk * mk_cell_bytes<HD>());
+            nsub = max(1, min(nsub, min(MK_CW / n_qblk, room)));
+        }
         if (SLOTS % nsub) nsub = 2;  // a slot's successive fills stay with one warp
-        const int qb = warp % n_qblk, sub = warp / n_qblk;
+        const int sub = n_qblk == 1 ? warp : warp / n_qblk, qb = warp - sub * n_qblk;
         // (the warps of a block all park its queries, the same numbers in the same place)
         kv_t *park = reinterpret_cast<kv_t *>(area) + (size_t)qb * 16 * (HD + 8);
         unsigned char *cells = area + n_qblk * mk_park_bytes<HD>();
         const size_t part = (size_t)(blockIdx.x + r.g * a.Hkv + r.hk) * stride;
         if (sub < nsub) {
-            const int row0 = sh->grp_row0[r.g], pos0 = sh->row_pos[row0];
             AtItem item;
-            item.qb = qb; item.hk = r.hk; item.row0 = row0; item.nrows = sh->grp_nrows[r.g]; item.pos0 = pos0; item.nq = nq;
-            item.w_end = min(pos0 + (min(qb * 16 + 16, nq) - 1) / G + 1, a.S);
+            item.qb = qb; item.hk = r.hk; item.row0 = r.row0; item.nrows = r.nrows; item.pos0 = r.pos0; item.nq = nq;
+            item.w_end = min(r.pos0 + (r.nrows == 1 ? 0 : (min(qb * 16 + 16, nq) - 1) / G) + 1, a.S);
             MkTiles<HD, SLOTS> tiles;
             tiles.ring = ring; tiles.sh = sh; tiles.status = a.status;
-            const size_t rows0 = ((size_t)sh->row_slot[row0] * a.Hkv + r.hk) * a.S;
-            tiles.kbase = a.kc + l * a.kv_layer + rows0 * HD; tiles.vbase = a.vc + l * a.kv_layer + rows0 * HD;
+            tiles.kbase = a.kc + l * a.kv_layer + (size_t)r.cache0 * HD; tiles.vbase = a.vc + l * a.kv_layer + (size_t)r.cache0 * HD;
             tiles.at0 = at; tiles.tile0 = r.tile0; tiles.sub = sub; tiles.nsub = nsub;
-            tiles.new0 = pos0; tiles.end = min(pos0 + item.nrows, a.S);
+            tiles.new0 = r.pos0; tiles.end = min(r.pos0 + r.nrows, a.S);
             tiles.arrivals = qb == 0 ? MK_CW - (n_qblk - 1) : 1;
-            const int mine = (n_items - sub + nsub - 1) / nsub;
-            tiles.n_tiles = 2 * mine - ((r.n & 1) && (n_items - 1) % nsub == sub ? 1 : 0);
+            const int mine = nsub == 1 ? n_items : (n_items - sub + nsub - 1) / nsub;
+            tiles.n_tiles = 2 * mine - ((r.n & 1) && sub + nsub * (mine - 1) == n_items - 1 ? 1 : 0);
             tiles.lane = lane;
             MkCells<HD> out;
             if (nsub > 1) {
@@ -156,9 +155,24 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
             }
             mk_consumer_sync();  // the next run may use the area
         }
+        t += r.n;
+        if (t < end) mk_run_at(a, sh, t, end, r);
     }
 }
 
+__device__ __forceinline__ MkMerge mk_merge_of(const MkArgs &a, const MkShared *sh, int h, int m)
+{
+    MkMerge r{0, -1, 0};
+    const int G = a.Hq / a.Hkv, hk = h / G;
+    const int g = m < a.n_rows && h < a.Hq ? sh->row_grp[m] : -1, tiles = g >= 0 ? sh->grp_tiles[g] : 0;
+    if (tiles > 0) {
+        const int t0 = sh->att_base[g] + hk * tiles;
+        r.cf = mk_run_cta(sh, t0);
+        r.cl = mk_run_cta(sh, t0 + tiles - 1);
+        r.cell0 = (g * a.Hkv + hk) * mk_part_rows(a) + (m - sh->grp_row0[g]) * G + h - hk * G;
+    }
+    return r;
+}
 // Merge of the partials of query heads hq and, with NH = 2, hq + 1, for all rows: 16 / (M NH) warps per row and head, a
 // share of the partials each, then the shares meet in scr.  Leaves the output of head i, row m at column c
 // through put(i, m, c, value).
@@ -166,24 +180,22 @@ template <int M, int HD, int NH, class Put>
 __device__ __forceinline__ void mk_merge_heads(const MkArgs &a, const MkShared *sh, int hq, float *scr, const Put &put)
 {
     constexpr int WPR = MK_CW / (M * NH), LN = HD / 4;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = a.Hq / a.Hkv;
-    const int hm = warp / WPR, h = hq + hm / M, hk = h / G, m = hm % M, wi = warp % WPR, stride = mk_part_rows(a);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int hm = warp / WPR, m = hm % M, wi = warp % WPR, stride = mk_part_rows(a);
     float2 *scr_ml = reinterpret_cast<float2 *>(scr + MK_CW * HD);
     float mx = -INFINITY, l = 0.f;
     float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-    const int g = m < a.n_rows ? sh->row_grp[m] : -1, tiles = g >= 0 ? sh->grp_tiles[g] : 0;
-    if (tiles > 0) {
-        const int t0 = sh->att_base[g] + hk * tiles;
-        const int cf = mk_run_cta(sh, t0), cl = mk_run_cta(sh, t0 + tiles - 1);
-        const size_t cell0 = (size_t)(g * a.Hkv + hk) * stride + (m - sh->grp_row0[g]) * G + h - hk * G;
+    const MkMerge p = hq == sh->head0 ? sh->merge[hm / M][m] : mk_merge_of(a, sh, hq + hm / M, m);
+    {
+        const int cl = p.cl;
         constexpr int U = 5;
-        for (int c0 = cf + wi; c0 <= cl; c0 += WPR * U) {
+        for (int c0 = p.cf + wi; c0 <= cl; c0 += WPR * U) {
             float2 ml[U];
             float4 v[U];
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 const int c = c0 + u * WPR;
-                const size_t cell = cell0 + (size_t)c * stride;
+                const size_t cell = (size_t)(p.cell0 + c * stride);
                 ml[u] = c <= cl ? a.part_ml[cell] : make_float2(-INFINITY, 0.f);
                 v[u] = c <= cl && lane < LN ? reinterpret_cast<const float4 *>(a.part_o + cell * HD)[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
             }

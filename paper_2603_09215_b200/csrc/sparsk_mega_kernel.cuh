@@ -31,8 +31,7 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
         return ok;
     };
     auto rows = [&](int type, const MkLayer *L) {
-        MkBands w;
-        w.init(type, a);
+        MkBands w = sh->bands[type == MK_QKV ? 0 : 1];
         for (; w.j < w.end; w.j += w.step)
             for (int ks = 0; ks < w.k_steps; ks++, idx++) {
                 if ((int)(idx % MK_PW) != p) continue;
@@ -65,11 +64,11 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
         const MkLayer *L = a.layers + l;
         rows(MK_QKV, L);
         if (!ok) break;
-        MkRuns runs;
-        runs.init(sh);
-        MkRun r;
-        while (ok && runs.next(sh, r)) {
-            const int y0 = (sh->row_slot[sh->grp_row0[r.g]] * a.Hkv + r.hk) * a.S;
+        MkRun r = sh->run0;
+        for (int t = sh->att_t0; ok && t < sh->att_t1;) {
+            if (t != sh->att_t0) mk_run_at(a, sh, t, sh->att_t1, r);
+            t += r.n;
+            const int y0 = r.cache0;
             for (int i = 0; i < r.n; i += 2, idx++) {
                 if ((int)(idx % MK_PW) != p) continue;
                 const int n = min(2, r.n - i);
@@ -84,14 +83,12 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
             }
         }
         if (!ok) break;
-        MkHeads w;
-        w.init(a);
+        const MkHeads w = sh->heads;
         for (int i = w.lo; i < w.hi && ok; i++) column_box(&L->map[MKW_O], HD, (i / w.boxes) * HD, (i % w.boxes) * MK_CBOX_ROWS);
         if (!ok) break;
         rows(MK_MLP, L);
         if (!ok) break;
-        MkBands b;
-        b.init(MK_MLP, a);
+        const MkBands b = sh->bands[1];
         if (b.j < b.end)
             for (int c = 0; c < a.cols.chunks && ok; c++)
                 for (int i = 0; i < w.boxes && ok; i++)
@@ -111,8 +108,7 @@ template <int M, int HD>
 __device__ __forceinline__ void mk_oproj(const MkArgs &a, unsigned char *area, unsigned char *ring, MkShared *sh,
                                          MkPos<mk_slots(M)> &at)
 {
-    MkHeads w;
-    w.init(a);
+    const MkHeads w = sh->heads;
     constexpr bool TC = M >= MK_TC_ROWS;
     constexpr int RS = HD + 8;
     // two merged heads, as fp32 rows or as two planes each
@@ -126,7 +122,7 @@ __device__ __forceinline__ void mk_oproj(const MkArgs &a, unsigned char *area, u
     };
     // a share reaches into a second head as often as not, into a third one only with more heads than CTAs
     for (int i = w.lo; i < w.hi;) {
-        const int hq = i / w.boxes;
+        const int hq = i == w.lo ? sh->head0 : i / w.boxes;
         if (i != w.lo) mk_consumer_sync();  // everyone is done with the heads before
         if ((hq + 1) * w.boxes < w.hi) mk_merge_heads<M, HD, 2>(a, sh, hq, scr, put);
         else mk_merge_heads<M, HD, 1>(a, sh, hq, scr, put);
@@ -145,8 +141,7 @@ __device__ __forceinline__ void mk_mlp(const MkArgs &a, int l, unsigned char *ar
                                        const MkGains &gains, MkPos<mk_slots(M)> &at)
 {
     const int boxes = (a.d + MK_CBOX_ROWS - 1) / MK_CBOX_ROWS;
-    MkBands w;
-    w.init(MK_MLP, a);
+    const MkBands w = sh->bands[1];
     if (w.j >= w.end) return;
     const bf16 *gain = a.layers[l].mlp_gain;
     // columns of the last box that are the next CTA's meet zeros
@@ -230,12 +225,18 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
             sh->att_ctas = (int)n;
             sh->att_t0 = c < n ? (int)(c * (unsigned)base / n) : 0;
             sh->att_t1 = c < n ? (int)((c + 1) * (unsigned)base / n) : 0;
+            if (sh->att_t0 < sh->att_t1) mk_run_at(a, sh, sh->att_t0, sh->att_t1, sh->run0);
+            sh->bands[0].init(MK_QKV, a);
+            sh->bands[1].init(MK_MLP, a);
+            sh->heads.init(a);
+            sh->head0 = sh->heads.lo / sh->heads.boxes;
         }
     }
-    if (warp >= 2 && warp < 2 + M && warp - 2 < a.n_rows) {
-        const int i = warp - 2, pos = a.row_pos[i];
-        for (int j = lane; j < HD / 2; j += 32) sh->rope[i][j] = pos >= 0 ? a.rope[(size_t)pos * (HD / 2) + j] : make_float2(1.f, 0.f);
-    }
+    __syncthreads();
+    if ((int)threadIdx.x < MK_BOX_ROWS * M)
+        sh->fin[threadIdx.x] = mk_fin(a, sh, blockIdx.x, (int)threadIdx.x / M, (int)threadIdx.x % M);
+    if (warp == MK_CW - 1 && lane < 2 * MK_MAX_ROWS)
+        sh->merge[lane / MK_MAX_ROWS][lane % MK_MAX_ROWS] = mk_merge_of(a, sh, sh->head0 + lane / MK_MAX_ROWS, lane % MK_MAX_ROWS);
     __syncthreads();
 
     if (warp >= MK_CW) {

@@ -199,34 +199,44 @@ __device__ __forceinline__ void mk_exchange(float (&v)[N], int lane)
 }
 
 // ------------------------------------------------------------------ what a finished pair of sums becomes
-// v0 = row `rib` of q/k/v band b's first box, v1 = the same row of its second box (a rotary pair or two
-// plain rows), for activation row m of layer l.
-__device__ __forceinline__ void mk_finish_qkv(const MkArgs &a, int l, const MkShared *sh, int b, int rib, int m, float v0, float v1)
+// Row `rib` of the two boxes of q/k/v band b, for activation row m.
+__device__ __forceinline__ MkFin mk_fin(const MkArgs &a, const MkShared *sh, int b, int rib, int m)
 {
+    MkFin f{make_float2(1.f, 0.f), 0, 0, MK_FIN_NONE};
+    if (m >= a.n_rows) return f;
     const int half = a.hd >> 1, per_head = half / MK_BOX_ROWS;
     const int nq = a.Hq * per_head, nk = a.Hkv * per_head;
-    const int slot_id = sh->row_slot[m], pos = sh->row_pos[m];
+    const int pos = sh->row_pos[m];
+    const size_t row = (size_t)sh->row_slot[m] * a.Hkv;
     if (b < nq + nk) {
-        const bool isq = b < nq;
-        const int bb = isq ? b : b - nq;
+        const int bb = b < nq ? b : b - nq;
         const int head = bb / per_head, i = (bb % per_head) * MK_BOX_ROWS + rib;
-        const float2 cs = sh->rope[m][i];
-        const float ra = v0 * cs.x - v1 * cs.y, rb = v1 * cs.x + v0 * cs.y;
-        if (isq) {
-            float *dst = a.q_buf + (size_t)m * a.Hq * a.hd + head * a.hd + i;
-            dst[0] = ra;
-            dst[half] = rb;
-        } else {
-            kv_t *dst = a.kc + l * a.kv_layer + (((size_t)slot_id * a.Hkv + head) * a.S + pos) * a.hd + i;
-            dst[0] = to_kv(ra);
-            dst[half] = to_kv(rb);
-        }
+        f.cs = a.rope[(size_t)pos * half + i];
+        f.second = half;
+        f.kind = b < nq ? MK_FIN_Q : MK_FIN_K;
+        f.off = b < nq ? ((size_t)m * a.Hq + head) * a.hd + i : ((row + head) * a.S + pos) * a.hd + i;
     } else {
-        const int n0 = (b - nq - nk) * 2 * MK_BOX_ROWS + rib, n1 = n0 + MK_BOX_ROWS;
-        const int kvd = a.Hkv * a.hd;
-        kv_t *vc = a.vc + l * a.kv_layer;
-        if (n0 < kvd) vc[(((size_t)slot_id * a.Hkv + n0 / a.hd) * a.S + pos) * a.hd + n0 % a.hd] = to_kv(v0);
-        if (n1 < kvd) vc[(((size_t)slot_id * a.Hkv + n1 / a.hd) * a.S + pos) * a.hd + n1 % a.hd] = to_kv(v1);
+        const int n = (b - nq - nk) * 2 * MK_BOX_ROWS + rib;   // (a head is a multiple of 32 numbers: n + 16 is in the same)
+        f.second = MK_BOX_ROWS;
+        f.kind = n < a.Hkv * a.hd ? MK_FIN_V : MK_FIN_NONE;
+        f.off = ((row + n / a.hd) * a.S + pos) * a.hd + n % a.hd;
+    }
+    return f;
+}
+__device__ __forceinline__ void mk_finish_qkv(const MkArgs &a, int l, const MkFin &f, float v0, float v1)
+{
+    const float ra = v0 * f.cs.x - v1 * f.cs.y, rb = v1 * f.cs.x + v0 * f.cs.y;
+    if (f.kind == MK_FIN_Q) {
+        a.q_buf[f.off] = ra;
+        a.q_buf[f.off + f.second] = rb;
+    } else if (f.kind == MK_FIN_K) {
+        kv_t *dst = a.kc + l * a.kv_layer + f.off;
+        dst[0] = to_kv(ra);
+        dst[f.second] = to_kv(rb);
+    } else if (f.kind == MK_FIN_V) {
+        kv_t *dst = a.vc + l * a.kv_layer + f.off;
+        dst[0] = to_kv(v0);
+        dst[f.second] = to_kv(v1);
     }
 }
 __device__ __forceinline__ float mk_silu_mul(float gate, float up) { return gate / (1.f + __expf(-gate)) * up; }
@@ -265,8 +275,7 @@ __device__ __forceinline__ void mk_rows(int type, const MkArgs &a, int l, float 
     constexpr int ROWS = MK_BOX_ROWS / (MK_CW / MK_GROUPS), N = 2 * ROWS * M;  // rows of a box per warp; sums per warp
     static_assert(ROWS == 4, "mk_take");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / MK_GROUPS, sub = warp % MK_GROUPS;
-    MkBands w;
-    w.init(type, a);
+    MkBands w = sh->bands[type == MK_QKV ? 0 : 1];
     if (w.j >= w.end) return;
     const int first = w.j, n_bands = (w.end - w.j + w.step - 1) / w.step, room = mk_act_window(M, own);
     const bool whole = w.k_steps <= room;
@@ -328,7 +337,7 @@ __device__ __forceinline__ void mk_rows(int type, const MkArgs &a, int l, float 
             const float4 s0 = reinterpret_cast<const float4 *>(sums)[(b * 2 * MK_BOX_ROWS + rib) * M + m];
             const float4 s1 = reinterpret_cast<const float4 *>(sums)[(b * 2 * MK_BOX_ROWS + MK_BOX_ROWS + rib) * M + m];
             const float v0 = (s0.x + s0.y) + (s0.z + s0.w), v1 = (s1.x + s1.y) + (s1.z + s1.w);
-            if (type == MK_QKV) mk_finish_qkv(a, l, sh, first + (b0 + b) * w.step, rib, m, v0, v1);
+            if (type == MK_QKV) mk_finish_qkv(a, l, b0 + b == 0 ? sh->fin[i] : mk_fin(a, sh, first + (b0 + b) * w.step, rib, m), v0, v1);
             else u[m * u_stride + (b0 + b) * MK_BOX_ROWS + rib] = mk_silu_mul(v0, v1);
         }
         if (b0 + MK_BATCH < n_bands) mk_consumer_sync();
@@ -429,8 +438,7 @@ __device__ __forceinline__ void mk_rows_tc(int type, const MkArgs &a, int l, bf1
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     const int grp = warp / MK_GROUPS, box = (warp >> 1) & 1, half = warp & 1;
-    MkBands w;
-    w.init(type, a);
+    MkBands w = sh->bands[type == MK_QKV ? 0 : 1];
     if (w.j >= w.end) return;
     // row stride: the padding spreads the rows over the banks
     const int first = w.j, ncols = w.k_steps * MK_BOX_COLS, rs = ncols + 8;
@@ -490,7 +498,7 @@ __device__ __forceinline__ void mk_rows_tc(int type, const MkArgs &a, int l, bf1
                 v1 += r1[sl * 16 * 8] + r1[sl * 16 * 8 + M];
             }
             if (type == MK_QKV) {
-                if (m < a.n_rows) mk_finish_qkv(a, l, sh, w.j, rib, m, v0, v1);
+                mk_finish_qkv(a, l, band_it == 0 ? sh->fin[threadIdx.x] : mk_fin(a, sh, w.j, rib, m), v0, v1);
             } else {
                 const int c = (w.j - first) * MK_BOX_ROWS + rib;
                 mk_put_planes<M>(u_planes, u_rs, m, c, mk_silu_mul(v0, v1));  // (rows beyond n_rows: their planes are zeros)
