@@ -57,7 +57,11 @@ constexpr int MK_BOX_ROWS = 16, MK_BOX_COLS = 256;           // row form: two su
 constexpr int MK_BOX_BYTES = MK_BOX_ROWS * MK_BOX_COLS * 2;  // 8 KB
 constexpr int MK_CBOX_ROWS = 64, MK_CBOX_COLS = 128;         // column form: one box of 64 rows and up to 128 columns per slot
 constexpr int MK_SLOT_BYTES = 2 * MK_BOX_BYTES;
-constexpr int MK_IN_FLIGHT = 8;                 // slots on their way at once
+constexpr int MK_IN_FLIGHT = 8;                 // slots on their way at once, in the MLP
+// and before it, with one row.  A trip to the L2 queues behind the copies on their way to the SM, 2.7 us of them at eight
+// slots, and the phases before the MLP are chains of such trips with little to stream: 81.7 us a layer with eight
+// throughout, 80.8 with four here.
+__host__ __device__ constexpr int mk_few_in_flight(int M) { return M == 1 ? 4 : MK_IN_FLIGHT; }
 constexpr int MK_MAX_ROWS = 4;
 constexpr int MK_TC_ROWS = 3;                   // rows from which the tensor-core form runs
 constexpr int MK_GROUPS = 4;                    // a slot of weights is the work of one of four groups of four warps
@@ -293,46 +297,6 @@ __device__ __forceinline__ int mk_run_cta(const MkShared *sh, int t)
 }
 // query vectors of a partial
 __device__ __forceinline__ int mk_part_rows(const MkArgs &a) { return a.n_rows * (a.Hq / a.Hkv); }
-
-// Consumers only: wait until every CTA has arrived at this barrier.  A warp whose wait for a ring slot ran out
-// stays until here, without working, because the barriers among the CTA's warps have no time limit;
-// here all of them learn of it and leave together.
-__device__ __forceinline__ bool mk_grid_barrier(const MkArgs &a, MkShared *sh, unsigned long long &epoch)
-{
-    mk_consumer_sync();
-    epoch += gridDim.x;
-    if (threadIdx.x == 0) {
-        // release: everything this CTA wrote (ordered before by the CTA barrier) is visible to
-        // whoever acquires the counter; no value comes back, so nothing waits on the round trip
-        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(a.bar), "l"(1ull) : "memory");
-        unsigned long long t0 = 0;
-        for (uint32_t spin = 0;; ++spin) {
-            if (ld_acquire_u64(a.bar) >= epoch) break;
-            if ((spin & 63u) == 63u) {
-                if (ld_volatile_i32(a.abort_word) || *(volatile int *)&sh->giving_up) {
-                    // this CTA or another (or an earlier launch that was never cleaned up after) gave up:
-                    // leave too, and say so, so that skipping the rest is never silent
-                    sh->giving_up = 1;
-                    atomicOr(a.status, ST_TIMEOUT);
-                    atomicExch(a.abort_word, 1);
-                    break;
-                }
-                const unsigned long long now = global_ns();
-                if (t0 == 0) t0 = now;
-                else if (now - t0 > GM_TIMEOUT_NS) {
-                    sh->giving_up = 1;
-                    atomicOr(a.status, ST_TIMEOUT);
-                    atomicExch(a.abort_word, 1);
-                    break;
-                }
-            }
-        }
-        sh->go_on = !*(volatile int *)&sh->giving_up;
-        if (blockIdx.x == 0 && a.trace) a.trace[(epoch - a.bar_base) / gridDim.x] = global_ns();
-    }
-    mk_consumer_sync();
-    return sh->go_on != 0;  // one answer for all warps
-}
 
 }  // namespace sparsk
 

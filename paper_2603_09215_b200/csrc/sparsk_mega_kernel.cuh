@@ -13,15 +13,16 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
     const int lane = threadIdx.x & 31;
     uint32_t idx = 0;   // ring item
     bool ok = true;
-    // waits until item idx's slot is free and no more than MK_IN_FLIGHT items (counting this one) are on
-    // their way, and announces `bytes`; item idx - MK_IN_FLIGHT was this warp's own
-    static_assert(MK_IN_FLIGHT % MK_PW == 0 && SLOTS % MK_PW == 0, "a producer waits for items of its own");
+    // waits until item idx's slot is free and no more than `flight` items (counting this one) are on
+    // their way, and announces `bytes`; item idx - flight was this warp's own
+    uint32_t flight = mk_few_in_flight(M);
+    static_assert(MK_IN_FLIGHT % MK_PW == 0 && mk_few_in_flight(M) % MK_PW == 0 && SLOTS % MK_PW == 0, "a producer waits for items of its own");
     auto open = [&](uint32_t bytes) {
         const int s = idx % SLOTS;
         int go = 1;
         if (lane == 0) {
-            if (SLOTS > MK_IN_FLIGHT && idx >= MK_IN_FLIGHT) {
-                const uint32_t o = idx - MK_IN_FLIGHT;
+            if (SLOTS > (int)flight && idx >= flight) {
+                const uint32_t o = idx - flight;
                 go = mbar_wait(&sh->full[o % SLOTS], (o / SLOTS) & 1, &sh->giving_up, a.status) ? 1 : 0;
             }
             if (go) go = mbar_wait(&sh->empty[s], ((idx / SLOTS) & 1) ^ 1, &sh->giving_up, a.status) ? 1 : 0;
@@ -32,8 +33,11 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
     };
     auto rows = [&](int type, const MkLayer *L) {
         MkBands w = sh->bands[type == MK_QKV ? 0 : 1];
+        const uint32_t idx0 = idx;
+        flight = mk_few_in_flight(M);
         for (; w.j < w.end; w.j += w.step)
             for (int ks = 0; ks < w.k_steps; ks++, idx++) {
+                if (idx - idx0 == SLOTS && type == MK_MLP) flight = MK_IN_FLIGHT;
                 if ((int)(idx % MK_PW) != p) continue;
                 if (!open(MK_SLOT_BYTES)) return;
                 if (lane < 2) {
@@ -137,13 +141,12 @@ __device__ __forceinline__ void mk_oproj(const MkArgs &a, unsigned char *area, u
 }
 
 template <int M>
-__device__ __forceinline__ void mk_mlp(const MkArgs &a, int l, unsigned char *area, unsigned char *ring, MkShared *sh,
+__device__ __forceinline__ void mk_mlp(const MkArgs &a, int l, const bf16 *gain, unsigned char *area, unsigned char *ring, MkShared *sh,
                                        const MkGains &gains, MkPos<mk_slots(M)> &at)
 {
     const int boxes = (a.d + MK_CBOX_ROWS - 1) / MK_CBOX_ROWS;
     const MkBands w = sh->bands[1];
     if (w.j >= w.end) return;
-    const bf16 *gain = a.layers[l].mlp_gain;
     // columns of the last box that are the next CTA's meet zeros
     if constexpr (M >= MK_TC_ROWS) {
         const int rs = a.cols.most + 8;
@@ -248,9 +251,10 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
         if (blockIdx.x == 0 && threadIdx.x == 0 && a.trace) a.trace[0] = global_ns();
         bool ok = true;
         MkGains gains;
-        gains.load(a.layers[a.layer_begin].attn_gain, a.d);
+        const bf16 *gain = a.layers[a.layer_begin].attn_gain;
+        gains.load(gain, a.d);
         for (int l = a.layer_begin; l < a.layer_end && ok; l++) {
-            const bf16 *gain = a.layers[l].attn_gain;
+            const bf16 *mlp_gain = a.layers[l].mlp_gain;
             if constexpr (TC) {
                 const int whole = (a.d + MK_BOX_COLS - 1) / MK_BOX_COLS * MK_BOX_COLS;
                 mk_rows_tc<M>(MK_QKV, a, l, reinterpret_cast<bf16 *>(area), reinterpret_cast<float *>(area + mk_tc_planes_bytes(M, whole)),
@@ -264,11 +268,10 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
             mk_attention<M, HD>(a, l, area, ring, sh, at);
             if (!(ok = mk_grid_barrier(a, sh, epoch))) break;
             mk_oproj<M, HD>(a, area, ring, sh, at);
-            gains.load(a.layers[l].mlp_gain, a.d);
-            if (!(ok = mk_grid_barrier(a, sh, epoch))) break;
-            mk_mlp<M>(a, l, area, ring, sh, gains, at);
-            if (l + 1 < a.layer_end) gains.load(a.layers[l + 1].attn_gain, a.d);
-            ok = mk_grid_barrier(a, sh, epoch);
+            if (!(ok = mk_grid_barrier(a, sh, epoch, &gains, mlp_gain))) break;
+            mk_mlp<M>(a, l, mlp_gain, area, ring, sh, gains, at);
+            gain = a.layers[min(l + 1, a.layer_end - 1)].attn_gain;
+            ok = mk_grid_barrier(a, sh, epoch, &gains, gain);
         }
         if (ok) mk_fold(a, (int)threadIdx.x, MK_CW * 32);
     }

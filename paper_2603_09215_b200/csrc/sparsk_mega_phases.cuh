@@ -42,6 +42,51 @@ struct MkGains {
     }
 };
 
+// Consumers only: wait until every CTA has arrived at this barrier.  A warp whose wait for a ring slot ran out
+// stays until here, without working, because the barriers among the CTA's warps have no time limit;
+// here all of them learn of it and leave together.  The gains of the norm behind the barrier are asked for between
+// arriving and waiting: a release waits for loads on their way as well.
+__device__ __forceinline__ bool mk_grid_barrier(const MkArgs &a, MkShared *sh, unsigned long long &epoch, MkGains *gains = nullptr,
+                                                const bf16 *gain = nullptr)
+{
+    mk_consumer_sync();
+    epoch += gridDim.x;
+    if (threadIdx.x == 0) {
+        // release: everything this CTA wrote (ordered before by the CTA barrier) is visible to
+        // whoever acquires the counter; no value comes back, so nothing waits on the round trip
+        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(a.bar), "l"(1ull) : "memory");
+    }
+    if (gains) gains->load(gain, a.d);
+    if (threadIdx.x == 0) {
+        unsigned long long t0 = 0;
+        for (uint32_t spin = 0;; ++spin) {
+            if (ld_acquire_u64(a.bar) >= epoch) break;
+            if ((spin & 63u) == 63u) {
+                if (ld_volatile_i32(a.abort_word) || *(volatile int *)&sh->giving_up) {
+                    // this CTA or another (or an earlier launch that was never cleaned up after) gave up:
+                    // leave too, and say so, so that skipping the rest is never silent
+                    sh->giving_up = 1;
+                    atomicOr(a.status, ST_TIMEOUT);
+                    atomicExch(a.abort_word, 1);
+                    break;
+                }
+                const unsigned long long now = global_ns();
+                if (t0 == 0) t0 = now;
+                else if (now - t0 > GM_TIMEOUT_NS) {
+                    sh->giving_up = 1;
+                    atomicOr(a.status, ST_TIMEOUT);
+                    atomicExch(a.abort_word, 1);
+                    break;
+                }
+            }
+        }
+        sh->go_on = !*(volatile int *)&sh->giving_up;
+        if (blockIdx.x == 0 && a.trace) a.trace[(epoch - a.bar_base) / gridDim.x] = global_ns();
+    }
+    mk_consumer_sync();
+    return sh->go_on != 0;  // one answer for all warps
+}
+
 // x = (h + h2) / sqrt(mean((h + h2)^2) + eps) * gain for the M rows, left through put(row, column, four numbers); columns at
 // or beyond K, up to ncols, and rows from n_rows on are zeros.  Rows of up to MK_KEEP float4s per thread stay in
 // registers between the sum of squares and the scaling: one trip to the L2.
