@@ -1021,7 +1021,7 @@ bool use_mega(const sparsk_ctx *c, int n_rows)
     return c->mega && c->mk_ok && c->mk_coop && n_rows >= 1 && n_rows <= c->mk_max_rows && (n_rows < MK_TC_ROWS || c->mk_tc_ok) &&
            c->attn_tma_ok && c->n_sm <= MK_MAX_CTAS &&
            (size_t)MK_MAX_ROWS * c->dm.n_kv_heads * (c->dm.max_seq_len / AT_TP + 1) * MK_MAX_CTAS < (1ull << 31) &&  // (32-bit shares)
-           mk_attn_fits(m, c->dm.n_q_heads / c->dm.n_kv_heads, c->dm.head_dim) &&
+           mk_attn_fits(m, c->dm.n_q_heads / c->dm.n_kv_heads) &&
            (n_rows >= MK_TC_ROWS || mk_act_window(m, m * c->mk_cols16.most * 4 + mk_sums_bytes(m)) >= 1);
 }
 

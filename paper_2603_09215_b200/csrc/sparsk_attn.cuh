@@ -20,7 +20,7 @@
 // sum) per (row, query head, split); a second kernel merges the splits.
 //
 // Two forms of the ring: coalesced 16-byte cp.async copies into padded rows (callers that pass
-// plain cache pointers: the stand-alone entry points, the persistent kernel), or one TMA box per
+// plain cache pointers: the stand-alone entry points), or one TMA box per
 // tile and matrix with the 128-byte swizzle and an mbarrier per stage (the decode path, which
 // holds tensor maps of its cache).  Two forms of an item: the one above, and a transposed one for
 // groups of at most eight query vectors (a single row at up to eight query heads per kv head),
@@ -445,13 +445,10 @@ struct AtCells {
 // One item, by one warp: query vectors [16 qb, 16 qb + 16) of a group (rows row0 .. row0 + nrows - 1
 // of slot `slot`, the first at position pos0) and kv head hk, over the tiles that `ring` (already
 // started) delivers, none of whose positions from w_end on counts.  Leaves the item's partial in `cells`.
-// QREG: the query fragments stay in registers for the whole item (32 registers at head dimension
-// 128); otherwise they are parked in `qs` ([16][HD + 8] of shared memory) and re-read per tile,
-// for callers whose register budget is spoken for.
-template <int HD, bool QREG, class Ring, class Cells>
-__device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, Ring &ring, const Cells &cells, kv_t *qs, int lane)
+// The query fragments stay in registers for the whole item (32 registers at head dimension 128).
+template <int HD, class Ring, class Cells>
+__device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, Ring &ring, const Cells &cells, int lane)
 {
-    constexpr int KP = HD + 8;      // padded row of the parked queries: ldmatrix rows fall into distinct banks
     constexpr float LOG2E = 1.4426950408889634f, LN2 = 0.6931471805599453f;
     const int G = a.Hq / a.Hkv;
     const int qb = it.qb, hk = it.hk, row0 = it.row0, pos0 = it.pos0;
@@ -461,7 +458,7 @@ __device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, R
 
     // the queries, as A fragments (row = lane / 4 and + 8, columns 2 (lane % 4) + {0, 1, 8, 9} of
     // every 16-column step), while the first tiles are on their way
-    uint32_t qa[QREG ? HD / 16 : 1][4];
+    uint32_t qa[HD / 16][4];
     const float qscale = rsqrtf((float)HD) * LOG2E;
     {
         const int qi0 = lane >> 2, qi1 = qi0 + 8, c0 = (lane & 3) * 2;
@@ -497,16 +494,8 @@ __device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, R
             }
             const uint32_t f0 = pack_h2(x00.x * qscale, x00.y * qscale), f1 = pack_h2(x10.x * qscale, x10.y * qscale);
             const uint32_t f2 = pack_h2(x01.x * qscale, x01.y * qscale), f3 = pack_h2(x11.x * qscale, x11.y * qscale);
-            if (QREG) {
-                qa[ks][0] = f0; qa[ks][1] = f1; qa[ks][2] = f2; qa[ks][3] = f3;
-            } else {
-                *reinterpret_cast<uint32_t *>(&qs[qi0 * KP + ks * 16 + c0]) = f0;
-                *reinterpret_cast<uint32_t *>(&qs[qi1 * KP + ks * 16 + c0]) = f1;
-                *reinterpret_cast<uint32_t *>(&qs[qi0 * KP + ks * 16 + c0 + 8]) = f2;
-                *reinterpret_cast<uint32_t *>(&qs[qi1 * KP + ks * 16 + c0 + 8]) = f3;
-            }
+            qa[ks][0] = f0; qa[ks][1] = f1; qa[ks][2] = f2; qa[ks][3] = f3;
         }
-        if (!QREG) __syncwarp();
     }
 
     float o[HD / 8][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
@@ -540,21 +529,10 @@ __device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, R
             const int krow = (lane & 7) + ((lane >> 4) << 3), kch = (lane >> 3) & 1;
             ldsm_x4(kb, &Kt[Ring::off(krow, ks * 2 + kch)]);
             ldsm_x4(kb2, &Kt[Ring::off(krow, (ks + 1) * 2 + kch)]);
-            if (QREG) {
-                mma_f16(s[0], qa[ks], kb[0], kb[1]);
-                mma_f16(s[1], qa[ks], kb[2], kb[3]);
-                mma_f16(s2[0], qa[ks + 1], kb2[0], kb2[1]);
-                mma_f16(s2[1], qa[ks + 1], kb2[2], kb2[3]);
-            } else {
-                uint32_t q1[4], q2[4];
-                const int qoff = ((lane & 7) + ((lane >> 3) & 1) * 8) * KP + (lane >> 4) * 8;
-                ldsm_x4(q1, &qs[qoff + ks * 16]);
-                ldsm_x4(q2, &qs[qoff + (ks + 1) * 16]);
-                mma_f16(s[0], q1, kb[0], kb[1]);
-                mma_f16(s[1], q1, kb[2], kb[3]);
-                mma_f16(s2[0], q2, kb2[0], kb2[1]);
-                mma_f16(s2[1], q2, kb2[2], kb2[3]);
-            }
+            mma_f16(s[0], qa[ks], kb[0], kb[1]);
+            mma_f16(s[1], qa[ks], kb[2], kb[3]);
+            mma_f16(s2[0], qa[ks + 1], kb2[0], kb2[1]);
+            mma_f16(s2[1], qa[ks + 1], kb2[2], kb2[3]);
         }
         // online softmax; P as the A operand of the second product.  A tile wholly inside what
         // every query vector of the item may see (all but the last of an item) needs no masking;
@@ -635,7 +613,7 @@ __device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, R
     }
 }
 
-// One item of at most eight query vectors, by one warp, in the transposed form: with few query
+// One item of at most eight query vectors (block it.qb of a group's), by one warp, in the transposed form: with few query
 // heads per kv head (a single row of a group) the sixteen-row M dimension of the form above is
 // half empty, so here the POSITIONS are the M dimension.  S^T = K Q^T (K tile as the A operand,
 // the queries as eight B columns, 16 registers for the whole item), the softmax runs down the
@@ -649,7 +627,7 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
     constexpr float LOG2E = 1.4426950408889634f, LN2 = 0.6931471805599453f;
     const int G = a.Hq / a.Hkv;
     const int hk = it.hk, row0 = it.row0, pos0 = it.pos0, w_end = it.w_end;
-    const int nq = it.nq;  // <= 8
+    const int q0 = it.qb * 8, nq = it.nq - q0;  // query vectors q0 .. q0 + min(nq, 8) - 1 of the group
 
     // the queries as B fragments: column lane / 4, elements 2 (lane % 4) + {0, 1, 8, 9} of every
     // 16-element step, scaled by log2(e) / sqrt(hd)
@@ -657,7 +635,7 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
     {
         const int qi = lane >> 2, c0 = (lane & 3) * 2;
         const bool have = qi < nq;
-        const size_t o = (size_t)(row0 + (have ? qi / G : 0)) * a.Hq * HD + (hk * G + (have ? qi % G : 0)) * HD + c0;
+        const size_t o = (size_t)(row0 + (have ? (q0 + qi) / G : 0)) * a.Hq * HD + (hk * G + (have ? (q0 + qi) % G : 0)) * HD + c0;
         const float qscale = rsqrtf((float)HD) * LOG2E;
 #pragma unroll
         for (int ks = 0; ks < HD / 16; ks++) {
@@ -682,8 +660,9 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
 #pragma unroll
     for (int e = 0; e < 2; e++) {
         const int qi = (lane & 3) * 2 + e;
-        limit[e] = qi < nq ? pos0 + qi / G : -1;
+        limit[e] = qi < nq ? pos0 + (q0 + qi) / G : -1;
     }
+    const int lim_min = pos0 + q0 / G;  // the smallest of all
     float o[HD / 16][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
 #pragma unroll
     for (int mt = 0; mt < HD / 16; mt++)
@@ -705,7 +684,7 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
             mma_f16(s1, kb, qf[ks + 1][0], qf[ks + 1][1]);
         }
         // online softmax down the columns; accumulator rows are positions lane / 4 and + 8
-        const bool full = p0 + AT_TP <= w_end && p0 + AT_TP - 1 <= pos0;
+        const bool full = p0 + AT_TP <= w_end && p0 + AT_TP - 1 <= lim_min;
         float pv[2][2], alpha[2];
 #pragma unroll
         for (int e = 0; e < 2; e++) {
@@ -762,8 +741,8 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
         l += __shfl_xor_sync(0xffffffffu, l, 16);
         const int qi = (lane & 3) * 2 + e;
         if (qi < nq) {
-            if ((lane >> 2) == 0) *cells.ml(qi) = make_float2(m_run[e] * LN2, l);
-            float *po = cells.o(qi) + (lane >> 2);
+            if ((lane >> 2) == 0) *cells.ml(q0 + qi) = make_float2(m_run[e] * LN2, l);
+            float *po = cells.o(q0 + qi) + (lane >> 2);
 #pragma unroll
             for (int mt = 0; mt < HD / 16; mt++) {
                 po[mt * 16] = o[mt][e];
@@ -786,7 +765,7 @@ __device__ __forceinline__ void attn_split_item(const AttnArgs &a, const AtItem 
     AtRing<HD, NS, TMA> ring(a, it, wr, lane, tm);
     ring.start();
     if (it.nq <= 8) attn_item_t<HD>(a, it, ring, cells, lane);
-    else attn_item<HD, true>(a, it, ring, cells, nullptr, lane);
+    else attn_item<HD>(a, it, ring, cells, lane);
 }
 
 // Persistent grid of warps; item i = ((sp * groups + g) * Hkv + hk) * n_qblk + qb: the query

@@ -66,12 +66,12 @@ constexpr int MK_MAX_ROWS = 4;
 constexpr int MK_TC_ROWS = 3;                   // rows from which the tensor-core form runs
 constexpr int MK_GROUPS = 4;                    // a slot of weights is the work of one of four groups of four warps
 constexpr int MK_MAX_CTAS = 192;                // bounds the number of attention partials
-constexpr int MK_SHARED_BYTES = 2560;           // MkShared, behind the area, with two to four rows
+constexpr int MK_SHARED_BYTES = 2688;           // MkShared, behind the area, with two to four rows
 constexpr int MK_SHARED_FEW_BYTES = 1536;       // the part of it that one row needs
 
 // The ring, then the area: the activations of a row-form phase (M rows; with one or two rows, when they
 // do not fit whole, a window of k-steps that is reloaded as the phase moves along) and what the CTA's
-// own bands make of them, or the attention's parked queries and partials, or the merged heads.
+// own bands make of them, or the attention's partials, or the merged heads.
 // Several rows' activations need the larger area.  A multiple of four slots: a weight slot always belongs
 // to the same four warps, so that nobody waits for a slot's next fill before its present one has landed.
 __host__ __device__ constexpr int mk_slots(int M) { return M >= 2 ? 8 : 12; }
@@ -214,7 +214,7 @@ struct MkHeads {
 struct MkRun {
     int g, hk, tile0, n;            // group, kv head, first tile, tiles
     int row0, nrows, pos0, cache0;  // the group's rows; first cache row of (slot, kv head)
-    int nq, n_qblk;                 // query vectors, blocks of sixteen of them
+    int nq, n_qblk;                 // query vectors, blocks of eight of them
 };
 // What a row of weights of the q/k/v projection becomes: a rotary pair of q or k, or two numbers of v.
 struct MkFin {
@@ -222,6 +222,7 @@ struct MkFin {
     size_t off;     // of the first number, the second is `second` behind it
     int second, kind;
 };
+constexpr int MK_RUNS = 4;
 enum { MK_FIN_Q = 0, MK_FIN_K, MK_FIN_V, MK_FIN_NONE };
 // The partials of one (row, query head): those of the CTAs [cf, cl], `cell0` plus the CTA's number times mk_part_rows.
 struct MkMerge {
@@ -239,7 +240,8 @@ struct MkShared {
     int att_base[MK_MAX_ROWS + 1];       // tiles x kv heads of the groups before this one
     int att_ctas;                        // CTAs that the tiles are dealt to: none of them goes without
     int att_t0, att_t1;                  // this CTA's share of them
-    MkRun run0;                          // its first run
+    int att_batch;                       // runs below when they are all of the share and are worked on side by side, or 0
+    MkRun runs[MK_RUNS];                 // its first runs
     MkBands bands[2];                    // this CTA's bands of q/k/v and of gate/up
     MkHeads heads;                       // and of the O-projection
     int head0;                           // first head of those
@@ -288,7 +290,7 @@ __device__ __forceinline__ void mk_run_at(const MkArgs &a, const MkShared *sh, i
     r.pos0 = sh->row_pos[r.row0];
     r.cache0 = (sh->row_slot[r.row0] * a.Hkv + r.hk) * a.S;
     r.nq = r.nrows * (a.Hq / a.Hkv);
-    r.n_qblk = (r.nq + 15) / 16;
+    r.n_qblk = (r.nq + 7) / 8;
 }
 // CTA whose share holds tile t
 __device__ __forceinline__ int mk_run_cta(const MkShared *sh, int t)

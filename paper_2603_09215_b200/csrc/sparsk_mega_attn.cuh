@@ -4,7 +4,7 @@
 namespace sparsk {
 
 // A warp's view of a run's ring items: items sub, sub + nsub, ... of the run, two 16-position tiles each (K and
-// V, with the 128-byte swizzle, as the producers' TMA copies leave them), in the form attn_item asks for.
+// V, with the 128-byte swizzle, as the producers' TMA copies leave them), in the form attn_item_t asks for.
 // The tiles were on their way before this launch's q/k/v projection had written the current rows' keys and
 // values: those rows are copied over from the cache, and value rows past the end are cleared (they meet a
 // weight of exactly zero, which must not meet a NaN).  Every warp that reads a tile does both for itself.
@@ -69,20 +69,16 @@ struct MkCells {
     __device__ __forceinline__ float *o(int qg) const { return po + (ptrdiff_t)qg * HD; }
     __device__ __forceinline__ float2 *ml(int qg) const { return pml + qg; }
 };
-// Parked queries of one block of sixteen; one warp's partial of such a block and its sums.
+// One warp's partial of a block of eight query vectors and its sums.
 template <int HD>
-__host__ __device__ constexpr int mk_park_bytes() { return 16 * (HD + 8) * 2; }
-template <int HD>
-__host__ __device__ constexpr int mk_cell_bytes() { return 16 * HD * 4 + 16 * 8; }
-// Shapes the phase can run: a warp and a place for its queries per block of query vectors of a group.
-inline bool mk_attn_fits(int M, int G, int head_dim)
-{
-    const int blocks = (M * G + 15) / 16;
-    return blocks <= MK_CW && blocks * (head_dim == 128 ? mk_park_bytes<128>() : mk_park_bytes<64>()) <= mk_area_bytes(M);
-}
+__host__ __device__ constexpr int mk_cell_bytes() { return 8 * HD * 4 + 8 * 8; }
+// Shapes the phase can run: a warp per block of query vectors of a group.
+inline bool mk_attn_fits(int M, int G) { return (M * G + 7) / 8 <= MK_CW; }
 
-// The CTA's runs, one after another.  Up to four warps per block of sixteen query vectors share a run (as many as the area
-// has room for partials), every nsub-th slot each; their partials meet in the area.
+// The CTA's runs, one after another.  Up to four warps per block of eight query vectors share a run (as many as the area
+// has room for partials, and two slots at least each), every nsub-th slot each; their partials meet in the area.
+// (Blocks of sixteen, positions as columns, cost 450 bytes of spills, and a reload behind a grid barrier is a trip to the L2: flushes of
+// four rows of the 28-layer shape 96.6 us a layer, so 90.9.)  Short runs go side by side, a warp per block.
 template <int M, int HD>
 __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned char *area, unsigned char *ring, MkShared *sh,
                                              MkPos<mk_slots(M)> &at)
@@ -93,58 +89,83 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
     aa.q32 = a.q_buf; aa.Hq = a.Hq; aa.Hkv = a.Hkv;
     const int stride = mk_part_rows(a), end = sh->att_t1;
     int t = sh->att_t0;
-    MkRun r = sh->run0;
+    MkRun r = sh->runs[0];
+    const int batch = M == 1 ? 0 : sh->att_batch; // (one row has one group: its runs are long or alone)
     while (t < end) {
-        const int nq = r.nq, n_qblk = r.n_qblk, n_items = (r.n + 1) / 2;
-        int nsub = min(4, n_items);
-        if (nsub > 1) {
-            const int room = (mk_area_bytes(M) - n_qblk * mk_park_bytes<HD>()) / (n_qblk * mk_cell_bytes<HD>());
-            nsub = max(1, min(nsub, min(MK_CW / n_qblk, room)));
+        int n_items = (r.n + 1) / 2, nsub = 1, sub = 0, qb = warp, before = 0;  // items before this warp's run
+        if (M > 1 && batch > 1) {
+            // (no more slots than the ring has, so none of them is filled twice before the warps meet again)
+            static_assert(2 * MK_RUNS <= SLOTS, "slots of a batch");
+            int mine = -1, w0 = 0;
+            n_items = 0;
+            for (int i = 0; i < batch; i++) {
+                const int nb = sh->runs[i].n_qblk;
+                if (warp >= w0 && warp < w0 + nb) {
+                    mine = i;
+                    qb = warp - w0;
+                    before = n_items;
+                }
+                w0 += nb;
+                n_items += (sh->runs[i].n + 1) / 2;
+            }
+            if (mine >= 0) r = sh->runs[mine];
+            else sub = 1;
+        } else {
+            nsub = min(4, (n_items + 1) / 2);
+            if (nsub > 1) {
+                const int room = mk_area_bytes(M) / (r.n_qblk * mk_cell_bytes<HD>());
+                nsub = max(1, min(nsub, min(MK_CW / r.n_qblk, room)));
+            }
+            if (SLOTS % nsub) nsub = 2;  // a slot's successive fills stay with one warp
+            if (r.n_qblk > 1) {
+                sub = warp / r.n_qblk;
+                qb = warp - sub * r.n_qblk;
+            } else {
+                sub = warp;
+                qb = 0;
+            }
         }
-        if (SLOTS % nsub) nsub = 2;  // a slot's successive fills stay with one warp
-        const int sub = n_qblk == 1 ? warp : warp / n_qblk, qb = warp - sub * n_qblk;
-        // (the warps of a block all park its queries, the same numbers in the same place)
-        kv_t *park = reinterpret_cast<kv_t *>(area) + (size_t)qb * 16 * (HD + 8);
-        unsigned char *cells = area + n_qblk * mk_park_bytes<HD>();
+        const int nq = r.nq, n_qblk = r.n_qblk, run_items = (r.n + 1) / 2;
         const size_t part = (size_t)(blockIdx.x + r.g * a.Hkv + r.hk) * stride;
         if (sub < nsub) {
             AtItem item;
             item.qb = qb; item.hk = r.hk; item.row0 = r.row0; item.nrows = r.nrows; item.pos0 = r.pos0; item.nq = nq;
-            item.w_end = min(r.pos0 + (r.nrows == 1 ? 0 : (min(qb * 16 + 16, nq) - 1) / G) + 1, a.S);
+            item.w_end = min(r.pos0 + (r.nrows == 1 ? 0 : (min(qb * 8 + 8, nq) - 1) / G) + 1, a.S);
             MkTiles<HD, SLOTS> tiles;
             tiles.ring = ring; tiles.sh = sh; tiles.status = a.status;
             tiles.kbase = a.kc + l * a.kv_layer + (size_t)r.cache0 * HD; tiles.vbase = a.vc + l * a.kv_layer + (size_t)r.cache0 * HD;
-            tiles.at0 = at; tiles.tile0 = r.tile0; tiles.sub = sub; tiles.nsub = nsub;
+            tiles.at0 = at;
+            tiles.at0.skip_many(before);
+            tiles.tile0 = r.tile0; tiles.sub = sub; tiles.nsub = nsub;
             tiles.new0 = r.pos0; tiles.end = min(r.pos0 + r.nrows, a.S);
             tiles.arrivals = qb == 0 ? MK_CW - (n_qblk - 1) : 1;
-            const int mine = nsub == 1 ? n_items : (n_items - sub + nsub - 1) / nsub;
-            tiles.n_tiles = 2 * mine - ((r.n & 1) && sub + nsub * (mine - 1) == n_items - 1 ? 1 : 0);
+            const int mine = nsub == 1 ? run_items : (run_items - sub + nsub - 1) / nsub;
+            tiles.n_tiles = 2 * mine - ((r.n & 1) && sub + nsub * (mine - 1) == run_items - 1 ? 1 : 0);
             tiles.lane = lane;
             MkCells<HD> out;
             if (nsub > 1) {
-                // query vector qg of block qb at row qg - 16 qb of the warp's cells
-                unsigned char *c = cells + (size_t)(sub * n_qblk + qb) * mk_cell_bytes<HD>();
-                out.po = reinterpret_cast<float *>(c) - (ptrdiff_t)qb * 16 * HD;
-                out.pml = reinterpret_cast<float2 *>(c + 16 * HD * 4) - qb * 16;
+                // query vector qg of block qb at row qg - 8 qb of the warp's cells
+                unsigned char *c = area + (size_t)(sub * n_qblk + qb) * mk_cell_bytes<HD>();
+                out.po = reinterpret_cast<float *>(c) - (ptrdiff_t)qb * 8 * HD;
+                out.pml = reinterpret_cast<float2 *>(c + 8 * HD * 4) - qb * 8;
             } else {
                 out.po = a.part_o + part * HD;
                 out.pml = a.part_ml + part;
             }
-            if (nq <= 8) attn_item_t<HD>(aa, item, tiles, out, lane);
-            else attn_item<HD, false>(aa, item, tiles, out, park, lane);
+            attn_item_t<HD>(aa, item, tiles, out, lane);
         }
         at.skip_many(n_items);
         mk_consumer_sync();
         if (nsub > 1) {
             for (int k = threadIdx.x; k < nq * (HD / 4); k += MK_CW * 32) {
-                const int qg = k / (HD / 4), c4 = k % (HD / 4), blk = qg / 16, ql = qg % 16;
+                const int qg = k / (HD / 4), c4 = k % (HD / 4), blk = qg / 8, ql = qg % 8;
                 float mx = -INFINITY, sum = 0.f;
                 float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
                 for (int s = 0; s < nsub; s++)
-                    mx = fmaxf(mx, reinterpret_cast<const float2 *>(cells + (size_t)(s * n_qblk + blk) * mk_cell_bytes<HD>() + 16 * HD * 4)[ql].x);
+                    mx = fmaxf(mx, reinterpret_cast<const float2 *>(area + (size_t)(s * n_qblk + blk) * mk_cell_bytes<HD>() + 8 * HD * 4)[ql].x);
                 for (int s = 0; s < nsub; s++) {
-                    const unsigned char *c = cells + (size_t)(s * n_qblk + blk) * mk_cell_bytes<HD>();
-                    const float2 ml = reinterpret_cast<const float2 *>(c + 16 * HD * 4)[ql];
+                    const unsigned char *c = area + (size_t)(s * n_qblk + blk) * mk_cell_bytes<HD>();
+                    const float2 ml = reinterpret_cast<const float2 *>(c + 8 * HD * 4)[ql];
                     const float w = ml.x == -INFINITY ? 0.f : __expf(ml.x - mx);
                     const float4 p = reinterpret_cast<const float4 *>(c)[ql * (HD / 4) + c4];
                     sum += ml.y * w;
@@ -155,6 +176,7 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
             }
             mk_consumer_sync();  // the next run may use the area
         }
+        if (batch > 1) break;
         t += r.n;
         if (t < end) mk_run_at(a, sh, t, end, r);
     }

@@ -68,7 +68,7 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
         const MkLayer *L = a.layers + l;
         rows(MK_QKV, L);
         if (!ok) break;
-        MkRun r = sh->run0;
+        MkRun r = sh->runs[0];
         for (int t = sh->att_t0; ok && t < sh->att_t1;) {
             if (t != sh->att_t0) mk_run_at(a, sh, t, sh->att_t1, r);
             t += r.n;
@@ -228,7 +228,17 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
             sh->att_ctas = (int)n;
             sh->att_t0 = c < n ? (int)(c * (unsigned)base / n) : 0;
             sh->att_t1 = c < n ? (int)((c + 1) * (unsigned)base / n) : 0;
-            if (sh->att_t0 < sh->att_t1) mk_run_at(a, sh, sh->att_t0, sh->att_t1, sh->run0);
+            // short runs (a slot or two each, a warp per block of query vectors) go side by side
+            int t = sh->att_t0, k = 0, warps = 0;
+            bool small = true;
+            for (; k < (M == 1 ? 1 : MK_RUNS) && t < sh->att_t1 && (k == 0 || small); k++) {
+                MkRun &r = sh->runs[k];
+                mk_run_at(a, sh, t, sh->att_t1, r);
+                t += r.n;
+                warps += r.n_qblk;
+                small = small && r.n <= 4 && warps <= MK_CW;
+            }
+            sh->att_batch = small && t >= sh->att_t1 ? k : 0;
             sh->bands[0].init(MK_QKV, a);
             sh->bands[1].init(MK_MLP, a);
             sh->heads.init(a);
