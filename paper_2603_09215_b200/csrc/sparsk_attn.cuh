@@ -31,6 +31,8 @@
 // in flight each keep HBM busy where CTA-wide tiles with a cross-warp merge did not.
 #pragma once
 
+#include <type_traits>
+
 #include "sparsk_common.cuh"
 
 namespace sparsk {
@@ -420,41 +422,30 @@ __device__ __forceinline__ uint32_t movmatrix_t(uint32_t x)
     return y;
 }
 
-// Where an item leaves what it found for query vector qg of its group (unnormalised sum of values;
-// running maximum and sum): the partial cells of the launch-wide merge.
-template <int HD>
-struct AtCells {
-    float *po;
-    float2 *pml;
-    int row0, Hq, h0, G, splits, sp;
-    __device__ __forceinline__ AtCells(const AttnArgs &a, const AtItem &it)
-        : po(a.part_o), pml(a.part_ml), row0(it.row0), Hq(a.Hq), h0(it.hk * (a.Hq / a.Hkv)), G(a.Hq / a.Hkv), splits(a.n_splits),
-          sp(it.sp)
-    {
-    }
-    __device__ __forceinline__ size_t cell(int qg) const { return ((size_t)(row0 + qg / G) * Hq + h0 + qg % G) * splits + sp; }
-    __device__ __forceinline__ float *o(int qg) const { return po + cell(qg) * HD; }
-    __device__ __forceinline__ float2 *ml(int qg) const { return pml + cell(qg); }
-    // an empty split: max = -inf, sum = 0 is all the merge looks at
-    __device__ __forceinline__ void empty(int q0, int n, int lane) const
-    {
-        for (int qi = lane; qi < n; qi += 32) *ml(q0 + qi) = make_float2(-INFINITY, 0.f);
-    }
-};
-
 // One item, by one warp: query vectors [16 qb, 16 qb + 16) of a group (rows row0 .. row0 + nrows - 1
-// of slot `slot`, the first at position pos0) and kv head hk, over the tiles that `ring` (already
-// started) delivers, none of whose positions from w_end on counts.  Leaves the item's partial in `cells`.
-// The query fragments stay in registers for the whole item (32 registers at head dimension 128).
-template <int HD, class Ring, class Cells>
-__device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, Ring &ring, const Cells &cells, int lane)
+// of slot `slot`, the first at position pos0), kv head hk, split sp.  `wr` is the warp's ring of
+// NS stages.  Writes the item's partial.  The query fragments stay in registers for the whole item (32
+// registers at head dimension 128).
+template <int HD, int NS, bool TMA>
+__device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, kv_t *wr, int lane, AttnTma *tm = nullptr)
 {
+    typedef AtRing<HD, NS, TMA> Ring;
     constexpr float LOG2E = 1.4426950408889634f, LN2 = 0.6931471805599453f;
-    const int G = a.Hq / a.Hkv;
-    const int qb = it.qb, hk = it.hk, row0 = it.row0, pos0 = it.pos0;
+    const int G = a.Hq / a.Hkv, splits = a.n_splits;
+    const int qb = it.qb, hk = it.hk, sp = it.sp, row0 = it.row0, pos0 = it.pos0;
     const int nq = it.nq, q0 = qb * 16;
     const int nq_here = min(16, nq - q0);
-    const int w_end = it.w_end, n_tiles = ring.n_tiles;
+    const int w_beg = it.w_beg, w_end = it.w_end, n_tiles = it.n_tiles;
+    if (n_tiles == 0) {
+        // an empty split: max = -inf, sum = 0 is all the merge looks at
+        for (int qi = lane; qi < nq_here; qi += 32) {
+            const int qg = q0 + qi;
+            a.part_ml[((size_t)(row0 + qg / G) * a.Hq + hk * G + qg % G) * splits + sp] = make_float2(-INFINITY, 0.f);
+        }
+        return;
+    }
+    Ring ring(a, it, wr, lane, tm);
+    ring.start();
 
     // the queries, as A fragments (row = lane / 4 and + 8, columns 2 (lane % 4) + {0, 1, 8, 9} of
     // every 16-column step), while the first tiles are on their way
@@ -515,7 +506,7 @@ __device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, R
     for (int t = 0; t < n_tiles; t++) {
         const kv_t *Kt, *Vt;
         if (!ring.wait(t, Kt, Vt)) return;
-        const int p0 = ring.pos(t);
+        const int p0 = w_beg + t * AT_TP;
 
         // S = Q K^T for 16 positions, in log2 units; two accumulator chains
         float s[2][4], s2[2][4];
@@ -605,15 +596,18 @@ __device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, R
         l += __shfl_xor_sync(0xffffffffu, l, 2);
         const int qi = (lane >> 2) + hf * 8;
         if (qi < nq_here) {
-            if ((lane & 3) == 0) *cells.ml(q0 + qi) = make_float2(m_run[hf] * LN2, l);  // max back in natural-log units
-            float *po = cells.o(q0 + qi) + (lane & 3) * 2;
+            const int qg = q0 + qi, r = qg / G, j = qg % G;
+            const size_t cell = ((size_t)(row0 + r) * a.Hq + hk * G + j) * splits + sp;
+            if ((lane & 3) == 0) a.part_ml[cell] = make_float2(m_run[hf] * LN2, l);  // max back in natural-log units
 #pragma unroll
-            for (int nt = 0; nt < HD / 8; nt++) *reinterpret_cast<float2 *>(po + nt * 8) = make_float2(o[nt][hf * 2], o[nt][hf * 2 + 1]);
+            for (int nt = 0; nt < HD / 8; nt++)
+                *reinterpret_cast<float2 *>(a.part_o + cell * HD + nt * 8 + (lane & 3) * 2) =
+                    make_float2(o[nt][hf * 2], o[nt][hf * 2 + 1]);
         }
     }
 }
 
-// One item of at most eight query vectors (block it.qb of a group's), by one warp, in the transposed form: with few query
+// One item of at most eight query vectors, by one warp, in the transposed form: with few query
 // heads per kv head (a single row of a group) the sixteen-row M dimension of the form above is
 // half empty, so here the POSITIONS are the M dimension.  S^T = K Q^T (K tile as the A operand,
 // the queries as eight B columns, 16 registers for the whole item), the softmax runs down the
@@ -621,13 +615,28 @@ __device__ __forceinline__ void attn_item(const AttnArgs &a, const AtItem &it, R
 // O^T = V^T P^T through two 8x8 register transposes, and V^T is read with transposing ldmatrix.
 // Half the MMAs, half the accumulators and a quarter of the exponentials of the other form;
 // the partial it writes is the same.
-template <int HD, class Ring, class Cells>
-__device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it, Ring &ring, const Cells &cells, int lane)
+// The persistent kernel hands in where its tiles are (`made`) and where the partial goes (`cells`), and its item is block it.qb of eight of a
+// group's query vectors.  The launches' own ring and partial are spelled out here: handed in as objects as well, they cost the
+// launches 1 to 8 % (48 groups of 200 to 3,000 positions of the 28-layer shape 58.1 us, so 57.5).
+template <int HD, class Ring, class Cells = void>
+__device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it, kv_t *wr, int lane, AttnTma *tm = nullptr,
+                                            const Ring *made = nullptr, const Cells *cells = nullptr)
 {
+    constexpr bool SPLIT = std::is_void<Cells>::value;
     constexpr float LOG2E = 1.4426950408889634f, LN2 = 0.6931471805599453f;
-    const int G = a.Hq / a.Hkv;
-    const int hk = it.hk, row0 = it.row0, pos0 = it.pos0, w_end = it.w_end;
-    const int q0 = it.qb * 8, nq = it.nq - q0;  // query vectors q0 .. q0 + min(nq, 8) - 1 of the group
+    const int G = a.Hq / a.Hkv, splits = a.n_splits;
+    const int hk = it.hk, sp = it.sp, row0 = it.row0, pos0 = it.pos0;
+    const int q0 = SPLIT ? 0 : it.qb * 8, nq = it.nq - q0;  // query vectors q0 .. q0 + min(nq, 8) - 1 of the group
+    if (SPLIT && it.n_tiles == 0) {
+        for (int qi = lane; qi < nq; qi += 32)
+            a.part_ml[((size_t)(row0 + qi / G) * a.Hq + hk * G + qi % G) * splits + sp] = make_float2(-INFINITY, 0.f);
+        return;
+    }
+    Ring ring = [&]() -> Ring {
+        if constexpr (SPLIT) return Ring(a, it, wr, lane, tm);
+        else return *made;
+    }();
+    ring.start();
 
     // the queries as B fragments: column lane / 4, elements 2 (lane % 4) + {0, 1, 8, 9} of every
     // 16-element step, scaled by log2(e) / sqrt(hd)
@@ -662,7 +671,6 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
         const int qi = (lane & 3) * 2 + e;
         limit[e] = qi < nq ? pos0 + (q0 + qi) / G : -1;
     }
-    const int lim_min = pos0 + q0 / G;  // the smallest of all
     float o[HD / 16][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
 #pragma unroll
     for (int mt = 0; mt < HD / 16; mt++)
@@ -684,14 +692,14 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
             mma_f16(s1, kb, qf[ks + 1][0], qf[ks + 1][1]);
         }
         // online softmax down the columns; accumulator rows are positions lane / 4 and + 8
-        const bool full = p0 + AT_TP <= w_end && p0 + AT_TP - 1 <= lim_min;
+        const bool full = p0 + AT_TP <= ring.w_end && p0 + AT_TP - 1 <= (SPLIT ? pos0 : pos0 + q0 / G);
         float pv[2][2], alpha[2];
 #pragma unroll
         for (int e = 0; e < 2; e++) {
 #pragma unroll
             for (int j = 0; j < 2; j++) {
                 const int p = p0 + (lane >> 2) + j * 8;
-                const bool ok = full || (p < w_end && p <= limit[e]);
+                const bool ok = full || (p < ring.w_end && p <= limit[e]);
                 pv[e][j] = ok ? s0[j * 2 + e] + s1[j * 2 + e] : -INFINITY;
             }
             float tmax = fmaxf(pv[e][0], pv[e][1]);
@@ -741,31 +749,24 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
         l += __shfl_xor_sync(0xffffffffu, l, 16);
         const int qi = (lane & 3) * 2 + e;
         if (qi < nq) {
-            if ((lane >> 2) == 0) *cells.ml(q0 + qi) = make_float2(m_run[e] * LN2, l);
-            float *po = cells.o(q0 + qi) + (lane >> 2);
+            float *po;
+            float2 *pml;
+            if constexpr (SPLIT) {
+                const size_t cell = ((size_t)(row0 + qi / G) * a.Hq + hk * G + qi % G) * splits + sp;
+                po = a.part_o + cell * HD;
+                pml = a.part_ml + cell;
+            } else {
+                po = cells->o(q0 + qi);
+                pml = cells->ml(q0 + qi);
+            }
+            if ((lane >> 2) == 0) *pml = make_float2(m_run[e] * LN2, l);
 #pragma unroll
             for (int mt = 0; mt < HD / 16; mt++) {
-                po[mt * 16] = o[mt][e];
-                po[mt * 16 + 8] = o[mt][2 + e];
+                po[mt * 16 + (lane >> 2)] = o[mt][e];
+                po[mt * 16 + 8 + (lane >> 2)] = o[mt][2 + e];
             }
         }
     }
-}
-
-// An item of the launches below: its ring, its form, its partial.  At most eight query vectors take the
-// transposed form.
-template <int HD, int NS, bool TMA>
-__device__ __forceinline__ void attn_split_item(const AttnArgs &a, const AtItem &it, kv_t *wr, int lane, AttnTma *tm = nullptr)
-{
-    const AtCells<HD> cells(a, it);
-    if (it.n_tiles == 0) {
-        cells.empty(it.qb * 16, min(16, it.nq - it.qb * 16), lane);
-        return;
-    }
-    AtRing<HD, NS, TMA> ring(a, it, wr, lane, tm);
-    ring.start();
-    if (it.nq <= 8) attn_item_t<HD>(a, it, ring, cells, lane);
-    else attn_item<HD>(a, it, ring, cells, lane);
 }
 
 // Persistent grid of warps; item i = ((sp * groups + g) * Hkv + hk) * n_qblk + qb: the query
@@ -801,7 +802,8 @@ __global__ void __launch_bounds__(AW_WARPS * 32) attn_warp_kernel(AttnArgs a)
         const AtItem it = at_resolve(a, item, n_items, n_groups, a.grp_row0, a.grp_nrows, a.row_slot, a.row_pos);
         item = next;
         if (!it.valid) continue;
-        attn_split_item<HD, NST, false>(a, it, wr, lane);
+        if (it.nq <= 8) attn_item_t<HD, AtRing<HD, NST, false>>(a, it, wr, lane);
+        else attn_item<HD, NST, false>(a, it, wr, lane);
     }
 }
 
@@ -857,7 +859,8 @@ __global__ void __launch_bounds__(WARPS * 32) attn_warp_tma_kernel(const __grid_
         item = next;
         // after a wait that ran out the warp keeps drawing (the ticket count must come out) but works no more
         if (!it.valid || giving_up_s) continue;
-        attn_split_item<HD, NST, true>(a, it, wr, lane, &tm);
+        if (it.nq <= 8) attn_item_t<HD, AtRing<HD, NST, true>>(a, it, wr, lane, &tm);
+        else attn_item<HD, NST, true>(a, it, wr, lane, &tm);
     }
 }
 inline size_t attn_warp_tma_bytes(int head_dim, int stages, int warps)

@@ -19,6 +19,7 @@ struct MkTiles {
     int tile0, sub, nsub;
     int new0, end;                // the pass's own positions: [new0, end), end = the prefix's length
     int arrivals;                 // this warp's share of a slot's release
+    int w_end;                    // no position from here on counts
     int n_tiles, lane;
 
     __device__ __forceinline__ static int off(int row, int c) { return at_swz<HD>(row, c); }
@@ -59,6 +60,7 @@ struct MkTiles {
             if (lane == 0) mbar_arrive_n(&sh->empty[place(t).s], (uint32_t)arrivals);
         }
     }
+    __device__ __forceinline__ void start() const {}
     __device__ __forceinline__ void finish() const {}
 };
 // Where it leaves its partial: the run's place in global memory, or the area, when several warps share the run.
@@ -130,7 +132,7 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
         if (sub < nsub) {
             AtItem item;
             item.qb = qb; item.hk = r.hk; item.row0 = r.row0; item.nrows = r.nrows; item.pos0 = r.pos0; item.nq = nq;
-            item.w_end = min(r.pos0 + (r.nrows == 1 ? 0 : (min(qb * 8 + 8, nq) - 1) / G) + 1, a.S);
+            const int w_end = min(r.pos0 + (r.nrows == 1 ? 0 : (min(qb * 8 + 8, nq) - 1) / G) + 1, a.S);
             MkTiles<HD, SLOTS> tiles;
             tiles.ring = ring; tiles.sh = sh; tiles.status = a.status;
             tiles.kbase = a.kc + l * a.kv_layer + (size_t)r.cache0 * HD; tiles.vbase = a.vc + l * a.kv_layer + (size_t)r.cache0 * HD;
@@ -141,7 +143,7 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
             tiles.arrivals = qb == 0 ? MK_CW - (n_qblk - 1) : 1;
             const int mine = nsub == 1 ? run_items : (run_items - sub + nsub - 1) / nsub;
             tiles.n_tiles = 2 * mine - ((r.n & 1) && sub + nsub * (mine - 1) == run_items - 1 ? 1 : 0);
-            tiles.lane = lane;
+            tiles.lane = lane; tiles.w_end = w_end;
             MkCells<HD> out;
             if (nsub > 1) {
                 // query vector qg of block qb at row qg - 8 qb of the warp's cells
@@ -152,7 +154,7 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
                 out.po = a.part_o + part * HD;
                 out.pml = a.part_ml + part;
             }
-            attn_item_t<HD>(aa, item, tiles, out, lane);
+            attn_item_t<HD>(aa, item, nullptr, lane, nullptr, &tiles, &out);
         }
         at.skip_many(n_items);
         mk_consumer_sync();
