@@ -209,7 +209,9 @@ int sparsk_set_debug(sparsk_ctx *ctx, float *exit_hidden /*device or NULL*/,
  * "time_kernel" (see sparsk_kernel_time), "inject_barrier_timeout" (test hook, 1: the next launch
  * of the persistent kernel is given a grid-barrier count that no CTA can reach, so its bounded
  * wait runs out after about two seconds, the kernel returns and the step reports
- * SPARSK_ETIMEOUT; nothing faults or hangs).  Returns SPARSK_EINVAL for an unknown name or value. */
+ * SPARSK_ETIMEOUT; nothing faults or hangs), "inject_short_copy" (test hook, 1: in the second layer of
+ * that kernel's next launch of two layers or more, one CTA waits for bytes that no copy brings; it gives up
+ * after two seconds and takes the others with it).  Returns SPARSK_EINVAL for an unknown name or value. */
 int sparsk_set_option(sparsk_ctx *ctx, const char *name /*host*/, int64_t value);
 
 /* Nucleus sampling (Sec. V-A: the 28-layer backbone is decoded with temperature 0.7 and top_p 0.9;

@@ -131,6 +131,7 @@ struct sparsk_ctx {
     std::vector<float> conf_trace; // last step: entropy seen at layer l (1-based, < L) by sequence i at [i * L + l], or -1
     float *conf_logits;            // device [B][V] when neither the parity hook nor a sampler lends a buffer
     int inject_timeout;            // test hook: the next persistent launch waits for a barrier count nobody reaches
+    int inject_short_copy;         // test hook: the next persistent launch of two layers waits for bytes that do not come
     int64_t route_layers[3];       // layer passes so far by implementation: see sparsk_route_counts
     std::vector<MkLayer> mk_host;
     float *qkv_part;  // fp32 sums of a q/k/v product whose inner dimension is cut across CTAs
@@ -1086,6 +1087,11 @@ cudaError_t run_mega(sparsk_ctx *c, int l_begin, int l_end, float *h, const RowS
         a.bar_base += 1ull << 40;
         c->inject_timeout = 0;
     }
+    a.short_copy_layer = -1;
+    if (c->inject_short_copy && l_end - l_begin >= 2) {
+        a.short_copy_layer = l_begin + 1;
+        c->inject_short_copy = 0;
+    }
     a.trace = c->mk_trace;
     c->mk_trace_n = 1 + MK_PHASES * (l_end - l_begin);
     c->mk_bar_base += (unsigned long long)MK_PHASES * (unsigned long long)(l_end - l_begin) * (unsigned long long)c->n_sm;
@@ -1221,7 +1227,7 @@ extern "C" int sparsk_create(const sparsk_dims *dims, const sparsk_weights *w, v
     ctx->gemm_cps = 1;
     ctx->mk_max_rows = MK_MAX_ROWS;
     ctx->attn_tc = 1; ctx->attn_tc_min_q = 33; ctx->attn_stages = AW_NST;
-    ctx->inject_timeout = 0;
+    ctx->inject_timeout = ctx->inject_short_copy = 0;
     ctx->attn_ticket_base = 0; ctx->attn_dynamic = 1; ctx->attn_ctas = 0;
     ctx->attn_tma = 1; ctx->attn_tma_ok = 0;
     ctx->trim_last = 1;
@@ -1405,6 +1411,7 @@ extern "C" int sparsk_set_option(sparsk_ctx *ctx, const char *name, int64_t valu
     else if (!strcmp(name, "gemm_smem_kb") && value >= 48 && value <= 220) ctx->gemm_smem_kb = (int)value;
     else if (!strcmp(name, "trim_last_layer") && value >= 0 && value <= 2) ctx->trim_last = (int)value;
     else if (!strcmp(name, "inject_barrier_timeout") && (value == 0 || value == 1)) ctx->inject_timeout = (int)value;
+    else if (!strcmp(name, "inject_short_copy") && (value == 0 || value == 1)) ctx->inject_short_copy = (int)value;
     else if (!strcmp(name, "gemv_r") && (value == 0 || value == 1 || value == 2 || value == 4)) ctx->gv_r = (int)value;
     else if (!strcmp(name, "time_kernel") && value >= 0 && value <= KC_ALL) {
         // start (or stop, with 0) timing every launch of one kernel class; resets the totals

@@ -136,6 +136,7 @@ struct MkArgs {
     unsigned long long bar_base;    // its value when this launch starts
     int *abort_word;                // nonzero: some CTA gave up
     int *status;
+    int short_copy_layer;           // test hook: the layer in which the first CTA's ring waits for bytes that do not come, or -1
     unsigned long long *trace;      // [1 + MK_PHASES * layers]: CTA 0's clock at the start and after every phase
 };
 

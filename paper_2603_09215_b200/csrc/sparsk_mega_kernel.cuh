@@ -33,13 +33,13 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
     };
     auto rows = [&](int type, const MkLayer *L) {
         MkBands w = sh->bands[type == MK_QKV ? 0 : 1];
-        const uint32_t idx0 = idx;
+        const uint32_t idx0 = idx, bytes = MK_SLOT_BYTES + (type == MK_QKV && L - a.layers == a.short_copy_layer && blockIdx.x == 0 ? 16 : 0);
         flight = mk_few_in_flight(M);
         for (; w.j < w.end; w.j += w.step)
             for (int ks = 0; ks < w.k_steps; ks++, idx++) {
                 if (idx - idx0 == SLOTS && type == MK_MLP) flight = MK_IN_FLIGHT;
                 if ((int)(idx % MK_PW) != p) continue;
-                if (!open(MK_SLOT_BYTES)) return;
+                if (!open(bytes)) return;
                 if (lane < 2) {
                     const CUtensorMap *map;
                     int row;

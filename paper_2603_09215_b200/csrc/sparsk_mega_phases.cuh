@@ -59,28 +59,26 @@ __device__ __forceinline__ bool mk_grid_barrier(const MkArgs &a, MkShared *sh, u
     if (gains) gains->load(gain, a.d);
     if (threadIdx.x == 0) {
         unsigned long long t0 = 0;
+        bool leave = false;
         for (uint32_t spin = 0;; ++spin) {
             if (ld_acquire_u64(a.bar) >= epoch) break;
             if ((spin & 63u) == 63u) {
-                if (ld_volatile_i32(a.abort_word) || *(volatile int *)&sh->giving_up) {
-                    // this CTA or another (or an earlier launch that was never cleaned up after) gave up:
-                    // leave too, and say so, so that skipping the rest is never silent
-                    sh->giving_up = 1;
-                    atomicOr(a.status, ST_TIMEOUT);
-                    atomicExch(a.abort_word, 1);
-                    break;
-                }
+                // this CTA or another (or an earlier launch that was never cleaned up after) gave up
+                if ((leave = ld_volatile_i32(a.abort_word) || *(volatile int *)&sh->giving_up)) break;
                 const unsigned long long now = global_ns();
                 if (t0 == 0) t0 = now;
-                else if (now - t0 > GM_TIMEOUT_NS) {
-                    sh->giving_up = 1;
-                    atomicOr(a.status, ST_TIMEOUT);
-                    atomicExch(a.abort_word, 1);
-                    break;
-                }
+                else if ((leave = now - t0 > GM_TIMEOUT_NS)) break;
             }
         }
-        sh->go_on = !*(volatile int *)&sh->giving_up;
+        if (leave || *(volatile int *)&sh->giving_up) {
+            // say so, also where all have arrived (with a wait for a ring slot that ran out on the way here): skipping the rest
+            // is never silent, and nobody sits out a time limit of his own at the next barrier
+            sh->giving_up = 1;
+            atomicOr(a.status, ST_TIMEOUT);
+            atomicExch(a.abort_word, 1);
+            leave = true;
+        }
+        sh->go_on = !leave;
         if (blockIdx.x == 0 && a.trace) a.trace[(epoch - a.bar_base) / gridDim.x] = global_ns();
     }
     mk_consumer_sync();

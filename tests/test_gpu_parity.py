@@ -559,6 +559,42 @@ def test_timeout_is_reported_once_and_the_context_recovers(util):
     P.close()
 
 
+@pytest.mark.parametrize("rows", [1, 2, 4])
+def test_a_ring_wait_that_runs_out_ends_the_launch_for_all(util, rows):
+    """One CTA of the persistent kernel waits for bytes that do not come, in a layer that begins with the sums of the
+    layer before still in their own buffer.  The other CTAs leave with it (two seconds; four where each sits out a limit of its
+    own at the next barrier), and after a reset decoding matches the oracle: nothing of those sums is left."""
+    import time
+    from paper_2603_09215_b200 import binding
+    dims = synth.model_dims(dict(MICRO256, n_layers=4), 2, 3, 0)
+    w = synth.make_weights(dims, seed=0)
+    prompts = [synth.make_prompts(dims, 1, 14, 14, seed=5 + i)[0] for i in range(rows)]
+    P = util.Pair(dims, w, rows, 64, 2)
+    P.prefill(prompts)
+    P.step([0] * rows, [0] * rows)
+    assert P.g.route_counts()["mega"] > 0
+    nt, dp = np.zeros(rows, np.int32), np.zeros(rows, np.int32)
+    P.g.set_option("inject_short_copy", 1)
+    t0 = time.perf_counter()
+    with pytest.raises(binding.SparskError) as ei:
+        P.g.decode_step_host(list(range(rows)), P.next_in, [0] * rows, [0] * rows, nt, dp)
+    took = time.perf_counter() - t0
+    assert ei.value.code == binding.ETIMEOUT
+    assert 1.5 < took < 3.0, took
+    P.g.check()
+    for s_ in range(rows):
+        P.g.reset_slot(s_)
+        P.os[s_] = P.om.new_seq(2)
+    P.prefill(prompts)
+    for g in range(7):
+        mc = [synth.interleave(g, 2, 4) for _ in range(rows)]
+        P.step([m for m, _ in mc], [c for _, c in mc])
+    for s_ in range(rows):
+        ln, pend = P.g.slot_state(s_)
+        P.check_cache(s_, range(1, 5), ln - pend)
+    P.close()
+
+
 @pytest.mark.parametrize("options", [{}, {"mega": 0}])
 @pytest.mark.parametrize("B", [2, 3])
 @pytest.mark.parametrize("hd", [64, 128])
