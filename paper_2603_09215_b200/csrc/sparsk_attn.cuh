@@ -671,6 +671,7 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
         const int qi = (lane & 3) * 2 + e;
         limit[e] = qi < nq ? pos0 + (q0 + qi) / G : -1;
     }
+    const int lim_min = SPLIT ? pos0 : pos0 + q0 / G;  // the smallest of all
     float o[HD / 16][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
 #pragma unroll
     for (int mt = 0; mt < HD / 16; mt++)
@@ -692,7 +693,7 @@ __device__ __forceinline__ void attn_item_t(const AttnArgs &a, const AtItem &it,
             mma_f16(s1, kb, qf[ks + 1][0], qf[ks + 1][1]);
         }
         // online softmax down the columns; accumulator rows are positions lane / 4 and + 8
-        const bool full = p0 + AT_TP <= ring.w_end && p0 + AT_TP - 1 <= (SPLIT ? pos0 : pos0 + q0 / G);
+        const bool full = p0 + AT_TP <= ring.w_end && p0 + AT_TP - 1 <= lim_min;
         float pv[2][2], alpha[2];
 #pragma unroll
         for (int e = 0; e < 2; e++) {
