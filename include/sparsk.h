@@ -312,7 +312,8 @@ int sparsk_check(sparsk_ctx *ctx);
 
 /* Phase clock of the persistent layer-range kernel: its first CTA records the GPU's nanosecond
  * timer when it starts and after each of the four phases of every layer (q/k/v; attention;
- * merge of its splits and O-projection; MLP).  Copies the entries of the most recent launch
+ * merge of its splits and O-projection; MLP) or five, where the MLP is wider than 128 columns an SM
+ * or a residual row than 7,168 numbers (gate/up; down).  Copies the entries of the most recent launch
  * to out_ns (host), synchronising the stream; returns how many were written (at most
  * `capacity`), or a negative code.  No counterpart in the paper: measurement only. */
 int sparsk_phase_trace(sparsk_ctx *ctx, int64_t *out_ns /*host*/, int32_t capacity);

@@ -114,9 +114,9 @@ struct sparsk_ctx {
     MkLayer *mk_layers;            // device [L]
     unsigned long long *mk_bar;    // device: grid barrier counter; mk_bar_base mirrors its value
     int *mk_abort;                 // device
-    float *mk_h2;                  // device fp32 [MK_MAX_ROWS][d] (see MkArgs)
+    float *mk_h2, *mk_act;         // device fp32 [MK_MAX_ROWS][d], [MK_MAX_ROWS][F] (see MkArgs)
     MkCols mk_cols16, mk_cols32;   // how the MLP's columns are dealt to the CTAs, at one and two and at three and four rows
-    unsigned long long *mk_trace;  // device [1 + MK_PHASES L]
+    unsigned long long *mk_trace;  // device [1 + MK_MAX_PHASES L]
     int mk_trace_n;                // entries the last launch wrote
     unsigned long long mk_bar_base;
     int mega, mk_ok, mk_coop, mk_max_rows;
@@ -255,8 +255,8 @@ size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
     unsigned long long *mkb = w.take<unsigned long long>(1);
     int *mka = w.take<int>(1);
     unsigned *atk = w.take<unsigned>(1);
-    float *mkh2 = w.take<float>((size_t)MK_MAX_ROWS * d->d_model);
-    unsigned long long *mkt = w.take<unsigned long long>(1 + MK_PHASES * L);
+    float *mkh2 = w.take<float>((size_t)MK_MAX_ROWS * d->d_model), *mkact = w.take<float>((size_t)MK_MAX_ROWS * d->d_ffn);
+    unsigned long long *mkt = w.take<unsigned long long>(1 + MK_MAX_PHASES * L);
     // attention partials: of the launches, and of the persistent kernel (see MkRun)
     const size_t runs = (size_t)MK_MAX_CTAS + (size_t)MK_MAX_ROWS * d->n_kv_heads;
     const size_t cells = std::max<size_t>(std::max(R, part_rows_of(d)) * d->n_q_heads, runs * MK_MAX_ROWS * (d->n_q_heads / d->n_kv_heads));
@@ -270,7 +270,7 @@ size_t carve(sparsk_ctx *c, const sparsk_dims *d, char *base)
         c->h_last = hlast; c->q_last = qlast; c->last_slot = lslot; c->last_pos = lpos;
         c->h_lo = hlo; c->h_up = hup; c->qbuf = q; c->attn_o = ao; c->act = act; c->xnorm = xn; c->qkv_part = qp;
         c->attn_o_lo = aol; c->act_lo = actl; c->xnorm_lo = xnl;
-        c->mk_layers = mkl; c->mk_bar = mkb; c->mk_abort = mka; c->mk_h2 = mkh2; c->mk_trace = mkt;
+        c->mk_layers = mkl; c->mk_bar = mkb; c->mk_abort = mka; c->mk_h2 = mkh2; c->mk_act = mkact; c->mk_trace = mkt;
         c->part_o = po; c->part_ml = pml; c->attn_ticket = atk;
     }
     return align_up(w.off, 256);
@@ -948,15 +948,15 @@ bool build_mega(sparsk_ctx *c)
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
-    c->mk_cols16 = mk_cols(d.d_ffn, MK_BOX_ROWS, c->n_sm);
-    c->mk_cols32 = mk_cols(d.d_ffn, 2 * MK_BOX_ROWS, c->n_sm);
+    c->mk_cols16 = mk_cols(d.d_ffn, d.d_model, MK_BOX_ROWS, c->n_sm);
+    c->mk_cols32 = mk_cols(d.d_ffn, d.d_model, 2 * MK_BOX_ROWS, c->n_sm);
     // The swizzled three-dimensional views need inner dimensions that are whole 64-element blocks, and
     // the RMSNorm of the form leaves whole residual rows in the activation area: 4,352 numbers.
     // Passes of three and four wider rows take the tcgen05 path, which is the faster one there in
     // any case.  us a layer at three / four rows: 4,352 numbers (MLP 11,776) 111 / 111 here and 117
     // there; a form that normalised a window at a time took 117 / 165 at 4,416, 142 / 204 at 5,120
     // (MLP 13,824) and 165 / 237 at 5,888 (15,360) where the tcgen05 path takes 113, 134 and 155.
-    c->mk_tc_ok = d.d_model % 64 == 0 && d.d_ffn % 64 == 0 && qd % 64 == 0 && mk_tc_fits(MK_MAX_ROWS, d.d_model, c->mk_cols32.most);
+    c->mk_tc_ok = d.d_model % 64 == 0 && d.d_ffn % 64 == 0 && qd % 64 == 0 && div_up(d.d_model, MK_BOX_COLS) <= MK_TC_STEPS;
     auto enc_sw = [&](CUtensorMap *m, const void *base, size_t rows, size_t cols) {
         const cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64)};
         const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, 128};
@@ -1018,21 +1018,18 @@ bool build_mega(sparsk_ctx *c)
 // Can a pass of n_rows rows go through the persistent kernel?
 bool use_mega(const sparsk_ctx *c, int n_rows)
 {
-    const int m = n_rows >= MK_TC_ROWS ? MK_MAX_ROWS : n_rows;  // (three rows run as four with one masked)
     return c->mega && c->mk_ok && c->mk_coop && n_rows >= 1 && n_rows <= c->mk_max_rows && (n_rows < MK_TC_ROWS || c->mk_tc_ok) &&
-           c->attn_tma_ok && c->n_sm <= MK_MAX_CTAS &&
-           (size_t)MK_MAX_ROWS * c->dm.n_kv_heads * (c->dm.max_seq_len / AT_TP + 1) * MK_MAX_CTAS < (1ull << 31) &&  // (32-bit shares)
-           mk_attn_fits(m, c->dm.n_q_heads / c->dm.n_kv_heads) &&
-           (n_rows >= MK_TC_ROWS || mk_act_window(m, m * c->mk_cols16.most * 4 + mk_sums_bytes(m)) >= 1);
+           c->attn_tma_ok && c->n_sm <= MK_MAX_CTAS && mk_attn_fits(n_rows >= MK_TC_ROWS ? MK_MAX_ROWS : n_rows, c->dm.n_q_heads / c->dm.n_kv_heads) &&
+           (size_t)MK_MAX_ROWS * c->dm.n_kv_heads * (c->dm.max_seq_len / AT_TP + 1) * MK_MAX_CTAS < (1ull << 31);  // (32-bit shares)
 }
 
-template <int M, int HD>
-cudaError_t launch_mega_inst(sparsk_ctx *c, const MkArgs &a)
+template <int M, int HD, bool WIDE>
+cudaError_t launch_mega_form(sparsk_ctx *c, const MkArgs &a)
 {
-    constexpr size_t smem = mk_smem_bytes(M);
+    constexpr size_t smem = mk_smem_bytes(M, WIDE);
     static PerDevice<int> grid_dev;  // 0: not asked yet, 1: one CTA per SM fits, 2: it does not
     int &grid_ok = grid_dev.here();
-    auto kern = mega_kernel<M, HD>;
+    auto kern = mega_kernel<M, HD, WIDE>;
     if (grid_ok == 0) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -1064,6 +1061,12 @@ cudaError_t launch_mega_inst(sparsk_ctx *c, const MkArgs &a)
     return e;
 }
 
+template <int M, int HD>
+cudaError_t launch_mega_inst(sparsk_ctx *c, const MkArgs &a)
+{
+    return a.cols.wide ? launch_mega_form<M, HD, true>(c, a) : launch_mega_form<M, HD, false>(c, a);
+}
+
 // Layers [l_begin, l_end) (0-based) over a row set of one to four rows, in one launch.
 cudaError_t run_mega(sparsk_ctx *c, int l_begin, int l_end, float *h, const RowSet &rs)
 {
@@ -1073,6 +1076,7 @@ cudaError_t run_mega(sparsk_ctx *c, int l_begin, int l_end, float *h, const RowS
     a.row_slot = rs.slot; a.row_pos = rs.pos; a.grp_row0 = rs.grp_row0; a.grp_nrows = rs.grp_nrows;
     a.n_rows = rs.n_rows; a.n_groups = rs.n_groups_h;
     a.h2 = c->mk_h2;
+    a.act = c->mk_act;
     a.kc = c->kcache; a.vc = c->vcache;
     a.kv_layer = (size_t)d.max_seqs * d.n_kv_heads * d.max_seq_len * d.head_dim;
     a.q_buf = c->qbuf; a.part_o = c->part_o; a.part_ml = c->part_ml;
@@ -1093,8 +1097,8 @@ cudaError_t run_mega(sparsk_ctx *c, int l_begin, int l_end, float *h, const RowS
         c->inject_short_copy = 0;
     }
     a.trace = c->mk_trace;
-    c->mk_trace_n = 1 + MK_PHASES * (l_end - l_begin);
-    c->mk_bar_base += (unsigned long long)MK_PHASES * (unsigned long long)(l_end - l_begin) * (unsigned long long)c->n_sm;
+    c->mk_trace_n = 1 + mk_phases(a.cols.wide) * (l_end - l_begin);
+    c->mk_bar_base += (unsigned long long)mk_phases(a.cols.wide) * (unsigned long long)(l_end - l_begin) * (unsigned long long)c->n_sm;
     // (three rows run as four with one masked)
     if (d.head_dim == 128) {
         switch (rs.n_rows) {

@@ -19,7 +19,7 @@
 //     attention's own cache reads by as much as it later saved.)
 //   * warps 0..15 are consumers.  Per layer they run four phases separated by grid-wide barriers:
 //     RMSNorm + q/k/v + rotary embedding + cache append; attention partials; O-projection;
-//     RMSNorm + gate/up + SiLU + down-projection.
+//     RMSNorm + gate/up + SiLU + down-projection (a phase of its own in the wide form, see MkCols).
 //     - Row form (q/k/v, gate/up: a sum is needed whole before anything can be done with it): a
 //       CTA owns "bands" of 32 weight rows in two 16-row boxes (rotary pairs, gate/up pairs, or
 //       plain rows) over the whole inner dimension.
@@ -36,7 +36,7 @@
 //     from the fp64 reference.
 //     While some CTA still reads the residual stream at the start of the MLP, another may be done with
 //     its gate/up bands: the down-projection therefore adds into a buffer of its own (h2), which the
-//     next layer's first RMSNorm reads along with h and the attention phase folds into h.
+//     next layer's first RMSNorm reads along with h and the attention phase folds into h.  (Not in the wide form.)
 //
 // Every wait (ring slot, grid barrier) is bounded by a wall-clock limit; on a timeout the CTA
 // raises ST_TIMEOUT, tells the other CTAs through the abort word, lets its copies land and
@@ -58,10 +58,10 @@ constexpr int MK_BOX_BYTES = MK_BOX_ROWS * MK_BOX_COLS * 2;  // 8 KB
 constexpr int MK_CBOX_ROWS = 64, MK_CBOX_COLS = 128;         // column form: one box of 64 rows and up to 128 columns per slot
 constexpr int MK_SLOT_BYTES = 2 * MK_BOX_BYTES;
 constexpr int MK_IN_FLIGHT = 8;                 // slots on their way at once, in the MLP
-// and before it, with one row.  A trip to the L2 queues behind the copies on their way to the SM, 2.7 us of them at eight
+// and before it, with one row (narrow form).  A trip to the L2 queues behind the copies on their way to the SM, 2.7 us of them at eight
 // slots, and the phases before the MLP are chains of such trips with little to stream: 81.7 us a layer with eight
 // throughout, 80.8 with four here.
-__host__ __device__ constexpr int mk_few_in_flight(int M) { return M == 1 ? 4 : MK_IN_FLIGHT; }
+constexpr int MK_FEW_IN_FLIGHT = 4;
 constexpr int MK_MAX_ROWS = 4;
 constexpr int MK_TC_ROWS = 3;                   // rows from which the tensor-core form runs
 constexpr int MK_GROUPS = 4;                    // a slot of weights is the work of one of four groups of four warps
@@ -69,22 +69,25 @@ constexpr int MK_MAX_CTAS = 192;                // bounds the number of attentio
 constexpr int MK_SHARED_BYTES = 2688;           // MkShared, behind the area, with two to four rows
 constexpr int MK_SHARED_FEW_BYTES = 1536;       // the part of it that one row needs
 
-// The ring, then the area: the activations of a row-form phase (M rows; with one or two rows, when they
-// do not fit whole, a window of k-steps that is reloaded as the phase moves along) and what the CTA's
-// own bands make of them, or the attention's partials, or the merged heads.
-// Several rows' activations need the larger area.  A multiple of four slots: a weight slot always belongs
-// to the same four warps, so that nobody waits for a slot's next fill before its present one has landed.
-__host__ __device__ constexpr int mk_slots(int M) { return M >= 2 ? 8 : 12; }
-__host__ __device__ constexpr int mk_area_bytes(int M) { return M >= 2 ? 88 * 1024 : 33792; }
-__host__ __device__ constexpr size_t mk_smem_bytes(int M)
+// The ring, then the area: the activations of a row-form phase (M rows) and what the CTA's own bands make of
+// them, or the attention's partials, or the merged heads, or (wide form) the activations of the CTA's share of the
+// down-projection.
+// Several rows' activations need the larger area, and so does one wide row.  (Wide form, one and two rows: activations that do
+// not fit even so, beyond 92 and 44 k-steps, come as a window that is reloaded as the phase moves along.)  A multiple of four
+// slots: a weight slot always belongs to the same four warps, so that nobody waits for a slot's next fill before its present
+// one has landed.
+__host__ __device__ constexpr int mk_slots(int M, bool wide) { return M >= 2 || wide ? 8 : 12; }
+__host__ __device__ constexpr int mk_area_bytes(int M, bool wide) { return wide ? 96 * 1024 : M >= 2 ? 88 * 1024 : 33792; }
+__host__ __device__ constexpr size_t mk_smem_bytes(int M, bool wide)
 {
-    return (size_t)mk_slots(M) * MK_SLOT_BYTES + mk_area_bytes(M) + (M >= 2 ? MK_SHARED_BYTES : MK_SHARED_FEW_BYTES);
+    return (size_t)mk_slots(M, wide) * MK_SLOT_BYTES + mk_area_bytes(M, wide) + (M >= 2 || wide ? MK_SHARED_BYTES : MK_SHARED_FEW_BYTES);
 }
 // k-steps of M fp32 activation rows that fit the area beside `own` bytes
-__host__ __device__ inline int mk_act_window(int M, int own) { return (mk_area_bytes(M) - own) / (M * MK_BOX_COLS * 4); }
+__host__ __device__ constexpr int mk_act_window(int M, bool wide, int own) { return (mk_area_bytes(M, wide) - own) / (M * MK_BOX_COLS * 4); }
 
 enum { MKW_Q = 0, MKW_K, MKW_V, MKW_O, MKW_G, MKW_U, MKW_D, MKW_N };
-enum { MK_QKV = 0, MK_ATTN = 1, MK_OPROJ = 2, MK_MLP = 3, MK_PHASES = 4 };
+enum { MK_QKV = 0, MK_ATTN = 1, MK_OPROJ = 2, MK_MLP = 3, MK_MAX_PHASES = 5 };
+inline int mk_phases(bool wide) { return wide ? 5 : 4; }
 
 // One layer's worth of what the phases need (device array, one entry per layer).
 struct MkLayer {
@@ -99,20 +102,26 @@ struct MkLayer {
 };
 
 // How the MLP's inner dimension is dealt: contiguous units of `unit` columns (16: a gate/up band; 32 with
-// three and four rows) to every CTA, at most `most` columns, walked in `chunks` boxes of `box` columns.
+// three and four rows) to every CTA, at most `box` columns, one box of the down-projection's columns.
 // A box may reach into the next CTA's columns; the activations that meet those are zeros.
+// The wide form: a CTA's columns are more than one box, or one activation row does not fit beside twelve slots.  Gate/up deals its bands
+// round-robin there and leaves the activation in memory, and the down-projection, a phase of its own, deals
+// (block of 128 columns, box of 64 weight rows) pairs evenly.  (Two boxes a CTA, of as many columns as the largest share needs in
+// halves, read a tenth too much in slots that are not full: a one-row layer of d_model 7,168, d_ffn 20,480 and 8 kv heads
+// after 100 positions 238 us, so 194; of 8,192 and 28,672, its row in windows besides, 369 and 282; two rows of 10,240 and
+// 27,648 531 and 374.)
 struct MkCols {
-    int unit, most, box, chunks;
+    int unit, box;
+    bool wide;
 };
-inline MkCols mk_cols(int F, int unit, int n_cta)
+constexpr int MK_NARROW_STEPS = (mk_area_bytes(1, false) - MK_CBOX_COLS * 4 - 4096) / (MK_BOX_COLS * 4);  // of one row, beside the CTA's columns and mk_sums_bytes(1)
+inline MkCols mk_cols(int F, int d, int unit, int n_cta)
 {
-    const int n = (F + unit - 1) / unit, per = (n + n_cta - 1) / n_cta, lim = MK_CBOX_COLS / unit;
+    const int n = (F + unit - 1) / unit, per = (n + n_cta - 1) / n_cta;
     MkCols c;
     c.unit = unit;
-    c.chunks = (per + lim - 1) / lim;
-    const int in_box = (per + c.chunks - 1) / c.chunks;
-    c.box = in_box * unit;
-    c.most = c.box * c.chunks;
+    c.wide = per * unit > MK_CBOX_COLS || (unit == MK_BOX_ROWS && d > MK_NARROW_STEPS * MK_BOX_COLS);
+    c.box = c.wide ? MK_CBOX_COLS : per * unit;
     return c;
 }
 
@@ -126,6 +135,7 @@ struct MkArgs {
     kv_t *kc, *vc;               // cache of the first layer [slot][Hkv][S][hd], and what lies between two layers'
     size_t kv_layer;             // (arithmetic: a pointer read from `layers` would be a trip to HBM in every layer)
     float *q_buf;                // [rows][Hq*hd]
+    float *act;                  // wide form: [rows][F], the MLP's activation
     float *part_o;               // attention partials, see MkRun
     float2 *part_ml;
     const float2 *rope;
@@ -137,7 +147,7 @@ struct MkArgs {
     int *abort_word;                // nonzero: some CTA gave up
     int *status;
     int short_copy_layer;           // test hook: the layer in which the first CTA's ring waits for bytes that do not come, or -1
-    unsigned long long *trace;      // [1 + MK_PHASES * layers]: CTA 0's clock at the start and after every phase
+    unsigned long long *trace;      // [1 + phases * layers]: CTA 0's clock at the start and after every phase
 };
 
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p)
@@ -155,17 +165,19 @@ __device__ __forceinline__ int ld_volatile_i32(const int *p)
 __device__ __forceinline__ void mk_consumer_sync() { asm volatile("bar.sync 2, %0;" ::"n"(MK_CW * 32) : "memory"); }
 
 // Row form: bands and k-steps.  q/k/v deals whole bands round-robin (144 bands fill 148 SMs well), gate/up
-// contiguous bands, because what they make is what the CTA's columns of the down-projection need.
+// contiguous bands, because what they make is what the CTA's columns of the down-projection need (wide form: round-robin as well).
 struct MkBands {
     int j, end, step, k_steps;
     __device__ void init(int type, const MkArgs &a)
     {
         const int half = a.hd >> 1;
         k_steps = (a.d + MK_BOX_COLS - 1) / MK_BOX_COLS;
+        j = blockIdx.x;
+        step = gridDim.x;
         if (type == MK_QKV) {
-            j = blockIdx.x;
             end = (a.Hq + a.Hkv) * (half / MK_BOX_ROWS) + (a.Hkv * a.hd + 2 * MK_BOX_ROWS - 1) / (2 * MK_BOX_ROWS);
-            step = gridDim.x;
+        } else if (a.cols.wide) {
+            end = (a.F + MK_BOX_ROWS - 1) / MK_BOX_ROWS;
         } else {
             const int per = a.cols.unit / MK_BOX_ROWS, n = (a.F + a.cols.unit - 1) / a.cols.unit;
             j = (int)(blockIdx.x * (unsigned)n / gridDim.x) * per;
@@ -196,13 +208,13 @@ __device__ __forceinline__ void mk_band(int type, const MkArgs &a, const MkLayer
 }
 
 // Column form, O-projection: the (head, box of 64 weight rows) pairs laid end to end, head by head, and cut
-// into equal contiguous shares [lo, hi).
-struct MkHeads {
+// into equal contiguous shares [lo, hi); of the wide form's down-projection the same with blocks of 128 columns.
+struct MkPairs {
     int boxes, lo, hi;
-    __device__ void init(const MkArgs &a)
+    __device__ void init(const MkArgs &a, int n)
     {
         boxes = (a.d + MK_CBOX_ROWS - 1) / MK_CBOX_ROWS;
-        const unsigned T = (unsigned)a.Hq * boxes;
+        const unsigned T = (unsigned)n * boxes;
         lo = (int)(blockIdx.x * T / gridDim.x);
         hi = (int)((blockIdx.x + 1) * T / gridDim.x);
     }
@@ -233,7 +245,7 @@ struct MkMerge {
 // A launch's constants are worked out once: a warp spends some ten cycles an instruction here, so the
 // divisions that turn a share into rows and heads held every layer up by 2 us.
 struct MkShared {
-    uint64_t full[mk_slots(1)], empty[mk_slots(1)];
+    uint64_t full[mk_slots(1, false)], empty[mk_slots(1, false)];
     int giving_up, never, go_on;
     int row_slot[MK_MAX_ROWS], row_pos[MK_MAX_ROWS], grp_row0[MK_MAX_ROWS], grp_nrows[MK_MAX_ROWS];  // copies of the row set
     int row_grp[MK_MAX_ROWS];            // group of a row
@@ -244,10 +256,11 @@ struct MkShared {
     int att_batch;                       // runs below when they are all of the share and are worked on side by side, or 0
     MkRun runs[MK_RUNS];                 // its first runs
     MkBands bands[2];                    // this CTA's bands of q/k/v and of gate/up
-    MkHeads heads;                       // and of the O-projection
+    MkPairs heads;                       // and of the O-projection
     int head0;                           // first head of those
     MkMerge merge[2][MK_MAX_ROWS];       // its first two heads
     float red_rows[MK_MAX_ROWS][MK_CW];  // per-row partial sums of squares
+    MkPairs downs;                       // and of the wide form's down-projection
     MkFin fin[MK_BOX_ROWS * MK_MAX_ROWS];  // of the first q/k/v band, [row of the box][activation row]; one row has room for as many
 };
 static_assert(sizeof(MkShared) <= MK_SHARED_BYTES, "MkShared outgrew its place");

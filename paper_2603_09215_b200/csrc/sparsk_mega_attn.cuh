@@ -81,11 +81,10 @@ inline bool mk_attn_fits(int M, int G) { return (M * G + 7) / 8 <= MK_CW; }
 // has room for partials, and two slots at least each), every nsub-th slot each; their partials meet in the area.
 // (Blocks of sixteen, positions as columns, cost 450 bytes of spills, and a reload behind a grid barrier is a trip to the L2: flushes of
 // four rows of the 28-layer shape 96.6 us a layer, so 90.9.)  Short runs go side by side, a warp per block.
-template <int M, int HD>
+template <int M, int HD, bool WIDE, int SLOTS>
 __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned char *area, unsigned char *ring, MkShared *sh,
-                                             MkPos<mk_slots(M)> &at)
+                                             MkPos<SLOTS> &at)
 {
-    constexpr int SLOTS = mk_slots(M);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = a.Hq / a.Hkv;
     AttnArgs aa{};
     aa.q32 = a.q_buf; aa.Hq = a.Hq; aa.Hkv = a.Hkv;
@@ -115,7 +114,7 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
         } else {
             nsub = min(4, (n_items + 1) / 2);
             if (nsub > 1) {
-                const int room = mk_area_bytes(M) / (r.n_qblk * mk_cell_bytes<HD>());
+                const int room = mk_area_bytes(M, WIDE) / (r.n_qblk * mk_cell_bytes<HD>());
                 nsub = max(1, min(nsub, min(MK_CW / r.n_qblk, room)));
             }
             if (SLOTS % nsub) nsub = 2;  // a slot's successive fills stay with one warp

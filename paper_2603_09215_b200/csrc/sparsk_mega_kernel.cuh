@@ -5,18 +5,19 @@ namespace sparsk {
 
 // ------------------------------------------------------------------ producers
 // One producer warp: walks the CTA's ring items in consumption order and issues every fourth.
-template <int M, int HD>
+template <int M, int HD, bool WIDE>
 __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring, MkShared *sh, int p)
 {
-    constexpr int SLOTS = mk_slots(M);
+    constexpr int SLOTS = mk_slots(M, WIDE);
     constexpr bool TC = M >= MK_TC_ROWS;
     const int lane = threadIdx.x & 31;
     uint32_t idx = 0;   // ring item
     bool ok = true;
     // waits until item idx's slot is free and no more than `flight` items (counting this one) are on
     // their way, and announces `bytes`; item idx - flight was this warp's own
-    uint32_t flight = mk_few_in_flight(M);
-    static_assert(MK_IN_FLIGHT % MK_PW == 0 && mk_few_in_flight(M) % MK_PW == 0 && SLOTS % MK_PW == 0, "a producer waits for items of its own");
+    constexpr uint32_t few = M == 1 && !WIDE ? MK_FEW_IN_FLIGHT : MK_IN_FLIGHT;
+    uint32_t flight = few;
+    static_assert(MK_IN_FLIGHT % MK_PW == 0 && MK_FEW_IN_FLIGHT % MK_PW == 0 && SLOTS % MK_PW == 0, "a producer waits for items of its own");
     auto open = [&](uint32_t bytes) {
         const int s = idx % SLOTS;
         int go = 1;
@@ -34,7 +35,7 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
     auto rows = [&](int type, const MkLayer *L) {
         MkBands w = sh->bands[type == MK_QKV ? 0 : 1];
         const uint32_t idx0 = idx, bytes = MK_SLOT_BYTES + (type == MK_QKV && L - a.layers == a.short_copy_layer && blockIdx.x == 0 ? 16 : 0);
-        flight = mk_few_in_flight(M);
+        flight = few;
         for (; w.j < w.end; w.j += w.step)
             for (int ks = 0; ks < w.k_steps; ks++, idx++) {
                 if (idx - idx0 == SLOTS && type == MK_MLP) flight = MK_IN_FLIGHT;
@@ -87,16 +88,19 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
             }
         }
         if (!ok) break;
-        const MkHeads w = sh->heads;
+        const MkPairs w = sh->heads;
         for (int i = w.lo; i < w.hi && ok; i++) column_box(&L->map[MKW_O], HD, (i / w.boxes) * HD, (i % w.boxes) * MK_CBOX_ROWS);
         if (!ok) break;
         rows(MK_MLP, L);
         if (!ok) break;
-        const MkBands b = sh->bands[1];
-        if (b.j < b.end)
-            for (int c = 0; c < a.cols.chunks && ok; c++)
-                for (int i = 0; i < w.boxes && ok; i++)
-                    column_box(&L->map[MKW_D], a.cols.box, b.j * MK_BOX_ROWS + c * a.cols.box, i * MK_CBOX_ROWS);
+        if constexpr (WIDE) {
+            const MkPairs v = sh->downs;
+            for (int i = v.lo; i < v.hi && ok; i++) column_box(&L->map[MKW_D], MK_CBOX_COLS, (i / v.boxes) * MK_CBOX_COLS, (i % v.boxes) * MK_CBOX_ROWS);
+        } else {
+            const MkBands b = sh->bands[1];
+            if (b.j < b.end)
+                for (int i = 0; i < w.boxes && ok; i++) column_box(&L->map[MKW_D], a.cols.box, b.j * MK_BOX_ROWS, i * MK_CBOX_ROWS);
+        }
     }
     // never leave with copies in flight: every slot this producer filled must have landed
     // (consumers that gave up no longer free slots, so wait on the full barriers, 2 ms each)
@@ -108,11 +112,10 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
 }
 
 // ------------------------------------------------------------------ consumers: O-projection and MLP
-template <int M, int HD>
-__device__ __forceinline__ void mk_oproj(const MkArgs &a, unsigned char *area, unsigned char *ring, MkShared *sh,
-                                         MkPos<mk_slots(M)> &at)
+template <int M, int HD, int SLOTS>
+__device__ __forceinline__ void mk_oproj(const MkArgs &a, unsigned char *area, unsigned char *ring, MkShared *sh, MkPos<SLOTS> &at)
 {
-    const MkHeads w = sh->heads;
+    const MkPairs w = sh->heads;
     constexpr bool TC = M >= MK_TC_ROWS;
     constexpr int RS = HD + 8;
     // two merged heads, as fp32 rows or as two planes each
@@ -140,34 +143,75 @@ __device__ __forceinline__ void mk_oproj(const MkArgs &a, unsigned char *area, u
     }
 }
 
-template <int M>
+// Gate/up, and in the narrow form the down-projection of what the CTA's own bands made.
+template <int M, bool WIDE, int SLOTS>
 __device__ __forceinline__ void mk_mlp(const MkArgs &a, int l, const bf16 *gain, unsigned char *area, unsigned char *ring, MkShared *sh,
-                                       const MkGains &gains, MkPos<mk_slots(M)> &at)
+                                       const MkGains &gains, MkPos<SLOTS> &at)
 {
     const int boxes = (a.d + MK_CBOX_ROWS - 1) / MK_CBOX_ROWS;
     const MkBands w = sh->bands[1];
     if (w.j >= w.end) return;
-    // columns of the last box that are the next CTA's meet zeros
+    // columns of the box that are the next CTA's meet zeros
     if constexpr (M >= MK_TC_ROWS) {
-        const int rs = a.cols.most + 8;
+        constexpr int RS = MK_CBOX_COLS + 8;
         bf16 *planes = reinterpret_cast<bf16 *>(area);
         float *red = reinterpret_cast<float *>(area + mk_tc_planes_bytes(M, w.k_steps * MK_BOX_COLS));
         bf16 *u = reinterpret_cast<bf16 *>(reinterpret_cast<unsigned char *>(red) + MK_TC_RED_BYTES);
-        for (int i = threadIdx.x; i < M * rs; i += MK_CW * 32) reinterpret_cast<uint32_t *>(u)[i] = 0u;
-        mk_rows_tc<M>(MK_MLP, a, l, planes, red, nullptr, gain, gains, u, rs, ring, sh, at);
-        mk_consumer_sync();
-        for (int c = 0; c < a.cols.chunks; c++, at.skip_many(boxes))
-            mk_columns_tc<M>(a, a.h2, 0, boxes, a.cols.box, u + c * a.cols.box, rs, ring, sh, at);
+        if (!WIDE)
+            for (int i = threadIdx.x; i < M * RS; i += MK_CW * 32) reinterpret_cast<uint32_t *>(u)[i] = 0u;
+        mk_rows_tc<M, WIDE>(MK_MLP, a, l, planes, red, nullptr, gain, gains, u, RS, ring, sh, at);
+        if constexpr (!WIDE) {
+            mk_consumer_sync();
+            mk_columns_tc<M>(a, a.h2, 0, boxes, a.cols.box, u, RS, ring, sh, at);
+            at.skip_many(boxes);
+        }
+    } else if constexpr (WIDE) {
+        mk_rows<M, true>(MK_MLP, a, l, reinterpret_cast<float *>(area), reinterpret_cast<float *>(area + mk_area_bytes(M, true) - mk_sums_bytes(M)),
+                         mk_act_window(M, true, mk_sums_bytes(M)), nullptr, gain, gains, nullptr, 0, ring, sh, at);
     } else {
-        const int own = M * a.cols.most * 4 + mk_sums_bytes(M);
-        float *u = reinterpret_cast<float *>(area + mk_area_bytes(M) - own), *sums = u + M * a.cols.most;
-        for (int i = threadIdx.x; i < M * a.cols.most; i += MK_CW * 32) u[i] = 0.f;
-        mk_rows<M>(MK_MLP, a, l, reinterpret_cast<float *>(area), sums, own, nullptr, gain, gains, u, a.cols.most, ring, sh, at);
+        constexpr int OWN = M * MK_CBOX_COLS * 4 + mk_sums_bytes(M);
+        float *u = reinterpret_cast<float *>(area + mk_area_bytes(M, false) - OWN), *sums = u + M * MK_CBOX_COLS;
+        for (int i = threadIdx.x; i < M * MK_CBOX_COLS; i += MK_CW * 32) u[i] = 0.f;
+        mk_rows<M, false>(MK_MLP, a, l, reinterpret_cast<float *>(area), sums, mk_act_window(M, false, OWN), nullptr, gain, gains, u, MK_CBOX_COLS, ring, sh, at);
         mk_consumer_sync();
-        for (int c = 0; c < a.cols.chunks; c++, at.skip_many(boxes)) {
-            const float *x = u + c * a.cols.box;
-            if (a.cols.box <= 64) mk_columns<M, 8>(a, a.h2, 0, boxes, a.cols.box, x, a.cols.most, ring, sh, at);
-            else mk_columns<M, 16>(a, a.h2, 0, boxes, a.cols.box, x, a.cols.most, ring, sh, at);
+        if (a.cols.box <= 64) mk_columns<M, 8>(a, a.h2, 0, boxes, a.cols.box, u, MK_CBOX_COLS, ring, sh, at);
+        else mk_columns<M, 16>(a, a.h2, 0, boxes, a.cols.box, u, MK_CBOX_COLS, ring, sh, at);
+        at.skip_many(boxes);
+    }
+}
+
+// Wide form: the CTA's share of the down-projection, the activations of its blocks of 128 columns a few at a time.
+template <int M, int SLOTS>
+__device__ __forceinline__ void mk_down(const MkArgs &a, unsigned char *area, unsigned char *ring, MkShared *sh, MkPos<SLOTS> &at)
+{
+    constexpr bool TC = M >= MK_TC_ROWS;
+    constexpr int C = MK_CBOX_COLS, RS = C + 8, NB = 4;
+    const MkPairs w = sh->downs;
+    float *const x = reinterpret_cast<float *>(area);
+    bf16 *const planes = reinterpret_cast<bf16 *>(area);
+    for (int i = w.lo; i < w.hi;) {
+        const int b0 = i / w.boxes, nb = min(NB, (w.hi - 1) / w.boxes - b0 + 1);
+        if (i != w.lo) mk_consumer_sync();  // everyone is done with the blocks before
+        for (int k = threadIdx.x; k < nb * M * (C / 4); k += MK_CW * 32) {
+            const int c = k % (C / 4) * 4, m = k / (C / 4) % M, b = k / (C / 4) / M, col = (b0 + b) * C + c;
+            const float4 v = col < a.F && m < a.n_rows ? *reinterpret_cast<const float4 *>(a.act + (size_t)m * a.F + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (TC) {
+                uint2 hi, lo;
+                split_pair(v.x, v.y, hi.x, lo.x);
+                split_pair(v.z, v.w, hi.y, lo.y);
+                *reinterpret_cast<uint2 *>(planes + (size_t)(b * 2 * M + m) * RS + c) = hi;
+                *reinterpret_cast<uint2 *>(planes + (size_t)(b * 2 * M + M + m) * RS + c) = lo;
+            } else {
+                *reinterpret_cast<float4 *>(x + (b * M + m) * C + c) = v;
+            }
+        }
+        mk_consumer_sync();
+        for (int k = 0; k < nb; k++) {
+            const int r0 = i - (b0 + k) * w.boxes, n = min(w.boxes - r0, w.hi - i);
+            if constexpr (TC) mk_columns_tc<M>(a, a.h, r0, r0 + n, C, planes + k * 2 * M * RS, RS, ring, sh, at);
+            else mk_columns<M, 16>(a, a.h, r0, r0 + n, C, x + k * M * C, C, ring, sh, at);
+            i += n;
+            at.skip_many(n);
         }
     }
 }
@@ -184,16 +228,17 @@ __device__ __forceinline__ void mk_fold(const MkArgs &a, int i, int n)
     }
 }
 
-template <int M, int HD>
+template <int M, int HD, bool WIDE>
 __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
 {
+    constexpr int SLOTS = mk_slots(M, WIDE), AREA = mk_area_bytes(M, WIDE);
     extern __shared__ __align__(1024) unsigned char mk_smem[];  // (nothing else is in shared memory: the swizzled boxes need 1024)
     unsigned char *ring = mk_smem;
-    unsigned char *area = ring + (size_t)mk_slots(M) * MK_SLOT_BYTES;
-    MkShared *sh = reinterpret_cast<MkShared *>(area + mk_area_bytes(M));
+    unsigned char *area = ring + (size_t)SLOTS * MK_SLOT_BYTES;
+    MkShared *sh = reinterpret_cast<MkShared *>(area + AREA);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < mk_slots(M); s++) {
+        for (int s = 0; s < SLOTS; s++) {
             mbar_init(&sh->full[s], 1);
             mbar_init(&sh->empty[s], MK_CW);
         }
@@ -241,7 +286,8 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
             sh->att_batch = small && t >= sh->att_t1 ? k : 0;
             sh->bands[0].init(MK_QKV, a);
             sh->bands[1].init(MK_MLP, a);
-            sh->heads.init(a);
+            sh->heads.init(a, a.Hq);
+            if (WIDE) sh->downs.init(a, (a.F + MK_CBOX_COLS - 1) / MK_CBOX_COLS);
             sh->head0 = sh->heads.lo / sh->heads.boxes;
         }
     }
@@ -253,10 +299,10 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
     __syncthreads();
 
     if (warp >= MK_CW) {
-        mk_produce<M, HD>(a, ring, sh, warp - MK_CW);
+        mk_produce<M, HD, WIDE>(a, ring, sh, warp - MK_CW);
     } else {
         constexpr bool TC = M >= MK_TC_ROWS;
-        MkPos<mk_slots(M)> at{0, 0u};
+        MkPos<SLOTS> at{0, 0u};
         unsigned long long epoch = a.bar_base;
         if (blockIdx.x == 0 && threadIdx.x == 0 && a.trace) a.trace[0] = global_ns();
         bool ok = true;
@@ -265,25 +311,30 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
         gains.load(gain, a.d);
         for (int l = a.layer_begin; l < a.layer_end && ok; l++) {
             const bf16 *mlp_gain = a.layers[l].mlp_gain;
+            const float *h2 = WIDE ? nullptr : a.h2;
             if constexpr (TC) {
                 const int whole = (a.d + MK_BOX_COLS - 1) / MK_BOX_COLS * MK_BOX_COLS;
-                mk_rows_tc<M>(MK_QKV, a, l, reinterpret_cast<bf16 *>(area), reinterpret_cast<float *>(area + mk_tc_planes_bytes(M, whole)),
-                              a.h2, gain, gains, nullptr, 0, ring, sh, at);
+                mk_rows_tc<M, WIDE>(MK_QKV, a, l, reinterpret_cast<bf16 *>(area), reinterpret_cast<float *>(area + mk_tc_planes_bytes(M, whole)),
+                                    h2, gain, gains, nullptr, 0, ring, sh, at);
             } else {
-                mk_rows<M>(MK_QKV, a, l, reinterpret_cast<float *>(area), reinterpret_cast<float *>(area + mk_area_bytes(M) - mk_sums_bytes(M)),
-                           mk_sums_bytes(M), a.h2, gain, gains, nullptr, 0, ring, sh, at);
+                mk_rows<M, WIDE>(MK_QKV, a, l, reinterpret_cast<float *>(area), reinterpret_cast<float *>(area + AREA - mk_sums_bytes(M)),
+                                 mk_act_window(M, WIDE, mk_sums_bytes(M)), h2, gain, gains, nullptr, 0, ring, sh, at);
             }
             if (!(ok = mk_grid_barrier(a, sh, epoch))) break;
-            if (warp == MK_CW - 1) mk_fold(a, lane, 32);
-            mk_attention<M, HD>(a, l, area, ring, sh, at);
+            if (!WIDE && warp == MK_CW - 1) mk_fold(a, lane, 32);
+            mk_attention<M, HD, WIDE>(a, l, area, ring, sh, at);
             if (!(ok = mk_grid_barrier(a, sh, epoch))) break;
             mk_oproj<M, HD>(a, area, ring, sh, at);
             if (!(ok = mk_grid_barrier(a, sh, epoch, &gains, mlp_gain))) break;
-            mk_mlp<M>(a, l, mlp_gain, area, ring, sh, gains, at);
+            mk_mlp<M, WIDE>(a, l, mlp_gain, area, ring, sh, gains, at);
+            if constexpr (WIDE) {
+                if (!(ok = mk_grid_barrier(a, sh, epoch))) break;
+                mk_down<M>(a, area, ring, sh, at);
+            }
             gain = a.layers[min(l + 1, a.layer_end - 1)].attn_gain;
             ok = mk_grid_barrier(a, sh, epoch, &gains, gain);
         }
-        if (ok) mk_fold(a, (int)threadIdx.x, MK_CW * 32);
+        if (ok && !WIDE) mk_fold(a, (int)threadIdx.x, MK_CW * 32);
     }
     __syncthreads();
 }

@@ -87,7 +87,8 @@ __device__ __forceinline__ bool mk_grid_barrier(const MkArgs &a, MkShared *sh, u
 
 // x = (h + h2) / sqrt(mean((h + h2)^2) + eps) * gain for the M rows, left through put(row, column, four numbers); columns at
 // or beyond K, up to ncols, and rows from n_rows on are zeros.  Rows of up to MK_KEEP float4s per thread stay in
-// registers between the sum of squares and the scaling: one trip to the L2.
+// registers between the sum of squares and the scaling: one trip to the L2.  (Wider rows parked in the area
+// meanwhile, instead of read again: no difference, 130 us a layer at one row of 5,120 numbers, 194 at 7,168.)
 template <int M, class Put>
 __device__ __forceinline__ void mk_norm(int ncols, int K, int n_rows, const float *h, const float *h2, const bf16 *gain,
                                         const MkGains &gains, float eps, MkShared *sh, const Put &put)
@@ -304,24 +305,24 @@ __device__ __forceinline__ bool mk_take(uint4 (&w)[8], const unsigned char *ring
 // meet in shared memory once per eight bands.  (All sixteen warps on every slot, a row of both boxes each, took
 // 0.35 us a slot from a full ring, as long as HBM takes to fill it; in groups 0.2: a warp spends some ten cycles an
 // instruction, and waiting, releasing and reading the activations cost as much as the products.)
-// If M rows of the whole inner dimension fit the area they are loaded once; otherwise the area
-// holds a window of k-steps that is reloaded as the phase moves along.  gate/up leaves its results in u: column
-// (band - first band) * 16 + row of the box, of activation row m at u + m * u_stride.
+// `room` k-steps of M rows fit the area.  If that is the whole inner dimension they are loaded once; otherwise (WIDE only) the area
+// holds a window that is reloaded as the phase moves along.  gate/up leaves its results in u: column
+// (band - first band) * 16 + row of the box, of activation row m at u + m * u_stride; WIDE: in a.act.
 constexpr int MK_BATCH = 8;  // bands whose sums wait in shared memory
 __host__ __device__ constexpr int mk_sums_bytes(int M) { return MK_BATCH * 2 * MK_BOX_ROWS * M * MK_GROUPS * 4; }
 
-template <int M>
-__device__ __forceinline__ void mk_rows(int type, const MkArgs &a, int l, float *act, float *sums, int own, const float *h2,
+template <int M, bool WIDE, int SLOTS>
+__device__ __forceinline__ void mk_rows(int type, const MkArgs &a, int l, float *act, float *sums, int room, const float *h2,
                                         const bf16 *gain, const MkGains &gains, float *u, int u_stride, unsigned char *ring,
-                                        MkShared *sh, MkPos<mk_slots(M)> &at)
+                                        MkShared *sh, MkPos<SLOTS> &at)
 {
     constexpr int ROWS = MK_BOX_ROWS / (MK_CW / MK_GROUPS), N = 2 * ROWS * M;  // rows of a box per warp; sums per warp
     static_assert(ROWS == 4, "mk_take");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / MK_GROUPS, sub = warp % MK_GROUPS;
     MkBands w = sh->bands[type == MK_QKV ? 0 : 1];
     if (w.j >= w.end) return;
-    const int first = w.j, n_bands = (w.end - w.j + w.step - 1) / w.step, room = mk_act_window(M, own);
-    const bool whole = w.k_steps <= room;
+    const int first = w.j, n_bands = (w.end - w.j + w.step - 1) / w.step;
+    const bool whole = !WIDE || w.k_steps <= room;
     const int window = whole ? w.k_steps : room, ncols = window * MK_BOX_COLS;
     bool live = true;        // false: a wait ran out, this warp only keeps the barriers whole
     if (whole)
@@ -339,7 +340,7 @@ __device__ __forceinline__ void mk_rows(int type, const MkArgs &a, int l, float 
                 const int n = min(window, w.k_steps - win0);
                 if (!whole) mk_norm_window<M>(act, win0 * MK_BOX_COLS, ncols, a.d, a.h, h2, gain, a.eps, sh);
                 const int ahead = (grp - at.s) & (MK_GROUPS - 1);
-                MkPos<mk_slots(M)> p = at;
+                MkPos<SLOTS> p = at;
                 p.skip(ahead);
                 for (int k = ahead; k < n && live; k += MK_GROUPS, p.skip(MK_GROUPS)) {
                     uint4 wt[2 * ROWS];
@@ -381,7 +382,8 @@ __device__ __forceinline__ void mk_rows(int type, const MkArgs &a, int l, float 
             const float4 s1 = reinterpret_cast<const float4 *>(sums)[(b * 2 * MK_BOX_ROWS + MK_BOX_ROWS + rib) * M + m];
             const float v0 = (s0.x + s0.y) + (s0.z + s0.w), v1 = (s1.x + s1.y) + (s1.z + s1.w);
             if (type == MK_QKV) mk_finish_qkv(a, l, b0 + b == 0 ? sh->fin[i] : mk_fin(a, sh, first + (b0 + b) * w.step, rib, m), v0, v1);
-            else u[m * u_stride + (b0 + b) * MK_BOX_ROWS + rib] = mk_silu_mul(v0, v1);
+            else if (!WIDE) u[m * u_stride + (b0 + b) * MK_BOX_ROWS + rib] = mk_silu_mul(v0, v1);
+            else if (const int c = (first + (b0 + b) * w.step) * MK_BOX_ROWS + rib; c < a.F) a.act[(size_t)m * a.F + c] = mk_silu_mul(v0, v1);
         }
         if (b0 + MK_BATCH < n_bands) mk_consumer_sync();
     }
@@ -393,9 +395,9 @@ __device__ __forceinline__ void mk_rows(int type, const MkArgs &a, int l, float 
 // warps of group s mod 4, sixteen rows each.  LPR lanes share a row, eight columns each, whose activations they hold
 // in registers: the products of a box need nothing but the weights from shared memory, and the sums of
 // sixteen rows meet in 8 (one row of activations) or 15 (two) shuffles.
-template <int M, int LPR>
+template <int M, int LPR, int SLOTS>
 __device__ __forceinline__ void mk_columns(const MkArgs &a, float *dst, int r0, int r1, int cols, const float *x, int x_stride,
-                                           unsigned char *ring, MkShared *sh, MkPos<mk_slots(M)> at)
+                                           unsigned char *ring, MkShared *sh, MkPos<SLOTS> at)
 {
     constexpr int RPL = 32 / LPR, NL = 16 / RPL;  // rows per load, loads per box
     static_assert(NL <= 8, "mk_take");
@@ -443,13 +445,11 @@ __device__ __forceinline__ void mk_columns(const MkArgs &a, float *dst, int r0, 
 // the end.  In the row form a warp of a slot's four takes one box and half of its columns, and the eight shares of a
 // box (four groups, two halves) meet in shared memory at the end of a band.
 constexpr int MK_TC_RED_BYTES = 2 * 2 * 8 * 16 * 8 * 4;  // [parity][box][share][16 rows][8 n] floats = 16 KB
-// The area with three and four rows: planes of d columns, the band sums, planes of the CTA's own `most` columns.
-__host__ __device__ inline size_t mk_tc_planes_bytes(int M, int cols) { return (size_t)2 * M * (cols + 8) * 2; }
-inline bool mk_tc_fits(int M, int d, int most)
-{
-    const int whole = (d + MK_BOX_COLS - 1) / MK_BOX_COLS * MK_BOX_COLS;
-    return mk_tc_planes_bytes(M, whole) + MK_TC_RED_BYTES + mk_tc_planes_bytes(M, most) <= (size_t)mk_area_bytes(M);
-}
+// The area with three and four rows: planes of d columns, the band sums, planes of the CTA's own columns.
+__host__ __device__ constexpr size_t mk_tc_planes_bytes(int M, int cols) { return (size_t)2 * M * (cols + 8) * 2; }
+constexpr int MK_TC_STEPS = 17;  // k-steps of a residual row
+static_assert(mk_tc_planes_bytes(MK_MAX_ROWS, MK_TC_STEPS * MK_BOX_COLS) + MK_TC_RED_BYTES + mk_tc_planes_bytes(MK_MAX_ROWS, MK_CBOX_COLS) <=
+                  (size_t)mk_area_bytes(MK_MAX_ROWS, false), "planes");
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -472,11 +472,11 @@ __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr)
                  : "memory");
 }
 
-// Row form.  gate/up leaves its results as planes of their own, u_planes, row stride u_rs.
-template <int M>
+// Row form.  gate/up leaves its results as planes of their own, u_planes, row stride u_rs; WIDE: as fp32 in a.act.
+template <int M, bool WIDE, int SLOTS>
 __device__ __forceinline__ void mk_rows_tc(int type, const MkArgs &a, int l, bf16 *planes, float *red, const float *h2,
                                            const bf16 *gain, const MkGains &gains, bf16 *u_planes, int u_rs, unsigned char *ring,
-                                           MkShared *sh, MkPos<mk_slots(M)> &at)
+                                           MkShared *sh, MkPos<SLOTS> &at)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
@@ -503,7 +503,7 @@ __device__ __forceinline__ void mk_rows_tc(int type, const MkArgs &a, int l, bf1
     for (; w.j < w.end; w.j += w.step) {
         float acc[4] = {0.f, 0.f, 0.f, 0.f}, acc2[4] = {0.f, 0.f, 0.f, 0.f};
         const int ahead = (grp - at.s) & (MK_GROUPS - 1);
-        MkPos<mk_slots(M)> p = at;
+        MkPos<SLOTS> p = at;
         p.skip(ahead);
         for (int ks = ahead; ks < w.k_steps && live; ks += MK_GROUPS, p.skip(MK_GROUPS)) {
             if (!(live = mbar_wait(&sh->full[p.s], p.ph, &sh->giving_up, a.status))) break;
@@ -542,6 +542,8 @@ __device__ __forceinline__ void mk_rows_tc(int type, const MkArgs &a, int l, bf1
             }
             if (type == MK_QKV) {
                 mk_finish_qkv(a, l, band_it == 0 ? sh->fin[threadIdx.x] : mk_fin(a, sh, w.j, rib, m), v0, v1);
+            } else if (WIDE) {
+                if (const int c = w.j * MK_BOX_ROWS + rib; c < a.F) a.act[(size_t)m * a.F + c] = mk_silu_mul(v0, v1);
             } else {
                 const int c = (w.j - first) * MK_BOX_ROWS + rib;
                 mk_put_planes<M>(u_planes, u_rs, m, c, mk_silu_mul(v0, v1));  // (rows beyond n_rows: their planes are zeros)
@@ -553,9 +555,9 @@ __device__ __forceinline__ void mk_rows_tc(int type, const MkArgs &a, int l, bf1
 
 // Column form (see mk_columns): a warp's sixteen rows are the A operand, the activations of the columns sit in
 // registers as B operands, and a box's sums need no other warp.  x: planes of M rows, row stride x_rs.
-template <int M>
+template <int M, int SLOTS>
 __device__ __forceinline__ void mk_columns_tc(const MkArgs &a, float *dst, int r0, int r1, int cols, const bf16 *x, int x_rs,
-                                              unsigned char *ring, MkShared *sh, MkPos<mk_slots(M)> at)
+                                              unsigned char *ring, MkShared *sh, MkPos<SLOTS> at)
 {
     constexpr int KS = MK_CBOX_COLS / 16;
     static_assert(2 * M == 8, "the exchange below adds column n + M to column n");

@@ -651,10 +651,10 @@ def test_persistent_kernel_tensor_core_form_for_three_and_four_rows(util, K, max
 
 
 @pytest.mark.parametrize("rows", [3, 4])
-@pytest.mark.parametrize("d_ffn", [4352, 4416, 9280])
-def test_persistent_kernel_mlp_windows(util, rows, d_ffn):
-    """Three and four rows in the persistent kernel with an MLP whose activations just fit the shared-memory
-    area (17 steps of 256 columns), just do not, and take several half windows with a ragged end."""
+@pytest.mark.parametrize("d_ffn", [4352, 9280, 18944, 18976 + 32])
+def test_persistent_kernel_mlp_shares(util, rows, d_ffn):
+    """Three and four rows in the persistent kernel with an MLP of which a CTA has one box of 128 columns at most, filled
+    to the last, and just more, which takes the wide form (148 SMs)."""
     dims = synth.model_dims(dict(MICRO256, d_ffn=d_ffn, n_layers=2), 1, 4, 0)
     w = synth.make_weights(dims, seed=19)
     prompts = synth.make_prompts(dims, rows, 5, 30, seed=4)
@@ -698,15 +698,24 @@ def test_three_and_four_wide_rows(util, rows, d_model, route):
     # a CTA's MLP columns: none for most CTAs, a lone band, boxes that reach into the next CTA's columns
     (dict(d_model=256, n_q_heads=4, n_kv_heads=2, head_dim=64, d_ffn=64), (1,)),
     (dict(d_model=200, n_q_heads=6, n_kv_heads=3, head_dim=64, d_ffn=712), (17, 30)),
-    # 148 SMs x 128 columns and a little: two boxes a CTA; nine bands a CTA meet in two batches of sums
+    # 148 SMs x 128 columns and a little: the wide form; nine bands a CTA meet in two batches of sums
     (dict(d_model=64, n_q_heads=2, n_kv_heads=1, head_dim=128, d_ffn=19200), (33,)),
     (dict(d_model=128, n_q_heads=2, n_kv_heads=2, head_dim=64, d_ffn=19008), (5, 64, 16)),
-    # sixteen query heads a kv head (blocks of sixteen query vectors) and more cache tiles than SMs, several a CTA
+    # sixteen query heads a kv head (two blocks of eight query vectors), fewer cache tiles than SMs; three or four tiles a CTA
     (dict(d_model=192, n_q_heads=16, n_kv_heads=1, head_dim=64, d_ffn=320), (900, 3)),
     (dict(d_model=128, n_q_heads=8, n_kv_heads=4, head_dim=64, d_ffn=256), (1300, 15, 48, 700)),
-    # a residual row wider than the registers of the norm hold, and with two rows than the area
+    # wide form with a last block of 128 columns that is ragged, one to four rows
+    (dict(d_model=136, n_q_heads=2, n_kv_heads=1, head_dim=128, d_ffn=19016), (21,)),
+    (dict(d_model=136, n_q_heads=2, n_kv_heads=1, head_dim=64, d_ffn=19016), (21, 5)),
+    (dict(d_model=192, n_q_heads=2, n_kv_heads=2, head_dim=128, d_ffn=38080), (21, 5, 30, 12)),
+    # a residual row wider than the registers of the norm hold; one that needs the wide form, just not and just so; whole with one row
+    # and two rows, and in windows
     (dict(d_model=4352, n_q_heads=2, n_kv_heads=1, head_dim=64, d_ffn=128), (20,)),
+    (dict(d_model=7168, n_q_heads=2, n_kv_heads=1, head_dim=64, d_ffn=2400), (20,)),
+    (dict(d_model=7176, n_q_heads=2, n_kv_heads=1, head_dim=128, d_ffn=2400), (20,)),
     (dict(d_model=11264, n_q_heads=2, n_kv_heads=1, head_dim=64, d_ffn=64), (18, 9)),
+    (dict(d_model=11520, n_q_heads=2, n_kv_heads=1, head_dim=64, d_ffn=256), (18, 9)),
+    (dict(d_model=23808, n_q_heads=2, n_kv_heads=1, head_dim=64, d_ffn=2400), (18,)),
 ])
 def test_persistent_kernel_at_the_edges_of_its_shares(util, shape, lens):
     """One to four rows through the persistent kernel (and the flushes of what they leave pending where those are
