@@ -58,9 +58,10 @@ constexpr int MK_BOX_BYTES = MK_BOX_ROWS * MK_BOX_COLS * 2;  // 8 KB
 constexpr int MK_CBOX_ROWS = 64, MK_CBOX_COLS = 128;         // column form: one box of 64 rows and up to 128 columns per slot
 constexpr int MK_SLOT_BYTES = 2 * MK_BOX_BYTES;
 constexpr int MK_IN_FLIGHT = 8;                 // slots on their way at once, in the MLP
-// and before it, with one row (narrow form).  A trip to the L2 queues behind the copies on their way to the SM, 2.7 us of them at eight
-// slots, and the phases before the MLP are chains of such trips with little to stream: 81.7 us a layer with eight
-// throughout, 80.8 with four here.
+// and before it, with one row (narrow form) and no more than one band of q/k/v a CTA.  A trip to the L2 queues behind the copies
+// on their way to the SM, 2.7 us of them at eight slots, and the phases before the MLP are chains of such trips with little to
+// stream: us a layer after 1,000 positions with eight / four here 92.8 / 91.4 (28 query heads, 4 kv heads), 84.5 / 82.7 (32, 2); with
+// two bands a CTA 94.4 / 95.4 (32, 8), with four 130.6 / 137.6 (40, 40).
 constexpr int MK_FEW_IN_FLIGHT = 4;
 constexpr int MK_MAX_ROWS = 4;
 constexpr int MK_TC_ROWS = 3;                   // rows from which the tensor-core form runs

@@ -15,7 +15,7 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
     bool ok = true;
     // waits until item idx's slot is free and no more than `flight` items (counting this one) are on
     // their way, and announces `bytes`; item idx - flight was this warp's own
-    constexpr uint32_t few = M == 1 && !WIDE ? MK_FEW_IN_FLIGHT : MK_IN_FLIGHT;
+    const uint32_t few = M == 1 && !WIDE && sh->bands[0].end <= (int)gridDim.x ? MK_FEW_IN_FLIGHT : MK_IN_FLIGHT;
     uint32_t flight = few;
     static_assert(MK_IN_FLIGHT % MK_PW == 0 && MK_FEW_IN_FLIGHT % MK_PW == 0 && SLOTS % MK_PW == 0, "a producer waits for items of its own");
     auto open = [&](uint32_t bytes) {
