@@ -226,9 +226,12 @@ struct MkPairs {
 // for as many SMs); a run is what a share has of one pair.  The run of pair p in CTA c leaves partial number
 // c + p (both only ever grow from one run to the next), for every query vector of the pair.
 struct MkRun {
+    int t;                          // where it begins in the CTA's share
     int g, hk, tile0, n;            // group, kv head, first tile, tiles
     int row0, nrows, pos0, cache0;  // the group's rows; first cache row of (slot, kv head)
     int nq, n_qblk;                 // query vectors, blocks of eight of them
+    int warp0, nsub, item0;         // first warp, warps a block, ring items of the runs beside it
+    int part;                       // its partial
 };
 // What a row of weights of the q/k/v projection becomes: a rotary pair of q or k, or two numbers of v.
 struct MkFin {

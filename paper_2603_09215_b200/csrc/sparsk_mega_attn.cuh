@@ -3,48 +3,53 @@
 
 namespace sparsk {
 
-// A warp's view of a run's ring items: items sub, sub + nsub, ... of the run, two 16-position tiles each (K and
+// A warp's view of a run's ring items: items first, first + nsub, ... behind `at`, two 16-position tiles each (K and
 // V, with the 128-byte swizzle, as the producers' TMA copies leave them), in the form attn_item_t asks for.
 // The tiles were on their way before this launch's q/k/v projection had written the current rows' keys and
 // values: those rows are copied over from the cache, and value rows past the end are cleared (they meet a
 // weight of exactly zero, which must not meet a NaN).  Every warp that reads a tile does both for itself.
+// What only a run's last tile or its end asks for is read from the run then: registers held across the tiles are spilled elsewhere, and a
+// reload behind a grid barrier is a trip to the L2.
 template <int HD, int SLOTS>
 struct MkTiles {
     static constexpr int TILE = AT_TP * HD;   // numbers of one matrix's tile
-    unsigned char *ring;
+    const MkArgs &a;
+    const MkRun *r;
     MkShared *sh;
-    int *status;
-    const kv_t *kbase, *vbase;    // the cache of (slot, kv head)
-    MkPos<SLOTS> at0;             // ring place of the run's first tiles
-    int tile0, sub, nsub;
-    int new0, end;                // the pass's own positions: [new0, end), end = the prefix's length
+    unsigned char *ring;
+    const MkPos<SLOTS> &at;       // the ring's place of item 0
+    int layer, lane;
+    int first, nsub;
+    int tile0;                    // first tile of item 0
+    int new0, w_end;              // the pass's own positions begin; no position from here on counts
     int arrivals;                 // this warp's share of a slot's release
-    int w_end;                    // no position from here on counts
-    int n_tiles, lane;
+    int n_tiles;
 
     __device__ __forceinline__ static int off(int row, int c) { return at_swz<HD>(row, c); }
-    __device__ __forceinline__ int item(int t) const { return sub + nsub * (t >> 1); }
+    __device__ __forceinline__ int item(int t) const { return first + nsub * (t >> 1); }
     __device__ __forceinline__ MkPos<SLOTS> place(int t) const
     {
-        MkPos<SLOTS> p = at0;
+        MkPos<SLOTS> p = at;
         p.skip_many(item(t));
         return p;
     }
     __device__ __forceinline__ int pos(int t) const { return (tile0 + 2 * item(t) + (t & 1)) * AT_TP; }
     __device__ __forceinline__ bool wait(int t, const kv_t *&Kt, const kv_t *&Vt) const
     {
-        const MkPos<SLOTS> at = place(t);
-        if (!(t & 1) && !mbar_wait(&sh->full[at.s], at.ph, &sh->giving_up, status)) return false;
-        kv_t *kt = reinterpret_cast<kv_t *>(ring + (size_t)at.s * MK_SLOT_BYTES) + (t & 1) * 2 * TILE, *vt = kt + TILE;
+        const MkPos<SLOTS> p = place(t);
+        if (!(t & 1) && !mbar_wait(&sh->full[p.s], p.ph, &sh->giving_up, a.status)) return false;
+        kv_t *kt = reinterpret_cast<kv_t *>(ring + (size_t)p.s * MK_SLOT_BYTES) + (t & 1) * 2 * TILE, *vt = kt + TILE;
         const int p0 = pos(t);
         if (p0 + AT_TP > new0) {
             constexpr int CH = HD / 8;
+            const int end = min(new0 + r->nrows, a.S);
+            const size_t base = layer * a.kv_layer + (size_t)r->cache0 * HD;
             for (int k = lane; k < AT_TP * CH; k += 32) {
-                const int r = k / CH, c = k % CH, p = p0 + r;
-                if (p < new0) continue;
-                const size_t o = (size_t)p * HD + c * 8;
-                if (p < end) *reinterpret_cast<uint4 *>(&kt[off(r, c)]) = __ldcg(reinterpret_cast<const uint4 *>(kbase + o));
-                *reinterpret_cast<uint4 *>(&vt[off(r, c)]) = p < end ? __ldcg(reinterpret_cast<const uint4 *>(vbase + o)) : make_uint4(0u, 0u, 0u, 0u);
+                const int row = k / CH, c = k % CH, q = p0 + row;
+                if (q < new0) continue;
+                const size_t o = base + (size_t)q * HD + c * 8;
+                if (q < end) *reinterpret_cast<uint4 *>(&kt[off(row, c)]) = __ldcg(reinterpret_cast<const uint4 *>(a.kc + o));
+                *reinterpret_cast<uint4 *>(&vt[off(row, c)]) = q < end ? __ldcg(reinterpret_cast<const uint4 *>(a.vc + o)) : make_uint4(0u, 0u, 0u, 0u);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the slot's next copy
         }
@@ -63,13 +68,20 @@ struct MkTiles {
     __device__ __forceinline__ void start() const {}
     __device__ __forceinline__ void finish() const {}
 };
-// Where it leaves its partial: the run's place in global memory, or the area, when several warps share the run.
+// Where it leaves its partial: the run's place in global memory, or, when several warps share the run, the warp's cell in the area.
 template <int HD>
 struct MkCells {
-    float *po;
-    float2 *pml;
-    __device__ __forceinline__ float *o(int qg) const { return po + (ptrdiff_t)qg * HD; }
-    __device__ __forceinline__ float2 *ml(int qg) const { return pml + qg; }
+    const MkArgs &a;
+    const MkRun *r;
+    unsigned char *cell;
+    __device__ __forceinline__ float *o(int qg) const
+    {
+        return r->nsub > 1 ? reinterpret_cast<float *>(cell) + (qg % 8) * HD : a.part_o + (size_t)(r->part + qg) * HD;
+    }
+    __device__ __forceinline__ float2 *ml(int qg) const
+    {
+        return r->nsub > 1 ? reinterpret_cast<float2 *>(cell + 8 * HD * 4) + qg % 8 : a.part_ml + r->part + qg;
+    }
 };
 // One warp's partial of a block of eight query vectors and its sums.
 template <int HD>
@@ -77,10 +89,76 @@ __host__ __device__ constexpr int mk_cell_bytes() { return 8 * HD * 4 + 8 * 8; }
 // Shapes the phase can run: a warp per block of query vectors of a group.
 inline bool mk_attn_fits(int M, int G) { return (M * G + 7) / 8 <= MK_CW; }
 
-// The CTA's runs, one after another.  Up to four warps per block of eight query vectors share a run (as many as the area
-// has room for partials, and two slots at least each), every nsub-th slot each; their partials meet in the area.
+// The run that begins with tile t of the CTA's share, on its own: up to four warps per block of eight query vectors share it (as many as the
+// area has room for partials, and two slots at least each), every nsub-th slot each.
+template <int M, int HD, bool WIDE>
+__device__ __forceinline__ void mk_run_alone(const MkArgs &a, MkShared *sh, int t, MkRun &r)
+{
+    constexpr int WARPS = mk_area_bytes(M, WIDE) / mk_cell_bytes<HD>() < MK_CW ? mk_area_bytes(M, WIDE) / mk_cell_bytes<HD>() : MK_CW;
+    mk_run_at(a, sh, t, sh->att_t1, r);
+    r.t = t;
+    r.warp0 = r.item0 = 0;
+    r.part = (int)(blockIdx.x + r.g * a.Hkv + r.hk) * mk_part_rows(a);
+    r.nsub = max(1, min(min(4, ((r.n + 1) / 2 + 1) / 2), WARPS / r.n_qblk));
+    if (mk_slots(M, WIDE) % r.nsub) r.nsub = 2;  // a slot's successive fills stay with one warp
+}
+// The first runs of the CTA (lane 0 of one warp, once a launch).  Are they worked on side by side?  If there are several, the ring holds all their
+// tiles (so none of its slots is filled twice before the warps meet again), and a warp per block of query vectors is to be had: then
+// with as many warps a block as above, or half as many, as long as there are warps and room for their partials.
+template <int M, int HD, bool WIDE>
+__device__ __forceinline__ void mk_runs(const MkArgs &a, MkShared *sh)
+{
+    constexpr int ROOM = mk_area_bytes(M, WIDE) / mk_cell_bytes<HD>();
+    int t = sh->att_t0, n = 0, items = 0, blocks = 0;
+    for (; n < MK_RUNS && t < sh->att_t1; n++) {
+        MkRun &r = sh->runs[n];
+        mk_run_alone<M, HD, WIDE>(a, sh, t, r);
+        t += r.n;
+        items += (r.n + 1) / 2;
+        blocks += r.n_qblk;
+    }
+    sh->att_batch = t >= sh->att_t1 && n > 1 && items <= mk_slots(M, WIDE) && blocks <= MK_CW ? n : 0;
+    if (!sh->att_batch) return;
+    for (int want = 4, warps = MK_CW + 1; want >= 1 && warps > min(MK_CW, ROOM); want /= 2) {
+        warps = items = 0;
+        for (int i = 0; i < n; i++) {
+            MkRun &r = sh->runs[i];
+            r.nsub = min(want, ((r.n + 1) / 2 + 1) / 2);
+            r.warp0 = warps;
+            r.item0 = items;
+            warps += r.nsub * r.n_qblk;
+            items += (r.n + 1) / 2;
+        }
+    }
+}
+
+// The n query vectors of a run whose `nb` blocks of eight had `nsub` warps each: their partials, merged, to number `part`.
+template <int HD>
+__device__ __forceinline__ void mk_meet(const MkArgs &a, const unsigned char *cells, int nb, int nsub, int n, size_t part)
+{
+    for (int k = threadIdx.x; k < n * (HD / 4); k += MK_CW * 32) {
+        const int ql = k / (HD / 4), c4 = k % (HD / 4);
+        const unsigned char *first = cells + (size_t)(ql / 8) * mk_cell_bytes<HD>();
+        float mx = -INFINITY, sum = 0.f;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int s = 0; s < nsub; s++)
+            mx = fmaxf(mx, reinterpret_cast<const float2 *>(first + (size_t)s * nb * mk_cell_bytes<HD>() + 8 * HD * 4)[ql % 8].x);
+        for (int s = 0; s < nsub; s++) {
+            const unsigned char *c = first + (size_t)s * nb * mk_cell_bytes<HD>();
+            const float2 ml = reinterpret_cast<const float2 *>(c + 8 * HD * 4)[ql % 8];
+            const float w = ml.x == -INFINITY ? 0.f : __expf(ml.x - mx);
+            const float4 p = reinterpret_cast<const float4 *>(c)[ql % 8 * (HD / 4) + c4];
+            sum += ml.y * w;
+            o.x += p.x * w; o.y += p.y * w; o.z += p.z * w; o.w += p.w * w;
+        }
+        *reinterpret_cast<float4 *>(a.part_o + (part + ql) * HD + c4 * 4) = o;
+        if (c4 == 0) a.part_ml[part + ql] = make_float2(mx, sum);
+    }
+}
+
+// The CTA's runs: side by side, or one after another (mk_runs); the partials of warps that share a run meet in the area.
 // (Blocks of sixteen, positions as columns, cost 450 bytes of spills, and a reload behind a grid barrier is a trip to the L2: flushes of
-// four rows of the 28-layer shape 96.6 us a layer, so 90.9.)  Short runs go side by side, a warp per block.
+// four rows of the 28-layer shape 96.6 us a layer, so 90.9.)
 template <int M, int HD, bool WIDE, int SLOTS>
 __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned char *area, unsigned char *ring, MkShared *sh,
                                              MkPos<SLOTS> &at)
@@ -88,98 +166,50 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = a.Hq / a.Hkv;
     AttnArgs aa{};
     aa.q32 = a.q_buf; aa.Hq = a.Hq; aa.Hkv = a.Hkv;
-    const int stride = mk_part_rows(a), end = sh->att_t1;
-    int t = sh->att_t0;
-    MkRun r = sh->runs[0];
-    const int batch = M == 1 ? 0 : sh->att_batch; // (one row has one group: its runs are long or alone)
-    while (t < end) {
-        int n_items = (r.n + 1) / 2, nsub = 1, sub = 0, qb = warp, before = 0;  // items before this warp's run
-        if (M > 1 && batch > 1) {
-            // (no more slots than the ring has, so none of them is filled twice before the warps meet again)
-            static_assert(2 * MK_RUNS <= SLOTS, "slots of a batch");
-            int mine = -1, w0 = 0;
-            n_items = 0;
-            for (int i = 0; i < batch; i++) {
-                const int nb = sh->runs[i].n_qblk;
-                if (warp >= w0 && warp < w0 + nb) {
-                    mine = i;
-                    qb = warp - w0;
-                    before = n_items;
-                }
-                w0 += nb;
-                n_items += (sh->runs[i].n + 1) / 2;
+    if (sh->att_t0 >= sh->att_t1) return;
+    // Nothing of a run is held in registers across its tiles: it is read from shared memory before and after.  The one behind it is
+    // worked out beside it, in the last three places in turn (whoever is late may still read the one before).
+    static_assert(MK_RUNS == 4, "places");
+    for (int at_run = 0;;) {
+        {
+            const MkRun *r = &sh->runs[at_run];
+            if (const int batch = sh->att_batch) {
+                for (int i = 1; i < batch; i++)
+                    if (warp >= sh->runs[i].warp0) r = &sh->runs[i];
+            } else if (threadIdx.x == (MK_CW - 1) * 32 && r->t + r->n < sh->att_t1) {
+                mk_run_alone<M, HD, WIDE>(a, sh, r->t + r->n, sh->runs[at_run == 3 ? 1 : at_run + 1]);
             }
-            if (mine >= 0) r = sh->runs[mine];
-            else sub = 1;
-        } else {
-            nsub = min(4, (n_items + 1) / 2);
-            if (nsub > 1) {
-                const int room = mk_area_bytes(M, WIDE) / (r.n_qblk * mk_cell_bytes<HD>());
-                nsub = max(1, min(nsub, min(MK_CW / r.n_qblk, room)));
-            }
-            if (SLOTS % nsub) nsub = 2;  // a slot's successive fills stay with one warp
-            if (r.n_qblk > 1) {
-                sub = warp / r.n_qblk;
-                qb = warp - sub * r.n_qblk;
-            } else {
-                sub = warp;
-                qb = 0;
+            const int nb = r->n_qblk, nsub = r->nsub, in_run = warp - r->warp0, sub = nb > 1 ? in_run / nb : in_run;
+            if (sub < nsub) {
+                const int qb = nb > 1 ? in_run - sub * nb : 0;
+                AtItem item;
+                item.qb = qb; item.hk = r->hk; item.row0 = r->row0; item.nrows = r->nrows; item.pos0 = r->pos0; item.nq = r->nq;
+                MkTiles<HD, SLOTS> tiles{a, r, sh, ring, at, l, lane};
+                tiles.first = r->item0 + sub; tiles.nsub = nsub; tiles.tile0 = r->tile0 - 2 * r->item0;
+                tiles.new0 = r->pos0;
+                tiles.w_end = min(r->pos0 + (r->nrows == 1 ? 0 : (min(qb * 8 + 8, r->nq) - 1) / G) + 1, a.S);
+                tiles.arrivals = qb == 0 ? MK_CW - (nb - 1) : 1;
+                const int run_items = (r->n + 1) / 2, mine = nsub == 1 ? run_items : (run_items - sub + nsub - 1) / nsub;
+                tiles.n_tiles = 2 * mine - ((r->n & 1) && sub + nsub * (mine - 1) == run_items - 1 ? 1 : 0);
+                const MkCells<HD> out{a, r, area + (size_t)warp * mk_cell_bytes<HD>()};
+                attn_item_t<HD>(aa, item, nullptr, lane, nullptr, &tiles, &out);
             }
         }
-        const int nq = r.nq, n_qblk = r.n_qblk, run_items = (r.n + 1) / 2;
-        const size_t part = (size_t)(blockIdx.x + r.g * a.Hkv + r.hk) * stride;
-        if (sub < nsub) {
-            AtItem item;
-            item.qb = qb; item.hk = r.hk; item.row0 = r.row0; item.nrows = r.nrows; item.pos0 = r.pos0; item.nq = nq;
-            const int w_end = min(r.pos0 + (r.nrows == 1 ? 0 : (min(qb * 8 + 8, nq) - 1) / G) + 1, a.S);
-            MkTiles<HD, SLOTS> tiles;
-            tiles.ring = ring; tiles.sh = sh; tiles.status = a.status;
-            tiles.kbase = a.kc + l * a.kv_layer + (size_t)r.cache0 * HD; tiles.vbase = a.vc + l * a.kv_layer + (size_t)r.cache0 * HD;
-            tiles.at0 = at;
-            tiles.at0.skip_many(before);
-            tiles.tile0 = r.tile0; tiles.sub = sub; tiles.nsub = nsub;
-            tiles.new0 = r.pos0; tiles.end = min(r.pos0 + r.nrows, a.S);
-            tiles.arrivals = qb == 0 ? MK_CW - (n_qblk - 1) : 1;
-            const int mine = nsub == 1 ? run_items : (run_items - sub + nsub - 1) / nsub;
-            tiles.n_tiles = 2 * mine - ((r.n & 1) && sub + nsub * (mine - 1) == run_items - 1 ? 1 : 0);
-            tiles.lane = lane; tiles.w_end = w_end;
-            MkCells<HD> out;
-            if (nsub > 1) {
-                // query vector qg of block qb at row qg - 8 qb of the warp's cells
-                unsigned char *c = area + (size_t)(sub * n_qblk + qb) * mk_cell_bytes<HD>();
-                out.po = reinterpret_cast<float *>(c) - (ptrdiff_t)qb * 8 * HD;
-                out.pml = reinterpret_cast<float2 *>(c + 8 * HD * 4) - qb * 8;
-            } else {
-                out.po = a.part_o + part * HD;
-                out.pml = a.part_ml + part;
-            }
-            attn_item_t<HD>(aa, item, nullptr, lane, nullptr, &tiles, &out);
-        }
-        at.skip_many(n_items);
         mk_consumer_sync();
-        if (nsub > 1) {
-            for (int k = threadIdx.x; k < nq * (HD / 4); k += MK_CW * 32) {
-                const int qg = k / (HD / 4), c4 = k % (HD / 4), blk = qg / 8, ql = qg % 8;
-                float mx = -INFINITY, sum = 0.f;
-                float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int s = 0; s < nsub; s++)
-                    mx = fmaxf(mx, reinterpret_cast<const float2 *>(area + (size_t)(s * n_qblk + blk) * mk_cell_bytes<HD>() + 8 * HD * 4)[ql].x);
-                for (int s = 0; s < nsub; s++) {
-                    const unsigned char *c = area + (size_t)(s * n_qblk + blk) * mk_cell_bytes<HD>();
-                    const float2 ml = reinterpret_cast<const float2 *>(c + 8 * HD * 4)[ql];
-                    const float w = ml.x == -INFINITY ? 0.f : __expf(ml.x - mx);
-                    const float4 p = reinterpret_cast<const float4 *>(c)[ql * (HD / 4) + c4];
-                    sum += ml.y * w;
-                    o.x += p.x * w; o.y += p.y * w; o.z += p.z * w; o.w += p.w * w;
-                }
-                *reinterpret_cast<float4 *>(a.part_o + (part + qg) * HD + c4 * 4) = o;
-                if (c4 == 0) a.part_ml[part + qg] = make_float2(mx, sum);
+        const int batch = sh->att_batch;
+        const MkRun *r = &sh->runs[batch ? batch - 1 : at_run];  // (the last of several)
+        at.skip_many(r->item0 + (r->n + 1) / 2);
+        bool met = false;
+        for (int i = batch ? 0 : at_run; i <= (batch ? batch - 1 : at_run); i++) {
+            const MkRun *b = &sh->runs[i];
+            if (b->nsub > 1) {
+                mk_meet<HD>(a, area + (size_t)b->warp0 * mk_cell_bytes<HD>(), b->n_qblk, b->nsub, b->nq, (size_t)b->part);
+                met = true;
             }
-            mk_consumer_sync();  // the next run may use the area
         }
-        if (batch > 1) break;
-        t += r.n;
-        if (t < end) mk_run_at(a, sh, t, end, r);
+        if (batch || r->t + r->n >= sh->att_t1) break;
+        at_run = at_run == 3 ? 1 : at_run + 1;
+        if (met) mk_consumer_sync();  // what comes next may use the area
     }
 }
 

@@ -273,17 +273,7 @@ __global__ void __launch_bounds__(MK_THREADS, 1) mega_kernel(const MkArgs a)
             sh->att_ctas = (int)n;
             sh->att_t0 = c < n ? (int)(c * (unsigned)base / n) : 0;
             sh->att_t1 = c < n ? (int)((c + 1) * (unsigned)base / n) : 0;
-            // short runs (a slot or two each, a warp per block of query vectors) go side by side
-            int t = sh->att_t0, k = 0, warps = 0;
-            bool small = true;
-            for (; k < (M == 1 ? 1 : MK_RUNS) && t < sh->att_t1 && (k == 0 || small); k++) {
-                MkRun &r = sh->runs[k];
-                mk_run_at(a, sh, t, sh->att_t1, r);
-                t += r.n;
-                warps += r.n_qblk;
-                small = small && r.n <= 4 && warps <= MK_CW;
-            }
-            sh->att_batch = small && t >= sh->att_t1 ? k : 0;
+            mk_runs<M, HD, WIDE>(a, sh);
             sh->bands[0].init(MK_QKV, a);
             sh->bands[1].init(MK_MLP, a);
             sh->heads.init(a, a.Hq);

@@ -735,3 +735,38 @@ def test_persistent_kernel_at_the_edges_of_its_shares(util, shape, lens):
         ln, pend = P.g.slot_state(s_)
         P.check_cache(s_, range(1, 4), ln - pend)
     P.close()
+
+
+@pytest.mark.parametrize("hd,n_kv,G,lens", [
+    # shares of five and six tiles (16 positions of a kv head) on 148 SMs: runs of one share side by side, two warps a run
+    (64, 16, 1, (760,)), (128, 16, 1, (900,)),
+    # of ten: three warps with twelve slots, two with eight; a share's runs have more tiles than the ring
+    (64, 16, 2, (1480,)), (128, 8, 4, (600, 700, 800, 900)), (64, 16, 2, (400, 1100)),
+    # of 34: a run goes round the ring more than once; of seventeen, four rows of four blocks of query vectors
+    (128, 16, 1, (5100,)), (64, 16, 2, (1300, 1290, 1280, 1310)), (64, 8, 8, (5100,)),
+])
+def test_persistent_kernel_long_runs(util, hd, n_kv, G, lens):
+    """Attention of the persistent kernel where a CTA's share of the cache is long, over imported prefixes: one to four
+    sequences, and the refresh passes of what they leave pending."""
+    dims = synth.model_dims(dict(n_layers=2, d_model=64, n_q_heads=n_kv * G, n_kv_heads=n_kv, head_dim=hd, d_ffn=128, vocab_text=96,
+                                 vocab_speech=64, rms_eps=1e-6, rope_base=10000.0), 1, 4, 0)
+    P = util.Pair(dims, synth.make_weights(dims, seed=3), len(lens), max(lens) + 16, 3, prefill_rows=64)
+    rng = np.random.default_rng(8)
+    for s_, n in enumerate(lens):
+        for layer in (1, 2):
+            k, v = (rng.standard_normal((n, n_kv * hd)).astype(np.float16) for _ in "kv")
+            P.g.import_kv(s_, layer, 0, torch.from_numpy(k).cuda(), torch.from_numpy(v).cuda())
+            kf, vf = k.astype(np.float64), v.astype(np.float64)
+            for p in range(n):
+                P.os[s_].set_kv(layer, p, kf[p], vf[p])
+        P.g.set_len(s_, n)
+        P.os[s_].set_len(n)
+    P.next_in = [int(t) for t in rng.integers(0, 160, size=len(lens))]
+    for g in range(6):
+        before = P.g.route_counts()
+        P.step([0 if g == 0 else 1] * len(lens), [0 if g == 0 else g - 1] * len(lens))
+        after = P.g.route_counts()
+        if g < 5 or len(lens) == 1:              # g = 5 is the refresh: three pending rows a sequence
+            assert after["mega"] > before["mega"] and after["tc"] == before["tc"] and after["gemv"] == before["gemv"]
+    assert P.stats["max_flush"] == 3
+    P.close()
