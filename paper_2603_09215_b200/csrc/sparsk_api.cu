@@ -1019,7 +1019,7 @@ bool build_mega(sparsk_ctx *c)
 bool use_mega(const sparsk_ctx *c, int n_rows)
 {
     return c->mega && c->mk_ok && c->mk_coop && n_rows >= 1 && n_rows <= c->mk_max_rows && (n_rows < MK_TC_ROWS || c->mk_tc_ok) &&
-           c->attn_tma_ok && c->n_sm <= MK_MAX_CTAS && mk_attn_fits(n_rows >= MK_TC_ROWS ? MK_MAX_ROWS : n_rows, c->dm.n_q_heads / c->dm.n_kv_heads) &&
+           c->attn_tma_ok && c->n_sm <= MK_MAX_CTAS &&
            (size_t)MK_MAX_ROWS * c->dm.n_kv_heads * (c->dm.max_seq_len / AT_TP + 1) * MK_MAX_CTAS < (1ull << 31);  // (32-bit shares)
 }
 

@@ -86,9 +86,6 @@ struct MkCells {
 // One warp's partial of a block of eight query vectors and its sums.
 template <int HD>
 __host__ __device__ constexpr int mk_cell_bytes() { return 8 * HD * 4 + 8 * 8; }
-// Shapes the phase can run: a warp per block of query vectors of a group.
-inline bool mk_attn_fits(int M, int G) { return (M * G + 7) / 8 <= MK_CW; }
-
 // The run that begins with tile t of the CTA's share, on its own: up to four warps per block of eight query vectors share it (as many as the
 // area has room for partials, and two slots at least each), every nsub-th slot each.
 template <int M, int HD, bool WIDE>
@@ -156,7 +153,8 @@ __device__ __forceinline__ void mk_meet(const MkArgs &a, const unsigned char *ce
     }
 }
 
-// The CTA's runs: side by side, or one after another (mk_runs); the partials of warps that share a run meet in the area.
+// The CTA's runs: side by side, or one after another (mk_runs); the partials of warps that share a run meet in the area.  More
+// than sixteen blocks have the run come by once for every sixteen.
 // (Blocks of sixteen, positions as columns, cost 450 bytes of spills, and a reload behind a grid barrier is a trip to the L2: flushes of
 // four rows of the 28-layer shape 96.6 us a layer, so 90.9.)
 template <int M, int HD, bool WIDE, int SLOTS>
@@ -170,7 +168,7 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
     // Nothing of a run is held in registers across its tiles: it is read from shared memory before and after.  The one behind it is
     // worked out beside it, in the last three places in turn (whoever is late may still read the one before).
     static_assert(MK_RUNS == 4, "places");
-    for (int at_run = 0;;) {
+    for (int at_run = 0, qb0 = 0;;) {  // qb0: first block of query vectors
         {
             const MkRun *r = &sh->runs[at_run];
             if (const int batch = sh->att_batch) {
@@ -179,16 +177,16 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
             } else if (threadIdx.x == (MK_CW - 1) * 32 && r->t + r->n < sh->att_t1) {
                 mk_run_alone<M, HD, WIDE>(a, sh, r->t + r->n, sh->runs[at_run == 3 ? 1 : at_run + 1]);
             }
-            const int nb = r->n_qblk, nsub = r->nsub, in_run = warp - r->warp0, sub = nb > 1 ? in_run / nb : in_run;
+            const int nb = min(MK_CW, r->n_qblk - qb0), nsub = r->nsub, in_run = warp - r->warp0, sub = nb > 1 ? in_run / nb : in_run;
             if (sub < nsub) {
-                const int qb = nb > 1 ? in_run - sub * nb : 0;
+                const int qb = qb0 + (nb > 1 ? in_run - sub * nb : 0);
                 AtItem item;
                 item.qb = qb; item.hk = r->hk; item.row0 = r->row0; item.nrows = r->nrows; item.pos0 = r->pos0; item.nq = r->nq;
                 MkTiles<HD, SLOTS> tiles{a, r, sh, ring, at, l, lane};
                 tiles.first = r->item0 + sub; tiles.nsub = nsub; tiles.tile0 = r->tile0 - 2 * r->item0;
                 tiles.new0 = r->pos0;
                 tiles.w_end = min(r->pos0 + (r->nrows == 1 ? 0 : (min(qb * 8 + 8, r->nq) - 1) / G) + 1, a.S);
-                tiles.arrivals = qb == 0 ? MK_CW - (nb - 1) : 1;
+                tiles.arrivals = qb == qb0 ? MK_CW - (nb - 1) : 1;
                 const int run_items = (r->n + 1) / 2, mine = nsub == 1 ? run_items : (run_items - sub + nsub - 1) / nsub;
                 tiles.n_tiles = 2 * mine - ((r->n & 1) && sub + nsub * (mine - 1) == run_items - 1 ? 1 : 0);
                 const MkCells<HD> out{a, r, area + (size_t)warp * mk_cell_bytes<HD>()};
@@ -207,8 +205,12 @@ __device__ __forceinline__ void mk_attention(const MkArgs &a, int l, unsigned ch
                 met = true;
             }
         }
-        if (batch || r->t + r->n >= sh->att_t1) break;
-        at_run = at_run == 3 ? 1 : at_run + 1;
+        if (batch) break;
+        if ((qb0 += MK_CW) >= r->n_qblk) {
+            if (r->t + r->n >= sh->att_t1) break;
+            qb0 = 0;
+            at_run = at_run == 3 ? 1 : at_run + 1;
+        }
         if (met) mk_consumer_sync();  // what comes next may use the area
     }
 }

@@ -70,9 +70,12 @@ __device__ __forceinline__ void mk_produce(const MkArgs &a, unsigned char *ring,
         rows(MK_QKV, L);
         if (!ok) break;
         MkRun r = sh->runs[0];
-        for (int t = sh->att_t0; ok && t < sh->att_t1;) {
-            if (t != sh->att_t0) mk_run_at(a, sh, t, sh->att_t1, r);
-            t += r.n;
+        for (int t = sh->att_t0, qb0 = 0; ok && t < sh->att_t1;) {
+            if (t != sh->att_t0 && qb0 == 0) mk_run_at(a, sh, t, sh->att_t1, r);
+            if ((qb0 += MK_CW) >= r.n_qblk) {  // (as often as it takes to have every block of query vectors see it)
+                t += r.n;
+                qb0 = 0;
+            }
             const int y0 = r.cache0;
             for (int i = 0; i < r.n; i += 2, idx++) {
                 if ((int)(idx % MK_PW) != p) continue;

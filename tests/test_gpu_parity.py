@@ -744,6 +744,8 @@ def test_persistent_kernel_at_the_edges_of_its_shares(util, shape, lens):
     (64, 16, 2, (1480,)), (128, 8, 4, (600, 700, 800, 900)), (64, 16, 2, (400, 1100)),
     # of 34: a run goes round the ring more than once; of seventeen, four rows of four blocks of query vectors
     (128, 16, 1, (5100,)), (64, 16, 2, (1300, 1290, 1280, 1310)), (64, 8, 8, (5100,)),
+    # more query vectors a group than a warp a block of eight takes in one go
+    (64, 1, 64, (3000,)), (64, 1, 72, (900, 2000)), (128, 1, 40, (12000,)),
 ])
 def test_persistent_kernel_long_runs(util, hd, n_kv, G, lens):
     """Attention of the persistent kernel where a CTA's share of the cache is long, over imported prefixes: one to four
