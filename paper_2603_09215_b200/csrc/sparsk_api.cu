@@ -1562,6 +1562,20 @@ extern "C" int sparsk_export_kv(sparsk_ctx *ctx, int32_t slot, int32_t layer, in
 }
 
 // --------------------------------------------------------------------------- prefill
+// Rows of the next pass when `left` prompt rows are to come and a pass takes up to `chunk`.  A block of few rows behind whole
+// ones costs a launch as much as a whole block, if its units need another wave: it is left for the next pass then, whose own launches
+// cut the inner dimension or go through the persistent kernel.  us a layer in one pass / in two: 257 rows 362 / 331, 288
+// rows 388 / 376, 320 rows 382 / 388 (28-layer shape; 40-layer shape 385 / 318, 383 / 363, 385 / 381); where the block finds
+// idle SMs (d_ffn 8,192: 32 pairs of units on 74) 257 rows 172 / 194, and 513 rows, another wave again, 253 / 235.
+constexpr int PREFILL_TAIL = 32;
+static int prefill_pass_rows(const sparsk_ctx *c, long left, int chunk)
+{
+    const int n = (int)std::min<long>(chunk, left), blocks = n / GM_MAX_N, tail = n % GM_MAX_N;
+    if (blocks == 0 || tail == 0 || tail > PREFILL_TAIL) return n;
+    const int pairs = std::max(1, c->n_sm / 2), units = div_up(c->dm.d_ffn, 2 * GM_BM);  // of gate/up, a block of rows
+    return div_up(units * (blocks + 1), pairs) > div_up(units * blocks, pairs) ? n - tail : n;
+}
+
 extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *slots, const int32_t *tokens,
                               const int32_t *offsets)
 {
@@ -1570,6 +1584,7 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
     if (n_seqs < 0 || n_seqs > d.max_seqs || (n_seqs && (!slots || !tokens || !offsets)))
         return fail(ctx, SPARSK_EINVAL, "prefill: bad arguments");
     std::vector<char> seen(d.max_seqs, 0);
+    long rows_left = 0;
     for (int i = 0; i < n_seqs; i++) {
         const int s = slots[i];
         if (s < 0 || s >= d.max_seqs || seen[s]) return fail(ctx, SPARSK_EINVAL, "prefill: slot %d invalid or repeated", s);
@@ -1578,6 +1593,7 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
         if (n < 0 || offsets[i] < 0) return fail(ctx, SPARSK_EINVAL, "prefill: offsets must not decrease");
         if (ctx->h_pend[s]) return fail(ctx, SPARSK_ESTATE, "prefill: slot %d has pending positions", s);
         if (ctx->h_len[s] + n > d.max_seq_len) return fail(ctx, SPARSK_ECAPACITY, "prefill: slot %d would hold %ld > %d positions", s, ctx->h_len[s] + n, d.max_seq_len);
+        rows_left += n;
     }
     // Passes of up to `chunk` rows, filled from the prompts in order: the end of one prompt, whole
     // short ones and the beginning of the next share a pass (each a group of its own), so that only
@@ -1595,8 +1611,10 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
             return launch(ctx, prompt_begin_kernel, dim3(rows), dim3(128), 0, in, pieces, first, last, tokens, r_slot, r_pos, r_g0,
                           r_gn, r_cnt, ctx->embed, ctx->h_up, d.d_model, d.vocab_text + d.vocab_speech, ctx->sd.counts + CNT_STATUS);
         };
-        while (i < n_seqs && n < chunk) {
-            const int s = slots[i], left = offsets[i + 1] - offsets[i] - done, take = std::min(chunk - n, left);
+        const int pass = prefill_pass_rows(ctx, rows_left, chunk);
+        rows_left -= pass;
+        while (i < n_seqs && n < pass) {
+            const int s = slots[i], left = offsets[i + 1] - offsets[i] - done, take = std::min(pass - n, left);
             if (take > 0) {
                 if (k == PP_MAX) CU(begin(false));
                 const int pos0 = ctx->h_len[s];

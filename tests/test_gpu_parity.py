@@ -772,3 +772,20 @@ def test_persistent_kernel_long_runs(util, hd, n_kv, G, lens):
             assert after["mega"] > before["mega"] and after["tc"] == before["tc"] and after["gemv"] == before["gemv"]
     assert P.stats["max_flush"] == 3
     P.close()
+
+
+@pytest.mark.parametrize("lens,passes", [((256,), 1), ((257,), 2), ((288,), 2), ((289,), 1), ((230, 40), 2), ((300, 229), 1), ((512, 100, 200), 1),
+                                         ((1030,), 2)])
+def test_prompt_rows_behind_whole_blocks(util, lens, passes):
+    """The library's own choice of rows a pass: few rows behind whole blocks of 256 go by themselves where their block would need
+    another wave of gate/up units (38 pairs of them on 74 pairs of SMs), the next prompt's rows with them."""
+    dims = synth.model_dims(dict(MICRO256, n_layers=2, d_ffn=9728), 1, 3, 0)
+    P = util.Pair(dims, synth.make_weights(dims, seed=9), len(lens), max(lens) + 4, 2)
+    rng = np.random.default_rng(6)
+    prompts = [rng.integers(0, 400, size=n + 1).astype(np.int32) for n in lens]
+    P.prefill(prompts)
+    assert sum(P.g.route_counts().values()) == 2 * passes
+    for s_, n in enumerate(lens):
+        P.check_cache(s_, (1, 2), n)
+    P.step([0] * len(lens), [0] * len(lens))
+    P.close()
