@@ -194,12 +194,15 @@ int sparsk_set_debug(sparsk_ctx *ctx, float *exit_hidden /*device or NULL*/,
  * four rows as one persistent kernel per layer range; default 1), "mega_max_rows" (1..4: the
  * largest pass that kernel takes; default 4. Passes of three and four rows use its tensor-core
  * inner loop, which needs d_model, d_ffn and n_heads * head_dim to be multiples of 64 and d_model
- * to be at most 4,352; other shapes stop at two rows), "gemm_kb" (1: one 64-element block of the inner
+ * to be at most 4,352; other shapes stop at two rows.  Caches of 2^31 rows (slots * n_kv_heads *
+ * max_seq_len) and prefixes of which 768 * n_kv_heads * max_seq_len / 16 reaches 2^31 do not go through it at all),
+ * "gemm_kb" (1: one 64-element block of the inner
  * dimension per TMA copy instead of two; 0 = automatic), "attn_split" (positions
- * per KV split), "attn_dynamic" (0/1: the attention kernel's warps draw their work items from a
+ * per KV split of the attention launches; the persistent kernel cuts its cache tiles evenly over the SMs,
+ * whatever this says), "attn_dynamic" (0/1: the attention kernel's warps draw their work items from a
  * counter as they finish instead of taking every n-th one; default 1), "attn_ctas" (CTAs of that
  * kernel; 0 = as many as fit the SMs), "attn_tma" (0/1: its K/V tiles arrive as TMA boxes with the
- * 128-byte swizzle instead of per-lane 16-byte copies; default 1), "attn_stages" (2 or 3 tiles per
+ * 128-byte swizzle instead of per-lane 16-byte copies; default 1; the persistent kernel's always do), "attn_stages" (2 or 3 tiles per
  * warp's ring), "pdl" (0/1, programmatic dependent launch between the kernels of a step; default 1),
  * "gemv_ks" / "gemv_r" (override the GEMV team width / rows per group; 0 = automatic),
  * "trim_last_layer" (0/1/2: in a full-depth step, pending rows leave layer L after its K/V

@@ -952,10 +952,10 @@ bool build_mega(sparsk_ctx *c)
     c->mk_cols32 = mk_cols(d.d_ffn, d.d_model, 2 * MK_BOX_ROWS, c->n_sm);
     // The swizzled three-dimensional views need inner dimensions that are whole 64-element blocks, and
     // the RMSNorm of the form leaves whole residual rows in the activation area: 4,352 numbers.
-    // Passes of three and four wider rows take the tcgen05 path, which is the faster one there in
-    // any case.  us a layer at three / four rows: 4,352 numbers (MLP 11,776) 111 / 111 here and 117
-    // there; a form that normalised a window at a time took 117 / 165 at 4,416, 142 / 204 at 5,120
-    // (MLP 13,824) and 165 / 237 at 5,888 (15,360) where the tcgen05 path takes 113, 134 and 155.
+    // Passes of three and four wider rows take the tcgen05 path.  us a layer after 1,000 positions at three / four rows, here
+    // and there: 3,584 numbers (MLP 18,944) 106 / 107 and 119 / 120, 4,096 (14,336) 109 / 109 and 117 / 118, 4,352 (11,776)
+    // 108 / 109 and 116 / 116, 4,352 (30,720) 179 / 180 and 189 / 189.  (Wider rows normalised a window at a time, in an earlier
+    // form of this kernel: 142 / 204 at 5,120 where the tcgen05 path takes 134.)
     c->mk_tc_ok = d.d_model % 64 == 0 && d.d_ffn % 64 == 0 && qd % 64 == 0 && div_up(d.d_model, MK_BOX_COLS) <= MK_TC_STEPS;
     auto enc_sw = [&](CUtensorMap *m, const void *base, size_t rows, size_t cols) {
         const cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64)};
