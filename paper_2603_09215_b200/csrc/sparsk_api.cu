@@ -1564,16 +1564,18 @@ extern "C" int sparsk_export_kv(sparsk_ctx *ctx, int32_t slot, int32_t layer, in
 // --------------------------------------------------------------------------- prefill
 // Rows of the next pass when `left` prompt rows are to come and a pass takes up to `chunk`.  A block of few rows behind whole
 // ones costs a launch as much as a whole block, if its units need another wave: it is left for the next pass then, whose own launches
-// cut the inner dimension or go through the persistent kernel.  us a layer in one pass / in two: 257 rows 362 / 331, 288
-// rows 388 / 376, 320 rows 382 / 388 (28-layer shape; 40-layer shape 385 / 318, 383 / 363, 385 / 381); where the block finds
-// idle SMs (d_ffn 8,192: 32 pairs of units on 74) 257 rows 172 / 194, and 513 rows, another wave again, 253 / 235.
+// cut the inner dimension or go through the persistent kernel.  us a layer in one pass / in two: 257 rows 359 / 319, 288
+// rows 384 / 356, 320 rows 396 / 380, 400 rows 399 / 454 (28-layer shape; 40-layer shape 372 / 318, 374 / 347, 388 / 376, 394 / 442).
+// More than 32 rows do so only if their block fills two fifths of a wave and more (those two shapes all of one and 34 of 74 pairs
+// of SMs; d_ffn 8,192 at three blocks 22: 517 rows 254 / 262); where the block finds idle SMs (d_ffn 8,192 at two) 257 rows take 168 / 194.
 constexpr int PREFILL_TAIL = 32;
 static int prefill_pass_rows(const sparsk_ctx *c, long left, int chunk)
 {
     const int n = (int)std::min<long>(chunk, left), blocks = n / GM_MAX_N, tail = n % GM_MAX_N;
-    if (blocks == 0 || tail == 0 || tail > PREFILL_TAIL) return n;
+    if (blocks == 0) return n;
     const int pairs = std::max(1, c->n_sm / 2), units = div_up(c->dm.d_ffn, 2 * GM_BM);  // of gate/up, a block of rows
-    return div_up(units * (blocks + 1), pairs) > div_up(units * blocks, pairs) ? n - tail : n;
+    const int beyond = units * (blocks + 1) - div_up(units * blocks, pairs) * pairs;     // those of the last block that the waves before it have no room for
+    return beyond > 0 && tail <= (beyond * 5 >= pairs * 2 ? 2 : 1) * PREFILL_TAIL ? n - tail : n;
 }
 
 extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *slots, const int32_t *tokens,
