@@ -376,6 +376,9 @@ int pick_r(const sparsk_ctx *c, int n_rows, bool paired)
     return 2;
 }
 
+struct PromptGroup {
+    int rows, len;  // of a prompt pass's group: rows, and positions the last of them attends to
+};
 struct RowSet {
     const int *slot, *pos, *grp_row0, *grp_nrows, *n_groups, *n_rows_dev;
     int n_rows;     // host count (sizes the launches)
@@ -386,6 +389,8 @@ struct RowSet {
     const float *q; // the rows' queries if they are not the context's query buffer (NULL: they are)
     long sum_len;   // total of the groups' prefix lengths (host; 0: unknown)
     bool rows_late; // the arrays are written by a kernel that may still run when the pass's kernels start
+    const PromptGroup *prompt;      // prompt passes: the groups (host), else NULL
+    mutable int splits_tc, splits_warp;  // prompt passes: even_splits' answers for the two attention kernels, once asked (0 before)
 };
 
 cudaError_t run_qkv(sparsk_ctx *c, int layer, const float *h, const RowSet &rs)
@@ -487,6 +492,42 @@ cudaError_t run_head(sparsk_ctx *c, int layer, const float *h, int list, int n_r
 }
 
 
+// Splits of a prompt pass whose groups are uneven.  The plans below take every group for the largest, in rows and in positions: where a few
+// rows behind a long prefix share a pass with many rows of a short one, that fills the machine on paper with one split, and one
+// worker is left with the whole prefix.  Here a plan's time is estimated, in positions of one item: whole rounds of its long items (or
+// the mean load, where that is more), `setup` for each round of items, `merge` for each split; `now` splits stay unless more of them
+// are better by a sixth.  us a layer, passes of 256 rows without this / one pass without / with it: two rows behind 60,000
+// positions and 700 without, 16 heads and kv heads of 64 739 / 2,243 / 334, 32 and 8 of 64 1,872 / 2,373 / 463; eight rows behind
+// 60,000 and three times 300, 28 and 4 heads of 128 1,104 / 1,842 / 946.
+int even_splits(const RowSet &rs, int q_min, int q_max, int G, int Hkv, int block, int workers, int tile, double setup, double merge,
+                int now, int max_splits)
+{
+    auto time = [&](int n) {
+        const int len = div_up(div_up(rs.max_len, n), tile) * tile;
+        double full = 0, items = 0, work = 0;
+        for (int g = 0; g < rs.n_groups_h; g++) {
+            const int q = rs.prompt[g].rows * G;
+            if (q < q_min || q > q_max) continue;
+            const double blocks = (double)div_up(q, block) * Hkv;
+            full += blocks * ((rs.prompt[g].len + len / 2) / len);
+            items += blocks * div_up(rs.prompt[g].len, len);
+            work += blocks * rs.prompt[g].len;
+        }
+        return std::max(std::ceil(full / workers) * len, work / workers) + std::ceil(items / workers) * setup + n * merge;
+    };
+    const double at_first = time(now);
+    double best = at_first;
+    int n_best = now;
+    for (int n = now + 1; n <= max_splits && div_up(rs.max_len, n) >= 8 * tile; n++) {
+        const double t = time(n);
+        if (t < best) {
+            best = t;
+            n_best = n;
+        }
+    }
+    return best < at_first * 5 / 6 ? n_best : now;
+}
+
 cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
 {
     const sparsk_dims &d = c->dm;
@@ -521,6 +562,17 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
     if (pl.n_splits > max_splits) {
         pl.split_len = div_up(div_up(rs.max_len, max_splits), AT_TP) * AT_TP;
         pl.n_splits = div_up(rs.max_len, pl.split_len);
+    }
+    // bytes of a split's partials, written and read, in us
+    const double merge_us = (double)rs.n_rows * d.n_q_heads * d.head_dim * 8 / 5e6;
+    if (rs.prompt && c->attn_split <= 0 && (!blocks_tc || n_small > 0)) {
+        if (!rs.splits_warp)  // (16 positions are 0.5 us, an item's set-up four tiles)
+            rs.splits_warp = even_splits(rs, 0, blocks_tc ? c->attn_tc_min_q - 1 : 1 << 30, G, d.n_kv_heads, 16, warp_ctas * AW_WARPS, AT_TP,
+                                         4 * AT_TP, merge_us * 32, pl.n_splits, max_splits);
+        if (rs.splits_warp > pl.n_splits) {
+            pl.split_len = div_up(div_up(rs.max_len, rs.splits_warp), AT_TP) * AT_TP;
+            pl.n_splits = div_up(rs.max_len, pl.split_len);
+        }
     }
     if (blocks_tc) {
         // Groups with many query vectors per kv head go to the tcgen05 kernel (one CTA per SM, tiles
@@ -559,6 +611,12 @@ cudaError_t run_attn(sparsk_ctx *c, int layer, const RowSet &rs)
         }
         if (c->attn_split > 0) s_tc = pl.n_splits;
         s_tc = std::min(s_tc, max_splits);
+        if (rs.prompt && c->attn_split <= 0) {  // (64 positions are 0.4 us, a set-up four tiles)
+            if (!rs.splits_tc)
+                rs.splits_tc = even_splits(rs, c->attn_tc_min_q, 1 << 30, G, d.n_kv_heads, TA_QB, c->n_sm, TA_NT, 4 * TA_NT, merge_us * 160, s_tc,
+                                           max_splits);
+            s_tc = rs.splits_tc;
+        }
         const int mult = n_small > 0 ? std::max(1, std::min(max_splits / s_tc, div_up(pl.n_splits, s_tc))) : 1;
         const int small_len = div_up(div_up(rs.max_len, s_tc * mult), TA_NT) * TA_NT;
         pl.split_len = small_len;
@@ -1604,7 +1662,9 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
     int *const r_slot = ctx->pf_rows, *const r_pos = r_slot + ctx->cap_rows, *const r_g0 = r_pos + ctx->cap_rows,
               *const r_gn = r_g0 + d.max_seqs, *const r_cnt = r_gn + d.max_seqs;
     PromptPieces in;
+    std::vector<PromptGroup> groups;  // of a pass
     for (int i = 0, done = 0; i < n_seqs;) {
+        groups.clear();
         int n = 0, ng = 0, k = 0, max_grp = 1, max_len = 0, n_big = 0;  // rows, groups (k of them in `in`) of the pass
         long sum_len = 0;
         auto begin = [&](bool last) {  // the k pieces in hand
@@ -1625,6 +1685,7 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
                 in.pos[k] = pos0;
                 in.token[k] = offsets[i] + done;
                 in.row0[++k] = n + take;
+                groups.push_back({take, pos0 + take});
                 ng++;
                 max_grp = std::max(max_grp, take);
                 max_len = std::max(max_len, pos0 + take);
@@ -1643,6 +1704,7 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
         CU(begin(true));
         RowSet rs{r_slot, r_pos, r_g0, r_gn, r_cnt, r_cnt + 1, n, ng, max_grp, max_len, n_big};
         rs.sum_len = sum_len;
+        rs.prompt = groups.data();
         CU(run_layers(ctx, 1, d.n_layers, ctx->h_up, rs));
         CU(launch(ctx, prefill_len_kernel, dim3((ng + 127) / 128), dim3(128), 0, ctx->kv_len, (const int *)r_slot, (const int *)r_pos,
                   (const int *)r_g0, (const int *)r_gn, ng));

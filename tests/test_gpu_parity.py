@@ -789,3 +789,28 @@ def test_prompt_rows_behind_whole_blocks(util, lens, passes):
         P.check_cache(s_, (1, 2), n)
     P.step([0] * len(lens), [0] * len(lens))
     P.close()
+
+
+@pytest.mark.parametrize("hd,G,short,n,passes", [(64, 2, 2, 4000, 1), (64, 2, 40, 4000, 1), (128, 2, 2, 4000, 1), (128, 2, 40, 4000, 1), (128, 8, 2, 4000, 1),
+                                                 (128, 8, 40, 4000, 1)])
+def test_few_prompt_rows_behind_a_long_prefix(util, hd, G, short, n, passes):
+    """A prompt pass whose groups are uneven (few rows behind n positions beside many rows of a new prompt) takes more splits
+    than the largest group alone would have, in either attention kernel and in both at once."""
+    dims = synth.model_dims(dict(n_layers=2, d_model=64, n_q_heads=8 * G, n_kv_heads=8, head_dim=hd, d_ffn=128, vocab_text=96,
+                                 vocab_speech=64, rms_eps=1e-6, rope_base=10000.0), 1, 4, 0)
+    rng = np.random.default_rng(12)
+    P = util.Pair(dims, synth.make_weights(dims, seed=3), 2, n + 64, 3)
+    for layer in (1, 2):
+        k, v = (rng.standard_normal((n, 8 * hd)).astype(np.float16) for _ in "kv")
+        P.g.import_kv(0, layer, 0, torch.from_numpy(k).cuda(), torch.from_numpy(v).cuda())
+        kf, vf = k.astype(np.float64), v.astype(np.float64)
+        for p in range(n):
+            P.os[0].set_kv(layer, p, kf[p], vf[p])
+    P.g.set_len(0, n)
+    P.os[0].set_len(n)
+    P.prefill([rng.integers(0, 160, size=m + 1).astype(np.int32) for m in (short, 600)])
+    assert sum(P.g.route_counts().values()) == 2 * passes
+    P.check_cache(0, (1, 2), n + short)
+    P.check_cache(1, (1, 2), 600)
+    P.step([0, 0], [0, 0])
+    P.close()
