@@ -1636,6 +1636,24 @@ static int prefill_pass_rows(const sparsk_ctx *c, long left, int chunk)
     return beyond > 0 && tail <= (beyond * 5 >= pairs * 2 ? 2 : 1) * PREFILL_TAIL ? n - tail : n;
 }
 
+// Few rows behind a long prefix beside a prompt's many rows: the partials have room for fewer splits the more rows a pass has
+// (part_rows_of), and where 256 rows' 32 splits would make the longest item this many positions shorter, the pass stays at 256.  us a
+// layer, two rows behind 60,000 positions and 700 without, 28-layer shape: 1,133 in one pass, 754 with the first 256 rows by themselves; behind 30,000 884 and 748,
+// behind 15,000 756 and 722.
+constexpr int PREFILL_LONG_ITEM = 1300;
+static bool wants_all_splits(const sparsk_ctx *c, const std::vector<PromptGroup> &groups, int n)
+{
+    const sparsk_dims &d = c->dm;
+    if (n <= GM_MAX_N || !c->attn_tc || !c->tc_ok || d.head_dim != TA_HD || c->attn_split > 0) return false;
+    int few_len = 0, many = 0;
+    for (const PromptGroup &g : groups) {
+        if (g.rows * (d.n_q_heads / d.n_kv_heads) < c->attn_tc_min_q) few_len = std::max(few_len, g.len);
+        else many = 1;
+    }
+    const int splits = (int)std::min<size_t>(AT_MAX_SPLITS, std::max<size_t>(1, part_rows_of(&d) / n));
+    return many && div_up(few_len, splits) - div_up(few_len, AT_MAX_SPLITS) > PREFILL_LONG_ITEM;
+}
+
 extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *slots, const int32_t *tokens,
                               const int32_t *offsets)
 {
@@ -1664,7 +1682,14 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
     PromptPieces in;
     std::vector<PromptGroup> groups;  // of a pass
     for (int i = 0, done = 0; i < n_seqs;) {
-        groups.clear();
+        auto next_groups = [&](int rows) {
+            groups.clear();
+            for (int j = i, had = done; rows > 0 && j < n_seqs; j++, had = 0) {
+                const int take = std::min(rows, offsets[j + 1] - offsets[j] - had);
+                if (take > 0) groups.push_back({take, ctx->h_len[slots[j]] + take});
+                rows -= take;
+            }
+        };
         int n = 0, ng = 0, k = 0, max_grp = 1, max_len = 0, n_big = 0;  // rows, groups (k of them in `in`) of the pass
         long sum_len = 0;
         auto begin = [&](bool last) {  // the k pieces in hand
@@ -1673,7 +1698,9 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
             return launch(ctx, prompt_begin_kernel, dim3(rows), dim3(128), 0, in, pieces, first, last, tokens, r_slot, r_pos, r_g0,
                           r_gn, r_cnt, ctx->embed, ctx->h_up, d.d_model, d.vocab_text + d.vocab_speech, ctx->sd.counts + CNT_STATUS);
         };
-        const int pass = prefill_pass_rows(ctx, rows_left, chunk);
+        int pass = prefill_pass_rows(ctx, rows_left, chunk);
+        next_groups(pass);
+        if (wants_all_splits(ctx, groups, pass)) next_groups(pass = GM_MAX_N);
         rows_left -= pass;
         while (i < n_seqs && n < pass) {
             const int s = slots[i], left = offsets[i + 1] - offsets[i] - done, take = std::min(pass - n, left);
@@ -1685,7 +1712,6 @@ extern "C" int sparsk_prefill(sparsk_ctx *ctx, int32_t n_seqs, const int32_t *sl
                 in.pos[k] = pos0;
                 in.token[k] = offsets[i] + done;
                 in.row0[++k] = n + take;
-                groups.push_back({take, pos0 + take});
                 ng++;
                 max_grp = std::max(max_grp, take);
                 max_len = std::max(max_len, pos0 + take);

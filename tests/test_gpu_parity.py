@@ -792,10 +792,11 @@ def test_prompt_rows_behind_whole_blocks(util, lens, passes):
 
 
 @pytest.mark.parametrize("hd,G,short,n,passes", [(64, 2, 2, 4000, 1), (64, 2, 40, 4000, 1), (128, 2, 2, 4000, 1), (128, 2, 40, 4000, 1), (128, 8, 2, 4000, 1),
-                                                 (128, 8, 40, 4000, 1)])
+                                                 (128, 8, 40, 4000, 1), (128, 2, 2, 30000, 2)])
 def test_few_prompt_rows_behind_a_long_prefix(util, hd, G, short, n, passes):
     """A prompt pass whose groups are uneven (few rows behind n positions beside many rows of a new prompt) takes more splits
-    than the largest group alone would have, in either attention kernel and in both at once."""
+    than the largest group alone would have, in either attention kernel and in both at once; where a pass of all rows has no
+    room for enough of them it has 256 of them."""
     dims = synth.model_dims(dict(n_layers=2, d_model=64, n_q_heads=8 * G, n_kv_heads=8, head_dim=hd, d_ffn=128, vocab_text=96,
                                  vocab_speech=64, rms_eps=1e-6, rope_base=10000.0), 1, 4, 0)
     rng = np.random.default_rng(12)
