@@ -1632,14 +1632,15 @@ static int prefill_pass_rows(const sparsk_ctx *c, long left, int chunk)
     const int n = (int)std::min<long>(chunk, left), blocks = n / GM_MAX_N, tail = n % GM_MAX_N;
     if (blocks == 0) return n;
     const int pairs = std::max(1, c->n_sm / 2), units = div_up(c->dm.d_ffn, 2 * GM_BM);  // of gate/up, a block of rows
-    const int beyond = units * (blocks + 1) - div_up(units * blocks, pairs) * pairs;     // those of the last block that the waves before it have no room for
+    // those of the last block for which the waves of the blocks before it have no room
+    const int beyond = units * (blocks + 1) - div_up(units * blocks, pairs) * pairs;
     return beyond > 0 && tail <= (beyond * 5 >= pairs * 2 ? 2 : 1) * PREFILL_TAIL ? n - tail : n;
 }
 
 // Few rows behind a long prefix beside a prompt's many rows: the partials have room for fewer splits the more rows a pass has
 // (part_rows_of), and where 256 rows' 32 splits would make the longest item this many positions shorter, the pass stays at 256.  us a
-// layer, two rows behind 60,000 positions and 700 without, 28-layer shape: 1,133 in one pass, 754 with the first 256 rows by themselves; behind 30,000 884 and 748,
-// behind 15,000 756 and 722.
+// layer, two rows behind 60,000 positions and 700 without, 28-layer shape: 1,133 in one pass, 748 with the first 256 rows by
+// themselves; behind 30,000 884 and 693, behind 15,000 756 and 717 (40-layer shape 694 and 735).
 constexpr int PREFILL_LONG_ITEM = 1300;
 static bool wants_all_splits(const sparsk_ctx *c, const std::vector<PromptGroup> &groups, int n)
 {

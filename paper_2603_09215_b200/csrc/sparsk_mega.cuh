@@ -115,7 +115,8 @@ struct MkCols {
     int unit, box;
     bool wide;
 };
-constexpr int MK_NARROW_STEPS = (mk_area_bytes(1, false) - MK_CBOX_COLS * 4 - 4096) / (MK_BOX_COLS * 4);  // of one row, beside the CTA's columns and mk_sums_bytes(1)
+// k-steps of one row that fit beside the CTA's columns and mk_sums_bytes(1)
+constexpr int MK_NARROW_STEPS = (mk_area_bytes(1, false) - MK_CBOX_COLS * 4 - 4096) / (MK_BOX_COLS * 4);
 inline MkCols mk_cols(int F, int d, int unit, int n_cta)
 {
     const int n = (F + unit - 1) / unit, per = (n + n_cta - 1) / n_cta;

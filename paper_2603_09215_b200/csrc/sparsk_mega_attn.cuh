@@ -86,6 +86,7 @@ struct MkCells {
 // One warp's partial of a block of eight query vectors and its sums.
 template <int HD>
 __host__ __device__ constexpr int mk_cell_bytes() { return 8 * HD * 4 + 8 * 8; }
+
 // The run that begins with tile t of the CTA's share, on its own: up to four warps per block of eight query vectors share it (as many as the
 // area has room for partials, and two slots at least each), every nsub-th slot each.
 template <int M, int HD, bool WIDE>

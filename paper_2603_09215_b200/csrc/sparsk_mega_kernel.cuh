@@ -173,6 +173,7 @@ __device__ __forceinline__ void mk_mlp(const MkArgs &a, int l, const bf16 *gain,
                          mk_act_window(M, true, mk_sums_bytes(M)), nullptr, gain, gains, nullptr, 0, ring, sh, at);
     } else {
         constexpr int OWN = M * MK_CBOX_COLS * 4 + mk_sums_bytes(M);
+        static_assert(mk_act_window(M, false, OWN) >= MK_NARROW_STEPS, "the narrow form's rows are whole");
         float *u = reinterpret_cast<float *>(area + mk_area_bytes(M, false) - OWN), *sums = u + M * MK_CBOX_COLS;
         for (int i = threadIdx.x; i < M * MK_CBOX_COLS; i += MK_CW * 32) u[i] = 0.f;
         mk_rows<M, false>(MK_MLP, a, l, reinterpret_cast<float *>(area), sums, mk_act_window(M, false, OWN), nullptr, gain, gains, u, MK_CBOX_COLS, ring, sh, at);

@@ -791,8 +791,10 @@ def test_prompt_rows_behind_whole_blocks(util, lens, passes):
     P.close()
 
 
-@pytest.mark.parametrize("hd,G,short,n,passes", [(64, 2, 2, 4000, 1), (64, 2, 40, 4000, 1), (128, 2, 2, 4000, 1), (128, 2, 40, 4000, 1), (128, 8, 2, 4000, 1),
-                                                 (128, 8, 40, 4000, 1), (128, 2, 2, 30000, 2)])
+@pytest.mark.parametrize("hd,G,short,n,passes", [
+    (64, 2, 2, 4000, 1), (64, 2, 40, 4000, 1), (128, 2, 2, 4000, 1), (128, 2, 40, 4000, 1), (128, 8, 2, 4000, 1), (128, 8, 40, 4000, 1),
+    (128, 2, 2, 30000, 2),
+])
 def test_few_prompt_rows_behind_a_long_prefix(util, hd, G, short, n, passes):
     """A prompt pass whose groups are uneven (few rows behind n positions beside many rows of a new prompt) takes more splits
     than the largest group alone would have, in either attention kernel and in both at once; where a pass of all rows has no
